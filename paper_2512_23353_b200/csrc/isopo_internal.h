@@ -181,13 +181,13 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
                                        const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout* L,
                                        void* const* G, const StoreFmt* fmt, int32_t* info, cudaStream_t st);
 // k_is_zero: the caller has already cleared K on this stream.  kpart != NULL (deterministic mode): every CTA
-// stores its partial upper triangle there ([kNtkMaxPartials][B * B] floats) and a second kernel sums them in order.
+// stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and a second kernel sums them in order.
 constexpr int kNtkMaxPartials = 160;
 isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_is_zero, float* kpart, const StoreFmt& fmt,
                       int32_t* info, cudaStream_t st);
 bool deterministic_mode();
-// K[i][j] = K[j][i] for j < i (the K kernels fill the upper triangle)
-isopo_status mirror_upper(float* K, int B, cudaStream_t st, const float* kdiag = nullptr);
+// K[i][j] = K[j][i] for j < i (the Gram kernels fill the upper triangle)
+isopo_status mirror_upper(float* K, int B, cudaStream_t st);
 isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out, int B, const float* coeffs, float* dW,
                           float beta, const WsTag* tag_dev, const WsTag& tag, const StoreFmt& fmt, int32_t* info,
                           cudaStream_t st);

@@ -6,7 +6,7 @@
 // (four per piece, so a CTA walks memory front to back) through a TMA ring, and uses every box as BOTH tcgen05 operands (K-major): rows 0..127 against all rows,
 // then rows 128..255 against rows 128..255 (the lower-left block is the mirror of the upper-right).
 // The float32 accumulators stay in tensor memory for the whole slab and are added into K once, with
-// reductions across CTAs by float atomics; a last tiny kernel mirrors the upper triangle.
+// reductions across CTAs by float atomics; a last tiny kernel mirrors the triangle.
 // For B <= 128 a box holds only the rows that exist (32, 64 or 128 >= B) but spans 8, 4 or 2 pieces, so
 // that every TMA copy still moves 32 KB (small boxes cost a fixed ~100 clocks each) and the stage is
 // again 256 rows: rows 0..127 and rows 128..255 each go through ONE 128 x 128 MMA per 16 elements,
@@ -130,7 +130,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
     } else {
       const int q = warp & 3;
       const int r = q * 32 + lane;
-      // every (CTA, entry of the upper triangle) is produced by exactly one thread, once
+      // every (CTA, entry of the lower triangle) is produced by exactly one thread, once.  Entry (r, c), c >= r, goes to
+      // K[c][r]: the 32 lanes of a warp own consecutive r, so one instruction adds 128 contiguous bytes.  (Adding to
+      // K[r][c] instead touched 32 rows per instruction: 89 us instead of 31 us for the whole pass at 256 sequences and
+      // a 128 x 896 layer, whose 59 MB stay in the L2.)
       float* const mine = p.kpart ? p.kpart + (size_t)blockIdx.x * p.B * p.B : nullptr;
       auto add_to_k = [&](size_t idx, float v) {
         if (mine) mine[idx] = v; else atomicAdd(&p.K[idx], v);
@@ -159,8 +162,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
               for (int e = 0; e < 32; ++e) {
                 const int c = c0 + e;
                 if (c >= r + (kE4m3 ? 1 : 0) && c < p.B &&
-                    ISOPO_IN_RANGE((long long)r * p.B + c, (long long)p.B * p.B, p.info, kIdNtk))
-                  add_to_k((size_t)r * p.B + c, unscale(r, c, __uint_as_float(v[e])));
+                    ISOPO_IN_RANGE((long long)c * p.B + r, (long long)p.B * p.B, p.info, kIdNtk))
+                  add_to_k((size_t)c * p.B + r, unscale(r, c, __uint_as_float(v[e])));
               }
             }
           }
@@ -175,8 +178,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
               for (int e = 0; e < 32; ++e) {
                 const int c = 128 + c0 + e;
                 if (c >= rr + (kE4m3 ? 1 : 0) && c < p.B &&
-                    ISOPO_IN_RANGE((long long)rr * p.B + c, (long long)p.B * p.B, p.info, kIdNtk))
-                  add_to_k((size_t)rr * p.B + c, unscale(rr, c, __uint_as_float(v[e])));
+                    ISOPO_IN_RANGE((long long)c * p.B + rr, (long long)p.B * p.B, p.info, kIdNtk))
+                  add_to_k((size_t)c * p.B + rr, unscale(rr, c, __uint_as_float(v[e])));
               }
             }
           }
@@ -204,11 +207,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
           if (ok) {
             for (int idx = r; idx < (ncol << lr); idx += 128) {
               const int sq = idx & (rows - 1), c = idx >> lr;
-              if (c < sq + (kE4m3 ? 1 : 0) || sq >= p.B) continue;  // upper triangle of the sequences that exist
+              if (c < sq + (kE4m3 ? 1 : 0) || sq >= p.B) continue;  // one triangle of the sequences that exist
               float sum = 0.f;
               for (int h = 0; h < ngroups; ++h) sum += red[(((h << lr) + c) << lr) + sq];
-              if (ISOPO_IN_RANGE((long long)sq * p.B + c, (long long)p.B * p.B, p.info, kIdNtk))
-                add_to_k((size_t)sq * p.B + c, unscale(sq, c, sum));
+              if (ISOPO_IN_RANGE((long long)c * p.B + sq, (long long)p.B * p.B, p.info, kIdNtk))
+                add_to_k((size_t)c * p.B + sq, unscale(sq, c, sum));
             }
           }
         }
@@ -222,14 +225,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
   if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
 }
 
-// Deterministic mode: K[i][j] = K[j][i] = sum over the CTAs, in CTA order, of their partial entry (i, j), i <= j.
-// One thread per entry of the upper triangle (its reads run along a row of every partial matrix), which also
+// Deterministic mode: K[i][j] = K[j][i] = sum over the CTAs, in CTA order, of their partial entry (i, j), i >= j.
+// One thread per entry of the lower triangle (its reads run along a row of every partial matrix), which also
 // writes the mirrored entry.
 __global__ void k_ntk_reduce(const float* __restrict__ kpart, int n_ctas, int B, float* __restrict__ K) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
   const int i = e / B, j = e % B;
-  if (j < i) return;
+  if (j > i) return;
   const size_t stride = (size_t)B * B;
   float s = 0.f;
   int c = 0;
@@ -245,12 +248,14 @@ __global__ void k_ntk_reduce(const float* __restrict__ kpart, int n_ctas, int B,
   K[(size_t)j * B + i] = s;
 }
 
+// Completes the triangle a K kernel left out (kFromLower: it filled i >= j, else i <= j).
 // kdiag != NULL (split store): the diagonal comes from the gradient GEMM's float32 sums of squares
-__global__ void k_mirror_upper(float* __restrict__ K, int B, const float* __restrict__ kdiag) {
+template <bool kFromLower>
+__global__ void k_mirror(float* __restrict__ K, int B, const float* __restrict__ kdiag) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
   const int i = e / B, j = e % B;
-  if (j < i) K[e] = K[(size_t)j * B + i];
+  if (kFromLower ? j > i : j < i) K[e] = K[(size_t)j * B + i];
   else if (j == i && kdiag) K[e] = kdiag[i];
 }
 
@@ -404,7 +409,12 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
     kernel<<<grid, kThreads, kSmemBytes, st>>>(mapG, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
-  if (!kpart) return mirror_upper(K, B, st, fmt.split ? fmt.kdiag : nullptr);
+  if (!kpart) {
+    LaunchScope scope(kIdMirror, st);
+    k_mirror<true><<<(B * B + 255) / 256, 256, 0, st>>>(K, B, fmt.split ? fmt.kdiag : nullptr);
+    ISOPO_CUDA_TRY(cudaGetLastError());
+    return ISOPO_OK;
+  }
   // CTAs whose slab of the contraction is empty wrote nothing: sum only those that had work
   const long long per = (p.nkb + grid - 1) / grid;
   const int n_active = (int)((p.nkb + per - 1) / per);
@@ -416,10 +426,10 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
   return ISOPO_OK;
 }
 
-isopo_status mirror_upper(float* K, int B, cudaStream_t st, const float* kdiag) {
+isopo_status mirror_upper(float* K, int B, cudaStream_t st) {
   {
     LaunchScope scope(kIdMirror, st);
-    k_mirror_upper<<<(B * B + 255) / 256, 256, 0, st>>>(K, B, kdiag);
+    k_mirror<false><<<(B * B + 255) / 256, 256, 0, st>>>(K, B, nullptr);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
