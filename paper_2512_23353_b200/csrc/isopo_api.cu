@@ -99,7 +99,7 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   if (dtype == ISOPO_BF16) {
     L.tiles_m = (d_out + kTileM - 1) / kTileM;
     L.tiles_n = (d_in + kTileN - 1) / kTileN;
-    L.n_pad = (int64_t)L.tiles_m * L.tiles_n * kTileElems;
+    L.n_pad = (int64_t)((d_out + 31) / 32 * 32) * d_in;  // pieces of 32 rows x 8 columns (tc_common.cuh)
     if (resolved == ISOPO_PATH_MATERIALISE) p = align_up(p + (size_t)2 * (size_t)B * (size_t)L.n_pad, 1024);
     L.off_kpart = p;
     if (resolved == ISOPO_PATH_MATERIALISE && deterministic_mode())

@@ -12,7 +12,6 @@ namespace isopo {
 // Tile of the stored per-sequence gradients on the bf16 path: one tensor-core accumulator tile.
 constexpr int kTileM = 128;  // rows of G (d_out)
 constexpr int kTileN = 256;  // columns of G (d_in)
-constexpr int kTileElems = kTileM * kTileN;
 
 // Kernel identifiers: written to *info together with ISOPO_INFO_TIMEOUT, and the index of the
 // per-kernel timing slots of isopo_profile_collect.

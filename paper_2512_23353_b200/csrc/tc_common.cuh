@@ -17,20 +17,38 @@ namespace tc {
 // ---------------------------------------------------------------------------------------------
 // Stored per-sequence gradients (bf16, materialised route; the order is private to the library).
 //
-// G_i is cut into 128 x 256 tiles (tile = tile_m * tiles_n + tile_n) and every tile into "pieces" of
-// 32 rows x 8 columns = 256 elements = 512 bytes: piece (tile, j, q) holds rows 32q .. 32q+31 and
-// columns 8j .. 8j+7 of the tile, row-major inside (row r at 16-byte slot r % 32).  That is exactly
+// G_i is cut into "pieces" of 32 rows x 8 columns = 256 elements = 512 bytes: piece (tm, c, q) holds rows
+// 128 tm + 32 q .. + 31 and columns 8 c .. 8 c + 7, row-major inside (row r at 16-byte slot r % 32).  That is exactly
 // what one epilogue warp writes with one 16-byte store per lane.  Pieces are the OUTER index and
 // the sequence the inner one:
-//     uint4 index of (piece p, sequence i, slot l) = (p * B + i) * 32 + l,   p = (tile * 32 + j) * 4 + q
+//     uint4 index of (piece p, sequence i, slot l) = (p * B + i) * 32 + l
 // so the B copies of one piece are contiguous (B x 512 bytes).  The NTK kernel contracts over
 // pieces and reads each such block once, front to back; the combine kernel sums over i inside it.
 // Any fixed order of the elements of G_i gives the same <G_i, G_j>.
+// Within a 128-row tile the column groups follow one another, its row quarters innermost.  Only pieces that hold
+// elements of G exist: d_in / 8 column groups and ceil(d_out / 32) row quarters, so a layer off the 128 x 256 tile
+// grid stores and re-reads no padding columns (896 columns padded to 1024 were 14 % of the bytes of three passes).
 // ---------------------------------------------------------------------------------------------
 constexpr int kPieceElems = 256;
-__host__ __device__ __forceinline__ size_t stored_piece(int tile, int j, int q) {
-  return ((size_t)tile * 32 + (size_t)j) * 4 + (size_t)q;
-}
+struct PieceGrid {
+  int groups;    // column groups: d_in / 8
+  int quarters;  // row quarters: ceil(d_out / 32)
+  __host__ __device__ __forceinline__ int quarters_of(int tm) const {  // row quarters of 128-row tile tm (none past the end)
+    const int left = quarters - 4 * tm;
+    return left > 4 ? 4 : left;
+  }
+  __host__ __device__ __forceinline__ size_t piece(int tm, int c, int q) const {
+    return (size_t)tm * 4 * (size_t)groups + (size_t)c * (size_t)quarters_of(tm) + (size_t)q;
+  }
+  // first row and first column of piece p
+  __device__ __forceinline__ void origin(int p, int& m, int& n) const {
+    const int per_tm = 4 * groups, tm = p / per_tm, rem = p - tm * per_tm, nq = quarters_of(tm);
+    const int c = nq == 4 ? rem >> 2 : rem / nq;
+    m = tm * kTileM + (rem - c * nq) * 32;
+    n = c * 8;
+  }
+};
+inline PieceGrid piece_grid(int d_in, int d_out) { return PieceGrid{d_in / 8, (d_out + 31) / 32}; }
 __host__ __device__ __forceinline__ size_t stored_slot(size_t piece, int i, int B, int l) {
   return (piece * (size_t)B + (size_t)i) * 32 + (size_t)l;
 }

@@ -265,7 +265,7 @@ __global__ void k_mirror(float* __restrict__ K, int B, const float* __restrict__
 constexpr int kCombineInFlight = ISOPO_COMBINE_IN_FLIGHT;  // 16-byte loads a thread has in flight
 // dW = beta dW + sum_i c_i G_i.  One thread per 16-byte slot (8 elements of every G_i) of the piece-blocked store.
 __global__ void __launch_bounds__(256) k_bf16_combine(const uint4* __restrict__ G, long long nchunks /* n_pad / 8 */,
-                                                       int B, int tiles_n, int d_in, int d_out,
+                                                       int B, PieceGrid grid, int d_in, int d_out,
                                                        const float* __restrict__ coeffs, float* __restrict__ dW,
                                                        float beta, const WsTag* __restrict__ tag_dev, WsTag tag,
                                                        int32_t* __restrict__ info) {
@@ -275,11 +275,12 @@ __global__ void __launch_bounds__(256) k_bf16_combine(const uint4* __restrict__ 
   __syncthreads();
   for (long long pos = blockIdx.x * (long long)blockDim.x + threadIdx.x; pos < nchunks;
        pos += (long long)gridDim.x * blockDim.x) {
-    // pos = piece * 32 + slot in the order of one sequence; piece = (tile * 32 + j) * 4 + q
-    const long long piece = pos >> 5;
-    const int l = (int)(pos & 31), q = (int)(piece & 3), j = (int)((piece >> 2) & 31), tile = (int)(piece >> 7);
-    const int m = (tile / tiles_n) * kTileM + q * 32 + l, n = (tile % tiles_n) * kTileN + j * 8;
-    if (m >= d_out || n >= d_in) continue;
+    // pos = piece * 32 + slot in the order of one sequence
+    const int piece = (int)(pos >> 5), l = (int)(pos & 31);
+    int m, n;
+    grid.origin(piece, m, n);
+    m += l;
+    if (m >= d_out) continue;
     if (!ISOPO_IN_RANGE((long long)stored_slot((size_t)piece, B - 1, B, l), nchunks * B, info, kIdCombine)) continue;
     if (!ISOPO_IN_RANGE((long long)m * d_in + n + 7, (long long)d_out * d_in, info, kIdCombine)) continue;
     float acc[8] = {};
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(256) k_bf16_combine(const uint4* __restrict__ 
 // columns), so that every load is 16 bytes per plane: with one slot per thread the two planes cost twice the load
 // instructions per byte of the bf16 store and the pass fell to 5.0 TB/s inside the step.
 __global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ planes, long long nchunks /* n_pad / 8 */,
-                                                       int B, int tiles_n, int d_in, int d_out,
+                                                       int B, PieceGrid grid, int d_in, int d_out,
                                                        const float* __restrict__ coeffs, const float* __restrict__ scales,
                                                        float* __restrict__ dW, float beta,
                                                        const WsTag* __restrict__ tag_dev, WsTag tag,
@@ -330,11 +331,12 @@ __global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ 
   const long long npairs = nchunks / 2;
   for (long long pos = blockIdx.x * (long long)blockDim.x + threadIdx.x; pos < npairs;
        pos += (long long)gridDim.x * blockDim.x) {
-    // pos = piece * 16 + pair of slots; piece = (tile * 32 + j) * 4 + q
-    const long long piece = pos >> 4;
-    const int l = (int)(pos & 15) * 2, q = (int)(piece & 3), j = (int)((piece >> 2) & 31), tile = (int)(piece >> 7);
-    const int m = (tile / tiles_n) * kTileM + q * 32 + l, n = (tile % tiles_n) * kTileN + j * 8;
-    if (m >= d_out || n >= d_in) continue;
+    // pos = piece * 16 + pair of slots
+    const int piece = (int)(pos >> 4), l = (int)(pos & 15) * 2;
+    int m, n;
+    grid.origin(piece, m, n);
+    m += l;
+    if (m >= d_out) continue;
     if (!ISOPO_IN_RANGE((long long)stored_slot((size_t)piece, B - 1, B, l + 1), nchunks * B, info, kIdCombine)) continue;
     if (!ISOPO_IN_RANGE((long long)m * d_in + n + 7, (long long)d_out * d_in, info, kIdCombine)) continue;
     float acc[16] = {};
@@ -440,6 +442,7 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
                           cudaStream_t st) {
   if (B > 256) return ISOPO_ERR_UNSUPPORTED;
   const long long chunks = L.n_pad / 8;
+  const PieceGrid pg = piece_grid(d_in, d_out);
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -447,10 +450,10 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
   {
     LaunchScope scope(kIdCombine, st);
     if (fmt.split)
-      k_e4m3_combine<<<grid, 256, 0, st>>>((const uint2*)G, chunks, B, L.tiles_n, d_in, d_out, coeffs, fmt.scales, dW, beta,
+      k_e4m3_combine<<<grid, 256, 0, st>>>((const uint2*)G, chunks, B, pg, d_in, d_out, coeffs, fmt.scales, dW, beta,
                                            tag_dev, tag, info);
     else
-      k_bf16_combine<<<grid, 256, 0, st>>>((const uint4*)G, chunks, B, L.tiles_n, d_in, d_out, coeffs, dW, beta, tag_dev, tag,
+      k_bf16_combine<<<grid, 256, 0, st>>>((const uint4*)G, chunks, B, pg, d_in, d_out, coeffs, dW, beta, tag_dev, tag,
                                            info);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());

@@ -53,7 +53,12 @@ struct SeqGradParams {
   float* dW;
   int64_t T, slab;  // tokens per work unit (a multiple of 64)
   int nslabs, d_in, d_out;
+  PieceGrid grid;   // per-sequence mode
 };
+
+// Columns of tile column tn that exist, in 16-column MMA steps: the last tile of a layer whose input width is off the
+// 256-column grid runs (and fetches) a narrower MMA.
+__device__ __forceinline__ int tile_cols(const SeqGradParams& p, int tn) { return min(kTileN, (p.d_in - tn * kTileN + 15) & ~15); }
 
 // Extents of the sequences in working order, staged in shared memory by the kernel (per-sequence mode).
 struct SeqInfo {
@@ -145,25 +150,24 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
         int64_t t0, t1;
         decode_unit<kFolded>(p, si, u, tiles_per_seq, tile, t0, t1, i);
         const int tm = tile / p.tiles_n, tn = tile % p.tiles_n;
-        const int nkb = (int)((t1 - t0 + kKB - 1) / kKB);
+        const int nkb = (int)((t1 - t0 + kKB - 1) / kKB), nchunks = (tile_cols(p, tn) + 63) >> 6;
         for (int kb = 0; kb < nkb; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.info, kIdSeqGrad))) break;
           const uint32_t a_dst = smem_base + stage * kStageBytes, b_dst = a_dst + kABytes;
           const int y = (int)(t0 + (int64_t)kb * kKB);
-          mbar_arrive_expect_tx(full_bar(stage), kStageBytes);
+          mbar_arrive_expect_tx(full_bar(stage), kABytes + nchunks * kChunkBytes);
 #pragma unroll
           for (int c = 0; c < kTileM / 64; ++c)
             tma_load_2d(a_dst + c * kChunkBytes, &mapY, tm * kTileM + c * 64, y, full_bar(stage));
 #pragma unroll
           for (int c = 0; c < kTileN / 64; ++c)
-            tma_load_2d(b_dst + c * kChunkBytes, &mapX, tn * kTileN + c * 64, y, full_bar(stage));
+            if (c < nchunks) tma_load_2d(b_dst + c * kChunkBytes, &mapX, tn * kTileN + c * 64, y, full_bar(stage));
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    constexpr uint32_t idesc = make_idesc_bf16(kTileM, kTileN, /*a_mn=*/true, /*b_mn=*/true);
     int stage = 0, acc = 0;
     uint32_t phase = 0, acc_phase = 0;
     bool ok = true;
@@ -176,6 +180,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
       if (!(ok = mbar_wait(accempty_bar(acc), acc_phase ^ 1u, abort_flag, p.info, kIdSeqGrad))) break;
       tc_fence_after_sync();
       const uint32_t d_tmem = tmem_base + (uint32_t)acc * kTileN;
+      const uint32_t idesc = make_idesc_bf16(kTileM, tile_cols(p, tile % p.tiles_n), /*a_mn=*/true, /*b_mn=*/true);
       for (int kb = 0; kb < nkb; ++kb) {
         // folded mode: the scaler warps hand the stage over (they have waited for the TMA bytes)
         if (!(ok = mbar_wait(kFolded ? scaled_bar(stage) : full_bar(stage), phase, abort_flag, p.info, kIdSeqGrad)))
@@ -226,8 +231,10 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kTileN;
       if (!kFolded) {
         uint4* dst = reinterpret_cast<uint4*>(p.G);
+        const int tm = tile / p.tiles_n, c0 = (tile % p.tiles_n) * (kTileN / 8);
+        const int ngroups = q < p.grid.quarters_of(tm) ? min(kTileN / 8, p.grid.groups - c0) : 0;  // pieces of this quarter
 #pragma unroll 2
-        for (int jc = 0; jc < kTileN / 32; ++jc) {
+        for (int jc = 0; jc * 4 < ngroups; ++jc) {
           uint32_t r[32];
           tmem_ld32(taddr + jc * 32, r);
           tmem_ld_wait();
@@ -238,8 +245,9 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
             o.y = pack_bf16x2(__uint_as_float(r[v * 8 + 2]), __uint_as_float(r[v * 8 + 3]));
             o.z = pack_bf16x2(__uint_as_float(r[v * 8 + 4]), __uint_as_float(r[v * 8 + 5]));
             o.w = pack_bf16x2(__uint_as_float(r[v * 8 + 6]), __uint_as_float(r[v * 8 + 7]));
-            const size_t slot = stored_slot(stored_piece(tile, jc * 4 + v, q), i, p.B, lane);
-            if (ISOPO_IN_RANGE(i < 0 || i >= p.B ? -1 : (long long)slot, (long long)p.B * p.n_pad / 8, p.info, kIdSeqGrad))
+            const size_t slot = stored_slot(p.grid.piece(tm, c0 + jc * 4 + v, q), i, p.B, lane);
+            if (jc * 4 + v < ngroups &&
+                ISOPO_IN_RANGE(i < 0 || i >= p.B ? -1 : (long long)slot, (long long)p.B * p.n_pad / 8, p.info, kIdSeqGrad))
               dst[slot] = o;
           }
         }
@@ -352,7 +360,7 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   SeqGradParams p{};
   p.off = off_dev; p.order = order_dev; p.G = (__nv_bfloat16*)G; p.n_pad = L.n_pad; p.B = B; p.tiles_m = L.tiles_m; p.tiles_n = L.tiles_n;
-  p.info = info;
+  p.info = info; p.d_in = d_in; p.d_out = d_out; p.grid = piece_grid(d_in, d_out);
   const long long units = (long long)B * L.tiles_m * L.tiles_n;
   const int grid = (int)std::min<long long>(units, sms);
   {

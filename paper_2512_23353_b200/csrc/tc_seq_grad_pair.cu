@@ -61,10 +61,11 @@ struct PairParams {
   const int64_t* off;
   const int32_t* order;     // the k-th sequence to work on (longest first)
   __nv_bfloat16* G[kMaxProj];   // stored gradients of every projection
-  int tiles_m[kMaxProj];        // stored 128-row tiles of every projection
+  PieceGrid grid[kMaxProj];     // pieces of every projection's stored gradients
+  int d_in;
   int ptm_first[kMaxProj + 1];  // first pair-tile row of every projection in the stacked grid
   int n_proj;
-  int B, tiles_n;           // sequences; stored 256-column tiles per gradient (X is common)
+  int B, tiles_n;           // sequences; 256-column tiles per gradient (X is common)
   int ptiles_m;             // pair-tile rows of the stacked grid = sum over projections of ceil(tiles_m / 2)
   int32_t* info;
   int group_m;              // pair-tile rows per group of the tile order
@@ -96,6 +97,10 @@ __device__ __forceinline__ void pair_tile(int pt, const PairParams& p, int& ptm,
   ptm = first + in_group % gm;
   tn = in_group / gm;
 }
+
+// Columns of tile column tn that exist, in the 32-column steps of a 2-CTA MMA: the last tile of a layer whose input
+// width is off the 256-column grid runs (and fetches) a narrower MMA, each CTA supplying half of these columns.
+__device__ __forceinline__ int tile_cols(const PairParams& p, int tn) { return min(kPairN, (p.d_in - tn * kPairN + 31) & ~31); }
 
 // Shape of one unit's token loop, identical in every role.
 struct UnitShape {
@@ -188,20 +193,23 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
         const UnitShape us = unit_shape(s_len[k]);
         const int h = proj_of(p, ptm);
         const CUtensorMap* mapY = h == 0 ? &mapY0 : h == 1 ? &mapY1 : &mapY2;
-        const int ycol = (2 * (ptm - (h == 0 ? 0 : (h == 1 ? p.ptm_first[1] : p.ptm_first[2]))) + (int)rank) * kHalf, xcol = tn * kPairN + (int)rank * kHalf;
+        const int ycol = (2 * (ptm - (h == 0 ? 0 : (h == 1 ? p.ptm_first[1] : p.ptm_first[2]))) + (int)rank) * kHalf, half_cols = tile_cols(p, tn) >> 1;
+        const int xcol = tn * kPairN + (int)rank * half_cols;
+        const bool two = half_cols > 64;  // 64-column boxes of X per CTA
+        const uint32_t x_bytes = two ? kOperandBytes : kChunkBytes;
         for (int kb = 0; kb < us.nkb; ++kb) {
           if (!(ok = mbar_wait_pair(empty_bar(stage), phase ^ 1u, abort_flag, peer_abort, p.info, kIdSeqGrad))) break;
           const uint32_t a_dst = smem_base + stage * kStageBytes, b_dst = a_dst + kOperandBytes;
           const int y = (int)(t0 + (int64_t)kb * kKB);
           const bool own_tail = us.fix && kb == us.nkb - 1;  // dY goes to this CTA's tail barrier
           if (own_tail) mbar_arrive_expect_tx(tail_bar(stage), kOperandBytes);
-          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), own_tail ? 2 * kOperandBytes : 2 * kStageBytes);
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * x_bytes + (own_tail ? 0 : 2 * kOperandBytes));
           const uint32_t fb = full_at_leader + 8u * stage;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             if (own_tail) tma_load_2d(a_dst + c * kChunkBytes, mapY, ycol + c * 64, y, tail_bar(stage));
             else tma_load_2d_pair(a_dst + c * kChunkBytes, mapY, ycol + c * 64, y, fb);
-            tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xcol + c * 64, y, fb);
+            if (c == 0 || two) tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xcol + c * 64, y, fb);
           }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -211,12 +219,14 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
     // ------------------------------------------------------------------ MMA issuer (one thread of CTA 0)
     // elected, not "lane 0": lets the compiler keep the MMA operands in uniform registers
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = make_idesc_bf16(256, kPairN, /*a_mn=*/true, /*b_mn=*/true);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, fixed_phase = 0;  // fixed_phase: one bit per stage
       bool ok = true;
       for (long long u = pair_id; u < total_units && ok; u += npairs) {
         const UnitShape us = unit_shape(s_len[u / ptiles]);
+        int ptm, tn;
+        pair_tile((int)(u % ptiles), p, ptm, tn);
+        const uint32_t idesc = make_idesc_bf16(256, tile_cols(p, tn), /*a_mn=*/true, /*b_mn=*/true);
         if (!(ok = mbar_wait_pair(accempty_bar(acc), acc_phase ^ 1u, abort_flag, peer_abort, p.info, kIdSeqGrad))) break;
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * kPairN;
         for (int kb = 0; kb < us.nkb; ++kb) {
@@ -257,11 +267,14 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
       pair_tile(pt, p, ptm, tn);
       const int h = proj_of(p, ptm);
       const int tm = 2 * (ptm - (h == 0 ? 0 : (h == 1 ? p.ptm_first[1] : p.ptm_first[2]))) + (int)rank;
-      const int tile = tm * p.tiles_n + tn;
+      const PieceGrid grid = pick(p.grid, h);
+      // pieces this warp stores: none past the last row quarter (an odd number of row tiles leaves the last pair's second
+      // half empty) or past the last column group
+      const int c0 = tn * (kPairN / 8), ngroups = q < grid.quarters_of(tm) ? min(kPairN / 8, grid.groups - c0) : 0;
       uint4* dst = reinterpret_cast<uint4*>(pick(p.G, h));
       if (!mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdSeqGrad)) break;
       tc_fence_after_sync();
-      if (kSplit && tm < pick(p.tiles_m, h)) {
+      if (kSplit && ngroups > 0) {
         // split store: hi = e4m3(s_i g), lo = e4m3(16 (s_i g - hi)), 8 bytes per lane and plane; the sum of g^2 goes to kdiag
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kPairN;
         const long long n_slots = pick(p.n_slots, h);
@@ -270,12 +283,13 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
         const float s_i = __ldg(pick(p.scales, h) + i);
         float ksum = 0.f, vmax = 0.f;
 #pragma unroll 2
-        for (int jc = 0; jc < kPairN / 32; ++jc) {
+        for (int jc = 0; jc * 4 < ngroups; ++jc) {
           uint32_t r[32];
           tmem_ld32(taddr + jc * 32, r);
           tmem_ld_wait();
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
+            if (jc * 4 + v >= ngroups) break;
             uint32_t hw[4], lw[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -287,7 +301,7 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
               const float2 hf = unpack_e4m3x2(hw[e]);
               lw[e] = pack_e4m3x2((v0 - hf.x) * kLoScale, (v1 - hf.y) * kLoScale);
             }
-            const size_t slot = stored_slot(stored_piece(tile, jc * 4 + v, q), i, p.B, lane);
+            const size_t slot = stored_slot(grid.piece(tm, c0 + jc * 4 + v, q), i, p.B, lane);
             if (ISOPO_IN_RANGE(i < 0 || i >= p.B ? -1 : (long long)slot, n_slots, p.info, kIdSeqGrad)) {
               hi_plane[slot] = make_uint2(hw[0] | (hw[1] << 16), hw[2] | (hw[3] << 16));
               lo_plane[slot] = make_uint2(lw[0] | (lw[1] << 16), lw[2] | (lw[3] << 16));
@@ -299,10 +313,10 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
         if (lane == 0 && ISOPO_IN_RANGE(i, p.B, p.info, kIdSeqGrad)) atomicAdd(pick(p.kdiag, h) + i, ksum);
         // an element beyond e4m3's largest value was clamped: K and dW are off by more than rounding, say so
         if (__any_sync(0xffffffffu, vmax > 448.f) && lane == 0) atomicCAS(p.info, 0, ISOPO_INFO_SATURATED | kIdSeqGrad);
-      } else if (!kSplit && tm < pick(p.tiles_m, h)) {  // an odd number of row tiles leaves the last pair's second half empty
+      } else if (!kSplit && ngroups > 0) {
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kPairN;
 #pragma unroll 2
-        for (int jc = 0; jc < kPairN / 32; ++jc) {
+        for (int jc = 0; jc * 4 < ngroups; ++jc) {
           uint32_t r[32];
           tmem_ld32(taddr + jc * 32, r);
           tmem_ld_wait();
@@ -313,8 +327,10 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
             o.y = pack_bf16x2(__uint_as_float(r[v * 8 + 2]), __uint_as_float(r[v * 8 + 3]));
             o.z = pack_bf16x2(__uint_as_float(r[v * 8 + 4]), __uint_as_float(r[v * 8 + 5]));
             o.w = pack_bf16x2(__uint_as_float(r[v * 8 + 6]), __uint_as_float(r[v * 8 + 7]));
-            const size_t slot = stored_slot(stored_piece(tile, jc * 4 + v, q), i, p.B, lane);
-            if (ISOPO_IN_RANGE(i < 0 || i >= p.B ? -1 : (long long)slot, pick(p.n_slots, h), p.info, kIdSeqGrad)) dst[slot] = o;
+            const size_t slot = stored_slot(grid.piece(tm, c0 + jc * 4 + v, q), i, p.B, lane);
+            if (jc * 4 + v < ngroups &&
+                ISOPO_IN_RANGE(i < 0 || i >= p.B ? -1 : (long long)slot, pick(p.n_slots, h), p.info, kIdSeqGrad))
+              dst[slot] = o;
           }
         }
       }
@@ -441,13 +457,13 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
     if (fmt[h].split != fmt[0].split) return ISOPO_ERR_INVALID_ARG;  // one store format per launch
   CUtensorMap mapY[kMaxProj], mapX;
   PairParams p{};
-  p.off = off_dev; p.order = order_dev; p.B = B; p.tiles_n = L[0].tiles_n; p.n_proj = n_proj; p.info = info;
+  p.off = off_dev; p.order = order_dev; p.B = B; p.tiles_n = L[0].tiles_n; p.n_proj = n_proj; p.info = info; p.d_in = d_in;
   for (int h = 0; h < kMaxProj; ++h) {
     const int hh = h < n_proj ? h : 0;  // unused slots repeat the first projection (never addressed)
     isopo_status s = make_map_2d_bf16(&mapY[h], dY[hh], (uint64_t)T, (uint64_t)d_out[hh], (uint64_t)d_out[hh], 64, kKB);
     if (s != ISOPO_OK) return s;
     p.G[h] = (__nv_bfloat16*)G[hh];
-    p.tiles_m[h] = L[hh].tiles_m;
+    p.grid[h] = piece_grid(d_in, d_out[hh]);
     p.n_slots[h] = (long long)B * L[hh].n_pad / 8;
     p.scales[h] = fmt[hh].scales;
     p.kdiag[h] = fmt[hh].kdiag;

@@ -69,6 +69,9 @@ __device__ __forceinline__ void pair_tile(int pt, const FoldParams& p, int& ptm,
   tn = in_group / gm;
 }
 
+// Columns of tile column tn that exist, in the 32-column steps of a 2-CTA MMA (see tc_seq_grad_pair.cu).
+__device__ __forceinline__ int tile_cols(const FoldParams& p, int tn) { return min(kPairN, (p.d_in - tn * kPairN + 31) & ~31); }
+
 // Shape of one segment's token loop, identical in every role.
 struct SegShape {
   int nkb;         // slabs
@@ -179,7 +182,10 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
         int ptm, tn, t0, t1;
         pair_tile((int)(u % ptiles), p, ptm, tn);
         unit_tokens(u, t0, t1);
-        const int ycol = (2 * ptm + (int)rank) * kHalf, xcol = tn * kPairN + (int)rank * kHalf;
+        const int ycol = (2 * ptm + (int)rank) * kHalf, half_cols = tile_cols(p, tn) >> 1;
+        const int xcol = tn * kPairN + (int)rank * half_cols;
+        const bool two = half_cols > 64;  // 64-column boxes of X per CTA
+        const uint32_t x_bytes = two ? kOperandBytes : kChunkBytes;
         for (SegWalk w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
           const SegShape ss = seg_shape(w.len());
           for (int kb = 0; kb < ss.nkb; ++kb) {
@@ -188,13 +194,13 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
             const int y = w.t + kb * kKB;  // rows past T and columns past the matrix read as zero
             const bool own_tail = ss.fix && kb == ss.nkb - 1;  // dY goes to this CTA's tail barrier
             if (own_tail) mbar_arrive_expect_tx(tail_bar(stage), kOperandBytes);
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), own_tail ? 2 * kOperandBytes : 2 * kStageBytes);
+            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * x_bytes + (own_tail ? 0 : 2 * kOperandBytes));
             const uint32_t fb = full_at_leader + 8u * stage;
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
               if (own_tail) tma_load_2d(a_dst + c * kChunkBytes, &mapY, ycol + c * 64, y, tail_bar(stage));
               else tma_load_2d_pair(a_dst + c * kChunkBytes, &mapY, ycol + c * 64, y, fb);
-              tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xcol + c * 64, y, fb);
+              if (c == 0 || two) tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xcol + c * 64, y, fb);
             }
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
@@ -204,12 +210,13 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (one thread of CTA 0)
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = make_idesc_bf16(256, kPairN, /*a_mn=*/true, /*b_mn=*/true);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, fixed_phase = 0;  // fixed_phase: one bit per stage
       bool ok = true;
       for (long long u = pair_id; u < total_units && ok; u += npairs) {
-        int t0, t1;
+        int ptm, tn, t0, t1;
+        pair_tile((int)(u % ptiles), p, ptm, tn);
+        const uint32_t idesc = make_idesc_bf16(256, tile_cols(p, tn), /*a_mn=*/true, /*b_mn=*/true);
         unit_tokens(u, t0, t1);
         for (SegWalk w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
           const SegShape ss = seg_shape(w.len());

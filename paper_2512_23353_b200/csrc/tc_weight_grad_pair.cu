@@ -53,6 +53,12 @@ struct FoldedPairParams {
   int32_t* info;
 };
 
+// Columns of the left / right accumulator of block column tn that exist, in the 32-column steps of a 2-CTA MMA (see
+// tc_seq_grad_pair.cu); the right one may have none.
+__device__ __forceinline__ int block_cols(const FoldedPairParams& p, int tn, int right) {
+  return max(0, min(kPairN, (p.d_in - (2 * tn + right) * kPairN + 31) & ~31));
+}
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX,
                         FoldedPairParams p) {
@@ -113,18 +119,20 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
         int64_t t0;
         int nkb;
         unit_tokens(u, t0, nkb);
-        const int ycol = (2 * ptm + (int)rank) * kHalf, xcol = tn * 2 * kPairN + (int)rank * kHalf;
+        const int ycol = (2 * ptm + (int)rank) * kHalf, hl = block_cols(p, tn, 0) >> 1, hr = block_cols(p, tn, 1) >> 1;
+        const int xl = tn * 2 * kPairN + (int)rank * hl, xr = (tn * 2 + 1) * kPairN + (int)rank * hr;
+        const uint32_t bytes = kOperandBytes + (uint32_t)(((hl + 63) >> 6) + ((hr + 63) >> 6)) * kChunkBytes;
         for (int kb = 0; kb < nkb; ++kb) {
           if (!(ok = mbar_wait_pair(empty_bar(stage), phase ^ 1u, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
           const uint32_t a_dst = smem_base + stage * kStageBytes, b_dst = a_dst + kOperandBytes;
           const int y = (int)(t0 + (int64_t)kb * kKB);  // rows past T and columns past d_in read as zero
-          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kStageBytes);
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * bytes);
           const uint32_t fb = full_at_leader + 8u * stage;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             tma_load_2d_pair(a_dst + c * kChunkBytes, &mapY, ycol + c * 64, y, fb);
-            tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xcol + c * 64, y, fb);
-            tma_load_2d_pair(b_dst + kOperandBytes + c * kChunkBytes, &mapX, xcol + kPairN + c * 64, y, fb);
+            if (c * 64 < hl) tma_load_2d_pair(b_dst + c * kChunkBytes, &mapX, xl + c * 64, y, fb);
+            if (c * 64 < hr) tma_load_2d_pair(b_dst + kOperandBytes + c * kChunkBytes, &mapX, xr + c * 64, y, fb);
           }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -133,7 +141,6 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (one thread of CTA 0)
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = make_idesc_bf16(256, kPairN, /*a_mn=*/true, /*b_mn=*/true);
       int stage = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
@@ -141,6 +148,9 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
         int64_t t0;
         int nkb;
         unit_tokens(u, t0, nkb);
+        const int tn = (int)(u % ptiles) % p.tiles_n, right = block_cols(p, tn, 1);
+        const uint32_t idesc = make_idesc_bf16(256, block_cols(p, tn, 0), /*a_mn=*/true, /*b_mn=*/true);
+        const uint32_t idesc2 = make_idesc_bf16(256, right, /*a_mn=*/true, /*b_mn=*/true);
         if (!(ok = mbar_wait_pair(accempty_bar(0), acc_phase ^ 1u, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base;
@@ -154,7 +164,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
             const uint64_t b_desc = make_sdesc_sw128(b_addr + k16 * 2048, kChunkBytes, 1024);
             const uint64_t b2_desc = make_sdesc_sw128(b_addr + kOperandBytes + k16 * 2048, kChunkBytes, 1024);
             mma_bf16_pair(d_tmem, a_desc, b_desc, idesc, (kb | k16) != 0);
-            mma_bf16_pair(d_tmem + kPairN, a_desc, b2_desc, idesc, (kb | k16) != 0);
+            if (right) mma_bf16_pair(d_tmem + kPairN, a_desc, b2_desc, idesc2, (kb | k16) != 0);
           }
           mma_commit_pair(empty_bar(stage));
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -178,7 +188,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
       float* dst = p.dW + (size_t)m * p.d_in + n0;
 #pragma unroll 2
-      for (int jc = 0; jc < 2 * kPairN / 32; ++jc) {
+      for (int jc = 0; jc < 2 * kPairN / 32 && n0 + jc * 32 < p.d_in; ++jc) {
         uint32_t r[32];
         tmem_ld32(taddr + jc * 32, r);
         tmem_ld_wait();
