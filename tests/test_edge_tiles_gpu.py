@@ -68,3 +68,17 @@ def test_stand_alone_weight_gradient(b, d_in, d_out, lens):
     ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, len(lens), b.PATH_GRAM)
     dW = _weight_grad(b, X, dY, off, c, ws, torch.zeros(1, dtype=torch.int32, device="cuda"), b.PATH_GRAM)
     assert rel_fro(dW, orc.weight_gradient(G, to_f64(c))) <= 6e-3
+
+
+# shares of the sequences in the combine: one (too few sequences / too many pieces), two, four and eight, even and uneven
+@pytest.mark.parametrize("B,d_in,d_out", [(15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
+def test_combine_shares(b, B, d_in, d_out):
+    X, dY, off, c, G = _problem(d_in, d_out, [2 + i % 3 for i in range(B)], B)
+    ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE)
+    K, info = torch.empty(B, B, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    b.isopo_layer_gram(X, dY, off, K, ws, info, b.PATH_MATERIALISE)
+    dW = torch.ones(d_out, d_in, device="cuda")
+    b.isopo_weight_grad(X, dY, c, off, dW, ws, info, b.PATH_MATERIALISE, 1.0)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    assert rel_fro(dW.cpu().numpy(), 1.0 + orc.weight_gradient(G, to_f64(c))) <= 6e-3
