@@ -91,7 +91,7 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   L.off_tokseq = p;
   p = align_up(p + sizeof(int32_t) * (size_t)T, 1024);
   L.off_kacc = p;
-  if (dtype == ISOPO_F32) p = align_up(p + sizeof(double) * (size_t)B * (size_t)B, 1024);
+  if (dtype == ISOPO_F32) p = align_up(p + sizeof(double) * ((size_t)B * (size_t)B + 1), 1024);
   L.off_scaled = p;
   if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM)
     p = align_up(p + (size_t)2 * (size_t)T * (size_t)std::min(d_in, d_out), 1024);
@@ -107,7 +107,7 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   } else {
     L.tiles_m = L.tiles_n = 0;
     L.off_kpart = p;
-    L.n_pad = (int64_t)d_in * d_out;
+    L.n_pad = ((int64_t)d_in * d_out + 3) / 4 * 4;
     if (resolved == ISOPO_PATH_MATERIALISE) p = align_up(p + (size_t)4 * (size_t)B * (size_t)L.n_pad, 1024);
   }
   L.total = p;
@@ -268,18 +268,17 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     if (s != ISOPO_OK) return s;
     return bf16_ntk(G, L, B, K, /*k_is_zero=*/true, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
   }
+  double* kacc = (double*)(w + L.off_kacc);
+  if (dtype == ISOPO_F32 && rp == ISOPO_PATH_MATERIALISE) {
+    float* G = (float*)(w + L.off_G);
+    uint32_t* done = (uint32_t*)(kacc + (size_t)B * B);
+    s = f32_seq_grad((const float*)X, (const float*)dY, d_in, d_out, seq_offsets_host, off_dev, B, G, L.n_pad, kacc, done,
+                     make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host), tag_dev, st);
+    return s != ISOPO_OK ? s : f32_ntk(G, L.n_pad, B, kacc, done, K, st);
+  }
   s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, st);
   if (s != ISOPO_OK) return s;
-  if (dtype == ISOPO_F32) {
-    if (rp == ISOPO_PATH_GRAM)
-      return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, (double*)(w + L.off_kacc), K, st);
-    s = store_tag(make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host), tag_dev, st);
-    if (s != ISOPO_OK) return s;
-    float* G = (float*)(w + L.off_G);
-    s = f32_seq_grad((const float*)X, (const float*)dY, d_in, d_out, off_dev, B, G, st);
-    if (s != ISOPO_OK) return s;
-    return f32_ntk(G, L.n_pad, B, K, st);
-  }
+  if (dtype == ISOPO_F32) return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);
   return bf16_gram(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
 }
 
@@ -507,7 +506,7 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
     const WsTag tag = make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host);
     const WsTag* tag_dev = (const WsTag*)(w + L.off_tag);
     if (dtype == ISOPO_F32)
-      return f32_combine((const float*)(w + L.off_G), L.n_pad, B, coeffs, dW, beta, tag_dev, tag, info, st);
+      return f32_combine((const float*)(w + L.off_G), (int64_t)d_in * d_out, L.n_pad, B, coeffs, dW, beta, tag_dev, tag, info, st);
     return bf16_combine(w + L.off_G, L, d_in, d_out, B, coeffs, dW, beta, tag_dev, tag, store_fmt(L, B, ws), info, st);
   }
   // GEMM over all tokens: refresh the token -> sequence map so the call also works on its own.

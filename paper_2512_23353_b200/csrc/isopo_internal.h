@@ -97,7 +97,7 @@ struct WsLayout {
   size_t off_offsets;  // int64 [B+1]
   size_t off_order;    // int32 [B]       (bf16 materialised path: sequences, longest first)
   size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here
-  size_t off_kacc;     // float64 [B*B]   (float32 path: K accumulators)
+  size_t off_kacc;     // float64 [B*B], uint32 (float32 path: K accumulators, CTAs of the K pass that are done)
   size_t off_scaled;   // bf16 [T, min(d_in, d_out)]  (bf16 Gram path: the pre-scaled operand of the weight-gradient GEMM)
   size_t off_G;        // stored gradients (materialised path only)
   size_t off_kpart;    // per-CTA partial K (bf16 materialised path in deterministic mode only)
@@ -135,7 +135,6 @@ isopo_status launch_prep_stored(const int64_t* off_host, int B, const WsTag& tag
                                 WsTag* tag_dev, float* K, cudaStream_t st);
 isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj, const WsTag* tag, int64_t* const* off_dev,
                                       int32_t* const* order_dev, WsTag* const* tag_dev, float* const* K, cudaStream_t st);
-isopo_status store_tag(const WsTag& tag, WsTag* tag_dev, cudaStream_t st);
 // offsets to the device and tokscale[t] = coeffs[sequence of token t] (float32 [T])
 isopo_status launch_tokscale(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs,
                              float* tokscale, cudaStream_t st);
@@ -151,14 +150,19 @@ __device__ __forceinline__ bool ws_tag_matches(const WsTag* __restrict__ have, c
   return ok;
 }
 
-// float32 SIMT path
-isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_dev, int B,
-                          float* G, cudaStream_t st);
-isopo_status f32_ntk(const float* G, int64_t N, int B, float* K, cudaStream_t st);
+// float32 path.  gstride: floats between the stored gradients of two sequences (WsLayout::n_pad, a multiple of 4)
+// f32_seq_grad also leaves the tag and clears kacc [B * B] and `done`, which f32_ntk adds into
+isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
+                          int B, float* G, int64_t gstride, double* kacc, uint32_t* done, const WsTag& tag, WsTag* tag_dev,
+                          cudaStream_t st);
+isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, cudaStream_t st);
+// M^T [n_samples, B] of the sampled rows a0, g0
+isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
+                         int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st);
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                       double* kacc, float* K, cudaStream_t st);
-isopo_status f32_combine(const float* G, int64_t N, int B, const float* coeffs, float* dW, float beta, const WsTag* tag_dev,
-                         const WsTag& tag, int32_t* info, cudaStream_t st);
+isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, const float* coeffs, float* dW, float beta,
+                         const WsTag* tag_dev, const WsTag& tag, int32_t* info, cudaStream_t st);
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* coeffs,
                              const int32_t* tokseq, float* dW, float beta, cudaStream_t st);
 

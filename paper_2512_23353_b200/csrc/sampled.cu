@@ -2,9 +2,9 @@
 // with a0 = X[samples], g0 = dY[samples] (the rows the caller drew),
 //   F_i^2 = sum_j (g0_j . G_i a0_j)^2 / sum_j (||g0_j|| ||a0_j||)^2 ,   c_i = A_i / sqrt(F_i^2 + lambda).
 // G_i is never formed: g0_j . G_i a0_j = sum_{t in i} (g0_j . dY_t)(a0_j . x_t) =: M^T[j, i] (Eq. one), a
-// rectangular cousin of the Gram route (tensor-core kernel in tc_gram.cu, float32 SIMT kernel here).
-// This file holds what surrounds it: gathering the sampled rows (and the denominator, Eq. two),
-// the float32 kernel, and the finishing step that turns M^T into F^2 and the coefficients.
+// rectangular cousin of the Gram route (tensor-core kernel in tc_gram.cu, float32 kernel in simt_f32.cu).
+// This file holds what surrounds it: gathering the sampled rows (and the denominator, Eq. two)
+// and the finishing step that turns M^T into F^2 and the coefficients.
 #include <algorithm>
 
 #include <cuda_bf16.h>
@@ -77,51 +77,6 @@ __global__ void __launch_bounds__(256) k_gather_samples(const T* __restrict__ X,
   if (threadIdx.x == 0) atomicAdd(den, na * ng);
 }
 
-// float32 route: for a 32 x 32 tile (samples x tokens) form P = a0 X^T and Q = g0 dY^T, multiply
-// elementwise and add into M^T[sample, sequence of the token] (float64 accumulators).
-constexpr int kST = 32;
-__global__ void __launch_bounds__(256) k_f32_sampled(const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
-                                                     int d_in, int d_out, const float* __restrict__ a0,
-                                                     const float* __restrict__ g0, int n_samples,
-                                                     const int32_t* __restrict__ tokseq, int B,
-                                                     double* __restrict__ Mt) {
-  __shared__ float sA[kST][kST + 1];
-  __shared__ float sB[kST][kST + 1];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int64_t j0 = (int64_t)blockIdx.y * kST, t0 = (int64_t)blockIdx.x * kST;
-  float h[2][2];
-  for (int pass = 0; pass < 2; ++pass) {
-    const float* R = pass == 0 ? a0 : g0;
-    const float* C = pass == 0 ? X : dY;
-    const int d = pass == 0 ? d_in : d_out;
-    float acc[2][2] = {};
-    for (int k0 = 0; k0 < d; k0 += kST) {
-      for (int e = tid; e < kST * kST; e += 256) {
-        const int r = e / kST, c = e % kST;
-        sA[r][c] = (j0 + r < n_samples && k0 + c < d) ? R[(j0 + r) * d + k0 + c] : 0.f;
-        sB[r][c] = (t0 + r < T && k0 + c < d) ? C[(t0 + r) * d + k0 + c] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int c = 0; c < kST; ++c) {
-        const float r0 = sA[ty * 2][c], r1 = sA[ty * 2 + 1][c], c0 = sB[tx * 2][c], c1 = sB[tx * 2 + 1][c];
-        acc[0][0] = fmaf(r0, c0, acc[0][0]);
-        acc[0][1] = fmaf(r0, c1, acc[0][1]);
-        acc[1][0] = fmaf(r1, c0, acc[1][0]);
-        acc[1][1] = fmaf(r1, c1, acc[1][1]);
-      }
-      __syncthreads();
-    }
-    for (int p = 0; p < 2; ++p)
-      for (int q = 0; q < 2; ++q) h[p][q] = pass == 0 ? acc[p][q] : h[p][q] * acc[p][q];
-  }
-  for (int p = 0; p < 2; ++p)
-    for (int q = 0; q < 2; ++q) {
-      const int64_t j = j0 + ty * 2 + p, t = t0 + tx * 2 + q;
-      if (j < n_samples && t < T) atomicAdd(&Mt[(size_t)j * B + tokseq[t]], (double)h[p][q]);
-    }
-}
-
 // F_i^2 = sum_j M^T[j, i]^2 / den,  c_i = A_i / sqrt(F_i^2 + lambda).  A block of 32 x 8 threads serves 32
 // sequences: thread (x, y) sums the samples j = y, y + 8, ... of sequence x (loads coalesced over x), the eight
 // partial sums meet in shared memory.
@@ -184,20 +139,13 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
     float* a0 = (float*)(ws + S.off_a0);
     float* g0 = (float*)(ws + S.off_g0);
     double* Mt = (double*)(ws + S.off_mt);
-    const int64_t nt = (T + kST - 1) / kST, ns = (n_samples + kST - 1) / kST;
-    if (ns > 65535) return ISOPO_ERR_UNSUPPORTED;
-    ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(double) * (size_t)n_samples * B, st));
     {
       LaunchScope scope(kIdSampledAux, st);
       k_gather_samples<float><<<n_samples, 256, 0, st>>>((const float*)X, (const float*)dY, d_in, d_out, rows, a0, g0, den);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
-    {
-      LaunchScope scope(kIdSampled, st);
-      k_f32_sampled<<<dim3((unsigned)nt, (unsigned)ns), 256, 0, st>>>((const float*)X, (const float*)dY, T, d_in, d_out, a0,
-                                                                      g0, n_samples, tokseq, B, Mt);
-    }
-    ISOPO_CUDA_TRY(cudaGetLastError());
+    s = f32_sampled((const float*)X, (const float*)dY, T, d_in, d_out, a0, g0, n_samples, tokseq, B, Mt, st);
+    if (s != ISOPO_OK) return s;
     {
       LaunchScope scope(kIdSampledAux, st);
       k_sampled_finish<double><<<(B + 31) / 32, 32 * kFinishSlices, 0, st>>>(Mt, n_samples, B, den, A, lambda, coeffs, F2);

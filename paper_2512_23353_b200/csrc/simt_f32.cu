@@ -1,6 +1,6 @@
-// float32 SIMT kernels of the ISOPO layer path (small layers, parity to 1e-5), plus the
-// token -> sequence map that both dtypes use.  Products are float32 FFMA; everything that sums
-// over many products of products (K) is accumulated in float64.
+// float32 kernels of the ISOPO layer path (parity to 1e-5), plus the token -> sequence map that both
+// dtypes use.  Token contractions are float32 FMA; everything that sums over many products of
+// products (K) is accumulated in float64.
 #include <algorithm>
 
 #include "isopo_internal.h"
@@ -8,9 +8,6 @@
 namespace isopo {
 
 namespace {
-
-constexpr int kT = 64;   // output tile edge of the SIMT GEMMs
-constexpr int kTK = 16;  // tokens staged per step
 
 // Host values travel to the device as kernel arguments (no host-to-device copy, so no hidden
 // synchronisation with the stream and nothing that reads the caller's array after the call returns).
@@ -43,10 +40,6 @@ __global__ void __launch_bounds__(256) k_prep_stored(StoredPrepArgs a, int B, in
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * B; e += gridDim.x * blockDim.x) a.K[h][e] = 0.f;
   }
 }
-__global__ void k_store_tag(WsTag t, WsTag* __restrict__ tag) {
-  if (threadIdx.x < 8) tag->v[threadIdx.x] = t.v[threadIdx.x];
-}
-
 __global__ void k_tokseq(const int64_t* __restrict__ off, int B, int64_t T, int32_t* __restrict__ tokseq) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
     int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
@@ -93,167 +86,562 @@ __global__ void __launch_bounds__(256) k_prep_small(OffsetArgs a, int B, int64_t
   }
 }
 
-// Accumulates, for tokens [t0, t1), acc[4][4] += w_t * dY[t, m0+4ty+a] * X[t, n0+4tx+b].
-template <bool kScaled>
-__device__ __forceinline__ void gemm_tokens(const float* __restrict__ X, const float* __restrict__ dY, int d_in,
-                                            int d_out, int64_t t0, int64_t t1, int m0, int n0,
-                                            const float* __restrict__ coeffs, const int32_t* __restrict__ tokseq,
-                                            float (&acc)[4][4]) {
-  __shared__ float sY[kTK][kT + 4];
-  __shared__ float sX[kTK][kT + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int64_t tb = t0; tb < t1; tb += kTK) {
-    for (int e = tid; e < kTK * kT; e += 256) {
-      const int r = e / kT, c = e % kT;
-      const int64_t t = tb + r;
-      float y = 0.f, x = 0.f;
-      if (t < t1) {
-        if (m0 + c < d_out) y = dY[t * d_out + m0 + c];
-        if (n0 + c < d_in) x = X[t * d_in + n0 + c];
-        if (kScaled) y *= coeffs[tokseq[t]];
-      }
-      sY[r][c] = y;
-      sX[r][c] = x;
+// ---------------------------------------------------------------------------------------------
+// Register-blocked float32 GEMM over tokens: acc[p][q] += w_t * dY[t, m] * X[t, n] for tokens [t0, t1), tile
+// kTile x kTile, kT x kT elements per thread.  Token rows are staged kTK at a time by cp.async, kStages deep (16-byte
+// copies where the row length allows, 4-byte ones otherwise; columns and tokens past the end arrive as zeros); a thread's
+// rows and columns come in groups of four, so that its operands are 16-byte shared loads.  Two neighbouring columns share
+// one packed fma (fma.rn.f32x2: the same two roundings, half the issue slots, which the shared loads need).
+// Bound by the float32 pipe: 64 sequences of 72 tokens, 896 x 896: 174 us (42 TFLOP/s with the 205 MB store of G) against
+// 342 us with a 64 x 64 tile loaded synchronously.  Stages of 8 tokens waste less of a short sequence's last stage
+// (G_i: 174 against 187 us with 16); over one long token range stages of 16 synchronise half as often (dW: 197 against 212 us).
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool live) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(live ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool live) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(live ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Stages rows [t, t + kRows) x columns [c0, c0 + kCols) of a row-major [., d] matrix into dst[kRows][kCols].
+template <int kRows, int kCols, int kThreadsF>
+__device__ __forceinline__ void stage_rows(float* dst, const float* __restrict__ M, int64_t t, int64_t t_end, int c0, int d) {
+  if ((d & 3) == 0) {
+#pragma unroll
+    for (int e = threadIdx.x; e < kRows * kCols / 4; e += kThreadsF) {
+      const int r = e / (kCols / 4), c = e % (kCols / 4) * 4;
+      const bool live = t + r < t_end && c0 + c < d;
+      cp_async16(dst + r * kCols + c, live ? M + (t + r) * d + c0 + c : M, live);
     }
-    __syncthreads();
+  } else {
 #pragma unroll
-    for (int r = 0; r < kTK; ++r) {
-      float a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { a[q] = sY[r][ty * 4 + q]; b[q] = sX[r][tx * 4 + q]; }
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
+    for (int e = threadIdx.x; e < kRows * kCols; e += kThreadsF) {
+      const int r = e / kCols, c = e % kCols;
+      const bool live = t + r < t_end && c0 + c < d;
+      cp_async4(dst + r * kCols + c, live ? M + (t + r) * d + c0 + c : M, live);
     }
-    __syncthreads();
   }
 }
 
-// G_i = dY_i^T X_i, one (64 x 64 tile, sequence) per CTA.
-__global__ void __launch_bounds__(256) k_f32_seq_grad(const float* __restrict__ X, const float* __restrict__ dY,
-                                                      int d_in, int d_out, const int64_t* __restrict__ off,
-                                                      float* __restrict__ G) {
-  const int i = blockIdx.z, m0 = blockIdx.y * kT, n0 = blockIdx.x * kT;
-  float acc[4][4] = {};
-  gemm_tokens<false>(X, dY, d_in, d_out, off[i], off[i + 1], m0, n0, nullptr, nullptr, acc);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float* Gi = G + (size_t)i * d_out * d_in;
-  for (int p = 0; p < 4; ++p)
-    for (int q = 0; q < 4; ++q) {
-      const int m = m0 + ty * 4 + p, n = n0 + tx * 4 + q;
-      if (m < d_out && n < d_in) Gi[(size_t)m * d_in + n] = acc[p][q];
+template <int kTile, int kT, int kTK, int kStages>
+struct TokenGemm {
+  static constexpr int kSide = kTile / kT;                        // threads along one side
+  static constexpr int kThr = kSide * kSide;
+  static constexpr int kStage = kTK * 2 * kTile;                  // floats
+  static constexpr int kSmem = kStages * (kStage + kTK) * 4;      // bytes (the last kTK floats: token weights)
+  static_assert(kSmem <= 99 * 1024, "two CTAs per SM");
+  f32x2 acc[kT][kT / 2];
+  // tile row of acc[p][.], tile column of the first element of a pair acc[.][q / 2]
+  __device__ __forceinline__ static int row(int p) { return (p / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x / kSide) * 4 + p % 4; }
+  __device__ __forceinline__ static int col(int q) { return (q / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x % kSide) * 4 + q % 4; }
+
+  // kScaled: the dY row of token t counts coeffs[tokseq[t]] times (rounded once, as a scaled copy of dY would be)
+  template <bool kScaled>
+  __device__ __forceinline__ void run(float* smem, const float* __restrict__ X, const float* __restrict__ dY, int d_in,
+                                      int d_out, int64_t t0, int64_t t1, int m0, int n0, const float* __restrict__ coeffs,
+                                      const int32_t* __restrict__ tokseq) {
+#pragma unroll
+    for (int p = 0; p < kT; ++p)
+#pragma unroll
+      for (int q = 0; q < kT / 2; ++q) acc[p][q] = 0ull;
+    const int nk = (int)((t1 - t0 + kTK - 1) / kTK);
+    float* sw = smem + kStages * kStage;
+    auto fetch = [&](int k) {
+      if (k < nk) {
+        float* s = smem + (k % kStages) * kStage;
+        const int64_t t = t0 + (int64_t)k * kTK;
+        stage_rows<kTK, kTile, kThr>(s, dY, t, t1, m0, d_out);
+        stage_rows<kTK, kTile, kThr>(s + kTK * kTile, X, t, t1, n0, d_in);
+        if (kScaled && threadIdx.x < kTK)
+          sw[(k % kStages) * kTK + threadIdx.x] = t + threadIdx.x < t1 ? coeffs[tokseq[t + threadIdx.x]] : 0.f;
+      }
+      cp_async_commit();
+    };
+#pragma unroll
+    for (int k = 0; k < kStages - 1; ++k) fetch(k);
+    for (int k = 0; k < nk; ++k) {
+      cp_async_wait<kStages - 2>();
+      __syncthreads();  // stage k is complete for everybody, and everybody is done with the stage fetched next
+      fetch(k + kStages - 1);
+      const float* sY = smem + (k % kStages) * kStage;
+      const float* sX = sY + kTK * kTile;
+#pragma unroll
+      for (int r = 0; r < kTK; ++r) {
+        float a[kT];
+        f32x2 b[kT / 2];
+#pragma unroll
+        for (int p = 0; p < kT; p += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(sY + r * kTile + row(p));
+          a[p] = v.x; a[p + 1] = v.y; a[p + 2] = v.z; a[p + 3] = v.w;
+        }
+        if (kScaled) {
+          const float w = sw[(k % kStages) * kTK + r];
+#pragma unroll
+          for (int p = 0; p < kT; ++p) a[p] *= w;
+        }
+#pragma unroll
+        for (int q = 0; q < kT; q += 4) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(sX + r * kTile + col(q));
+          b[q / 2] = v.x; b[q / 2 + 1] = v.y;
+        }
+#pragma unroll
+        for (int p = 0; p < kT; ++p) {
+          const f32x2 ap = pack2(a[p], a[p]);
+#pragma unroll
+          for (int q = 0; q < kT / 2; ++q) acc[p][q] = fma2(ap, b[q], acc[p][q]);
+        }
+      }
     }
+  }
+};
+template <int kTile, int kT> using SeqGemm = TokenGemm<kTile, kT, 8, 4>;
+template <int kTile, int kT> using SlabGemm = TokenGemm<kTile, kT, 16, 3>;
+
+// G_i = dY_i^T X_i, one (tile, sequence) per CTA.  The launch also leaves the workspace tag and clears the accumulators
+// that the K pass behind it adds into.  Offsets come as kernel arguments when they fit (kArgOff), else from `off`.
+struct F32StoredArgs {
+  const float* X;
+  const float* dY;
+  int d_in, d_out, B;
+  int64_t gstride;   // floats between the gradients of two sequences (a multiple of 4)
+  const int64_t* off;
+  float* G;
+  double* kacc;      // [B * B]
+  uint32_t* done;    // CTAs of the K pass that have finished
+  WsTag tag;
+  WsTag* tag_dev;
+};
+template <bool kArgOff> struct OffsetParam { int64_t v[1]; };
+template <> struct OffsetParam<true> { int64_t v[kArgChunk]; };
+static_assert(sizeof(F32StoredArgs) + sizeof(OffsetParam<true>) <= 4096, "kernel arguments");
+
+template <int kTile, int kT, bool kArgOff>
+__global__ void __launch_bounds__(SeqGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
+k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ OffsetParam<kArgOff> o) {
+  extern __shared__ __align__(16) float smem[];
+  const int i = blockIdx.z, m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
+  const int64_t cta = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  const int64_t threads = (int64_t)gridDim.x * gridDim.y * gridDim.z * blockDim.x;
+  for (int64_t e = cta * blockDim.x + threadIdx.x; e < (int64_t)a.B * a.B; e += threads) a.kacc[e] = 0.0;
+  if (cta == 0) {
+    if (threadIdx.x < 8) a.tag_dev->v[threadIdx.x] = a.tag.v[threadIdx.x];
+    if (threadIdx.x == 8) *a.done = 0u;
+  }
+  const int64_t t0 = kArgOff ? o.v[i] : a.off[i], t1 = kArgOff ? o.v[i + 1] : a.off[i + 1];
+  SeqGemm<kTile, kT> g;
+  g.template run<false>(smem, a.X, a.dY, a.d_in, a.d_out, t0, t1, m0, n0, nullptr, nullptr);
+  float* Gi = a.G + (size_t)i * a.gstride;
+#pragma unroll
+  for (int p = 0; p < kT; ++p) {
+    const int m = m0 + g.row(p);
+    if (m >= a.d_out) continue;
+#pragma unroll
+    for (int q = 0; q < kT; q += 4) {
+      const int n = n0 + g.col(q);
+      float4 v;
+      unpack2(g.acc[p][q / 2], v.x, v.y);
+      unpack2(g.acc[p][q / 2 + 1], v.z, v.w);
+      float* dst = Gi + (size_t)m * a.d_in + n;
+      if ((a.d_in & 3) == 0) {
+        if (n < a.d_in) *reinterpret_cast<float4*>(dst) = v;
+      } else {
+        if (n < a.d_in) dst[0] = v.x;
+        if (n + 1 < a.d_in) dst[1] = v.y;
+        if (n + 2 < a.d_in) dst[2] = v.z;
+        if (n + 3 < a.d_in) dst[3] = v.w;
+      }
+    }
+  }
+  // the K pass reads whole groups of four: the padding of a gradient is zero
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) {
+    const int64_t e = (int64_t)a.d_in * a.d_out + threadIdx.x;
+    if (e < a.gstride) Gi[e] = 0.f;
+  }
 }
 
 // dW += (c_seq(t) dY)^T X over a slab of tokens (split over blockIdx.z), float atomics.
-__global__ void __launch_bounds__(256) k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY,
-                                                         int64_t T, int d_in, int d_out,
-                                                         const float* __restrict__ coeffs,
-                                                         const int32_t* __restrict__ tokseq, float* __restrict__ dW,
-                                                         int64_t slab) {
-  const int m0 = blockIdx.y * kT, n0 = blockIdx.x * kT;
+template <int kTile, int kT>
+__global__ void __launch_bounds__(SlabGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
+k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int64_t T, int d_in, int d_out,
+                  const float* __restrict__ coeffs, const int32_t* __restrict__ tokseq, float* __restrict__ dW, int64_t slab) {
+  extern __shared__ __align__(16) float smem[];
+  const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t t0 = blockIdx.z * slab, t1 = min(T, t0 + slab);
-  float acc[4][4] = {};
-  gemm_tokens<true>(X, dY, d_in, d_out, t0, t1, m0, n0, coeffs, tokseq, acc);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int p = 0; p < 4; ++p)
-    for (int q = 0; q < 4; ++q) {
-      const int m = m0 + ty * 4 + p, n = n0 + tx * 4 + q;
-      if (m < d_out && n < d_in) atomicAdd(&dW[(size_t)m * d_in + n], acc[p][q]);
+  SlabGemm<kTile, kT> g;
+  g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, m0, n0, coeffs, tokseq);
+#pragma unroll
+  for (int p = 0; p < kT; ++p) {
+    const int m = m0 + g.row(p);
+#pragma unroll
+    for (int q = 0; q < kT; q += 2) {
+      const int n = n0 + g.col(q);
+      float v0, v1;
+      unpack2(g.acc[p][q / 2], v0, v1);
+      if (m < d_out && n < d_in) atomicAdd(&dW[(size_t)m * d_in + n], v0);
+      if (m < d_out && n + 1 < d_in) atomicAdd(&dW[(size_t)m * d_in + n + 1], v1);
     }
-}
-
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  v = l < (blockDim.x >> 5) ? red[l] : 0.0;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// K_ij = sum(G_i * G_j) for j >= i, mirrored.
-__global__ void __launch_bounds__(256) k_f32_ntk(const float* __restrict__ G, int64_t N, int B, float* __restrict__ K) {
-  const int i = blockIdx.y, j = blockIdx.x;
-  if (j < i) return;
-  const float* gi = G + (size_t)i * N;
-  const float* gj = G + (size_t)j * N;
-  double s = 0.0;
-  for (int64_t e = threadIdx.x; e < N; e += blockDim.x) s += (double)(gi[e] * gj[e]);
-  s = block_sum(s);
-  if (threadIdx.x == 0) {
-    K[(size_t)i * B + j] = (float)s;
-    K[(size_t)j * B + i] = (float)s;
   }
 }
 
-// Gram route: for a pair of 32-token tiles (I <= J) form P = X_I X_J^T and Q = dY_I dY_J^T, multiply
-// elementwise and add into the (seq t, seq s) accumulators.  Only token pairs t <= s are used; a
-// pair inside one sequence with t < s stands for (t,s) and (s,t) and counts twice.
-constexpr int kGT = 32;
-__global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
+// ---------------------------------------------------------------------------------------------
+// K_ij = sum(G_i * G_j), i <= j, products and sums in float64 (mma.sync m16n8k8.f64: the exact product of two floats,
+// accumulated in float64).  A CTA takes every gridDim.y-th 64-column chunk of a pair of row blocks of G_flat, staged by
+// cp.async as floats; its four warps share the columns of a chunk, each holding the whole block of K in registers, so a
+// fragment is read and widened once for many MMAs.  kDiag: 8 kNB rows against themselves, only the 16 x 8 blocks on and
+// above the diagonal; otherwise 16 kMA rows against 8 kNB others.  The CTAs meet in kacc by float64 atomics; with one
+// row block the last CTA to finish rounds K to float32.
+// Bound by the float64 pipe.  One CTA per pair (i, j) with scalar float64 additions re-read G B / 2 times: 1384 us at 64
+// sequences of an 896 x 896 layer against 146 us, 3694 against 500 us at 256 sequences of 300 x 500.  One CTA of eight
+// warps per SM instead of two of four: 162 and 715 us.  Few sequences leave the pass to HBM and need more loads in flight: kPerSm.
+// ---------------------------------------------------------------------------------------------
+constexpr int kNtkKC = 64;             // columns per chunk
+constexpr int kNtkPitch = kNtkKC + 4;  // floats: the 32 lanes of a fragment read hit 32 banks
+constexpr int kNtkStages = 3;
+constexpr int kNtkRows = 64;           // sequences per row block
+constexpr int kNtkThreads = 128;
+
+__device__ __forceinline__ void dmma16x8x8(double (&c)[4], double a0, double a1, double a2, double a3, double b0, double b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+      : "d"(a0), "d"(a1), "d"(a2), "d"(a3), "d"(b0), "d"(b1));
+}
+
+template <int kMA, int kNB, bool kDiag>
+struct NtkShape {
+  static constexpr int kRowsStaged = kDiag ? 8 * kNB : 16 * kMA + 8 * kNB;
+  static constexpr int kStageFloats = kRowsStaged * kNtkPitch;
+  static constexpr int kSmemStages = kNtkStages * kStageFloats * 4;
+  static constexpr int kBlocks = kDiag ? kMA * (kMA + 1) : kMA * kNB;  // 16 x 8 blocks of K in a warp's registers
+  static constexpr int kSmemRed = 2 * kBlocks * 128 * 8;               // two warps' blocks
+  static constexpr int kSmem = kSmemStages > kSmemRed ? kSmemStages : kSmemRed;
+  static constexpr int kPerSm = kNB == 2 ? 8 : kNB == 4 ? 4 : 2;       // resident CTAs per SM
+};
+
+template <int kMA, int kNB, bool kDiag>
+__global__ void __launch_bounds__(kNtkThreads, NtkShape<kMA, kNB, kDiag>::kPerSm)
+k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uint32_t* done, float* __restrict__ K) {
+  typedef NtkShape<kMA, kNB, kDiag> S;
+  extern __shared__ __align__(16) float smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  // the pair of row blocks: diagonal blocks in order; otherwise pairs I < J of 64-row blocks, I in two halves of 32 rows
+  int i0, j0;
+  if (kDiag) {
+    i0 = j0 = blockIdx.x * kNtkRows;
+  } else {
+    int J = 1, r = blockIdx.x >> 1;
+    while (r >= J) { r -= J; ++J; }
+    i0 = r * kNtkRows + (blockIdx.x & 1) * 32;
+    j0 = J * kNtkRows;
+  }
+  const int64_t nchunks = (gstride + kNtkKC - 1) / kNtkKC;
+  auto fetch = [&](int64_t ch, int stage) {
+    if (ch < nchunks) {
+      float* s = smem + stage * S::kStageFloats;
+      for (int e = tid; e < S::kRowsStaged * (kNtkKC / 4); e += kNtkThreads) {
+        const int r = e / (kNtkKC / 4), c = e % (kNtkKC / 4) * 4;
+        const int seq = kDiag || r < 16 * kMA ? i0 + r : j0 + r - 16 * kMA;
+        const int64_t x = ch * kNtkKC + c;
+        const bool live = seq < B && x < gstride;
+        cp_async16(s + r * kNtkPitch + c, live ? G + (size_t)seq * gstride + x : G, live);
+      }
+    }
+    cp_async_commit();
+  };
+  double acc[kMA][kNB][4];
+#pragma unroll
+  for (int p = 0; p < kMA; ++p)
+#pragma unroll
+    for (int n = 0; n < kNB; ++n)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[p][n][q] = 0.0;
+#pragma unroll
+  for (int k = 0; k < kNtkStages - 1; ++k) fetch(blockIdx.y + (int64_t)k * gridDim.y, k);
+  int stage = 0;
+  for (int64_t ch = blockIdx.y; ch < nchunks; ch += gridDim.y) {
+    cp_async_wait<kNtkStages - 2>();
+    __syncthreads();
+    fetch(ch + (int64_t)(kNtkStages - 1) * gridDim.y, (stage + kNtkStages - 1) % kNtkStages);
+    const float* s = smem + stage * S::kStageFloats;
+    if (++stage == kNtkStages) stage = 0;
+#pragma unroll
+    for (int h = 0; h < kNtkKC / 32; ++h) {
+      const int k0 = (warp + 4 * h) * 8 + t;
+      double b[kNB][2];
+      const float* sb = s + (kDiag ? 0 : 16 * kMA) * kNtkPitch;
+#pragma unroll
+      for (int n = 0; n < kNB; ++n) {
+        b[n][0] = (double)sb[(n * 8 + g) * kNtkPitch + k0];
+        b[n][1] = (double)sb[(n * 8 + g) * kNtkPitch + k0 + 4];
+      }
+#pragma unroll
+      for (int p = 0; p < kMA; ++p) {
+        double a0, a1, a2, a3;
+        if (kDiag) {  // rows and columns are the same sequences, and a fragment of either holds the same elements
+          a0 = b[2 * p][0]; a1 = b[2 * p + 1][0]; a2 = b[2 * p][1]; a3 = b[2 * p + 1][1];
+        } else {
+          a0 = (double)s[(p * 16 + g) * kNtkPitch + k0];
+          a1 = (double)s[(p * 16 + 8 + g) * kNtkPitch + k0];
+          a2 = (double)s[(p * 16 + g) * kNtkPitch + k0 + 4];
+          a3 = (double)s[(p * 16 + 8 + g) * kNtkPitch + k0 + 4];
+        }
+#pragma unroll
+        for (int n = kDiag ? 2 * p : 0; n < kNB; ++n) dmma16x8x8(acc[p][n], a0, a1, a2, a3, b[n][0], b[n][1]);
+      }
+    }
+  }
+  cp_async_wait<0>();
+  // the warps' shares meet in shared memory (4 -> 2 -> 1), the CTAs' in kacc
+  double2* red = reinterpret_cast<double2*>(smem);
+  for (int half = 2; half >= 1; half >>= 1) {
+    __syncthreads();
+    if (warp >= half && warp < 2 * half) {
+      int blk = (warp - half) * S::kBlocks;
+#pragma unroll
+      for (int p = 0; p < kMA; ++p)
+#pragma unroll
+        for (int n = kDiag ? 2 * p : 0; n < kNB; ++n, ++blk) {
+          red[blk * 64 + lane] = make_double2(acc[p][n][0], acc[p][n][1]);
+          red[blk * 64 + 32 + lane] = make_double2(acc[p][n][2], acc[p][n][3]);
+        }
+    }
+    __syncthreads();
+    if (warp < half) {
+      int blk = warp * S::kBlocks;
+#pragma unroll
+      for (int p = 0; p < kMA; ++p)
+#pragma unroll
+        for (int n = kDiag ? 2 * p : 0; n < kNB; ++n, ++blk) {
+          const double2 lo = red[blk * 64 + lane], hi = red[blk * 64 + 32 + lane];
+          acc[p][n][0] += lo.x; acc[p][n][1] += lo.y; acc[p][n][2] += hi.x; acc[p][n][3] += hi.y;
+        }
+    }
+  }
+  if (warp == 0) {
+#pragma unroll
+    for (int p = 0; p < kMA; ++p)
+#pragma unroll
+      for (int n = kDiag ? 2 * p : 0; n < kNB; ++n)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + p * 16 + g + (q >> 1) * 8, j = j0 + n * 8 + 2 * t + (q & 1);
+          if (i <= j && j < B) atomicAdd(&kacc[(size_t)i * B + j], acc[p][n][q]);
+        }
+  }
+  if (kDiag && gridDim.x == 1) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(done, 1u) == gridDim.y - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int e = tid; e < B * B; e += kNtkThreads) {
+      const int i = e / B, j = e % B;
+      K[e] = (float)__ldcg(&kacc[i <= j ? (size_t)i * B + j : (size_t)j * B + i]);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Products over token pairs: for a 64 x 64 tile (row tokens x column tokens) P = RX X^T and Q = RY dY^T, multiplied
+// elementwise and summed per (row segment, column sequence) in float64.  Operand rows are staged 16 features at a time
+// by cp.async and read four features at once (16-byte shared loads, rows 20 floats apart: no bank conflicts); an element
+// is a sum over the even and one over the odd features, the two halves of a packed fma.
+//   Gram (kSampled = false): rows and columns are both tokens, tile pairs I <= J.  Only token pairs t <= s are used; a
+//     pair inside one sequence with t < s stands for (t,s) and (s,t) and counts twice.
+//   Sampled estimator (kSampled = true): the rows are the gathered sample rows, out = M^T[sample, sequence], no weights.
+// The tile's products go through shared memory; a warp owns 32 rows x 16 columns of them, walks the columns (sequence
+// boundaries are the same for all its lanes), and adds the lanes of one row sequence together before it issues one
+// float64 atomic.  Bound by the float32 pipe: 896 -> 896, 4608 tokens: 1207 us against 3246 us for 32 x 32 tiles loaded
+// synchronously with an atomic per token pair.
+// ---------------------------------------------------------------------------------------------
+constexpr int kGT = 64;   // tokens per tile
+constexpr int kGK = 16;   // features per stage
+constexpr int kGPitch = kGK + 4;
+constexpr int kGramStages = 3;
+
+template <bool kSampled>
+__global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
+                                                  const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
                                                   int d_in, int d_out, const int32_t* __restrict__ tokseq, int B,
-                                                  double* __restrict__ kacc) {
+                                                  double* __restrict__ out) {
   const int I = blockIdx.y, J = blockIdx.x;
-  if (J < I) return;
-  __shared__ float sA[kGT][kGT + 1];
-  __shared__ float sB[kGT][kGT + 1];
+  if (!kSampled && J < I) return;
+  __shared__ __align__(16) float stage_mem[kGramStages][2][kGT * kGPitch];
+  __shared__ int s_col[kGT];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int64_t tI = (int64_t)I * kGT, tJ = (int64_t)J * kGT;
-  float h[2][2];
-  for (int pass = 0; pass < 2; ++pass) {
-    const float* M = pass == 0 ? X : dY;
-    const int d = pass == 0 ? d_in : d_out;
-    float acc[2][2] = {};
-    for (int k0 = 0; k0 < d; k0 += kGT) {
-      for (int e = tid; e < kGT * kGT; e += 256) {
-        const int r = e / kGT, c = e % kGT;
-        sA[r][c] = (tI + r < T && k0 + c < d) ? M[(tI + r) * d + k0 + c] : 0.f;
-        sB[r][c] = (tJ + r < T && k0 + c < d) ? M[(tJ + r) * d + k0 + c] : 0.f;
+  const int64_t r0 = (int64_t)I * kGT, c0 = (int64_t)J * kGT;
+  if (tid < kGT) s_col[tid] = c0 + tid < T ? tokseq[c0 + tid] : -1;
+  const int nkx = (d_in + kGK - 1) / kGK, nky = (d_out + kGK - 1) / kGK;
+  auto fetch = [&](int k) {
+    if (k < nkx + nky) {
+      const bool second = k >= nkx;
+      const int d = second ? d_out : d_in, f0 = (second ? k - nkx : k) * kGK;
+      for (int side = 0; side < 2; ++side) {
+        const float* M = side == 0 ? (second ? RY : RX) : (second ? dY : X);
+        const int64_t first = side == 0 ? r0 : c0, end = side == 0 ? n_rows : T;
+        float* dst = stage_mem[k % kGramStages][side];
+        if ((d & 3) == 0) {
+          const int r = tid >> 2, c = (tid & 3) * 4;
+          const bool live = first + r < end && f0 + c < d;
+          cp_async16(dst + r * kGPitch + c, live ? M + (first + r) * d + f0 + c : M, live);
+        } else {
+#pragma unroll
+          for (int e = tid; e < kGT * kGK; e += 256) {
+            const int r = e / kGK, c = e % kGK;
+            const bool live = first + r < end && f0 + c < d;
+            cp_async4(dst + r * kGPitch + c, live ? M + (first + r) * d + f0 + c : M, live);
+          }
+        }
       }
-      __syncthreads();
-#pragma unroll 8
-      for (int c = 0; c < kGT; ++c) {
-        const float a0 = sA[ty * 2][c], a1 = sA[ty * 2 + 1][c], b0 = sB[tx * 2][c], b1 = sB[tx * 2 + 1][c];
-        acc[0][0] = fmaf(a0, b0, acc[0][0]);
-        acc[0][1] = fmaf(a0, b1, acc[0][1]);
-        acc[1][0] = fmaf(a1, b0, acc[1][0]);
-        acc[1][1] = fmaf(a1, b1, acc[1][1]);
-      }
-      __syncthreads();
     }
-    for (int p = 0; p < 2; ++p)
-      for (int q = 0; q < 2; ++q) h[p][q] = pass == 0 ? acc[p][q] : h[p][q] * acc[p][q];
+    cp_async_commit();
+  };
+  float h[4][4];
+  f32x2 acc[4][4] = {};
+  auto total = [](f32x2 v) { float lo, hi; unpack2(v, lo, hi); return lo + hi; };
+  for (int k = 0; k < kGramStages - 1; ++k) fetch(k);
+  for (int k = 0; k < nkx + nky; ++k) {
+    cp_async_wait<kGramStages - 2>();
+    __syncthreads();
+    fetch(k + kGramStages - 1);
+    if (k == nkx) {
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { h[p][q] = total(acc[p][q]); acc[p][q] = 0ull; }
+    }
+    const float* sA = stage_mem[k % kGramStages][0];
+    const float* sB = stage_mem[k % kGramStages][1];
+#pragma unroll
+    for (int c = 0; c < kGK; c += 4) {
+      ulonglong2 a[4], b[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        a[p] = *reinterpret_cast<const ulonglong2*>(sA + (ty + 16 * p) * kGPitch + c);
+        b[p] = *reinterpret_cast<const ulonglong2*>(sB + (tx + 16 * p) * kGPitch + c);
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = fma2(a[p].y, b[q].y, fma2(a[p].x, b[q].x, acc[p][q]));
+    }
   }
-  for (int p = 0; p < 2; ++p)
-    for (int q = 0; q < 2; ++q) {
-      const int64_t t = tI + ty * 2 + p, s = tJ + tx * 2 + q;
-      if (t >= T || s >= T || t > s) continue;
-      const int st = tokseq[t], ss = tokseq[s];
-      const double w = (st == ss && t < s) ? 2.0 : 1.0;
-      atomicAdd(&kacc[(size_t)st * B + ss], w * (double)h[p][q]);
+  cp_async_wait<0>();
+  __syncthreads();
+  float* tile = &stage_mem[0][0][0];  // [row][kGT + 1]
+  static_assert(kGT * (kGT + 1) <= kGramStages * 2 * kGT * kGPitch, "the tile reuses the stages");
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tile[(ty + 16 * p) * (kGT + 1) + tx + 16 * q] = h[p][q] * total(acc[p][q]);
+  __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31, row = (warp & 1) * 32 + lane, cb = (warp >> 1) * 16;
+  const int64_t t = r0 + row;
+  const int rseq = t < n_rows ? (kSampled ? (int)t : tokseq[t]) : -1;  // rows past the end form a run of their own, unused
+  int same = 0;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int other = __shfl_down_sync(0xffffffffu, rseq, 1 << k);
+    if (lane + (1 << k) < 32 && other == rseq) same |= 1 << k;
+  }
+  const int up = __shfl_up_sync(0xffffffffu, rseq, 1);
+  const bool head = (lane == 0 || up != rseq) && rseq >= 0;
+  double run = 0.0;
+  for (int c = 0; c < 16; ++c) {
+    const int cs = s_col[cb + c];
+    if (cs < 0) break;
+    const int64_t s = c0 + cb + c;
+    const double v = (double)tile[row * (kGT + 1) + cb + c];
+    if (kSampled) run += v;
+    else if (t <= s) run += rseq == cs && t < s ? 2.0 * v : v;
+    if (c == 15 || s_col[cb + c + 1] != cs) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const double o = __shfl_down_sync(0xffffffffu, run, 1 << k);
+        if ((same >> k) & 1) run += o;
+      }
+      if (head && run != 0.0) atomicAdd(&out[(size_t)rseq * B + cs], run);
+      run = 0.0;
     }
+  }
 }
 
 __global__ void k_f32_gram_finish(const double* __restrict__ kacc, int B, float* __restrict__ K) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= B * B) return;
-  const int i = e / B, j = e % B;
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= (int64_t)B * B) return;
+  const int i = (int)(e / B), j = (int)(e % B);
   K[e] = (float)(i <= j ? kacc[(size_t)i * B + j] : kacc[(size_t)j * B + i]);
 }
 
-__global__ void k_f32_combine(const float* __restrict__ G, int64_t N, int B, const float* __restrict__ coeffs,
-                              float* __restrict__ dW, float beta, const WsTag* __restrict__ tag_dev, WsTag tag,
-                              int32_t* __restrict__ info) {
+// dW = beta dW + sum_i c_i G_i, four elements per lane, eight 16-byte loads in flight, float64 sums.  HBM stream: 205 MB in
+// 29 us against 60 us with one 4-byte load per thread and sequence.  As in the bf16 combine a small layer splits the
+// sequences over the warps of a block (kSlices of them) and adds the shares in shared memory: 300 x 500 at 256 sequences
+// 28 us split, 120 us whole.
+template <int kSlices>
+__global__ void __launch_bounds__(256) k_f32_combine(const float* __restrict__ G, int64_t N, int64_t gstride, int B,
+                                                     const float* __restrict__ coeffs, float* __restrict__ dW, float beta,
+                                                     const WsTag* __restrict__ tag_dev, WsTag tag,
+                                                     int32_t* __restrict__ info) {
   if (!ws_tag_matches(tag_dev, tag, info)) return;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int i = 0; i < B; ++i) s += (double)coeffs[i] * (double)G[(size_t)i * N + e];
-    dW[e] = (float)(beta != 0.f ? (double)dW[e] + s : s);
+  constexpr int kLanes = 256 / kSlices;
+  __shared__ double4 part[kSlices > 1 ? 256 : 1];
+  const int x = threadIdx.x % kLanes, slice = threadIdx.x / kLanes;
+  const int per = (B + kSlices - 1) / kSlices, i1 = min(B, (slice + 1) * per);
+  for (int64_t e0 = 4 * (int64_t)blockIdx.x * kLanes; e0 < N; e0 += 4 * (int64_t)gridDim.x * kLanes) {
+    const int64_t e = e0 + 4 * x;
+    double4 s = make_double4(0.0, 0.0, 0.0, 0.0);
+    auto add = [&](const float4& v, float c) {
+      s.x += (double)c * (double)v.x; s.y += (double)c * (double)v.y;
+      s.z += (double)c * (double)v.z; s.w += (double)c * (double)v.w;
+    };
+    const float* src = G + e;
+    int i = e < N ? slice * per : i1;
+    for (; i + 8 <= i1; i += 8) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(src + (size_t)(i + u) * gstride));
+#pragma unroll
+      for (int u = 0; u < 8; ++u) add(v[u], __ldg(coeffs + i + u));
+    }
+    for (; i < i1; ++i) add(__ldcs(reinterpret_cast<const float4*>(src + (size_t)i * gstride)), __ldg(coeffs + i));
+    if (kSlices > 1) {
+      part[threadIdx.x] = s;
+      __syncthreads();
+      if (slice == 0)
+#pragma unroll
+        for (int k = 1; k < kSlices; ++k) {
+          const double4 o = part[k * kLanes + x];
+          s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+        }
+      __syncthreads();
+      if (slice != 0) continue;
+    }
+    const double v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (e + k < N) dW[e + k] = (float)(beta != 0.f ? (double)dW[e + k] + v[k] : v[k]);
   }
 }
 
@@ -339,32 +727,76 @@ isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj
   return ISOPO_OK;
 }
 
-isopo_status store_tag(const WsTag& tag, WsTag* tag_dev, cudaStream_t st) {
-  k_store_tag<<<1, 32, 0, st>>>(tag, tag_dev);
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
-}
-
-isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_dev, int B,
-                          float* G, cudaStream_t st) {
-  dim3 grid((d_in + kT - 1) / kT, (d_out + kT - 1) / kT, B);
+template <int kTile, int kT, bool kArgOff>
+static isopo_status launch_f32_seq_grad(const F32StoredArgs& a, const OffsetParam<kArgOff>& o, cudaStream_t st) {
+  typedef SeqGemm<kTile, kT> Gemm;
+  const dim3 grid((a.d_in + kTile - 1) / kTile, (a.d_out + kTile - 1) / kTile, a.B);
   if (grid.y > 65535 || grid.z > 65535) return ISOPO_ERR_UNSUPPORTED;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_seq_grad<kTile, kT, kArgOff>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   {
     LaunchScope scope(kIdF32SeqGrad, st);
-    k_f32_seq_grad<<<grid, 256, 0, st>>>(X, dY, d_in, d_out, off_dev, G);
+    k_f32_seq_grad<kTile, kT, kArgOff><<<grid, Gemm::kThr, Gemm::kSmem, st>>>(a, o);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 
-isopo_status f32_ntk(const float* G, int64_t N, int B, float* K, cudaStream_t st) {
-  if (B > 65535) return ISOPO_ERR_UNSUPPORTED;
+// 128 x 128 tiles (8 x 8 per thread) where they fill the machine twice and pad little, else 64 x 64 (4 x 4).
+static bool f32_wide_tiles(int d_in, int d_out, int64_t copies) {
+  const int64_t gx = (d_in + 127) / 128, gy = (d_out + 127) / 128, hx = (d_in + 63) / 64, hy = (d_out + 63) / 64;
+  return gx * gy * copies >= 296 && gx * gy * 4 * 4 <= hx * hy * 5;
+}
+
+isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
+                          int B, float* G, int64_t gstride, double* kacc, uint32_t* done, const WsTag& tag, WsTag* tag_dev,
+                          cudaStream_t st) {
+  F32StoredArgs a{X, dY, d_in, d_out, B, gstride, off_dev, G, kacc, done, tag, tag_dev};
+  const bool wide = f32_wide_tiles(d_in, d_out, B);
+  if (B + 1 <= kArgChunk) {
+    OffsetParam<true> o;
+    for (int i = 0; i <= B; ++i) o.v[i] = off_host[i];
+    return wide ? launch_f32_seq_grad<128, 8, true>(a, o, st) : launch_f32_seq_grad<64, 4, true>(a, o, st);
+  }
+  isopo_status s = store_i64(off_host, (int64_t)B + 1, off_dev, st);
+  if (s != ISOPO_OK) return s;
+  const OffsetParam<false> o{};
+  return wide ? launch_f32_seq_grad<128, 8, false>(a, o, st) : launch_f32_seq_grad<64, 4, false>(a, o, st);
+}
+
+template <int kMA, int kNB, bool kDiag>
+static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, int64_t pairs,
+                                   cudaStream_t st) {
+  constexpr int smem = NtkShape<kMA, kNB, kDiag>::kSmem;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_ntk<kMA, kNB, kDiag>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // every SM full over all pairs; at least eight chunks each, or the reduction outweighs the stream
+  constexpr int64_t ctas = 148 * NtkShape<kMA, kNB, kDiag>::kPerSm;
+  const int64_t chunks = (gstride + kNtkKC - 1) / kNtkKC;
+  const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + 7) / 8));
   {
     LaunchScope scope(kIdF32Ntk, st);
-    k_f32_ntk<<<dim3(B, B), 256, 0, st>>>(G, N, B, K);
+    k_f32_ntk<kMA, kNB, kDiag><<<dim3((unsigned)pairs, (unsigned)slabs), kNtkThreads, smem, st>>>(G, gstride, B, kacc, done, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
+}
+
+static isopo_status launch_f32_finish(const double* kacc, int B, float* K, cudaStream_t st) {
+  {
+    LaunchScope scope(kIdMirror, st);
+    k_f32_gram_finish<<<(unsigned)(((int64_t)B * B + 255) / 256), 256, 0, st>>>(kacc, B, K);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
+}
+
+isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, cudaStream_t st) {
+  if (B <= 16) return launch_f32_ntk<1, 2, true>(G, gstride, B, kacc, done, K, 1, st);
+  if (B <= 32) return launch_f32_ntk<2, 4, true>(G, gstride, B, kacc, done, K, 1, st);
+  const int64_t nb = (B + kNtkRows - 1) / kNtkRows;
+  isopo_status s = launch_f32_ntk<4, 8, true>(G, gstride, B, kacc, done, K, nb, st);
+  if (s != ISOPO_OK || nb == 1) return s;
+  s = launch_f32_ntk<2, 8, false>(G, gstride, B, kacc, done, K, nb * (nb - 1), st);  // two halves of nb (nb - 1) / 2 pairs
+  return s != ISOPO_OK ? s : launch_f32_finish(kacc, B, K, st);
 }
 
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
@@ -374,23 +806,54 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
   ISOPO_CUDA_TRY(cudaMemsetAsync(kacc, 0, sizeof(double) * (size_t)B * B, st));
   {
     LaunchScope scope(kIdF32Gram, st);
-    k_f32_gram<<<dim3((unsigned)nt, (unsigned)nt), 256, 0, st>>>(X, dY, T, d_in, d_out, tokseq, B, kacc);
+    k_f32_gram<false><<<dim3((unsigned)nt, (unsigned)nt), 256, 0, st>>>(X, dY, T, X, dY, T, d_in, d_out, tokseq, B, kacc);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
+  return launch_f32_finish(kacc, B, K, st);
+}
+
+isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
+                         int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st) {
+  const int64_t nt = (T + kGT - 1) / kGT, ns = (n_samples + kGT - 1) / kGT;
+  if (ns > 65535) return ISOPO_ERR_UNSUPPORTED;
+  ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(double) * (size_t)n_samples * B, st));
   {
-    LaunchScope scope(kIdMirror, st);
-    k_f32_gram_finish<<<(B * B + 255) / 256, 256, 0, st>>>(kacc, B, K);
+    LaunchScope scope(kIdSampled, st);
+    k_f32_gram<true><<<dim3((unsigned)nt, (unsigned)ns), 256, 0, st>>>(a0, g0, n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 
-isopo_status f32_combine(const float* G, int64_t N, int B, const float* coeffs, float* dW, float beta, const WsTag* tag_dev,
-                         const WsTag& tag, int32_t* info, cudaStream_t st) {
-  const int grid = (int)std::min<int64_t>((N + 255) / 256, 148 * 8);
+isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, const float* coeffs, float* dW, float beta,
+                         const WsTag* tag_dev, const WsTag& tag, int32_t* info, cudaStream_t st) {
+  // split while whole lanes would leave the machine (about 2^17 lanes of four elements in flight) mostly empty
+  const bool split = N < ((int64_t)1 << 19) && B >= 4;
+  const int64_t per_block = split ? 128 : 1024;
+  const int grid = (int)std::min<int64_t>((N + per_block - 1) / per_block, 148 * 16);
   {
     LaunchScope scope(kIdF32Combine, st);
-    k_f32_combine<<<grid, 256, 0, st>>>(G, N, B, coeffs, dW, beta, tag_dev, tag, info);
+    (split ? k_f32_combine<8> : k_f32_combine<1>)<<<grid, 256, 0, st>>>(G, N, gstride, B, coeffs, dW, beta, tag_dev, tag, info);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
+}
+
+template <int kTile, int kT>
+static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out,
+                                           const float* coeffs, const int32_t* tokseq, float* dW, cudaStream_t st) {
+  typedef SlabGemm<kTile, kT> Gemm;
+  const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
+  if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
+  // enough token slabs to fill the machine, each a multiple of the staging depth
+  int64_t splits = std::max<int64_t>(1, std::min<int64_t>((T + 255) / 256, (148 * 4 + gx * gy - 1) / (gx * gy)));
+  int64_t slab = ((T + splits - 1) / splits + 15) / 16 * 16;
+  splits = (T + slab - 1) / slab;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_weight_grad<kTile, kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
+  {
+    LaunchScope scope(kIdF32WeightGrad, st);
+    k_f32_weight_grad<kTile, kT><<<dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st>>>(X, dY, T, d_in, d_out, coeffs,
+                                                                                                  tokseq, dW, slab);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -399,18 +862,8 @@ isopo_status f32_combine(const float* G, int64_t N, int B, const float* coeffs, 
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* coeffs,
                              const int32_t* tokseq, float* dW, float beta, cudaStream_t st) {
   if (beta == 0.f) ISOPO_CUDA_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)d_in * d_out, st));
-  const int gx = (d_in + kT - 1) / kT, gy = (d_out + kT - 1) / kT;
-  if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
-  // enough token slabs to fill the machine, each a multiple of the staging depth
-  int64_t splits = std::max<int64_t>(1, std::min<int64_t>((T + 255) / 256, (148 * 4 + gx * gy - 1) / (gx * gy)));
-  int64_t slab = ((T + splits - 1) / splits + kTK - 1) / kTK * kTK;
-  splits = (T + slab - 1) / slab;
-  {
-    LaunchScope scope(kIdF32WeightGrad, st);
-    k_f32_weight_grad<<<dim3(gx, gy, (unsigned)splits), 256, 0, st>>>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, slab);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
+  return f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st)
+                                                      : launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st);
 }
 
 }  // namespace isopo
