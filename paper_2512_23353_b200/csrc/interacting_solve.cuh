@@ -221,12 +221,12 @@ __device__ __noinline__ void block_cholesky_solve(typename BlkPtr<kW>::ro Lb, co
 
 // Interacting variant, (K + lambda I) c = A: blocked Cholesky of the lower block triangle held at Lb (nb(nb+1)/2
 // blocks; shared memory, or the workspace with kW), the inverse diagonal factors at InvD, then the solve and up to
-// two refinement rounds.  Called by every thread of the CTA; `layer` tags a failed pivot in *info.
-template <bool kW>
+// two refinement rounds.  Called by every thread of a CTA of kThr; `layer` tags a failed pivot in *info.
+template <bool kW, int kThr = kSolveThreads>
 __device__ __forceinline__ void interacting_solve(const TransformParams& P, typename BlkPtr<kW>::rw Lb, float* InvD,
                                                   float* vec, double* sol, float* rdiag, double& s_trace, double& s_res,
                                                   int& s_fail, int layer) {
-  const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kSolveThreads / 32;
+  const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThr / 32;
   const float* __restrict__ K = P.K;
   const int nb = (B + kNB - 1) / kNB, Bp = nb * kNB;
   if (tid == 0) s_fail = 0;
@@ -234,16 +234,16 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
   // the blocks; float4 loads, eight in flight per thread, when B is a multiple of 4.
   if ((B & 3) == 0) {
     const int nvec = B * B / 4;
-    for (int base = tid; base < nvec; base += kSolveThreads * 8) {
+    for (int base = tid; base < nvec; base += kThr * 8) {
       float4 val[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int e = base + u * kSolveThreads;
+        const int e = base + u * kThr;
         val[u] = e < nvec ? __ldg(reinterpret_cast<const float4*>(K) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int e = base + u * kSolveThreads;
+        const int e = base + u * kThr;
         if (e >= nvec) continue;
         const int j = (e * 4) / B, i = (e * 4) % B, I = i / kNB, J = j / kNB;
         if (I < J) continue;
@@ -256,13 +256,13 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
       }
     }
   } else {
-    for (int e = tid; e < B * B; e += kSolveThreads) {
+    for (int e = tid; e < B * B; e += kThr) {
       const int j = e / B, i = e % B, I = i / kNB, J = j / kNB;
       if (I >= J) Lb[blk_slot(I, J) * kBlk + (j % kNB) * kNB + (i % kNB)] = K[e] + (i == j ? P.lambda : 0.f);
     }
   }
   // identity padding of the last block row / column
-  for (int e = tid; e < (Bp - B) * Bp; e += kSolveThreads) {
+  for (int e = tid; e < (Bp - B) * Bp; e += kThr) {
     const int i = B + e / Bp, j = e % Bp;  // rows B..Bp-1, all columns j <= i
     if (j <= i || j / kNB == i / kNB)
       Lb[blk_slot(i / kNB, j / kNB) * kBlk + (j % kNB) * kNB + (i % kNB)] = i == j ? 1.f : 0.f;
@@ -288,7 +288,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
       // all warps: rank-32 update of the next diagonal block, kNB / nwarps columns each (lane = row)
       float* Dn = Lb + blk_slot(J + 1, J + 1) * kBlk;
       const float* Pn = Lb + blk_slot(J + 1, J) * kBlk;
-      constexpr int kColsPerWarp = kNB / (kSolveThreads / 32);
+      constexpr int kColsPerWarp = kNB / (kThr / 32);
       float acc[kColsPerWarp];
 #pragma unroll
       for (int c = 0; c < kColsPerWarp; ++c) acc[c] = Dn[(warp * kColsPerWarp + c) * kNB + lane];
@@ -318,12 +318,12 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
   __syncthreads();
   if (s_fail) {
     if (tid == 0) atomicCAS(P.info, 0, s_fail + (layer << 16));
-    for (int i = tid; i < B; i += kSolveThreads) P.coeffs[i] = 0.f;
+    for (int i = tid; i < B; i += kThr) P.coeffs[i] = 0.f;
     return;
   }
   // solve, then refinement rounds with a float64 residual while it is above float32 round-off
   double anorm2 = 0.0;
-  for (int i = tid; i < Bp; i += kSolveThreads) {
+  for (int i = tid; i < Bp; i += kThr) {
     const float a = i < B ? P.A[i] : 0.f;
     vec[i] = a;
     sol[i] = 0.0;
@@ -337,7 +337,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
   anorm2 = s_trace;
   for (int round = 0; round < 3; ++round) {
     block_cholesky_solve<kW>(Lb, InvD, vec, nb);
-    for (int i = tid; i < Bp; i += kSolveThreads) sol[i] += (double)vec[i];
+    for (int i = tid; i < Bp; i += kThr) sol[i] += (double)vec[i];
     __syncthreads();
     if (round == 2) break;
     double rn2 = 0.0;
@@ -390,7 +390,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
     if (tid == 0) s_res = 0.0;
     if (done) break;
   }
-  for (int i = tid; i < B; i += kSolveThreads) P.coeffs[i] = (float)sol[i];
+  for (int i = tid; i < B; i += kThr) P.coeffs[i] = (float)sol[i];
 }
 
 // Dynamic shared memory of a CTA that runs interacting_solve<false>, and its layout.
