@@ -1,6 +1,7 @@
 // Advantage transform: one CTA turns (K, A) into the per-sequence coefficients.
-//   simple variants  - per-row sums of K in float64, one warp per row
-//   interacting      - blocked Cholesky of K + lambda*I with refinement (interacting_solve.cuh)
+//   simple variants  - per-row sums of K in float64, a few rows per warp
+//   interacting      - up to 128 sequences L D L^T in float64; more: blocked Cholesky of K + lambda*I with refinement
+//                      (interacting_solve.cuh)
 #include "interacting_solve.cuh"
 
 namespace isopo {
@@ -19,17 +20,13 @@ struct TransformBatch {
   float lambda[ISOPO_MAX_BATCH];
 };
 
-__global__ void __launch_bounds__(kThreads) k_transform(const __grid_constant__ TransformBatch batch) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+// The parameters of one layer of the batch, regularisers made absolute.
+__device__ __forceinline__ TransformParams layer_params(const TransformBatch& batch, int layer) {
   TransformParams P = batch.common;
-  P.K = batch.K[blockIdx.x];
-  P.coeffs = batch.coeffs[blockIdx.x];
-  P.rel_state = batch.rel_state[blockIdx.x];
-  P.lambda = batch.lambda[blockIdx.x];
-  __shared__ double s_trace, s_res;
-  __shared__ int s_fail;
-  const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThreads / 32;
-  const float* __restrict__ K = P.K;
+  P.K = batch.K[layer];
+  P.coeffs = batch.coeffs[layer];
+  P.rel_state = batch.rel_state[layer];
+  P.lambda = batch.lambda[layer];
   if (P.rel_state) {
     // reg(val) = val + regularization * expectation(val) of the generalised re-scaling figure: each
     // regulariser is its factor times the running mean of the quantity it is added to
@@ -43,55 +40,192 @@ __global__ void __launch_bounds__(kThreads) k_transform(const __grid_constant__ 
       default: P.reg_F *= eF; P.reg_G *= eG; P.reg_rel *= eR;
     }
   }
+  return P;
+}
 
+// Sums of squares of the rows i0, i0 + step, .. of K (four at a time, so that the loads of four rows are in flight), row by
+// row to f(i, sum) in lane 0 of the calling warp.
+template <typename F>
+__device__ __forceinline__ void row_square_sums(const float* __restrict__ K, int B, int first, int last, F f) {
+  const int lane = threadIdx.x & 31;
+  for (int i0 = first; i0 < last; i0 += 4) {
+    double sq[4] = {};
+    if ((B & 3) == 0) {
+#pragma unroll 2
+      for (int j = lane * 4; j < B; j += 128) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(K + (size_t)min(i0 + u, last - 1) * B + j));
+          sq[u] += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+        }
+      }
+    } else {
+      for (int j = lane; j < B; j += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double v = (double)__ldg(K + (size_t)min(i0 + u, last - 1) * B + j);
+          sq[u] += v * v;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sq[u] = warp_sum(sq[u]);
+    if (lane == 0)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < last) f(i0 + u, sq[u]);
+  }
+}
+// Sum over a block of kWarps warps, in the same order in every thread.
+template <int kWarps>
+__device__ __forceinline__ double block_total(double v, double* s_part) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) t += s_part[w];
+  return t;
+}
+
+// Simple variants.  Block (l, y): rows 32 y .. 32 y + 31 of layer l, four per warp; every block adds the trace up for
+// itself.  Bound by latency: the seven layers of a block at 256 sequences took 25 us with one CTA per layer.
+constexpr int kSimpleRows = 32;
+__global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant__ TransformBatch batch) {
+  const TransformParams P = layer_params(batch, blockIdx.x);
+  __shared__ double s_part[8];
+  const int B = P.B, tid = threadIdx.x, first = blockIdx.y * kSimpleRows;
+  const float* __restrict__ K = P.K;
   if (P.variant == ISOPO_VAR_REINFORCE) {
-    for (int i = tid; i < B; i += kThreads) P.coeffs[i] = P.A[i];
+    if (tid < kSimpleRows && first + tid < B) P.coeffs[first + tid] = P.A[first + tid];
     return;
   }
+  double tr = 0.0;
+  for (int i = tid; i < B; i += 256) tr += (double)__ldg(K + (size_t)i * B + i);
+  __shared__ double s_sq[kSimpleRows];
+  const int r0 = first + (tid >> 5) * 4;
+  row_square_sums(K, B, r0, min(B, r0 + 4), [&](int i, double sq) { s_sq[i - first] = sq; });
+  const double trace = block_total<8>(tr, s_part);
+  const int i = first + tid;
+  if (tid >= kSimpleRows || i >= B) return;
+  const double sq = s_sq[tid], n2 = (double)K[(size_t)i * B + i];
+  const double F2 = P.variant == ISOPO_VAR_NORMALISED_RAW ? sq / (double)B : sq / trace;
+  const double a = (double)P.A[i], lam = (double)P.lambda;
+  double c;
+  switch (P.variant) {
+    case ISOPO_VAR_NORMALISED:
+    case ISOPO_VAR_NORMALISED_RAW: c = a / sqrt(F2 + lam); break;
+    case ISOPO_VAR_DIRECTION: c = a / (F2 / n2 + lam); break;
+    case ISOPO_VAR_EUCLID: c = a / sqrt(n2 + lam); break;
+    default: {  // ISOPO_VAR_GENERAL
+      const double eps = 1e-8;
+      const double rF = sqrt(F2 + (double)P.reg_F + eps);
+      const double rG = sqrt(n2 + (double)P.reg_G + eps);
+      const double rR = sqrt(F2 / n2 + (double)P.reg_rel + eps);
+      c = a * pow(rF, (double)P.p) * pow(rG, (double)P.q) * pow(rR, (double)P.r);
+    }
+  }
+  P.coeffs[i] = (float)c;
+}
 
-  if (P.variant != ISOPO_VAR_INTERACTING) {
-    // trace of K
-    double tr = 0.0;
-    for (int i = tid; i < B; i += kThreads) tr += (double)K[(size_t)i * B + i];
-    tr = warp_sum(tr);
-    if (tid == 0) s_trace = 0.0;
-    __syncthreads();
-    if (lane == 0) atomicAdd(&s_trace, tr);
-    __syncthreads();
-    const double trace = s_trace;
-    for (int i = warp; i < B; i += nwarps) {
-      double sq = 0.0;
-      for (int j = lane; j < B; j += 32) {
-        const double kij = (double)K[(size_t)i * B + j];
-        sq += kij * kij;
-      }
-      sq = warp_sum(sq);
-      if (lane == 0) {
-        const double n2 = (double)K[(size_t)i * B + i];
-        const double F2 = P.variant == ISOPO_VAR_NORMALISED_RAW ? sq / (double)B : sq / trace;
-        const double a = (double)P.A[i], lam = (double)P.lambda;
-        double c;
-        switch (P.variant) {
-          case ISOPO_VAR_NORMALISED:
-          case ISOPO_VAR_NORMALISED_RAW: c = a / sqrt(F2 + lam); break;
-          case ISOPO_VAR_DIRECTION: c = a / (F2 / n2 + lam); break;
-          case ISOPO_VAR_EUCLID: c = a / sqrt(n2 + lam); break;
-          default: {  // ISOPO_VAR_GENERAL
-            const double eps = 1e-8;
-            const double rF = sqrt(F2 + (double)P.reg_F + eps);
-            const double rG = sqrt(n2 + (double)P.reg_G + eps);
-            const double rR = sqrt(F2 / n2 + (double)P.reg_rel + eps);
-            c = a * pow(rF, (double)P.p) * pow(rG, (double)P.q) * pow(rR, (double)P.r);
-          }
+// Interacting variant, up to 128 sequences: (K + lambda I) c = A by L D L^T in float64, one CTA per layer.
+// Thread (ty, tx) of a 16 x 16 grid keeps the elements (ty + 16 p, tx + 16 q) in registers; step k publishes column k in
+// shared memory (where L stays for the backward solve), and after ONE barrier everybody subtracts its rank-1 share; the
+// right-hand side rides along, one element per thread.  The backward solve is one warp's work.
+// Bound by latency: per column a barrier, a shared load, a division and two multiply-adds follow one another.  In float64
+// the solution needs no refinement.  The blocked float32 kernel below spends most of its time, at these sizes, on fetching
+// its unrolled code once and on refinement: 64 sequences 34 us there, 128 sequences 45 us.
+template <int kA>
+__global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__ TransformBatch batch) {
+  extern __shared__ __align__(16) double smem_d[];
+  const TransformParams P = layer_params(batch, blockIdx.x);
+  const int B = P.B, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, pitch = B | 1;
+  double* col = smem_d;             // [k * pitch + i], i >= k: column k before its division by the pivot
+  double* y = col + (size_t)B * pitch;
+  double* inv_d = y + B;
+  double a[kA][kA];
+#pragma unroll
+  for (int p = 0; p < kA; ++p)
+#pragma unroll
+    for (int q = 0; q <= p; ++q) {
+      const int i = ty + 16 * p, j = tx + 16 * q;
+      a[p][q] = i < B && j < B ? (double)__ldg(P.K + (size_t)i * B + j) + (i == j ? (double)P.lambda : 0.0) : 0.0;
+    }
+  double rhs = tid < B ? (double)P.A[tid] : 0.0;
+  int fail = 0;
+#pragma unroll
+  for (int q = 0; q < kA; ++q) {
+#pragma unroll 1
+    for (int k = 16 * q; k < min(B, 16 * q + 16) && !fail; ++k) {
+      double* ck = col + (size_t)k * pitch;
+      if (tx == (k & 15)) {
+#pragma unroll
+        for (int p = q; p < kA; ++p) {
+          const int i = ty + 16 * p;
+          if (i >= k && i < B) ck[i] = a[p][q];
         }
-        P.coeffs[i] = (float)c;
+      }
+      if (tid == k) y[k] = rhs;
+      __syncthreads();
+      const double d = ck[k];
+      if (!(d > 0.0)) { fail = k + 1; break; }  // the same in every thread
+      const double inv = 1.0 / d;
+      if (tid == 0) inv_d[k] = inv;
+      double cj[kA];  // rows and columns up to k, and past B, take part with whatever they hold: nothing reads them again
+#pragma unroll
+      for (int p = q; p < kA; ++p) cj[p] = ck[min(tx + 16 * p, B - 1)];
+#pragma unroll
+      for (int p = q; p < kA; ++p) {
+        const double t = ck[min(ty + 16 * p, B - 1)] * inv;
+#pragma unroll
+        for (int r = q; r <= p; ++r) a[p][r] -= t * cj[r];
+      }
+      if (tid > k && tid < B) rhs -= ck[tid] * inv * y[k];
+    }
+  }
+  if (fail) {
+    if (tid == 0) atomicCAS(P.info, 0, fail + ((int)blockIdx.x << 16));
+    if (tid < B) P.coeffs[tid] = 0.f;
+    return;
+  }
+  __syncthreads();
+  if (tid >= 32) return;
+  // L^T x = D^-1 y, lane l holds the elements l + 32 c
+  constexpr int kC = (kA + 1) / 2;
+  double x[kC], w[kC], l[kC];
+#pragma unroll
+  for (int c = 0; c < kC; ++c) {
+    const int j = tid + 32 * c;
+    w[c] = j < B ? inv_d[j] : 0.0;
+    x[c] = j < B ? y[j] * w[c] : 0.0;
+    l[c] = j < B - 1 ? col[(size_t)j * pitch + B - 1] : 0.0;
+  }
+#pragma unroll
+  for (int c = kC - 1; c >= 0; --c) {
+#pragma unroll 1
+    for (int k = min(B, 32 * c + 32) - 1; k >= 32 * c; --k) {
+      const double xk = __shfl_sync(0xffffffffu, x[c], k & 31);
+#pragma unroll
+      for (int b = 0; b <= c; ++b) {
+        const int j = tid + 32 * b;
+        x[b] -= l[b] * w[b] * xk;
+        l[b] = j < k - 1 ? col[(size_t)j * pitch + k - 1] : 0.0;  // row k - 1 of L D
       }
     }
-    return;
   }
+#pragma unroll
+  for (int c = 0; c < kC; ++c)
+    if (tid + 32 * c < B) P.coeffs[tid + 32 * c] = (float)x[c];
+}
+constexpr int kMaxSmallB = 128;
+inline size_t small_smem_bytes(int B) { return sizeof(double) * ((size_t)B * (B | 1) + 2 * (size_t)B); }
 
-  // ---------------- interacting: (K + lambda I) c = A ----------------
-  const SolveSmem m = solve_smem(smem_raw, B);
+// Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
+__global__ void __launch_bounds__(kThreads) k_transform(const __grid_constant__ TransformBatch batch) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const TransformParams P = layer_params(batch, blockIdx.x);
+  __shared__ double s_trace, s_res;
+  __shared__ int s_fail;
+  const SolveSmem m = solve_smem(smem_raw, P.B);
   interacting_solve<false>(P, m.Lb, m.InvD, m.vec, m.sol, m.rdiag, s_trace, s_res, s_fail, (int)blockIdx.x);
 }
 
@@ -112,34 +246,26 @@ __global__ void __launch_bounds__(kThreads) k_transform_large(const TransformPar
 
 // Running means for the relative regulariser.  state = {E[F^2], E[||G||^2], E[F^2 / ||G||^2], number of updates};
 // the first update stores this microbatch's means, later ones blend: s <- decay * s + (1 - decay) * mean.
-__global__ void __launch_bounds__(kThreads) k_reg_ema(const float* __restrict__ K, int B, float decay,
-                                                      float* __restrict__ state) {
-  __shared__ double s_trace, s_f2, s_rel;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThreads / 32;
-  double tr = 0.0;
-  for (int i = tid; i < B; i += kThreads) tr += (double)K[(size_t)i * B + i];
+// One pass: F_i^2 = sum_j K_ij^2 / tr K, so all three means follow from sums of row sums.
+constexpr int kEmaThreads = 1024;
+__global__ void __launch_bounds__(kEmaThreads) k_reg_ema(const float* __restrict__ K, int B, float decay,
+                                                         float* __restrict__ state) {
+  __shared__ double s_part[3][kEmaThreads / 32];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  double tr = 0.0, f2 = 0.0, rel = 0.0;
+  for (int i = tid; i < B; i += kEmaThreads) tr += (double)__ldg(K + (size_t)i * B + i);
+  for (int i0 = warp * 4; i0 < B; i0 += kEmaThreads / 8)
+    row_square_sums(K, B, i0, min(B, i0 + 4), [&](int i, double sq) {
+      f2 += sq;
+      rel += sq / (double)__ldg(K + (size_t)i * B + i);
+    });
   tr = warp_sum(tr);
-  if (tid == 0) { s_trace = 0.0; s_f2 = 0.0; s_rel = 0.0; }
+  if ((tid & 31) == 0) { s_part[0][warp] = tr; s_part[1][warp] = f2; s_part[2][warp] = rel; }
   __syncthreads();
-  if (lane == 0) atomicAdd(&s_trace, tr);
-  __syncthreads();
-  const double trace = s_trace;
-  double f2_sum = 0.0, rel_sum = 0.0;
-  for (int i = warp; i < B; i += nwarps) {
-    double sq = 0.0;
-    for (int j = lane; j < B; j += 32) {
-      const double kij = (double)K[(size_t)i * B + j];
-      sq += kij * kij;
-    }
-    sq = warp_sum(sq);
-    const double F2 = sq / trace;
-    f2_sum += F2;
-    rel_sum += F2 / (double)K[(size_t)i * B + i];
-  }
-  if (lane == 0) { atomicAdd(&s_f2, f2_sum); atomicAdd(&s_rel, rel_sum); }
-  __syncthreads();
+  if (warp != 0) return;
+  const double trace = warp_sum(s_part[0][tid]), f2_sum = warp_sum(s_part[1][tid]) / trace, rel_sum = warp_sum(s_part[2][tid]) / trace;
   if (tid == 0) {
-    const double m[3] = {s_f2 / B, trace / B, s_rel / B};
+    const double m[3] = {f2_sum / B, trace / B, rel_sum / B};
     const bool first = state[3] == 0.f;
     for (int k = 0; k < 3; ++k)
       state[k] = (float)(first ? m[k] : (double)decay * (double)state[k] + (1.0 - (double)decay) * m[k]);
@@ -152,7 +278,7 @@ __global__ void __launch_bounds__(kThreads) k_reg_ema(const float* __restrict__ 
 isopo_status reg_ema_update(const float* K, int B, float decay, float* state, cudaStream_t st) {
   {
     LaunchScope scope(kIdTransform, st);
-    k_reg_ema<<<1, kThreads, 0, st>>>(K, B, decay, state);
+    k_reg_ema<<<1, kEmaThreads, 0, st>>>(K, B, decay, state);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -171,15 +297,20 @@ isopo_status transform_batched(int n, const float* const* K, const float* A, int
     T.rel_state[l] = rel_state ? rel_state[l] : nullptr;
     T.lambda[l] = lambda[l];
   }
-  size_t smem = 0;
-  if (v == ISOPO_VAR_INTERACTING) {
-    if (B > kMaxB) return ISOPO_ERR_UNSUPPORTED;
-    smem = solve_smem_bytes(B);
-    ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  }
-  {
+  if (v != ISOPO_VAR_INTERACTING) {
     LaunchScope scope(kIdTransform, st);
-    k_transform<<<n, kThreads, smem, st>>>(T);
+    k_transform_simple<<<dim3(n, (B + kSimpleRows - 1) / kSimpleRows), 256, 0, st>>>(T);
+  } else if (B <= kMaxSmallB) {
+    auto kernel = B <= 16 ? k_transform_small<1> : B <= 32 ? k_transform_small<2> : B <= 64 ? k_transform_small<4> : k_transform_small<8>;
+    const size_t smem = small_smem_bytes(B);
+    if (smem > 48 * 1024) ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    LaunchScope scope(kIdTransform, st);
+    kernel<<<n, 256, smem, st>>>(T);
+  } else {
+    if (B > kMaxB) return ISOPO_ERR_UNSUPPORTED;
+    ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    LaunchScope scope(kIdTransform, st);
+    k_transform<<<n, kThreads, solve_smem_bytes(B), st>>>(T);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -193,6 +324,7 @@ size_t transform_large_workspace_bytes(int B) {
 isopo_status transform_large(const float* K, const float* A, int B, float lambda, float* coeffs, float* scratch,
                              int32_t* info, cudaStream_t st) {
   if (B < 1 || B > kMaxLargeB) return ISOPO_ERR_UNSUPPORTED;
+  if (B <= kMaxSmallB) return transform(K, A, B, ISOPO_VAR_INTERACTING, lambda, nullptr, nullptr, coeffs, info, st);
   TransformParams P{};
   P.K = K; P.A = A; P.coeffs = coeffs; P.info = info; P.B = B; P.variant = (int)ISOPO_VAR_INTERACTING; P.lambda = lambda;
   const size_t nb = (size_t)(B + kNB - 1) / kNB;
