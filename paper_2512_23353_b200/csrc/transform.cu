@@ -127,60 +127,86 @@ __global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant_
   P.coeffs[i] = (float)c;
 }
 
-// Interacting variant, up to 128 sequences: (K + lambda I) c = A by L D L^T in float64, one CTA per layer.
-// Thread (ty, tx) of a 16 x 16 grid keeps the elements (ty + 16 p, tx + 16 q) in registers; step k publishes column k in
-// shared memory (where L stays for the backward solve), and after ONE barrier everybody subtracts its rank-1 share; the
-// right-hand side rides along, one element per thread.  The backward solve is one warp's work.
-// Bound by latency: per column a barrier, a shared load, a division and two multiply-adds follow one another.  In float64
-// the solution needs no refinement.  The blocked float32 kernel below spends most of its time, at these sizes, on fetching
-// its unrolled code once and on refinement: 64 sequences 34 us there, 128 sequences 45 us.
+// Interacting variant, up to 128 sequences: (K + lambda I) c = A in float64 by block elimination with 2 x 2 pivots (a
+// block L D L^T), one CTA per layer.  Thread (ty, tx) of a 16 x 16 grid keeps the elements (ty + 16 p, tx + 16 q) in
+// registers.  A step publishes two columns C in shared memory, and after ONE barrier everybody forms the rows of
+// T = C P^-1, P the pivot, that it needs and subtracts T C^T from its elements; the right-hand side rides along, one
+// element per thread.  T stays in shared memory for the backward solve, one warp's work.  An odd last row gets a unit row.
+// Bound by latency: a step's barrier, shared load, reciprocal and some ten dependent float64 operations.  Single columns
+// (one reciprocal and one barrier each) took 16.4 us at 64 and 41 us at 128 sequences, this 14.7 and 36.9.  In float64 the
+// solution needs no refinement; the blocked float32 kernel below, which does, takes 21.5 and 39 us when its unrolled code
+// is in the instruction cache and about twice that when a GEMM ran before it.
+// 1 / d by Newton's iteration from the hardware's approximation (about 20 bits; twice gives all 53).
+__device__ __forceinline__ double newton_rcp(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
+}
 template <int kA>
 __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__ TransformBatch batch) {
   extern __shared__ __align__(16) double smem_d[];
   const TransformParams P = layer_params(batch, blockIdx.x);
-  const int B = P.B, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, pitch = B | 1;
-  double* col = smem_d;             // [k * pitch + i], i >= k: column k before its division by the pivot
-  double* y = col + (size_t)B * pitch;
-  double* inv_d = y + B;
+  const int B = P.B, n = B + (B & 1), tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, pitch = n + 1;
+  double* T = smem_d;                            // [k * pitch + i]: T(i, k), i > k
+  double* y = T + (size_t)n * pitch;             // D^-1 y
+  double2* col = reinterpret_cast<double2*>(y + n);  // [2][n]: the two columns of a step, two buffers
+  double2* ycol = col + 2 * n;                   // [2]: the right-hand side's two elements
   double a[kA][kA];
 #pragma unroll
   for (int p = 0; p < kA; ++p)
 #pragma unroll
     for (int q = 0; q <= p; ++q) {
       const int i = ty + 16 * p, j = tx + 16 * q;
-      a[p][q] = i < B && j < B ? (double)__ldg(P.K + (size_t)i * B + j) + (i == j ? (double)P.lambda : 0.0) : 0.0;
+      a[p][q] = i < B && j < B ? (double)__ldg(P.K + (size_t)i * B + j) + (i == j ? (double)P.lambda : 0.0) : i == j ? 1.0 : 0.0;
     }
+  int iy[kA], jx[kA];  // this thread's rows and columns, kept inside the matrix
+#pragma unroll
+  for (int p = 0; p < kA; ++p) { iy[p] = min(ty + 16 * p, n - 1); jx[p] = min(tx + 16 * p, n - 1); }
   double rhs = tid < B ? (double)P.A[tid] : 0.0;
   int fail = 0;
 #pragma unroll
   for (int q = 0; q < kA; ++q) {
 #pragma unroll 1
-    for (int k = 16 * q; k < min(B, 16 * q + 16) && !fail; ++k) {
-      double* ck = col + (size_t)k * pitch;
-      if (tx == (k & 15)) {
+    for (int k = 16 * q; k < min(n, 16 * q + 16); k += 2) {
+      double2* c = col + ((k >> 1) & 1) * n;
+      double2* yc = ycol + ((k >> 1) & 1);
+      if ((tx & ~1) == (k & 15)) {
+        double* half = reinterpret_cast<double*>(c) + (tx & 1);
 #pragma unroll
         for (int p = q; p < kA; ++p) {
           const int i = ty + 16 * p;
-          if (i >= k && i < B) ck[i] = a[p][q];
+          if (i >= k && i < n) half[2 * i] = a[p][q];
         }
       }
-      if (tid == k) y[k] = rhs;
+      if ((tid & ~1) == k) reinterpret_cast<double*>(yc)[tid & 1] = rhs;
       __syncthreads();
-      const double d = ck[k];
-      if (!(d > 0.0)) { fail = k + 1; break; }  // the same in every thread
-      const double inv = 1.0 / d;
-      if (tid == 0) inv_d[k] = inv;
-      double cj[kA];  // rows and columns up to k, and past B, take part with whatever they hold: nothing reads them again
+      const double2 r0 = c[k], r1 = c[k + 1];  // P = [r0.x r1.x; r1.x r1.y]
+      const double det = fma(r0.x, r1.y, -(r1.x * r1.x));
+      if (!(r0.x > 0.0)) fail = k + 1;
+      else if (!(det > 0.0)) fail = k + 2;
+      if (fail) break;  // the same in every thread
+      const double inv = newton_rcp(det);
+      const double p00 = r1.y * inv, p01 = -r1.x * inv, p11 = r0.x * inv;  // P^-1
+      const double2 yk = *yc;
+      if (tid == 0) { y[k] = p00 * yk.x + p01 * yk.y; y[k + 1] = p01 * yk.x + p11 * yk.y; }
+      double2 cj[kA];  // rows and columns up to k + 1 take part with whatever they hold: nothing reads them again
 #pragma unroll
-      for (int p = q; p < kA; ++p) cj[p] = ck[min(tx + 16 * p, B - 1)];
+      for (int p = q; p < kA; ++p) cj[p] = c[jx[p]];
 #pragma unroll
       for (int p = q; p < kA; ++p) {
-        const double t = ck[min(ty + 16 * p, B - 1)] * inv;
+        const double2 ci = c[iy[p]];
+        const double t0 = fma(p00, ci.x, p01 * ci.y), t1 = fma(p01, ci.x, p11 * ci.y);
 #pragma unroll
-        for (int r = q; r <= p; ++r) a[p][r] -= t * cj[r];
+        for (int r = q; r <= p; ++r) a[p][r] = fma(-t1, cj[r].y, fma(-t0, cj[r].x, a[p][r]));
+        if (tx < 2 && ty + 16 * p < n) T[(size_t)(k + tx) * pitch + ty + 16 * p] = tx ? t1 : t0;
       }
-      if (tid > k && tid < B) rhs -= ck[tid] * inv * y[k];
+      if (tid > k + 1 && tid < B) {
+        const double2 ci = c[tid];
+        rhs = fma(-fma(p01, ci.x, p11 * ci.y), yk.y, fma(-fma(p00, ci.x, p01 * ci.y), yk.x, rhs));
+      }
     }
+    if (fail) break;
   }
   if (fail) {
     if (tid == 0) atomicCAS(P.info, 0, fail + ((int)blockIdx.x << 16));
@@ -189,26 +215,27 @@ __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__
   }
   __syncthreads();
   if (tid >= 32) return;
-  // L^T x = D^-1 y, lane l holds the elements l + 32 c
+  // x_J = P_J^-1 y_J - sum over later rows k of T(k, J) x_k; lane l holds the elements l + 32 c
   constexpr int kC = (kA + 1) / 2;
-  double x[kC], w[kC], l[kC];
+  double x[kC], l0[kC], l1[kC];
 #pragma unroll
   for (int c = 0; c < kC; ++c) {
     const int j = tid + 32 * c;
-    w[c] = j < B ? inv_d[j] : 0.0;
-    x[c] = j < B ? y[j] * w[c] : 0.0;
-    l[c] = j < B - 1 ? col[(size_t)j * pitch + B - 1] : 0.0;
+    x[c] = j < n ? y[j] : 0.0;
+    l0[c] = j < n - 2 ? T[(size_t)j * pitch + n - 2] : 0.0;
+    l1[c] = j < n - 2 ? T[(size_t)j * pitch + n - 1] : 0.0;
   }
 #pragma unroll
   for (int c = kC - 1; c >= 0; --c) {
 #pragma unroll 1
-    for (int k = min(B, 32 * c + 32) - 1; k >= 32 * c; --k) {
-      const double xk = __shfl_sync(0xffffffffu, x[c], k & 31);
+    for (int k = min(n, 32 * c + 32) - 2; k >= 32 * c; k -= 2) {
+      const double x0 = __shfl_sync(0xffffffffu, x[c], k & 31), x1 = __shfl_sync(0xffffffffu, x[c], (k & 31) + 1);
 #pragma unroll
       for (int b = 0; b <= c; ++b) {
         const int j = tid + 32 * b;
-        x[b] -= l[b] * w[b] * xk;
-        l[b] = j < k - 1 ? col[(size_t)j * pitch + k - 1] : 0.0;  // row k - 1 of L D
+        x[b] = fma(-l1[b], x1, fma(-l0[b], x0, x[b]));
+        l0[b] = j < k - 2 ? T[(size_t)j * pitch + k - 2] : 0.0;
+        l1[b] = j < k - 2 ? T[(size_t)j * pitch + k - 1] : 0.0;
       }
     }
   }
@@ -217,7 +244,10 @@ __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__
     if (tid + 32 * c < B) P.coeffs[tid + 32 * c] = (float)x[c];
 }
 constexpr int kMaxSmallB = 128;
-inline size_t small_smem_bytes(int B) { return sizeof(double) * ((size_t)B * (B | 1) + 2 * (size_t)B); }
+inline size_t small_smem_bytes(int B) {
+  const size_t n = (size_t)B + (B & 1);
+  return sizeof(double) * (n * (n + 1) + n + 4 * n + 4);
+}
 
 // Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
 __global__ void __launch_bounds__(kThreads) k_transform(const __grid_constant__ TransformBatch batch) {
