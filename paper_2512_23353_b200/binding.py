@@ -153,8 +153,18 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+# The current stream's handle without building a torch.cuda.Stream object: 0.2 us instead of 3 us per call, of a call that
+# takes 5 us on the host otherwise.
+_current_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
+
+
+def _addr(a: np.ndarray) -> int:
+    """Address of an array's data (`a.ctypes.data` builds two objects to get at it)."""
+    return a.__array_interface__["data"][0]
 
 
 def _offsets(seq_offsets) -> np.ndarray:
@@ -190,9 +200,9 @@ def isopo_layer_gram(X: torch.Tensor, dY: torch.Tensor, seq_offsets, K: torch.Te
     assert X.is_cuda and dY.is_cuda and X.is_contiguous() and dY.is_contiguous() and X.dtype == dY.dtype
     assert K.dtype == torch.float32 and K.is_contiguous() and K.numel() == B * B
     assert info.dtype == torch.int32 and ws.dtype == torch.uint8
-    st = lib.isopo_layer_gram(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1], dY.shape[1],
-                              off.ctypes.data, B, path, K.data_ptr(), ws.data_ptr(), ws.numel(), info.data_ptr(),
-                              _stream())
+    T, d_in = X.shape
+    st = lib.isopo_layer_gram(X.data_ptr(), dY.data_ptr(), _dtype_code(X), T, d_in, dY.shape[1], _addr(off), B, path,
+                              K.data_ptr(), ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_layer_gram")
 
 
@@ -208,8 +218,8 @@ def isopo_layer_gram_shared_x(X: torch.Tensor, dYs, seq_offsets, Ks, ws: torch.T
     dy_ptrs = np.array([d.data_ptr() for d in dYs], dtype=np.uint64)
     k_ptrs = np.array([K.data_ptr() for K in Ks], dtype=np.uint64)
     widths = np.array([d.shape[1] for d in dYs], dtype=np.int32)
-    st = lib.isopo_layer_gram_shared_x(X.data_ptr(), n, dy_ptrs.ctypes.data, widths.ctypes.data, _dtype_code(X),
-                                       X.shape[0], X.shape[1], off.ctypes.data, B, k_ptrs.ctypes.data, ws.data_ptr(),
+    st = lib.isopo_layer_gram_shared_x(X.data_ptr(), n, _addr(dy_ptrs), _addr(widths), _dtype_code(X),
+                                       X.shape[0], X.shape[1], _addr(off), B, _addr(k_ptrs), ws.data_ptr(),
                                        ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_layer_gram_shared_x")
 
@@ -229,9 +239,9 @@ def isopo_layer_gram_shared_x_stored(X: torch.Tensor, dYs, seq_offsets, Ks, wss,
     ws_ptrs = np.array([w.data_ptr() for w in wss], dtype=np.uint64)
     ws_sizes = np.array([w.numel() for w in wss], dtype=np.uint64)
     widths = np.array([d.shape[1] for d in dYs], dtype=np.int32)
-    st = lib.isopo_layer_gram_shared_x_stored(X.data_ptr(), n, dy_ptrs.ctypes.data, widths.ctypes.data, _dtype_code(X),
-                                              X.shape[0], X.shape[1], off.ctypes.data, B, k_ptrs.ctypes.data,
-                                              ws_ptrs.ctypes.data, ws_sizes.ctypes.data, info.data_ptr(), _stream())
+    st = lib.isopo_layer_gram_shared_x_stored(X.data_ptr(), n, _addr(dy_ptrs), _addr(widths), _dtype_code(X),
+                                              X.shape[0], X.shape[1], _addr(off), B, _addr(k_ptrs),
+                                              _addr(ws_ptrs), _addr(ws_sizes), info.data_ptr(), _stream())
     _check(st, "isopo_layer_gram_shared_x_stored")
 
 
@@ -245,7 +255,7 @@ def isopo_layer_gram_static(X: torch.Tensor, dY: torch.Tensor, seq_offsets, K: t
     assert X.is_cuda and dY.is_cuda and X.is_contiguous() and dY.is_contiguous() and X.dtype == dY.dtype
     assert K.dtype == torch.float32 and K.is_contiguous() and K.numel() == B * B and info.dtype == torch.int32
     st = lib.isopo_layer_gram_static(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1],
-                                     dY.shape[1], off.ctypes.data, B, K.data_ptr(), info.data_ptr(), _stream())
+                                     dY.shape[1], _addr(off), B, K.data_ptr(), info.data_ptr(), _stream())
     if st == ERR_UNSUPPORTED:
         raise IsopoError(st, f"isopo_layer_gram_static: ISOPO_ERR_UNSUPPORTED [{lib.isopo_last_cuda_error().decode()}]")
     _check(st, "isopo_layer_gram_static")
@@ -261,7 +271,7 @@ def isopo_transform_advantages(K: torch.Tensor, A: torch.Tensor, variant: int, l
         g = np.ascontiguousarray(np.asarray(pqr_regs, dtype=np.float32))
         assert g.shape == (6,)
     st = lib.isopo_transform_advantages(K.data_ptr(), A.data_ptr(), B, variant, float(lam),
-                                        g.ctypes.data if g is not None else None, coeffs.data_ptr(),
+                                        _addr(g) if g is not None else None, coeffs.data_ptr(),
                                         info.data_ptr(), _stream())
     _check(st, "isopo_transform_advantages")
 
@@ -299,7 +309,7 @@ def isopo_transform_advantages_rel(K: torch.Tensor, A: torch.Tensor, variant: in
         g = np.ascontiguousarray(np.asarray(pqr_factors, dtype=np.float32))
         assert g.shape == (6,)
     st = lib.isopo_transform_advantages_rel(K.data_ptr(), A.data_ptr(), B, variant, float(factor),
-                                            g.ctypes.data if g is not None else None, state.data_ptr(),
+                                            _addr(g) if g is not None else None, state.data_ptr(),
                                             coeffs.data_ptr(), info.data_ptr(), _stream())
     _check(st, "isopo_transform_advantages_rel")
 
@@ -326,10 +336,10 @@ def isopo_transform_advantages_batched(Ks, A: torch.Tensor, variant: int, lams, 
     if pqr_regs is not None:
         g = np.ascontiguousarray(np.asarray(pqr_regs, dtype=np.float32))
         assert g.shape == (6,)
-    st = lib.isopo_transform_advantages_batched(n, k_ptrs.ctypes.data, A.data_ptr(), B, variant, lam.ctypes.data,
-                                                g.ctypes.data if g is not None else None,
-                                                s_ptrs.ctypes.data if s_ptrs is not None else None,
-                                                c_ptrs.ctypes.data, info.data_ptr(), _stream())
+    st = lib.isopo_transform_advantages_batched(n, _addr(k_ptrs), A.data_ptr(), B, variant, _addr(lam),
+                                                _addr(g) if g is not None else None,
+                                                _addr(s_ptrs) if s_ptrs is not None else None,
+                                                _addr(c_ptrs), info.data_ptr(), _stream())
     _check(st, "isopo_transform_advantages_batched")
 
 
@@ -369,8 +379,8 @@ def isopo_transform_spectral_batched(Ks, A: torch.Tensor, lams, coeffs, info: to
     lam = np.ascontiguousarray(np.asarray(lams, dtype=np.float32))
     if ws is None:
         ws = torch.empty(n * lib.isopo_spectral_workspace_bytes(), dtype=torch.uint8, device=A.device)
-    st = lib.isopo_transform_spectral_batched(n, k_ptrs.ctypes.data, A.data_ptr(), B, lam.ctypes.data, float(rel_cutoff),
-                                              c_ptrs.ctypes.data, e_ptrs.ctypes.data if e_ptrs is not None else None,
+    st = lib.isopo_transform_spectral_batched(n, _addr(k_ptrs), A.data_ptr(), B, _addr(lam), float(rel_cutoff),
+                                              _addr(c_ptrs), _addr(e_ptrs) if e_ptrs is not None else None,
                                               ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_transform_spectral_batched")
 
@@ -379,10 +389,11 @@ def isopo_weight_grad(X: torch.Tensor, dY: torch.Tensor, coeffs: torch.Tensor, s
                       ws: torch.Tensor, info: torch.Tensor, path: int = PATH_AUTO, beta: float = 0.0) -> None:
     off = _offsets(seq_offsets)
     B = off.shape[0] - 1
-    assert dW.dtype == torch.float32 and dW.is_contiguous() and dW.shape == (dY.shape[1], X.shape[1])
+    (T, d_in), d_out = X.shape, dY.shape[1]
+    assert dW.dtype == torch.float32 and dW.is_contiguous() and dW.shape == (d_out, d_in)
     assert coeffs.dtype == torch.float32 and coeffs.numel() == B
-    st = lib.isopo_weight_grad(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1], dY.shape[1],
-                               coeffs.data_ptr(), off.ctypes.data, B, path, dW.data_ptr(), float(beta),
+    st = lib.isopo_weight_grad(X.data_ptr(), dY.data_ptr(), _dtype_code(X), T, d_in, d_out,
+                               coeffs.data_ptr(), _addr(off), B, path, dW.data_ptr(), float(beta),
                                ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_weight_grad")
 
@@ -410,7 +421,7 @@ def isopo_sampled_coefficients(X: torch.Tensor, dY: torch.Tensor, seq_offsets, s
     assert A.dtype == torch.float32 and coeffs.dtype == torch.float32 and A.numel() == B and coeffs.numel() == B
     assert F2 is None or (F2.dtype == torch.float32 and F2.numel() == B)
     st = lib.isopo_sampled_coefficients(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1], dY.shape[1],
-                                        off.ctypes.data, B, rows.ctypes.data, rows.shape[0], A.data_ptr(), float(lam),
+                                        _addr(off), B, _addr(rows), rows.shape[0], A.data_ptr(), float(lam),
                                         coeffs.data_ptr(), F2.data_ptr() if F2 is not None else None, ws.data_ptr(),
                                         ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_sampled_coefficients")
@@ -447,7 +458,7 @@ def isopo_profile_collect() -> dict:
     """{kernel name: (total ms, launches)} since the last collect; synchronises the recorded events."""
     ms = np.zeros(NUM_KERNELS, dtype=np.float64)
     n = np.zeros(NUM_KERNELS, dtype=np.int64)
-    _check(lib.isopo_profile_collect(ms.ctypes.data, n.ctypes.data), "isopo_profile_collect")
+    _check(lib.isopo_profile_collect(_addr(ms), _addr(n)), "isopo_profile_collect")
     return {lib.isopo_kernel_name(k).decode(): (float(ms[k]), int(n[k])) for k in range(NUM_KERNELS) if n[k] or ms[k]}
 
 

@@ -115,11 +115,16 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
 }
 
 WsTag make_ws_tag(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, const int64_t* off_host) {
-  uint64_t h = 1469598103934665603ull;  // FNV-1a over the offsets' bytes
+  // four interleaved multiply-xorshift chains over the offsets, one word at a time (a byte at a time, each multiplication
+  // waiting for the one before, took 2.5 us at 256 sequences)
+  uint64_t lane[4] = {1469598103934665603ull, 0x9e3779b97f4a7c15ull, 0xc2b2ae3d27d4eb4full, 0x165667b19e3779f9ull};
   for (int i = 0; i <= B; ++i) {
-    uint64_t w = (uint64_t)off_host[i];
-    for (int b = 0; b < 8; ++b) { h ^= w & 0xffu; h *= 1099511628211ull; w >>= 8; }
+    uint64_t& h = lane[i & 3];
+    h = (h ^ (uint64_t)off_host[i]) * 0xff51afd7ed558ccdull;
+    h ^= h >> 32;
   }
+  uint64_t h = lane[0];
+  for (int k = 1; k < 4; ++k) { h = (h ^ lane[k]) * 0xff51afd7ed558ccdull; h ^= h >> 32; }
   WsTag t{};
   t.v[0] = 0x49534f504f5f4753ll;
   t.v[1] = (int64_t)dtype; t.v[2] = T; t.v[3] = d_in; t.v[4] = d_out; t.v[5] = B; t.v[6] = (int64_t)h;
