@@ -2,13 +2,12 @@
 //   simple variants  - per-row sums of K in float64, a few rows per warp
 //   interacting      - up to 128 sequences L D L^T in float64; more: blocked Cholesky of K + lambda*I with refinement
 //                      (interacting_solve.cuh)
-#include "interacting_solve.cuh"
+#include "cluster_solve.cuh"
 
 namespace isopo {
 
 namespace {
 
-constexpr int kThreads = kSolveThreads;
 constexpr int kMaxB = 256;
 
 // One launch serves up to ISOPO_MAX_BATCH layers that share A and the variant: CTA l works on layer l.
@@ -250,28 +249,21 @@ inline size_t small_smem_bytes(int B) {
 }
 
 // Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
-__global__ void __launch_bounds__(kThreads) k_transform(const __grid_constant__ TransformBatch batch) {
+__global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_constant__ TransformBatch batch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TransformParams P = layer_params(batch, blockIdx.x);
   __shared__ double s_trace, s_res;
   __shared__ int s_fail;
   const SolveSmem m = solve_smem(smem_raw, P.B);
-  interacting_solve<false>(P, m.Lb, m.InvD, m.vec, m.sol, m.rdiag, s_trace, s_res, s_fail, (int)blockIdx.x);
+  interacting_solve(P, m.Lb, m.InvD, m.vec, m.sol, m.rdiag, s_trace, s_res, s_fail, (int)blockIdx.x);
 }
 
-// The interacting variant for more sequences than the shared-memory kernel holds: the block triangle (2.1 MB at
-// 1024 sequences) lives in a workspace that stays in the L2, everything else as above.  One CTA.
+// 257 to 1024 sequences: a cluster of sixteen, the factor's blocks also in a workspace that stays in the L2 (2.1 MB at 1024).
 constexpr int kMaxLargeB = ISOPO_MAX_LARGE_SEQS;
-__global__ void __launch_bounds__(kThreads) k_transform_large(const TransformParams P, float* scratch) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double s_trace, s_res;
-  __shared__ int s_fail;
-  const int nb = (P.B + kNB - 1) / kNB, Bp = nb * kNB;
-  float* InvD = reinterpret_cast<float*>(smem_raw);         // nb inverse diagonal factors
-  float* vec = InvD + (size_t)nb * kBlk;                    // Bp floats
-  double* sol = reinterpret_cast<double*>(vec + Bp);        // Bp doubles
-  float* rdiag = reinterpret_cast<float*>(sol + Bp);        // Bp floats
-  interacting_solve<true>(P, scratch, InvD, vec, sol, rdiag, s_trace, s_res, s_fail, 0);
+constexpr int kLargeCluster = 16;
+__global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const TransformParams P, float* scratch) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cluster_solve<kLargeCluster>(P, scratch, smem_raw, 0);
 }
 
 // Running means for the relative regulariser.  state = {E[F^2], E[||G||^2], E[F^2 / ||G||^2], number of updates};
@@ -340,7 +332,7 @@ isopo_status transform_batched(int n, const float* const* K, const float* A, int
     if (B > kMaxB) return ISOPO_ERR_UNSUPPORTED;
     ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     LaunchScope scope(kIdTransform, st);
-    k_transform<<<n, kThreads, solve_smem_bytes(B), st>>>(T);
+    k_transform<<<n, kSolveThreads, solve_smem_bytes(B), st>>>(T);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -354,15 +346,24 @@ size_t transform_large_workspace_bytes(int B) {
 isopo_status transform_large(const float* K, const float* A, int B, float lambda, float* coeffs, float* scratch,
                              int32_t* info, cudaStream_t st) {
   if (B < 1 || B > kMaxLargeB) return ISOPO_ERR_UNSUPPORTED;
-  if (B <= kMaxSmallB) return transform(K, A, B, ISOPO_VAR_INTERACTING, lambda, nullptr, nullptr, coeffs, info, st);
+  if (B <= kMaxB) return transform(K, A, B, ISOPO_VAR_INTERACTING, lambda, nullptr, nullptr, coeffs, info, st);
   TransformParams P{};
   P.K = K; P.A = A; P.coeffs = coeffs; P.info = info; P.B = B; P.variant = (int)ISOPO_VAR_INTERACTING; P.lambda = lambda;
-  const size_t nb = (size_t)(B + kNB - 1) / kNB;
-  const size_t smem = sizeof(float) * (nb * kBlk + 2 * nb * kNB) + sizeof(double) * nb * kNB;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform_large, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform_large, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kLargeCluster);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = cl_smem_bytes<kLargeCluster>(B);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kLargeCluster; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   {
     LaunchScope scope(kIdTransform, st);
-    k_transform_large<<<1, kThreads, smem, st>>>(P, scratch);
+    ISOPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_transform_large, P, scratch));
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -138,3 +138,18 @@ def test_gram_route_with_300_sequences_end_to_end(b):
     assert errs["K"] <= 2e-2 and errs["dW_own_c"] <= 2e-2
     assert errs["c_from_K"] <= 1e-5 + 2e-7 * cond
     assert errs["c"] <= 2e-2 * max(1.0, cond / 1e3)
+
+
+@pytest.mark.parametrize("B", [258, 288, 289, 511, 513, 544, 992, 993, 1023])
+def test_block_rows_dealt_to_the_cluster(b, B):
+    """Sizes at which the snake of block rows over sixteen CTAs starts, turns and ends with a full or a padded block row, on
+    a matrix that needs a refinement round (K + lambda I with a condition number of about 1e4): bounds as above."""
+    K = _spd(B, 2 * B, 8600 + B, 3.0)
+    A = np.random.default_rng(B).standard_normal(B).astype(np.float32)
+    lam = float(np.float32(1e-3 * np.mean(np.diag(K))))
+    c, info = _solve(b, K, A, lam)
+    assert info == 0
+    K64 = K.astype(np.float64) + lam * np.eye(B)
+    cond = float(np.linalg.cond(K64))
+    assert rel_fro(c, np.linalg.solve(K64, A.astype(np.float64))) <= 1e-5 + 2e-7 * cond
+    assert float(np.linalg.norm(K64 @ c.astype(np.float64) - A) / np.linalg.norm(A)) <= 2e-6 + 1e-7 * cond
