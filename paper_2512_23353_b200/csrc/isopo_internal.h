@@ -127,6 +127,32 @@ void set_cuda_error(cudaError_t e, const char* where);
     }                                                         \
   } while (0)
 
+// ---- programmatic dependent launch ----
+// A layer is a chain of five to ten dependent kernels, several of them a few microseconds long.  Every kernel of the
+// library is launched so that its CTAs may be set up while its predecessor in the stream still runs, lets its own
+// successor do the same from its first instruction, and waits for everything before it to be complete and visible before
+// it touches memory (all of its CTAs do, so that the chain stays ordered end to end).  Work of other origin in the stream
+// is ordered as always.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// The kernel must call pdl_wait().  Errors are picked up by the cudaGetLastError() that follows every launch.
+template <typename... Params, typename... Args>
+inline void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // ---- launchers (each enqueues on `st` and returns a status; none synchronises) ----
 
 isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, cudaStream_t st);

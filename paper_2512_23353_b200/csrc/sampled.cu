@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(256) k_gather_samples(const T* __restrict__ X,
                                                         int d_out, const int64_t* __restrict__ rows,
                                                         T* __restrict__ a0, T* __restrict__ g0,
                                                         double* __restrict__ den) {
+  pdl_wait();
   const int j = blockIdx.x;
   const int64_t t = rows[j];
   double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * d_in, d_in);
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(32 * kFinishSlices) k_sampled_finish(const TM*
                                                                        const double* __restrict__ den,
                                                                        const float* __restrict__ A, float lambda,
                                                                        float* __restrict__ coeffs, float* __restrict__ F2) {
+  pdl_wait();
   __shared__ double part[kFinishSlices][32];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + x;
@@ -141,14 +143,14 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
     double* Mt = (double*)(ws + S.off_mt);
     {
       LaunchScope scope(kIdSampledAux, st);
-      k_gather_samples<float><<<n_samples, 256, 0, st>>>((const float*)X, (const float*)dY, d_in, d_out, rows, a0, g0, den);
+      launch(k_gather_samples<float>, n_samples, 256, 0, st, (const float*)X, (const float*)dY, d_in, d_out, rows, a0, g0, den);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     s = f32_sampled((const float*)X, (const float*)dY, T, d_in, d_out, a0, g0, n_samples, tokseq, B, Mt, st);
     if (s != ISOPO_OK) return s;
     {
       LaunchScope scope(kIdSampledAux, st);
-      k_sampled_finish<double><<<(B + 31) / 32, 32 * kFinishSlices, 0, st>>>(Mt, n_samples, B, den, A, lambda, coeffs, F2);
+      launch(k_sampled_finish<double>, (B + 31) / 32, 32 * kFinishSlices, 0, st, Mt, n_samples, B, den, A, lambda, coeffs, F2);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     return ISOPO_OK;
@@ -158,7 +160,7 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
   float* Mt = (float*)(ws + S.off_mt);
   {
     LaunchScope scope(kIdSampledAux, st);
-    k_gather_samples<__nv_bfloat16><<<n_samples, 256, 0, st>>>((const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out,
+    launch(k_gather_samples<__nv_bfloat16>, n_samples, 256, 0, st, (const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out,
                                                                rows, a0, g0, den);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
@@ -166,7 +168,7 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
   if (s != ISOPO_OK) return s;
   {
     LaunchScope scope(kIdSampledAux, st);
-    k_sampled_finish<float><<<(B + 31) / 32, 32 * kFinishSlices, 0, st>>>(Mt, n_samples, B, den, A, lambda, coeffs, F2);
+    launch(k_sampled_finish<float>, (B + 31) / 32, 32 * kFinishSlices, 0, st, Mt, n_samples, B, den, A, lambda, coeffs, F2);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -14,6 +14,7 @@ namespace {
 constexpr int kArgChunk = 384;
 struct OffsetArgs { int64_t v[kArgChunk]; };
 __global__ void k_store_offsets(OffsetArgs a, int base, int n, int64_t* __restrict__ off) {
+  pdl_wait();
   const int t = threadIdx.x;
   if (t < n) off[base + t] = a.v[t];
 }
@@ -31,6 +32,7 @@ struct StoredPrepArgs {
   uint8_t order[256];
 };
 __global__ void __launch_bounds__(256) k_prep_stored(StoredPrepArgs a, int B, int n_proj) {
+  pdl_wait();
   for (int h = 0; h < n_proj; ++h) {
     if (blockIdx.x == 0) {
       for (int i = threadIdx.x; i <= B; i += blockDim.x) a.off_dev[h][i] = a.off[i];
@@ -41,6 +43,7 @@ __global__ void __launch_bounds__(256) k_prep_stored(StoredPrepArgs a, int B, in
   }
 }
 __global__ void k_tokseq(const int64_t* __restrict__ off, int B, int64_t T, int32_t* __restrict__ tokseq) {
+  pdl_wait();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
     int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
     while (hi - lo > 1) {
@@ -54,6 +57,7 @@ __global__ void k_tokseq(const int64_t* __restrict__ off, int B, int64_t T, int3
 // tokscale[t] = coeffs[sequence of token t]: what the folded weight-gradient GEMM multiplies row t by.
 __global__ void k_tokscale(const int64_t* __restrict__ off, int B, int64_t T, const float* __restrict__ coeffs,
                            float* __restrict__ tokscale) {
+  pdl_wait();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
     int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
     while (hi - lo > 1) {
@@ -69,6 +73,7 @@ __global__ void k_tokscale(const int64_t* __restrict__ off, int B, int64_t T, co
 template <bool kScale>
 __global__ void __launch_bounds__(256) k_prep_small(OffsetArgs a, int B, int64_t T, int64_t* __restrict__ off_dev,
                                                     const float* __restrict__ coeffs, void* __restrict__ out) {
+  pdl_wait();
   __shared__ int64_t s_off[kArgChunk];
   for (int i = threadIdx.x; i <= B; i += blockDim.x) {
     s_off[i] = a.v[i];
@@ -238,6 +243,7 @@ static_assert(sizeof(F32StoredArgs) + sizeof(OffsetParam<true>) <= 4096, "kernel
 template <int kTile, int kT, bool kArgOff>
 __global__ void __launch_bounds__(SeqGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
 k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ OffsetParam<kArgOff> o) {
+  pdl_wait();
   extern __shared__ __align__(16) float smem[];
   const int i = blockIdx.z, m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t cta = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -284,6 +290,7 @@ template <int kTile, int kT>
 __global__ void __launch_bounds__(SlabGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
 k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int64_t T, int d_in, int d_out,
                   const float* __restrict__ coeffs, const int32_t* __restrict__ tokseq, float* __restrict__ dW, int64_t slab) {
+  pdl_wait();
   extern __shared__ __align__(16) float smem[];
   const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t t0 = blockIdx.z * slab, t1 = min(T, t0 + slab);
@@ -341,6 +348,7 @@ struct NtkShape {
 template <int kMA, int kNB, bool kDiag>
 __global__ void __launch_bounds__(kNtkThreads, NtkShape<kMA, kNB, kDiag>::kPerSm)
 k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uint32_t* done, float* __restrict__ K) {
+  pdl_wait();
   typedef NtkShape<kMA, kNB, kDiag> S;
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -486,6 +494,7 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
                                                   const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
                                                   int d_in, int d_out, const int32_t* __restrict__ tokseq, int B,
                                                   double* __restrict__ out) {
+  pdl_wait();
   const int I = blockIdx.y, J = blockIdx.x;
   if (!kSampled && J < I) return;
   __shared__ __align__(16) float stage_mem[kGramStages][2][kGT * kGPitch];
@@ -589,6 +598,7 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
 }
 
 __global__ void k_f32_gram_finish(const double* __restrict__ kacc, int B, float* __restrict__ K) {
+  pdl_wait();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)B * B) return;
   const int i = (int)(e / B), j = (int)(e % B);
@@ -604,6 +614,7 @@ __global__ void __launch_bounds__(256) k_f32_combine(const float* __restrict__ G
                                                      const float* __restrict__ coeffs, float* __restrict__ dW, float beta,
                                                      const WsTag* __restrict__ tag_dev, WsTag tag,
                                                      int32_t* __restrict__ info) {
+  pdl_wait();
   if (!ws_tag_matches(tag_dev, tag, info)) return;
   constexpr int kLanes = 256 / kSlices;
   __shared__ double4 part[kSlices > 1 ? 256 : 1];
@@ -652,7 +663,7 @@ isopo_status store_i64(const int64_t* host, int64_t n, int64_t* dev, cudaStream_
     OffsetArgs a;
     const int m = (int)std::min<int64_t>(kArgChunk, n - base);
     for (int t = 0; t < m; ++t) a.v[t] = host[base + t];
-    k_store_offsets<<<1, kArgChunk, 0, st>>>(a, (int)base, m, dev);
+    launch(k_store_offsets, 1, kArgChunk, 0, st, a, (int)base, m, dev);
     ISOPO_CUDA_TRY(cudaGetLastError());
   }
   return ISOPO_OK;
@@ -666,7 +677,7 @@ static isopo_status launch_prep_small(const int64_t* off_host, int B, int64_t T,
   const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
   {
     LaunchScope scope(kIdPrep, st);
-    k_prep_small<kScale><<<grid, 256, 0, st>>>(a, B, T, off_dev, coeffs, out);
+    launch(k_prep_small<kScale>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -680,7 +691,7 @@ isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off
   const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
   {
     LaunchScope scope(kIdPrep, st);
-    k_tokseq<<<grid, 256, 0, st>>>(off_dev, B, T, tokseq);
+    launch(k_tokseq, grid, 256, 0, st, off_dev, B, T, tokseq);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -694,7 +705,7 @@ isopo_status launch_tokscale(const int64_t* off_host, int B, int64_t T, int64_t*
   const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
   {
     LaunchScope scope(kIdPrep, st);
-    k_tokscale<<<grid, 256, 0, st>>>(off_dev, B, T, coeffs, tokscale);
+    launch(k_tokscale, grid, 256, 0, st, off_dev, B, T, coeffs, tokscale);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -721,7 +732,7 @@ isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj
   for (int i = 0; i < B; ++i) a.order[i] = (uint8_t)idx[i];
   {
     LaunchScope scope(kIdPrep, st);
-    k_prep_stored<<<std::max(1, (B * B + 2047) / 2048), 256, 0, st>>>(a, B, n_proj);
+    launch(k_prep_stored, std::max(1, (B * B + 2047) / 2048), 256, 0, st, a, B, n_proj);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -735,7 +746,7 @@ static isopo_status launch_f32_seq_grad(const F32StoredArgs& a, const OffsetPara
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_seq_grad<kTile, kT, kArgOff>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   {
     LaunchScope scope(kIdF32SeqGrad, st);
-    k_f32_seq_grad<kTile, kT, kArgOff><<<grid, Gemm::kThr, Gemm::kSmem, st>>>(a, o);
+    launch(k_f32_seq_grad<kTile, kT, kArgOff>, grid, Gemm::kThr, Gemm::kSmem, st, a, o);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -774,7 +785,7 @@ static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, doubl
   const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + 7) / 8));
   {
     LaunchScope scope(kIdF32Ntk, st);
-    k_f32_ntk<kMA, kNB, kDiag><<<dim3((unsigned)pairs, (unsigned)slabs), kNtkThreads, smem, st>>>(G, gstride, B, kacc, done, K);
+    launch(k_f32_ntk<kMA, kNB, kDiag>, dim3((unsigned)pairs, (unsigned)slabs), kNtkThreads, smem, st, G, gstride, B, kacc, done, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -783,7 +794,7 @@ static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, doubl
 static isopo_status launch_f32_finish(const double* kacc, int B, float* K, cudaStream_t st) {
   {
     LaunchScope scope(kIdMirror, st);
-    k_f32_gram_finish<<<(unsigned)(((int64_t)B * B + 255) / 256), 256, 0, st>>>(kacc, B, K);
+    launch(k_f32_gram_finish, (unsigned)(((int64_t)B * B + 255) / 256), 256, 0, st, kacc, B, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -806,7 +817,7 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
   ISOPO_CUDA_TRY(cudaMemsetAsync(kacc, 0, sizeof(double) * (size_t)B * B, st));
   {
     LaunchScope scope(kIdF32Gram, st);
-    k_f32_gram<false><<<dim3((unsigned)nt, (unsigned)nt), 256, 0, st>>>(X, dY, T, X, dY, T, d_in, d_out, tokseq, B, kacc);
+    launch(k_f32_gram<false>, dim3((unsigned)nt, (unsigned)nt), 256, 0, st, X, dY, T, X, dY, T, d_in, d_out, tokseq, B, kacc);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return launch_f32_finish(kacc, B, K, st);
@@ -819,7 +830,7 @@ isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, i
   ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(double) * (size_t)n_samples * B, st));
   {
     LaunchScope scope(kIdSampled, st);
-    k_f32_gram<true><<<dim3((unsigned)nt, (unsigned)ns), 256, 0, st>>>(a0, g0, n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
+    launch(k_f32_gram<true>, dim3((unsigned)nt, (unsigned)ns), 256, 0, st, a0, g0, n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -833,7 +844,7 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
   const int grid = (int)std::min<int64_t>((N + per_block - 1) / per_block, 148 * 16);
   {
     LaunchScope scope(kIdF32Combine, st);
-    (split ? k_f32_combine<8> : k_f32_combine<1>)<<<grid, 256, 0, st>>>(G, N, gstride, B, coeffs, dW, beta, tag_dev, tag, info);
+    launch((split ? k_f32_combine<8> : k_f32_combine<1>), grid, 256, 0, st, G, N, gstride, B, coeffs, dW, beta, tag_dev, tag, info);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -852,7 +863,7 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_weight_grad<kTile, kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   {
     LaunchScope scope(kIdF32WeightGrad, st);
-    k_f32_weight_grad<kTile, kT><<<dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st>>>(X, dY, T, d_in, d_out, coeffs,
+    launch(k_f32_weight_grad<kTile, kT>, dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st, X, dY, T, d_in, d_out, coeffs,
                                                                                                   tokseq, dW, slab);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());

@@ -87,6 +87,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -225,7 +226,7 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   p.strip = gram_strip_width(2.0 * kTT * (d_in + d_out), grid);
   {
     LaunchScope scope(kIdGram, st);
-    k_bf16_gram<false><<<grid, kThreads, kSmemBytes, st>>>(mapX, mapY, mapX, mapY, p);
+    launch(k_bf16_gram<false>, grid, kThreads, kSmemBytes, st, mapX, mapY, mapX, mapY, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return mirror_upper(K, B, st);
@@ -250,7 +251,7 @@ isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, in
   const int grid = (int)std::min<long long>(units, sms);
   {
     LaunchScope scope(kIdSampled, st);
-    k_bf16_gram<true><<<grid, kThreads, kSmemBytes, st>>>(mapRX, mapRY, mapX, mapY, p);
+    launch(k_bf16_gram<true>, grid, kThreads, kSmemBytes, st, mapRX, mapRY, mapX, mapY, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -63,6 +63,7 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -240,7 +241,7 @@ isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, i
   p.strip = gram_strip_width(2.0 * kTT * d_sum, grid);
   {
     LaunchScope scope(kIdGram, st);
-    k_bf16_gram_shared<<<grid, kThreads, kSmemBytes, st>>>(mapX, mapY[0], mapY[1], mapY[2], p);
+    launch(k_bf16_gram_shared, grid, kThreads, kSmemBytes, st, mapX, mapY[0], mapY[1], mapY[2], p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   for (int h = 0; h < n_heads; ++h) {

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
 // One thread per entry of the lower triangle (its reads run along a row of every partial matrix), which also
 // writes the mirrored entry.
 __global__ void k_ntk_reduce(const float* __restrict__ kpart, int n_ctas, int B, float* __restrict__ K) {
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
   const int i = e / B, j = e % B;
@@ -252,6 +254,7 @@ __global__ void k_ntk_reduce(const float* __restrict__ kpart, int n_ctas, int B,
 // kdiag != NULL (split store): the diagonal comes from the gradient GEMM's float32 sums of squares
 template <bool kFromLower>
 __global__ void k_mirror(float* __restrict__ K, int B, const float* __restrict__ kdiag) {
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
   const int i = e / B, j = e % B;
@@ -274,6 +277,7 @@ __global__ void __launch_bounds__(256, kSlices > 1 ? 4 : 1) k_bf16_combine(const
                                                        const float* __restrict__ coeffs, float* __restrict__ dW,
                                                        float beta, const WsTag* __restrict__ tag_dev, WsTag tag,
                                                        int32_t* __restrict__ info) {
+  pdl_wait();
   if (!ws_tag_matches(tag_dev, tag, info)) return;  // another layer's or microbatch's gradients: touch nothing
   constexpr int kPieces = 8 / kSlices;  // pieces a block works on at a time
   constexpr int kF = kSlices > 1 ? 8 : kCombineInFlight;
@@ -373,6 +377,7 @@ __global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ 
                                                        float* __restrict__ dW, float beta,
                                                        const WsTag* __restrict__ tag_dev, WsTag tag,
                                                        int32_t* __restrict__ info) {
+  pdl_wait();
   if (!ws_tag_matches(tag_dev, tag, info)) return;  // another layer's or microbatch's gradients: touch nothing
   __shared__ float sc[256];
   for (int i = threadIdx.x; i < B; i += blockDim.x) sc[i] = coeffs[i] / scales[i];
@@ -457,12 +462,12 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
   if (kpart) grid = std::min(grid, kNtkMaxPartials);
   {
     LaunchScope scope(kIdNtk, st);
-    kernel<<<grid, kThreads, kSmemBytes, st>>>(mapG, p);
+    launch(kernel, grid, kThreads, kSmemBytes, st, mapG, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   if (!kpart) {
     LaunchScope scope(kIdMirror, st);
-    k_mirror<true><<<(B * B + 255) / 256, 256, 0, st>>>(K, B, fmt.split ? fmt.kdiag : nullptr);
+    launch(k_mirror<true>, (B * B + 255) / 256, 256, 0, st, K, B, fmt.split ? fmt.kdiag : nullptr);
     ISOPO_CUDA_TRY(cudaGetLastError());
     return ISOPO_OK;
   }
@@ -471,7 +476,7 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
   const int n_active = (int)((p.nkb + per - 1) / per);
   {
     LaunchScope scope(kIdMirror, st);
-    k_ntk_reduce<<<(B * B + 255) / 256, 256, 0, st>>>(kpart, n_active, B, K);
+    launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, n_active, B, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -480,7 +485,7 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
 isopo_status mirror_upper(float* K, int B, cudaStream_t st) {
   {
     LaunchScope scope(kIdMirror, st);
-    k_mirror<false><<<(B * B + 255) / 256, 256, 0, st>>>(K, B, nullptr);
+    launch(k_mirror<false>, (B * B + 255) / 256, 256, 0, st, K, B, nullptr);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -500,13 +505,13 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
   {
     LaunchScope scope(kIdCombine, st);
     if (fmt.split)
-      k_e4m3_combine<<<grid, 256, 0, st>>>((const uint2*)G, chunks, B, pg, d_in, d_out, coeffs, fmt.scales, dW, beta,
+      launch(k_e4m3_combine, grid, 256, 0, st, (const uint2*)G, chunks, B, pg, d_in, d_out, coeffs, fmt.scales, dW, beta,
                                            tag_dev, tag, info);
     else
-      (slices == 1   ? k_bf16_combine<1>
+      launch((slices == 1   ? k_bf16_combine<1>
        : slices == 2 ? k_bf16_combine<2>
        : slices == 4 ? k_bf16_combine<4>
-                     : k_bf16_combine<8>)<<<grid, 256, 0, st>>>((const uint4*)G, chunks, B, pg, d_in, d_out, coeffs, dW, beta,
+                     : k_bf16_combine<8>), grid, 256, 0, st, (const uint4*)G, chunks, B, pg, d_in, d_out, coeffs, dW, beta,
                                                                 tag_dev, tag, info);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());

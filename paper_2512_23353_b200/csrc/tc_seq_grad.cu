@@ -106,15 +106,6 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
   int64_t* s_first = reinterpret_cast<int64_t*>(smem + kStages * kStageBytes + 256);
   int* s_len = reinterpret_cast<int*>(s_first + kMaxSeqs);
   int* s_seq = s_len + kMaxSeqs;
-  if (!kFolded) {
-    for (int k = threadIdx.x; k < p.B; k += blockDim.x) {
-      const int i = p.order[k];
-      const int64_t t0 = p.off[i];
-      s_first[k] = t0;
-      s_len[k] = (int)(p.off[i + 1] - t0);
-      s_seq[k] = i;
-    }
-  }
   const SeqInfo si{s_first, s_len, s_seq};
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -129,6 +120,16 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
+  if (!kFolded) {
+    for (int k = threadIdx.x; k < p.B; k += blockDim.x) {
+      const int i = p.order[k];
+      const int64_t t0 = p.off[i];
+      s_first[k] = t0;
+      s_len[k] = (int)(p.off[i + 1] - t0);
+      s_seq[k] = i;
+    }
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -365,7 +366,7 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   const int grid = (int)std::min<long long>(units, sms);
   {
     LaunchScope scope(kIdSeqGrad, st);
-    k_bf16_seq_grad<false><<<grid, kThreads, kSmemBytes, st>>>(mapY, mapX, p);
+    launch(k_bf16_seq_grad<false>, grid, kThreads, kSmemBytes, st, mapY, mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -399,7 +400,7 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   const int grid = (int)std::min<long long>(tiles * nslabs, sms);
   {
     LaunchScope scope(kIdWeightGrad, st);
-    k_bf16_seq_grad<true><<<grid, kThreadsFolded, kSmemBytes, st>>>(mapY, mapX, p);
+    launch(k_bf16_seq_grad<true>, grid, kThreadsFolded, kSmemBytes, st, mapY, mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

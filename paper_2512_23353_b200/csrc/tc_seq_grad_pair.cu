@@ -140,13 +140,6 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
   int64_t* s_first = reinterpret_cast<int64_t*>(smem + kStages * kStageBytes + 512);
   int* s_len = reinterpret_cast<int*>(s_first + kMaxSeqs);
   int* s_seq = s_len + kMaxSeqs;
-  for (int k = threadIdx.x; k < p.B; k += kThreads) {
-    const int i = p.order[k];
-    const int64_t t0 = p.off[i];
-    s_first[k] = t0;
-    s_len[k] = (int)(p.off[i + 1] - t0);
-    s_seq[k] = i;
-  }
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();  // 0 issues the MMAs
@@ -163,6 +156,14 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
+  for (int k = threadIdx.x; k < p.B; k += kThreads) {
+    const int i = p.order[k];
+    const int64_t t0 = p.off[i];
+    s_first[k] = t0;
+    s_len[k] = (int)(p.off[i + 1] - t0);
+    s_seq[k] = i;
+  }
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -399,6 +400,7 @@ __device__ __forceinline__ float sum_sq8(const uint4& v) {
 __global__ void __launch_bounds__(512) k_seq_scales(const uint4* __restrict__ X, const uint4* __restrict__ dY, int d_in8,
                                                     int d_out8, const int64_t* __restrict__ off,
                                                     float* __restrict__ scales, float* __restrict__ kdiag) {
+  pdl_wait();
   const int i = blockIdx.x;
   const int64_t t0 = off[i], len = off[i + 1] - t0;
   const int n = (int)min((int64_t)16, len);
@@ -434,7 +436,7 @@ isopo_status launch_seq_scales(const void* X, const void* dY, int d_in, int d_ou
                                float* kdiag, cudaStream_t st) {
   {
     LaunchScope scope(kIdPrep, st);
-    k_seq_scales<<<B, 512, 0, st>>>((const uint4*)X, (const uint4*)dY, d_in / 8, d_out / 8, off_dev, scales, kdiag);
+    launch(k_seq_scales, B, 512, 0, st, (const uint4*)X, (const uint4*)dY, d_in / 8, d_out / 8, off_dev, scales, kdiag);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -505,7 +507,7 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
   p.group_m = std::max(1, std::min(g, p.ptiles_m));
   {
     LaunchScope scope(kIdSeqGrad, st);
-    kernel<<<2 * npairs, kThreads, kSmemBytes, st>>>(mapY[0], mapY[1], mapY[2], mapX, p);
+    launch(kernel, 2 * npairs, kThreads, kSmemBytes, st, mapY[0], mapY[1], mapY[2], mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

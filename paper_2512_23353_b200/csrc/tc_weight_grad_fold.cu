@@ -134,8 +134,6 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
   // segment, and a global load there would stall the MMA thread for longer than its queue of MMAs lasts
   int* s_off = reinterpret_cast<int*>(smem + kStages * kStageBytes + 512);
   float* s_coef = reinterpret_cast<float*>(smem + kStages * kStageBytes + 512 + kOffBytes);
-  for (int k = threadIdx.x; k <= p.B; k += kThreads) s_off[k] = (int)p.off[k];
-  for (int k = threadIdx.x; k < p.B; k += kThreads) s_coef[k] = p.coeffs[k];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();  // 0 issues the MMAs
@@ -152,6 +150,9 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
+  for (int k = threadIdx.x; k <= p.B; k += kThreads) s_off[k] = (int)p.off[k];
+  for (int k = threadIdx.x; k < p.B; k += kThreads) s_coef[k] = p.coeffs[k];
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -413,7 +414,7 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   p.group_m = std::max(1, std::min(g, p.ptiles_m));
   {
     LaunchScope scope(kIdWeightGrad, st);
-    k_bf16_weight_grad_fold<<<2 * npairs, kThreads, kSmemBytes, st>>>(mapY, mapX, p);
+    launch(k_bf16_weight_grad_fold, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -88,6 +88,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+  pdl_wait();
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -224,6 +225,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
 // dst[t, :] = bf16(tokscale[t] * src[t, :]) (round to nearest even), 8 elements per thread.
 __global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src, const float* __restrict__ tokscale,
                                                     int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst) {
+  pdl_wait();
   const int64_t n = T * d8;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const float c = __ldg(tokscale + e / d8);
@@ -249,7 +251,7 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
     const int grid = (int)std::min<int64_t>((T * d8 + 255) / 256, (int64_t)sms * 16);
     {
       LaunchScope scope(kIdScaleRows, st);
-      k_scale_rows<<<grid, 256, 0, st>>>((const uint4*)(scale_y ? dY : X), tokscale, T, d8, (uint4*)scaled);
+      launch(k_scale_rows, grid, 256, 0, st, (const uint4*)(scale_y ? dY : X), tokscale, T, d8, (uint4*)scaled);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     if (scale_y) dY = scaled; else X = scaled;
@@ -301,7 +303,7 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
   const int npairs = (int)std::max<long long>(1, std::min<long long>(ptiles * nslabs, pairs));
   {
     LaunchScope scope(kIdWeightGrad, st);
-    k_bf16_weight_grad_pair<<<2 * npairs, kThreads, kSmemBytes, st>>>(mapY, mapX, p);
+    launch(k_bf16_weight_grad_pair, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

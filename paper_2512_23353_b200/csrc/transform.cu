@@ -90,6 +90,7 @@ __device__ __forceinline__ double block_total(double v, double* s_part) {
 // itself.  Bound by latency: the seven layers of a block at 256 sequences took 25 us with one CTA per layer.
 constexpr int kSimpleRows = 32;
 __global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant__ TransformBatch batch) {
+  pdl_wait();
   const TransformParams P = layer_params(batch, blockIdx.x);
   __shared__ double s_part[8];
   const int B = P.B, tid = threadIdx.x, first = blockIdx.y * kSimpleRows;
@@ -144,6 +145,7 @@ __device__ __forceinline__ double newton_rcp(double d) {
 }
 template <int kA>
 __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__ TransformBatch batch) {
+  pdl_wait();
   extern __shared__ __align__(16) double smem_d[];
   const TransformParams P = layer_params(batch, blockIdx.x);
   const int B = P.B, n = B + (B & 1), tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, pitch = n + 1;
@@ -250,6 +252,7 @@ inline size_t small_smem_bytes(int B) {
 
 // Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
 __global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_constant__ TransformBatch batch) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TransformParams P = layer_params(batch, blockIdx.x);
   __shared__ double s_trace, s_res;
@@ -262,6 +265,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_consta
 constexpr int kMaxLargeB = ISOPO_MAX_LARGE_SEQS;
 constexpr int kLargeCluster = 16;
 __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const TransformParams P, float* scratch) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   cluster_solve<kLargeCluster>(P, scratch, smem_raw, 0);
 }
@@ -272,6 +276,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const Transfo
 constexpr int kEmaThreads = 1024;
 __global__ void __launch_bounds__(kEmaThreads) k_reg_ema(const float* __restrict__ K, int B, float decay,
                                                          float* __restrict__ state) {
+  pdl_wait();
   __shared__ double s_part[3][kEmaThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5;
   double tr = 0.0, f2 = 0.0, rel = 0.0;
@@ -300,7 +305,7 @@ __global__ void __launch_bounds__(kEmaThreads) k_reg_ema(const float* __restrict
 isopo_status reg_ema_update(const float* K, int B, float decay, float* state, cudaStream_t st) {
   {
     LaunchScope scope(kIdTransform, st);
-    k_reg_ema<<<1, kEmaThreads, 0, st>>>(K, B, decay, state);
+    launch(k_reg_ema, 1, kEmaThreads, 0, st, K, B, decay, state);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -321,18 +326,18 @@ isopo_status transform_batched(int n, const float* const* K, const float* A, int
   }
   if (v != ISOPO_VAR_INTERACTING) {
     LaunchScope scope(kIdTransform, st);
-    k_transform_simple<<<dim3(n, (B + kSimpleRows - 1) / kSimpleRows), 256, 0, st>>>(T);
+    launch(k_transform_simple, dim3(n, (B + kSimpleRows - 1) / kSimpleRows), 256, 0, st, T);
   } else if (B <= kMaxSmallB) {
     auto kernel = B <= 16 ? k_transform_small<1> : B <= 32 ? k_transform_small<2> : B <= 64 ? k_transform_small<4> : k_transform_small<8>;
     const size_t smem = small_smem_bytes(B);
     if (smem > 48 * 1024) ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     LaunchScope scope(kIdTransform, st);
-    kernel<<<n, 256, smem, st>>>(T);
+    launch(kernel, n, 256, smem, st, T);
   } else {
     if (B > kMaxB) return ISOPO_ERR_UNSUPPORTED;
     ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     LaunchScope scope(kIdTransform, st);
-    k_transform<<<n, kSolveThreads, solve_smem_bytes(B), st>>>(T);
+    launch(k_transform, n, kSolveThreads, solve_smem_bytes(B), st, T);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
