@@ -472,63 +472,77 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uin
 }
 
 // ---------------------------------------------------------------------------------------------
-// Products over token pairs: for a 64 x 64 tile (row tokens x column tokens) P = RX X^T and Q = RY dY^T, multiplied
+// Products over token pairs: for a kGT x kGT tile (row tokens x column tokens) P = RX X^T and Q = RY dY^T, multiplied
 // elementwise and summed per (row segment, column sequence) in float64.  Operand rows are staged 16 features at a time
 // by cp.async and read four features at once (16-byte shared loads, rows 20 floats apart: no bank conflicts); an element
 // is a sum over the even and one over the odd features, the two halves of a packed fma.
 //   Gram (kSampled = false): rows and columns are both tokens, tile pairs I <= J.  Only token pairs t <= s are used; a
 //     pair inside one sequence with t < s stands for (t,s) and (s,t) and counts twice.
 //   Sampled estimator (kSampled = true): the rows are the gathered sample rows, out = M^T[sample, sequence], no weights.
-// The tile's products go through shared memory; a warp owns 32 rows x 16 columns of them, walks the columns (sequence
+// The tile's products go through shared memory; a warp owns 32 rows x kGT / 4 columns of them, walks the columns (sequence
 // boundaries are the same for all its lanes), and adds the lanes of one row sequence together before it issues one
-// float64 atomic.  Bound by the float32 pipe: 896 -> 896, 4608 tokens: 1207 us against 3246 us for 32 x 32 tiles loaded
-// synchronously with an atomic per token pair.
+// float64 atomic.  Bound by the float32 pipe: 896 -> 896, 4608 tokens: 1151 us against 3246 us for 32 x 32 tiles loaded
+// synchronously with an atomic per token pair.  Too few tiles of 64 to fill the machine leave the kernel to the latency of
+// one CTA's walk over the features: tiles of 32 then (f32_gram_tile).
 // ---------------------------------------------------------------------------------------------
-constexpr int kGT = 64;   // tokens per tile
 constexpr int kGK = 16;   // features per stage
 constexpr int kGPitch = kGK + 4;
-constexpr int kGramStages = 3;
 
-template <bool kSampled>
-__global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
+template <int kGT>
+struct GramTile {
+  static constexpr int kRows = kGT / 16, kCols = 4;                 // elements of a thread
+  static constexpr int kTx = kGT / kCols, kThr = 16 * kTx;          // 64: 16 x 16 threads; 32: 16 x 8
+  static constexpr int kStages = kGT == 64 ? 3 : 6;                 // 30 KB either way
+};
+template <bool kSampled, int kGT>
+__global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
                                                   const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
                                                   int d_in, int d_out, const int32_t* __restrict__ tokseq, int B,
                                                   double* __restrict__ out) {
   pdl_wait();
+  constexpr int kRows = GramTile<kGT>::kRows, kTx = GramTile<kGT>::kTx, kThr = GramTile<kGT>::kThr;
+  constexpr int kGramStages = GramTile<kGT>::kStages;
   const int I = blockIdx.y, J = blockIdx.x;
   if (!kSampled && J < I) return;
   __shared__ __align__(16) float stage_mem[kGramStages][2][kGT * kGPitch];
   __shared__ int s_col[kGT];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, tx = tid % kTx, ty = tid / kTx;
   const int64_t r0 = (int64_t)I * kGT, c0 = (int64_t)J * kGT;
   if (tid < kGT) s_col[tid] = c0 + tid < T ? tokseq[c0 + tid] : -1;
   const int nkx = (d_in + kGK - 1) / kGK, nky = (d_out + kGK - 1) / kGK;
+  // a thread copies one column (group) of a stage, every kThr / kGK-th (4-byte copies) or 4 kThr / kGK-th row
+  const int c1 = tid % kGK, r1 = tid / kGK, c4 = tid % (kGK / 4) * 4, r4 = tid / (kGK / 4);
   auto fetch = [&](int k) {
     if (k < nkx + nky) {
       const bool second = k >= nkx;
       const int d = second ? d_out : d_in, f0 = (second ? k - nkx : k) * kGK;
+#pragma unroll
       for (int side = 0; side < 2; ++side) {
         const float* M = side == 0 ? (second ? RY : RX) : (second ? dY : X);
-        const int64_t first = side == 0 ? r0 : c0, end = side == 0 ? n_rows : T;
+        const int64_t first = side == 0 ? r0 : c0;
+        const int rows = (int)min((int64_t)kGT, (side == 0 ? n_rows : T) - first);  // rows of the tile that exist
         float* dst = stage_mem[k % kGramStages][side];
         if ((d & 3) == 0) {
-          const int r = tid >> 2, c = (tid & 3) * 4;
-          const bool live = first + r < end && f0 + c < d;
-          cp_async16(dst + r * kGPitch + c, live ? M + (first + r) * d + f0 + c : M, live);
-        } else {
+          const float* src = M + (first + r4) * d + f0 + c4;
 #pragma unroll
-          for (int e = tid; e < kGT * kGK; e += 256) {
-            const int r = e / kGK, c = e % kGK;
-            const bool live = first + r < end && f0 + c < d;
-            cp_async4(dst + r * kGPitch + c, live ? M + (first + r) * d + f0 + c : M, live);
+          for (int i = 0; i < kGT; i += 4 * kThr / kGK, src += (int64_t)(4 * kThr / kGK) * d) {
+            const bool live = r4 + i < rows && f0 + c4 < d;
+            cp_async16(dst + (r4 + i) * kGPitch + c4, live ? src : M, live);
+          }
+        } else {
+          const float* src = M + (first + r1) * d + f0 + c1;
+#pragma unroll
+          for (int i = 0; i < kGT; i += kThr / kGK, src += (int64_t)(kThr / kGK) * d) {
+            const bool live = r1 + i < rows && f0 + c1 < d;
+            cp_async4(dst + (r1 + i) * kGPitch + c1, live ? src : M, live);
           }
         }
       }
     }
     cp_async_commit();
   };
-  float h[4][4];
-  f32x2 acc[4][4] = {};
+  float h[kRows][4];
+  f32x2 acc[kRows][4] = {};
   auto total = [](f32x2 v) { float lo, hi; unpack2(v, lo, hi); return lo + hi; };
   for (int k = 0; k < kGramStages - 1; ++k) fetch(k);
   for (int k = 0; k < nkx + nky; ++k) {
@@ -537,7 +551,7 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
     fetch(k + kGramStages - 1);
     if (k == nkx) {
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+      for (int p = 0; p < kRows; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) { h[p][q] = total(acc[p][q]); acc[p][q] = 0ull; }
     }
@@ -545,14 +559,13 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
     const float* sB = stage_mem[k % kGramStages][1];
 #pragma unroll
     for (int c = 0; c < kGK; c += 4) {
-      ulonglong2 a[4], b[4];
+      ulonglong2 a[kRows], b[4];
 #pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        a[p] = *reinterpret_cast<const ulonglong2*>(sA + (ty + 16 * p) * kGPitch + c);
-        b[p] = *reinterpret_cast<const ulonglong2*>(sB + (tx + 16 * p) * kGPitch + c);
-      }
+      for (int p = 0; p < kRows; ++p) a[p] = *reinterpret_cast<const ulonglong2*>(sA + (ty + 16 * p) * kGPitch + c);
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+      for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(sB + (tx + kTx * q) * kGPitch + c);
+#pragma unroll
+      for (int p = 0; p < kRows; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[p][q] = fma2(a[p].y, b[q].y, fma2(a[p].x, b[q].x, acc[p][q]));
     }
@@ -562,11 +575,11 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
   float* tile = &stage_mem[0][0][0];  // [row][kGT + 1]
   static_assert(kGT * (kGT + 1) <= kGramStages * 2 * kGT * kGPitch, "the tile reuses the stages");
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
+  for (int p = 0; p < kRows; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) tile[(ty + 16 * p) * (kGT + 1) + tx + 16 * q] = h[p][q] * total(acc[p][q]);
+    for (int q = 0; q < 4; ++q) tile[(ty + 16 * p) * (kGT + 1) + tx + kTx * q] = h[p][q] * total(acc[p][q]);
   __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, row = (warp & 1) * 32 + lane, cb = (warp >> 1) * 16;
+  const int warp = tid >> 5, lane = tid & 31, row = (warp % (kGT / 32)) * 32 + lane, cb = warp / (kGT / 32) * (kGT / 4);
   const int64_t t = r0 + row;
   const int rseq = t < n_rows ? (kSampled ? (int)t : tokseq[t]) : -1;  // rows past the end form a run of their own, unused
   int same = 0;
@@ -578,14 +591,14 @@ __global__ void __launch_bounds__(256) k_f32_gram(const float* __restrict__ RX, 
   const int up = __shfl_up_sync(0xffffffffu, rseq, 1);
   const bool head = (lane == 0 || up != rseq) && rseq >= 0;
   double run = 0.0;
-  for (int c = 0; c < 16; ++c) {
+  for (int c = 0; c < kGT / 4; ++c) {
     const int cs = s_col[cb + c];
     if (cs < 0) break;
     const int64_t s = c0 + cb + c;
     const double v = (double)tile[row * (kGT + 1) + cb + c];
     if (kSampled) run += v;
     else if (t <= s) run += rseq == cs && t < s ? 2.0 * v : v;
-    if (c == 15 || s_col[cb + c + 1] != cs) {
+    if (c == kGT / 4 - 1 || s_col[cb + c + 1] != cs) {
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const double o = __shfl_down_sync(0xffffffffu, run, 1 << k);
@@ -810,14 +823,20 @@ isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint3
   return s != ISOPO_OK ? s : launch_f32_finish(kacc, B, K, st);
 }
 
+// Tokens per tile: 64, or 32 where `tiles` of 64 would not give every SM two CTAs.
+static bool f32_gram_small_tiles(int64_t tiles) { return tiles < 2 * 148; }
+
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                       double* kacc, float* K, cudaStream_t st) {
-  const int64_t nt = (T + kGT - 1) / kGT;
+  const int64_t n64 = (T + 63) / 64;
+  const bool small = f32_gram_small_tiles(n64 * (n64 + 1) / 2);
+  const int64_t nt = small ? (T + 31) / 32 : n64;
   if (nt > 65535) return ISOPO_ERR_UNSUPPORTED;
   ISOPO_CUDA_TRY(cudaMemsetAsync(kacc, 0, sizeof(double) * (size_t)B * B, st));
   {
     LaunchScope scope(kIdF32Gram, st);
-    launch(k_f32_gram<false>, dim3((unsigned)nt, (unsigned)nt), 256, 0, st, X, dY, T, X, dY, T, d_in, d_out, tokseq, B, kacc);
+    launch(small ? k_f32_gram<false, 32> : k_f32_gram<false, 64>, dim3((unsigned)nt, (unsigned)nt), small ? 128 : 256, 0, st, X, dY,
+           T, X, dY, T, d_in, d_out, tokseq, B, kacc);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return launch_f32_finish(kacc, B, K, st);
@@ -825,12 +844,14 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
 
 isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
                          int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st) {
-  const int64_t nt = (T + kGT - 1) / kGT, ns = (n_samples + kGT - 1) / kGT;
+  const bool small = f32_gram_small_tiles((T + 63) / 64 * ((n_samples + 63) / 64));
+  const int64_t nt = small ? (T + 31) / 32 : (T + 63) / 64, ns = small ? (n_samples + 31) / 32 : (n_samples + 63) / 64;
   if (ns > 65535) return ISOPO_ERR_UNSUPPORTED;
   ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(double) * (size_t)n_samples * B, st));
   {
     LaunchScope scope(kIdSampled, st);
-    launch(k_f32_gram<true>, dim3((unsigned)nt, (unsigned)ns), 256, 0, st, a0, g0, n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
+    launch(small ? k_f32_gram<true, 32> : k_f32_gram<true, 64>, dim3((unsigned)nt, (unsigned)ns), small ? 128 : 256, 0, st, a0, g0,
+           (int64_t)n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -59,6 +59,7 @@ SHAPES = [
     ([1 + i % 3 for i in range(200)], 36, 20),
     ([1 + i % 2 for i in range(400)], 20, 12),   # offsets through device memory
     ([2, 5], 900, 640),                          # combine whole (over 2^19 elements)
+    ([300, 299, 301, 633], 40, 21),              # Gram tiles of 64 (300 of them), the last one ragged
 ]
 
 
@@ -77,8 +78,9 @@ def test_layer(b, case, route):
 
 @pytest.mark.parametrize("n_samples", [1, 63, 65, 130])
 @pytest.mark.parametrize("d_in,d_out", [(64, 48), (37, 130)])
-def test_sampled(b, n_samples, d_in, d_out):
-    X, dY, off, A, G = _problem(d_in, d_out, [1, 70, 64, 33, 129], n_samples + d_in)
+@pytest.mark.parametrize("lens", [[1, 70, 64, 33, 129], [4000, 5000, 600, 1]])  # tiles of 32; of 64 for 65 and 130 samples
+def test_sampled(b, n_samples, d_in, d_out, lens):
+    X, dY, off, A, G = _problem(d_in, d_out, lens, n_samples + d_in)
     B, T = len(off) - 1, int(off[-1])
     rows = np.random.default_rng(n_samples).permutation(T)[:n_samples].astype(np.int64)
     ws = b.alloc_sampled_workspace(b.F32, T, d_in, d_out, B, n_samples)
