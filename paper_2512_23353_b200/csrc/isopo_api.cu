@@ -271,7 +271,7 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     }
     s = bf16_seq_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, order, B, L, G, fmt, info, st);
     if (s != ISOPO_OK) return s;
-    return bf16_ntk(G, L, B, K, /*k_is_zero=*/true, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
+    return bf16_ntk(G, L, B, K, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
   }
   double* kacc = (double*)(w + L.off_kacc);
   if (dtype == ISOPO_F32 && rp == ISOPO_PATH_MATERIALISE) {
@@ -281,7 +281,8 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
                      make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host), tag_dev, st);
     return s != ISOPO_OK ? s : f32_ntk(G, L.n_pad, B, kacc, done, K, st);
   }
-  s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, st);
+  const int64_t bb = (int64_t)B * B;
+  s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, dtype == ISOPO_F32 ? Clear{{(float*)kacc}, {2 * bb}} : Clear{{K}, {bb}}, st);
   if (s != ISOPO_OK) return s;
   if (dtype == ISOPO_F32) return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);
   return bf16_gram(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
@@ -305,7 +306,9 @@ isopo_status isopo_layer_gram_shared_x(const void* X, int n_proj, const void* co
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* w = (char*)ws;
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
-  isopo_status s = launch_prep(seq_offsets_host, B, T, (int64_t*)(w + L.off_offsets), tokseq, st);
+  Clear clear{};
+  for (int h = 0; h < n_proj; ++h) { clear.p[h] = K[h]; clear.n[h] = (int64_t)B * B; }
+  isopo_status s = launch_prep(seq_offsets_host, B, T, (int64_t*)(w + L.off_offsets), tokseq, clear, st);
   if (s != ISOPO_OK) return s;
   return bf16_gram_shared(X, dY, T, d_in, d_out, n_proj, tokseq, B, K, info, st);
 }
@@ -361,7 +364,7 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
   }
   for (int h = 0; h < n_proj; ++h) {
     float* kpart = deterministic_mode() ? (float*)((char*)ws[h] + L[h].off_kpart) : nullptr;
-    s = bf16_ntk(G[h], L[h], B, K[h], /*k_is_zero=*/true, kpart, fmt[h], info, st);
+    s = bf16_ntk(G[h], L[h], B, K[h], kpart, fmt[h], info, st);
     if (s != ISOPO_OK) return s;
   }
   return ISOPO_OK;
@@ -390,7 +393,9 @@ isopo_status isopo_sampled_coefficients(const void* X, const void* dY, isopo_dty
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* w = (char*)ws;
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
-  s = launch_prep(seq_offsets_host, B, T, (int64_t*)(w + L.off_offsets), tokseq, st);
+  const int64_t mt = (int64_t)n_samples * B * (dtype == ISOPO_F32 ? 2 : 1);  // M^T and its float64 denominator, in floats
+  s = launch_prep(seq_offsets_host, B, T, (int64_t*)(w + L.off_offsets), tokseq,
+                  Clear{{(float*)(w + S.off_mt), (float*)(w + S.off_den)}, {mt, 2}}, st);
   if (s != ISOPO_OK) return s;
   return sampled_coefficients(X, dY, dtype, T, d_in, d_out, tokseq, B, sample_rows_host, n_samples, w, S, A, lambda, coeffs,
                               F2, info, st);
@@ -514,25 +519,27 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
       return f32_combine((const float*)(w + L.off_G), (int64_t)d_in * d_out, L.n_pad, B, coeffs, dW, beta, tag_dev, tag, info, st);
     return bf16_combine(w + L.off_G, L, d_in, d_out, B, coeffs, dW, beta, tag_dev, tag, store_fmt(L, B, ws), info, st);
   }
-  // GEMM over all tokens: refresh the token -> sequence map so the call also works on its own.
+  // GEMM over all tokens: refresh the token -> sequence map so the call also works on its own.  The kernels add their
+  // token slabs into dW.
+  const Clear clear = beta == 0.f ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
   int64_t* off_dev = (int64_t*)(w + L.off_offsets);
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
   if (dtype == ISOPO_F32) {
-    s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, st);
+    s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, clear, st);
     if (s != ISOPO_OK) return s;
-    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, coeffs, tokseq, dW, beta, st);
+    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, coeffs, tokseq, dW, st);
   }
   if (bf16_weight_grad_fold_applies(T, d_in, d_out, B)) {
-    s = store_i64(seq_offsets_host, (int64_t)B + 1, off_dev, st);
+    s = launch_offsets(seq_offsets_host, B, off_dev, clear, st);
     if (s != ISOPO_OK) return s;
-    return bf16_weight_grad_fold(X, dY, T, d_in, d_out, off_dev, coeffs, B, dW, beta, info, st);
+    return bf16_weight_grad_fold(X, dY, T, d_in, d_out, off_dev, coeffs, B, dW, info, st);
   }
   // one scale per token, so that the kernel's scaler warps need a single independent load per row
   float* tokscale = (float*)tokseq;
-  s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, st);
+  s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);
   if (s != ISOPO_OK) return s;
   void* scaled = w + L.off_scaled;
-  return bf16_weight_grad(X, dY, T, d_in, d_out, tokscale, scaled, dW, beta, info, st);
+  return bf16_weight_grad(X, dY, T, d_in, d_out, tokscale, scaled, dW, info, st);
 }
 
 }  // extern "C"

@@ -111,9 +111,9 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved);
 
 // Workspace of isopo_sampled_coefficients: the Gram-route prefix (offsets, order, token map), then
-// the sampled row indices, the gathered rows a0 / g0, M^T and the denominator.
+// the gathered rows a0 / g0, M^T and the denominator.
 struct SampledLayout {
-  size_t off_rows, off_a0, off_g0, off_mt, off_den, total;
+  size_t off_a0, off_g0, off_mt, off_den, total;
 };
 SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples);
 
@@ -129,15 +129,20 @@ void set_cuda_error(cudaError_t e, const char* where);
 
 // ---- programmatic dependent launch ----
 // A layer is a chain of five to ten dependent kernels, several of them a few microseconds long.  Every kernel of the
-// library is launched so that its CTAs may be set up while its predecessor in the stream still runs, lets its own
-// successor do the same from its first instruction, and waits for everything before it to be complete and visible before
-// it touches memory (all of its CTAs do, so that the chain stays ordered end to end).  Work of other origin in the stream
-// is ordered as always.
-__device__ __forceinline__ void pdl_wait() {
+// library is launched so that its CTAs may be set up as soon as its predecessor in the stream lets them, and waits for
+// everything before it to be complete and visible before it touches memory (all of its CTAs do, so that the chain stays
+// ordered end to end).  Work of other origin in the stream is ordered as always.
+//   pdl_begin  waits, then lets the successor in while this kernel runs: kernels of one CTA per SM, which leave no room
+//              beside them, and kernels of a few CTAs
+//   pdl_wait   waits; the successor is let in when the last CTA leaves.  Kernels of several CTAs per SM: a successor let
+//              in earlier finds a few SMs with room and is crowded onto them (a float32 layer of 102 sequences, 789
+//              tokens: 184 us a pass when every kernel let its successor in at once, 133 us so)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
-// The kernel must call pdl_wait().  Errors are picked up by the cudaGetLastError() that follows every launch.
+// The kernel must call pdl_begin() or pdl_wait().  Errors are picked up by the cudaGetLastError() that follows every launch.
 template <typename... Params, typename... Args>
 inline void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -155,17 +160,24 @@ inline void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem
 
 // ---- launchers (each enqueues on `st` and returns a status; none synchronises) ----
 
-isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, cudaStream_t st);
+// Up to three float32 regions that a launch clears for the kernels behind it (n = 0: none).
+struct Clear {
+  float* p[3];
+  int64_t n[3];
+};
+// offsets and the token -> sequence map to the device, `clear` cleared
+isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, const Clear& clear,
+                         cudaStream_t st);
+// the offsets alone
+isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, const Clear& clear, cudaStream_t st);
 // bf16 materialised path (B <= 256) in one launch: offsets, the longest-first order, the workspace tag, K = 0
 isopo_status launch_prep_stored(const int64_t* off_host, int B, const WsTag& tag, int64_t* off_dev, int32_t* order_dev,
                                 WsTag* tag_dev, float* K, cudaStream_t st);
 isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj, const WsTag* tag, int64_t* const* off_dev,
                                       int32_t* const* order_dev, WsTag* const* tag_dev, float* const* K, cudaStream_t st);
-// offsets to the device and tokscale[t] = coeffs[sequence of token t] (float32 [T])
+// offsets and tokscale[t] = coeffs[sequence of token t] (float32 [T])
 isopo_status launch_tokscale(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs,
-                             float* tokscale, cudaStream_t st);
-// n host values -> device array, passed as kernel arguments (no host-to-device copy)
-isopo_status store_i64(const int64_t* host, int64_t n, int64_t* dev, cudaStream_t st);
+                             float* tokscale, const Clear& clear, cudaStream_t st);
 // true when every word of the tag in the workspace equals `want`; otherwise the first thread of the grid
 // records ISOPO_INFO_STALE_WORKSPACE (device code, used by the combine kernels)
 __device__ __forceinline__ bool ws_tag_matches(const WsTag* __restrict__ have, const WsTag& want, int32_t* info) {
@@ -182,7 +194,7 @@ isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, 
                           int B, float* G, int64_t gstride, double* kacc, uint32_t* done, const WsTag& tag, WsTag* tag_dev,
                           cudaStream_t st);
 isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, cudaStream_t st);
-// M^T [n_samples, B] of the sampled rows a0, g0
+// M^T [n_samples, B] += of the sampled rows a0, g0
 isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
                          int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st);
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
@@ -190,7 +202,7 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
 isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, const float* coeffs, float* dW, float beta,
                          const WsTag* tag_dev, const WsTag& tag, int32_t* info, cudaStream_t st);
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* coeffs,
-                             const int32_t* tokseq, float* dW, float beta, cudaStream_t st);
+                             const int32_t* tokseq, float* dW, cudaStream_t st);
 
 // bf16 tcgen05 path
 isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
@@ -209,10 +221,10 @@ isopo_status launch_seq_scales(const void* X, const void* dY, int d_in, int d_ou
 isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* const* dY, const int* d_out, int64_t T, int d_in,
                                        const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout* L,
                                        void* const* G, const StoreFmt* fmt, int32_t* info, cudaStream_t st);
-// k_is_zero: the caller has already cleared K on this stream.  kpart != NULL (deterministic mode): every CTA
+// Adds into K, which the caller has cleared on this stream.  kpart != NULL (deterministic mode): every CTA
 // stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and a second kernel sums them in order.
 constexpr int kNtkMaxPartials = 160;
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_is_zero, float* kpart, const StoreFmt& fmt,
+isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, float* kpart, const StoreFmt& fmt,
                       int32_t* info, cudaStream_t st);
 bool deterministic_mode();
 // K[i][j] = K[j][i] for j < i (the Gram kernels fill the upper triangle)
@@ -220,19 +232,21 @@ isopo_status mirror_upper(float* K, int B, cudaStream_t st);
 isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out, int B, const float* coeffs, float* dW,
                           float beta, const WsTag* tag_dev, const WsTag& tag, const StoreFmt& fmt, int32_t* info,
                           cudaStream_t st);
+// The Gram, sampled and weight-gradient kernels ADD into K, M^T and dW: the caller has cleared them on this stream (or wants
+// the sum).
 isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                        float* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              void* scaled, float* dW, float beta, int32_t* info, cudaStream_t st);
+                              void* scaled, float* dW, int32_t* info, cudaStream_t st);
 
 // dW with the per-sequence coefficient applied when a segment's accumulator is drained (no scaled operand copy)
 bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, float* dW, float beta, int32_t* info, cudaStream_t st);
+                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st);
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                                   void* scaled, float* dW, float beta, int32_t* info, cudaStream_t st);
+                                   void* scaled, float* dW, int32_t* info, cudaStream_t st);
 
 // token-sampled estimator of Algorithm 1
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,

@@ -62,15 +62,18 @@ __device__ __forceinline__ double copy_row_sq(const T* __restrict__ src, T* __re
   return acc;
 }
 
+// The sample rows, as kernel arguments (token indices are below 2^31).
+template <int kN> struct RowArgs { int32_t v[kN]; };
+
 // Block j copies token row rows[j] of X and dY into a0[j], g0[j] and adds ||g0_j||^2 ||a0_j||^2 to *den.
-template <typename T>
+template <typename T, int kN>
 __global__ void __launch_bounds__(256) k_gather_samples(const T* __restrict__ X, const T* __restrict__ dY, int d_in,
-                                                        int d_out, const int64_t* __restrict__ rows,
+                                                        int d_out, const __grid_constant__ RowArgs<kN> rows,
                                                         T* __restrict__ a0, T* __restrict__ g0,
                                                         double* __restrict__ den) {
   pdl_wait();
   const int j = blockIdx.x;
-  const int64_t t = rows[j];
+  const int64_t t = rows.v[j];
   double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * d_in, d_in);
   double ng = copy_row_sq(dY + t * d_out, g0 + (size_t)j * d_out, d_out);
   na = block_sum_d(na);
@@ -108,14 +111,31 @@ __global__ void __launch_bounds__(32 * kFinishSlices) k_sampled_finish(const TM*
   coeffs[i] = (float)((double)A[i] / sqrt(f2 + (double)lambda));
 }
 
+template <int kN, typename T>
+isopo_status gather_with(const T* X, const T* dY, int d_in, int d_out, const int64_t* rows_host, int n_samples, T* a0, T* g0,
+                         double* den, cudaStream_t st) {
+  RowArgs<kN> rows;
+  for (int j = 0; j < n_samples; ++j) rows.v[j] = (int32_t)rows_host[j];
+  {
+    LaunchScope scope(kIdSampledAux, st);
+    launch(k_gather_samples<T, kN>, n_samples, 256, 0, st, X, dY, d_in, d_out, rows, a0, g0, den);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
+}
+template <typename T>
+isopo_status gather_samples(const T* X, const T* dY, int d_in, int d_out, const int64_t* rows_host, int n_samples, T* a0, T* g0,
+                            double* den, cudaStream_t st) {
+  return n_samples <= 256 ? gather_with<256>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st)
+                          : gather_with<ISOPO_MAX_SAMPLES>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st);
+}
+
 }  // namespace
 
 SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples) {
   SampledLayout S{};
   const size_t elt = dtype == ISOPO_BF16 ? 2 : 4;
   size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM).total;  // offsets, order, token map (+ kacc)
-  S.off_rows = p;
-  p = align_up(p + sizeof(int64_t) * (size_t)n_samples, 1024);
   S.off_a0 = p;
   p = align_up(p + elt * (size_t)n_samples * d_in, 1024);
   S.off_g0 = p;
@@ -132,20 +152,13 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
                                   const int32_t* tokseq, int B, const int64_t* rows_host, int n_samples, char* ws,
                                   const SampledLayout& S, const float* A, float lambda, float* coeffs, float* F2,
                                   int32_t* info, cudaStream_t st) {
-  int64_t* rows = (int64_t*)(ws + S.off_rows);
-  double* den = (double*)(ws + S.off_den);
-  isopo_status s = store_i64(rows_host, n_samples, rows, st);
-  if (s != ISOPO_OK) return s;
-  ISOPO_CUDA_TRY(cudaMemsetAsync(den, 0, sizeof(double), st));
+  double* den = (double*)(ws + S.off_den);  // cleared, like M^T
+  isopo_status s;
   if (dtype == ISOPO_F32) {
     float* a0 = (float*)(ws + S.off_a0);
     float* g0 = (float*)(ws + S.off_g0);
     double* Mt = (double*)(ws + S.off_mt);
-    {
-      LaunchScope scope(kIdSampledAux, st);
-      launch(k_gather_samples<float>, n_samples, 256, 0, st, (const float*)X, (const float*)dY, d_in, d_out, rows, a0, g0, den);
-    }
-    ISOPO_CUDA_TRY(cudaGetLastError());
+    if ((s = gather_samples((const float*)X, (const float*)dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st)) != ISOPO_OK) return s;
     s = f32_sampled((const float*)X, (const float*)dY, T, d_in, d_out, a0, g0, n_samples, tokseq, B, Mt, st);
     if (s != ISOPO_OK) return s;
     {
@@ -158,12 +171,8 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
   __nv_bfloat16* a0 = (__nv_bfloat16*)(ws + S.off_a0);
   __nv_bfloat16* g0 = (__nv_bfloat16*)(ws + S.off_g0);
   float* Mt = (float*)(ws + S.off_mt);
-  {
-    LaunchScope scope(kIdSampledAux, st);
-    launch(k_gather_samples<__nv_bfloat16>, n_samples, 256, 0, st, (const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out,
-                                                               rows, a0, g0, den);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
+  s = gather_samples((const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st);
+  if (s != ISOPO_OK) return s;
   s = bf16_sampled(X, dY, T, d_in, d_out, tokseq, B, a0, g0, n_samples, Mt, info, st);
   if (s != ISOPO_OK) return s;
   {

@@ -11,12 +11,27 @@ namespace {
 
 // Host values travel to the device as kernel arguments (no host-to-device copy, so no hidden
 // synchronisation with the stream and nothing that reads the caller's array after the call returns).
-constexpr int kArgChunk = 384;
-struct OffsetArgs { int64_t v[kArgChunk]; };
-__global__ void k_store_offsets(OffsetArgs a, int base, int n, int64_t* __restrict__ off) {
+// Token offsets are below 2^31 and travel as 32-bit values.
+constexpr int kArgChunk = 384;    // the usual case; 1.5 KB of arguments
+constexpr int kArgLarge = 2048;   // up to here still one launch
+template <int kN> struct OffsetArgs { int32_t v[kN]; };
+template <int kN>
+__global__ void __launch_bounds__(256) k_store_offsets(const __grid_constant__ OffsetArgs<kN> a, int64_t base, int n,
+                                                       int64_t* __restrict__ off) {
   pdl_wait();
-  const int t = threadIdx.x;
-  if (t < n) off[base + t] = a.v[t];
+  for (int t = threadIdx.x; t < n; t += blockDim.x) off[base + t] = a.v[t];
+}
+
+// Clears the regions that the kernels behind this one add into (in place of a memset for each).
+__device__ __forceinline__ void clear_regions(const Clear& c) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (c.n[k] == 0) continue;
+    const int64_t quads = (reinterpret_cast<uintptr_t>(c.p[k]) & 15) == 0 ? c.n[k] / 4 : 0;
+    for (int64_t e = first; e < quads; e += step) reinterpret_cast<float4*>(c.p[k])[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t e = 4 * quads + first; e < c.n[k]; e += step) c.p[k][e] = 0.f;
+  }
 }
 
 // Everything the bf16 stored-gradient kernels need before they start, in one launch (B <= 256):
@@ -42,53 +57,43 @@ __global__ void __launch_bounds__(256) k_prep_stored(StoredPrepArgs a, int B, in
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * B; e += gridDim.x * blockDim.x) a.K[h][e] = 0.f;
   }
 }
-__global__ void k_tokseq(const int64_t* __restrict__ off, int B, int64_t T, int32_t* __restrict__ tokseq) {
-  pdl_wait();
+// What a kernel over all tokens needs before it starts, in one launch: the offsets in the workspace, the regions it adds
+// into cleared, and per token its sequence (kOut = kTokSeq) or that sequence's coefficient (kTokScale).
+enum PrepOut { kOffsetsOnly, kTokSeq, kTokScale };
+template <int kOut, typename Off>
+__device__ __forceinline__ void fill_tokens(const Off* off, int B, int64_t T, const float* __restrict__ coeffs, void* __restrict__ out) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
     int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
     while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (off[mid] <= t) lo = mid; else hi = mid;
+      const int mid = (lo + hi) >> 1;
+      if (off[mid] <= (Off)t) lo = mid; else hi = mid;
     }
-    tokseq[t] = lo;
-  }
-}
-
-// tokscale[t] = coeffs[sequence of token t]: what the folded weight-gradient GEMM multiplies row t by.
-__global__ void k_tokscale(const int64_t* __restrict__ off, int B, int64_t T, const float* __restrict__ coeffs,
-                           float* __restrict__ tokscale) {
-  pdl_wait();
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (off[mid] <= t) lo = mid; else hi = mid;
-    }
-    tokscale[t] = coeffs[lo];
-  }
-}
-
-// k_store_offsets + k_tokseq / k_tokscale in one launch when all B + 1 offsets fit one argument block:
-// every CTA copies them to shared memory and searches there; CTA 0 also leaves them in the workspace.
-template <bool kScale>
-__global__ void __launch_bounds__(256) k_prep_small(OffsetArgs a, int B, int64_t T, int64_t* __restrict__ off_dev,
-                                                    const float* __restrict__ coeffs, void* __restrict__ out) {
-  pdl_wait();
-  __shared__ int64_t s_off[kArgChunk];
-  for (int i = threadIdx.x; i <= B; i += blockDim.x) {
-    s_off[i] = a.v[i];
-    if (blockIdx.x == 0) off_dev[i] = a.v[i];
-  }
-  __syncthreads();
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (s_off[mid] <= t) lo = mid; else hi = mid;
-    }
-    if (kScale) static_cast<float*>(out)[t] = coeffs[lo];
+    if (kOut == kTokScale) static_cast<float*>(out)[t] = coeffs[lo];
     else static_cast<int32_t*>(out)[t] = lo;
   }
+}
+// offsets in the arguments: every CTA copies them to shared memory and searches there; CTA 0 also leaves them in the workspace
+template <int kOut, int kN>
+__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ OffsetArgs<kN> a, int B, int64_t T,
+                                              int64_t* __restrict__ off_dev, const float* __restrict__ coeffs,
+                                              void* __restrict__ out, const __grid_constant__ Clear clear) {
+  __shared__ int32_t s_off[kN];
+  for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = a.v[i];
+  pdl_wait();
+  __syncthreads();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= B; i += blockDim.x) off_dev[i] = s_off[i];
+  clear_regions(clear);
+  if (kOut != kOffsetsOnly) fill_tokens<kOut>(s_off, B, T, coeffs, out);
+}
+// more sequences than the arguments hold: k_store_offsets has left the offsets in the workspace
+template <int kOut>
+__global__ void __launch_bounds__(256) k_prep_many(const int64_t* __restrict__ off_dev, int B, int64_t T,
+                                                   const float* __restrict__ coeffs, void* __restrict__ out,
+                                                   const __grid_constant__ Clear clear) {
+  pdl_wait();
+  clear_regions(clear);
+  if (kOut != kOffsetsOnly) fill_tokens<kOut>(off_dev, B, T, coeffs, out);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -237,7 +242,7 @@ struct F32StoredArgs {
   WsTag* tag_dev;
 };
 template <bool kArgOff> struct OffsetParam { int64_t v[1]; };
-template <> struct OffsetParam<true> { int64_t v[kArgChunk]; };
+template <> struct OffsetParam<true> { int32_t v[kArgChunk]; };
 static_assert(sizeof(F32StoredArgs) + sizeof(OffsetParam<true>) <= 4096, "kernel arguments");
 
 template <int kTile, int kT, bool kArgOff>
@@ -671,57 +676,47 @@ __global__ void __launch_bounds__(256) k_f32_combine(const float* __restrict__ G
 
 }  // namespace
 
-isopo_status store_i64(const int64_t* host, int64_t n, int64_t* dev, cudaStream_t st) {
-  for (int64_t base = 0; base < n; base += kArgChunk) {
-    OffsetArgs a;
-    const int m = (int)std::min<int64_t>(kArgChunk, n - base);
-    for (int t = 0; t < m; ++t) a.v[t] = host[base + t];
-    launch(k_store_offsets, 1, kArgChunk, 0, st, a, (int)base, m, dev);
+template <int kOut>
+static isopo_status prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs, void* out,
+                         const Clear& clear, cudaStream_t st) {
+  const int64_t work = std::max<int64_t>(kOut == kOffsetsOnly ? 1 : T, (clear.n[0] + clear.n[1] + clear.n[2]) / 4);
+  const int grid = (int)std::min<int64_t>((work + 255) / 256, 1184);
+  LaunchScope scope(kIdPrep, st);
+  if (B + 1 <= kArgChunk) {
+    OffsetArgs<kArgChunk> a;
+    for (int t = 0; t <= B; ++t) a.v[t] = (int32_t)off_host[t];
+    launch(k_prep<kOut, kArgChunk>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out, clear);
+  } else if (B + 1 <= kArgLarge) {
+    OffsetArgs<kArgLarge> a;
+    for (int t = 0; t <= B; ++t) a.v[t] = (int32_t)off_host[t];
+    launch(k_prep<kOut, kArgLarge>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out, clear);
+  } else {
+    for (int64_t base = 0; base <= B; base += kArgLarge) {
+      OffsetArgs<kArgLarge> a;
+      const int m = (int)std::min<int64_t>(kArgLarge, B + 1 - base);
+      for (int t = 0; t < m; ++t) a.v[t] = (int32_t)off_host[base + t];
+      launch(k_store_offsets<kArgLarge>, 1, 256, 0, st, a, base, m, off_dev);
+    }
     ISOPO_CUDA_TRY(cudaGetLastError());
-  }
-  return ISOPO_OK;
-}
-
-template <bool kScale>
-static isopo_status launch_prep_small(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs,
-                                      void* out, cudaStream_t st) {
-  OffsetArgs a;
-  for (int t = 0; t <= B; ++t) a.v[t] = off_host[t];
-  const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
-  {
-    LaunchScope scope(kIdPrep, st);
-    launch(k_prep_small<kScale>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out);
+    if (kOut != kOffsetsOnly || clear.n[0] + clear.n[1] + clear.n[2] > 0)
+      launch(k_prep_many<kOut>, grid, 256, 0, st, off_dev, B, T, coeffs, out, clear);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 
-isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq,
+isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, const Clear& clear,
                          cudaStream_t st) {
-  if (B + 1 <= kArgChunk) return launch_prep_small<false>(off_host, B, T, off_dev, nullptr, tokseq, st);
-  isopo_status s = store_i64(off_host, (int64_t)B + 1, off_dev, st);
-  if (s != ISOPO_OK) return s;
-  const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
-  {
-    LaunchScope scope(kIdPrep, st);
-    launch(k_tokseq, grid, 256, 0, st, off_dev, B, T, tokseq);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
+  return prep<kTokSeq>(off_host, B, T, off_dev, nullptr, tokseq, clear, st);
 }
 
 isopo_status launch_tokscale(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs,
-                             float* tokscale, cudaStream_t st) {
-  if (B + 1 <= kArgChunk) return launch_prep_small<true>(off_host, B, T, off_dev, coeffs, tokscale, st);
-  isopo_status s = store_i64(off_host, (int64_t)B + 1, off_dev, st);
-  if (s != ISOPO_OK) return s;
-  const int grid = (int)std::min<int64_t>((T + 255) / 256, 1184);
-  {
-    LaunchScope scope(kIdPrep, st);
-    launch(k_tokscale, grid, 256, 0, st, off_dev, B, T, coeffs, tokscale);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
+                             float* tokscale, const Clear& clear, cudaStream_t st) {
+  return prep<kTokScale>(off_host, B, T, off_dev, coeffs, tokscale, clear, st);
+}
+
+isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, const Clear& clear, cudaStream_t st) {
+  return prep<kOffsetsOnly>(off_host, B, 0, off_dev, nullptr, nullptr, clear, st);
 }
 
 isopo_status launch_prep_stored(const int64_t* off_host, int B, const WsTag& tag, int64_t* off_dev, int32_t* order_dev,
@@ -778,10 +773,10 @@ isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, 
   const bool wide = f32_wide_tiles(d_in, d_out, B);
   if (B + 1 <= kArgChunk) {
     OffsetParam<true> o;
-    for (int i = 0; i <= B; ++i) o.v[i] = off_host[i];
+    for (int i = 0; i <= B; ++i) o.v[i] = (int32_t)off_host[i];
     return wide ? launch_f32_seq_grad<128, 8, true>(a, o, st) : launch_f32_seq_grad<64, 4, true>(a, o, st);
   }
-  isopo_status s = store_i64(off_host, (int64_t)B + 1, off_dev, st);
+  isopo_status s = launch_offsets(off_host, B, off_dev, Clear{}, st);
   if (s != ISOPO_OK) return s;
   const OffsetParam<false> o{};
   return wide ? launch_f32_seq_grad<128, 8, false>(a, o, st) : launch_f32_seq_grad<64, 4, false>(a, o, st);
@@ -832,7 +827,6 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
   const bool small = f32_gram_small_tiles(n64 * (n64 + 1) / 2);
   const int64_t nt = small ? (T + 31) / 32 : n64;
   if (nt > 65535) return ISOPO_ERR_UNSUPPORTED;
-  ISOPO_CUDA_TRY(cudaMemsetAsync(kacc, 0, sizeof(double) * (size_t)B * B, st));
   {
     LaunchScope scope(kIdF32Gram, st);
     launch(small ? k_f32_gram<false, 32> : k_f32_gram<false, 64>, dim3((unsigned)nt, (unsigned)nt), small ? 128 : 256, 0, st, X, dY,
@@ -847,7 +841,6 @@ isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, i
   const bool small = f32_gram_small_tiles((T + 63) / 64 * ((n_samples + 63) / 64));
   const int64_t nt = small ? (T + 31) / 32 : (T + 63) / 64, ns = small ? (n_samples + 31) / 32 : (n_samples + 63) / 64;
   if (ns > 65535) return ISOPO_ERR_UNSUPPORTED;
-  ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(double) * (size_t)n_samples * B, st));
   {
     LaunchScope scope(kIdSampled, st);
     launch(small ? k_f32_gram<true, 32> : k_f32_gram<true, 64>, dim3((unsigned)nt, (unsigned)ns), small ? 128 : 256, 0, st, a0, g0,
@@ -892,8 +885,7 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
 }
 
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* coeffs,
-                             const int32_t* tokseq, float* dW, float beta, cudaStream_t st) {
-  if (beta == 0.f) ISOPO_CUDA_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)d_in * d_out, st));
+                             const int32_t* tokseq, float* dW, cudaStream_t st) {
   return f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st)
                                                       : launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st);
 }

@@ -78,9 +78,11 @@ extern "C" ISOPO_API isopo_status isopo_layer_gram_static(const void* X, const v
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   ProfilingPause pause;  // event timing would create events: keep this call free of any allocation
-  // Every region that is read is rewritten first: the offsets and the map for [0, T) here, the
-  // accumulators by a memset inside the float32 route.  Nothing left by an earlier call is used.
-  s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, st);
+  // Every region that is read is rewritten first: the offsets, the map for [0, T) and the accumulators.
+  // Nothing left by an earlier call is used.
+  const int64_t bb = (int64_t)B * B;
+  const Clear clear = dtype == ISOPO_F32 ? Clear{{(float*)kacc}, {2 * bb}} : Clear{{K}, {bb}};
+  s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, clear, st);
   if (s != ISOPO_OK) return s;
   if (dtype == ISOPO_F32)
     return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);

@@ -87,7 +87,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -219,7 +219,6 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  ISOPO_CUDA_TRY(cudaMemsetAsync(K, 0, sizeof(float) * (size_t)B * B, st));
   GramParams p{tokseq, K, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, 0, 0, 0};
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms);
@@ -245,7 +244,6 @@ isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, in
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  ISOPO_CUDA_TRY(cudaMemsetAsync(Mt, 0, sizeof(float) * (size_t)n_samples * B, st));
   GramParams p{tokseq, Mt, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, n_samples, (n_samples + kTT - 1) / kTT, 0};
   const long long units = (long long)p.n_row_tiles * p.nT;
   const int grid = (int)std::min<long long>(units, sms);

@@ -63,7 +63,7 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -234,7 +234,6 @@ isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, i
     p.K[h] = K[h];
     p.d_out[h] = d_out[h];
     d_sum += d_out[h];
-    ISOPO_CUDA_TRY(cudaMemsetAsync(K[h], 0, sizeof(float) * (size_t)B * B, st));
   }
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms);

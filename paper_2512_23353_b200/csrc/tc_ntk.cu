@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ 
 
 }  // namespace
 
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_is_zero, float* kpart, const StoreFmt& fmt,
+isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, float* kpart, const StoreFmt& fmt,
                       int32_t* info, cudaStream_t st) {
   if (B > 256) return ISOPO_ERR_UNSUPPORTED;
   if (fmt.split && kpart) return ISOPO_ERR_INVALID_ARG;  // the split store's diagonal is summed with float atomics
@@ -454,7 +454,6 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, bool k_
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   auto kernel = fmt.split ? k_bf16_ntk<true> : k_bf16_ntk<false>;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  if (!k_is_zero && !kpart) ISOPO_CUDA_TRY(cudaMemsetAsync(K, 0, sizeof(float) * (size_t)B * B, st));
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
   NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, (pieces + ppb - 1) / ppb * (fmt.split ? 2 : 4), info, (int)rows,
               (int)ppb};

@@ -120,7 +120,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   if (!kFolded) {
     for (int k = threadIdx.x; k < p.B; k += blockDim.x) {
       const int i = p.order[k];
@@ -373,10 +373,10 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
 }
 
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              void* scaled, float* dW, float beta, int32_t* info, cudaStream_t st) {
+                              void* scaled, float* dW, int32_t* info, cudaStream_t st) {
   {  // 2-CTA tiles when they waste little (see bf16_seq_grad)
     const int tiles_m = (d_out + kTileM - 1) / kTileM;
-    if (tiles_m % 2 == 0 || tiles_m >= 7) return bf16_weight_grad_pair(X, dY, T, d_in, d_out, tokscale, scaled, dW, beta, info, st);
+    if (tiles_m % 2 == 0 || tiles_m >= 7) return bf16_weight_grad_pair(X, dY, T, d_in, d_out, tokscale, scaled, dW, info, st);
   }
   CUtensorMap mapY, mapX;
   isopo_status s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out);
@@ -384,7 +384,6 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   int sms = 0;
   if ((s = sm_count(&sms)) != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  if (beta == 0.f) ISOPO_CUDA_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)d_in * d_out, st));
   SeqGradParams p{};
   p.tiles_m = (d_out + kTileM - 1) / kTileM;
   p.tiles_n = (d_in + kTileN - 1) / kTileN;

@@ -156,7 +156,7 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   for (int k = threadIdx.x; k < p.B; k += kThreads) {
     const int i = p.order[k];
     const int64_t t0 = p.off[i];

@@ -150,7 +150,7 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   for (int k = threadIdx.x; k <= p.B; k += kThreads) s_off[k] = (int)p.off[k];
   for (int k = threadIdx.x; k < p.B; k += kThreads) s_coef[k] = p.coeffs[k];
   tc_fence_before_sync();
@@ -360,7 +360,7 @@ bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B) {
 }
 
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, float* dW, float beta, int32_t* info, cudaStream_t st) {
+                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -370,7 +370,6 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
   if (s != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  if (beta == 0.f) ISOPO_CUDA_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)d_in * d_out, st));
   static int resident_pairs[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident_pairs[dev] == 0) {

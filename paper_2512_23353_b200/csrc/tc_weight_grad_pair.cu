@@ -88,7 +88,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
-  pdl_wait();
+  pdl_begin();
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ sr
 }  // namespace
 
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                                   void* scaled, float* dW, float beta, int32_t* info, cudaStream_t st) {
+                                   void* scaled, float* dW, int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -262,7 +262,6 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
   s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
   if (s != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  if (beta == 0.f) ISOPO_CUDA_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)d_in * d_out, st));
   static int resident_pairs[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident_pairs[dev] == 0) {

@@ -90,7 +90,7 @@ __device__ __forceinline__ double block_total(double v, double* s_part) {
 // itself.  Bound by latency: the seven layers of a block at 256 sequences took 25 us with one CTA per layer.
 constexpr int kSimpleRows = 32;
 __global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant__ TransformBatch batch) {
-  pdl_wait();
+  pdl_begin();
   const TransformParams P = layer_params(batch, blockIdx.x);
   __shared__ double s_part[8];
   const int B = P.B, tid = threadIdx.x, first = blockIdx.y * kSimpleRows;
@@ -145,7 +145,7 @@ __device__ __forceinline__ double newton_rcp(double d) {
 }
 template <int kA>
 __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__ TransformBatch batch) {
-  pdl_wait();
+  pdl_begin();
   extern __shared__ __align__(16) double smem_d[];
   const TransformParams P = layer_params(batch, blockIdx.x);
   const int B = P.B, n = B + (B & 1), tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, pitch = n + 1;
@@ -252,7 +252,7 @@ inline size_t small_smem_bytes(int B) {
 
 // Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
 __global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_constant__ TransformBatch batch) {
-  pdl_wait();
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TransformParams P = layer_params(batch, blockIdx.x);
   __shared__ double s_trace, s_res;
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_consta
 constexpr int kMaxLargeB = ISOPO_MAX_LARGE_SEQS;
 constexpr int kLargeCluster = 16;
 __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const TransformParams P, float* scratch) {
-  pdl_wait();
+  pdl_begin();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   cluster_solve<kLargeCluster>(P, scratch, smem_raw, 0);
 }
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const Transfo
 constexpr int kEmaThreads = 1024;
 __global__ void __launch_bounds__(kEmaThreads) k_reg_ema(const float* __restrict__ K, int B, float decay,
                                                          float* __restrict__ state) {
-  pdl_wait();
+  pdl_begin();
   __shared__ double s_part[3][kEmaThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5;
   double tr = 0.0, f2 = 0.0, rel = 0.0;
