@@ -81,13 +81,11 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   WsLayout L{};
   size_t p = 0;
   L.off_tag = p;
-  p = align_up(p + sizeof(WsTag), 1024);
+  p = align_up(p + sizeof(WsHead), 1024);
   L.off_aux = p;
   if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_MATERIALISE) p = align_up(p + 2 * sizeof(float) * (size_t)B, 1024);
   L.off_offsets = p;
   p = align_up(p + sizeof(int64_t) * (size_t)(B + 1), 1024);
-  L.off_order = p;
-  p = align_up(p + sizeof(int32_t) * (size_t)B, 1024);
   L.off_tokseq = p;
   p = align_up(p + sizeof(int32_t) * (size_t)T, 1024);
   L.off_kacc = p;
@@ -258,20 +256,20 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
   WsTag* tag_dev = (WsTag*)(w + L.off_tag);
   if (dtype == ISOPO_BF16 && rp == ISOPO_PATH_MATERIALISE) {
-    // the stored-gradient kernels need the offsets and the longest-first order, not the token map
     void* G = w + L.off_G;
-    int32_t* order = (int32_t*)(w + L.off_order);
-    s = launch_prep_stored(seq_offsets_host, B, make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host), off_dev, order,
-                           tag_dev, K, st);
-    if (s != ISOPO_OK) return s;
+    WsHead* head = (WsHead*)(w + L.off_tag);
+    const WsTag tag = make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host);
+    StoredIntake in;
+    make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &K);
     const StoreFmt fmt = store_fmt(L, B, ws);
     if (fmt.split) {
-      s = launch_seq_scales(X, dY, d_in, d_out, off_dev, B, (float*)fmt.scales, fmt.kdiag, st);
+      s = launch_offsets(seq_offsets_host, B, off_dev, Clear{}, st);
+      if (s == ISOPO_OK) s = launch_seq_scales(X, dY, d_in, d_out, off_dev, B, (float*)fmt.scales, fmt.kdiag, st);
       if (s != ISOPO_OK) return s;
     }
-    s = bf16_seq_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, order, B, L, G, fmt, info, st);
+    s = bf16_seq_grad(X, dY, T, d_in, d_out, in, B, L, G, fmt, info, st);
     if (s != ISOPO_OK) return s;
-    return bf16_ntk(G, L, B, K, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
+    return bf16_ntk(G, L, B, K, head, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
   }
   double* kacc = (double*)(w + L.off_kacc);
   if (dtype == ISOPO_F32 && rp == ISOPO_PATH_MATERIALISE) {
@@ -322,9 +320,8 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
   if (dtype != ISOPO_BF16 || B > 256) return ISOPO_ERR_UNSUPPORTED;
   WsLayout L[3];
   WsTag tag[3];
-  int64_t* off_dev[3];
-  int32_t* order[3];
-  WsTag* tag_dev[3];
+  int64_t* off_dev = nullptr;
+  WsHead* head[3];
   void* G[3];
   StoreFmt fmt[3];
   bool pairs_fit = true;
@@ -338,33 +335,37 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
     if (ws_bytes[h] < L[h].total) return ISOPO_ERR_WORKSPACE;
     char* w = (char*)ws[h];
     tag[h] = make_ws_tag(dtype, T, d_in, d_out[h], B, seq_offsets_host);
-    off_dev[h] = (int64_t*)(w + L[h].off_offsets);
-    order[h] = (int32_t*)(w + L[h].off_order);
-    tag_dev[h] = (WsTag*)(w + L[h].off_tag);
+    if (h == 0) off_dev = (int64_t*)(w + L[h].off_offsets);
+    head[h] = (WsHead*)(w + L[h].off_tag);
     G[h] = w + L[h].off_G;
     fmt[h] = store_fmt(L[h], B, ws[h]);
     pairs_fit = pairs_fit && (L[h].tiles_m % 2 == 0 || L[h].tiles_m >= 7);
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  isopo_status s = launch_prep_stored_multi(seq_offsets_host, B, n_proj, tag, off_dev, order, tag_dev, K, st);
-  if (s != ISOPO_OK) return s;
+  isopo_status s = ISOPO_OK;
+  bool have_offsets = false;
   for (int h = 0; h < n_proj; ++h)
     if (fmt[h].split) {
-      s = launch_seq_scales(X, dY[h], d_in, d_out[h], off_dev[0], B, (float*)fmt[h].scales, fmt[h].kdiag, st);
+      if (!have_offsets) s = launch_offsets(seq_offsets_host, B, off_dev, Clear{}, st);
+      have_offsets = true;
+      if (s == ISOPO_OK) s = launch_seq_scales(X, dY[h], d_in, d_out[h], off_dev, B, (float*)fmt[h].scales, fmt[h].kdiag, st);
       if (s != ISOPO_OK) return s;
     }
+  StoredIntake in;
   if (pairs_fit) {
-    s = bf16_seq_grad_pair_shared(X, n_proj, dY, d_out, T, d_in, off_dev[0], order[0], B, L, G, fmt, info, st);
+    make_stored_intake(&in, seq_offsets_host, B, n_proj, tag, head, K);
+    s = bf16_seq_grad_pair_shared(X, n_proj, dY, d_out, T, d_in, in, B, L, G, fmt, info, st);
     if (s != ISOPO_OK) return s;
   } else {  // a projection with an odd, small number of 128-row tiles would idle half of its pairs: one launch each
     for (int h = 0; h < n_proj; ++h) {
-      s = bf16_seq_grad(X, dY[h], T, d_in, d_out[h], seq_offsets_host, off_dev[h], order[h], B, L[h], G[h], fmt[h], info, st);
+      make_stored_intake(&in, seq_offsets_host, B, 1, tag + h, head + h, K + h);
+      s = bf16_seq_grad(X, dY[h], T, d_in, d_out[h], in, B, L[h], G[h], fmt[h], info, st);
       if (s != ISOPO_OK) return s;
     }
   }
   for (int h = 0; h < n_proj; ++h) {
     float* kpart = deterministic_mode() ? (float*)((char*)ws[h] + L[h].off_kpart) : nullptr;
-    s = bf16_ntk(G[h], L[h], B, K[h], kpart, fmt[h], info, st);
+    s = bf16_ntk(G[h], L[h], B, K[h], head[h], kpart, fmt[h], info, st);
     if (s != ISOPO_OK) return s;
   }
   return ISOPO_OK;

@@ -81,6 +81,54 @@ struct WsTag {
 };
 WsTag make_ws_tag(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, const int64_t* off_host);
 
+// What lies at the head of a workspace on the materialised route.
+struct WsHead {
+  WsTag tag;
+  uint32_t done;  // CTAs of the K pass that have added their share (bf16)
+};
+
+// What the bf16 gradient kernel takes as arguments besides its matrices, so that no launch of its own prepares it: the
+// token offsets, the sequences longest first, and per projection the head to leave in its workspace and the K to clear for
+// the K pass behind it.
+struct StoredIntake {
+  int32_t off[257];
+  uint8_t order[256];
+  int n_proj;
+  WsTag tag[3];
+  WsHead* head[3];
+  float* K[3];
+};
+void make_stored_intake(StoredIntake* a, const int64_t* off_host, int B, int n_proj, const WsTag* tag, WsHead* const* head,
+                        float* const* K);
+// Extents of the sequences in working order to shared memory (`raw`: scratch there, kIntakeRawBytes).  Arguments are no
+// memory of any predecessor's, so this may run before the wait for them.  The arguments are read as ordinary memory, a word
+// per thread: indexing them directly goes through the constant cache, one word at a time (2.5 us at 236 sequences).
+constexpr int kIntakeRawBytes = 257 * 4 + 256;
+__device__ __forceinline__ void stored_extents(const StoredIntake& a, int B, int32_t* raw, int64_t* s_first, int* s_len, int* s_seq) {
+  static_assert(offsetof(StoredIntake, order) == 257 * 4, "one run of words");
+  const int32_t* src = a.off;
+  asm volatile("" : "+l"(src));  // an address like any other
+  for (int k = threadIdx.x; k < kIntakeRawBytes / 4; k += blockDim.x) raw[k] = src[k];
+  __syncthreads();
+  const uint8_t* order = reinterpret_cast<const uint8_t*>(raw + 257);
+  for (int k = threadIdx.x; k < B; k += blockDim.x) {
+    const int i = order[k], t0 = raw[i];
+    s_first[k] = t0;
+    s_len[k] = raw[i + 1] - t0;
+    s_seq[k] = i;
+  }
+}
+// The grid's share of the clearing; CTA 0 leaves the heads.
+__device__ __forceinline__ void stored_heads(const StoredIntake& a, int B) {
+  for (int h = 0; h < a.n_proj; ++h) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * B; e += gridDim.x * blockDim.x) a.K[h][e] = 0.f;
+    if (blockIdx.x == 0) {
+      if (threadIdx.x < 8) a.head[h]->tag.v[threadIdx.x] = a.tag[h].v[threadIdx.x];
+      if (threadIdx.x == 8) a.head[h]->done = 0u;
+    }
+  }
+}
+
 // How the bf16 stored route keeps G_i.  Split (isopo_set_store_format(ISOPO_STORE_E4M3_SPLIT)): two e4m3 planes of
 // one byte per element each - `hi` = round(s_i G_i), `lo` = round(16 (s_i G_i - hi)) with a power-of-two scale s_i per
 // sequence - in the same piece order.  The K pass reads only `hi` (half the bytes, kind::f8f6f4 MMAs) and takes the
@@ -92,10 +140,9 @@ struct StoreFmt {
 };
 
 struct WsLayout {
-  size_t off_tag;      // WsTag (materialised path)
+  size_t off_tag;      // WsHead (materialised path)
   size_t off_aux;      // float scales[B] | float kdiag[B]  (bf16 materialised path, split store)
   size_t off_offsets;  // int64 [B+1]
-  size_t off_order;    // int32 [B]       (bf16 materialised path: sequences, longest first)
   size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here
   size_t off_kacc;     // float64 [B*B], uint32 (float32 path: K accumulators, CTAs of the K pass that are done)
   size_t off_scaled;   // bf16 [T, min(d_in, d_out)]  (bf16 Gram path: the pre-scaled operand of the weight-gradient GEMM)
@@ -170,11 +217,6 @@ isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off
                          cudaStream_t st);
 // the offsets alone
 isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, const Clear& clear, cudaStream_t st);
-// bf16 materialised path (B <= 256) in one launch: offsets, the longest-first order, the workspace tag, K = 0
-isopo_status launch_prep_stored(const int64_t* off_host, int B, const WsTag& tag, int64_t* off_dev, int32_t* order_dev,
-                                WsTag* tag_dev, float* K, cudaStream_t st);
-isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj, const WsTag* tag, int64_t* const* off_dev,
-                                      int32_t* const* order_dev, WsTag* const* tag_dev, float* const* K, cudaStream_t st);
 // offsets and tokscale[t] = coeffs[sequence of token t] (float32 [T])
 isopo_status launch_tokscale(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, const float* coeffs,
                              float* tokscale, const Clear& clear, cudaStream_t st);
@@ -205,12 +247,8 @@ isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_i
                              const int32_t* tokseq, float* dW, cudaStream_t st);
 
 // bf16 tcgen05 path
-isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                           const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout& L, void* G,
-                           const StoreFmt& fmt, int32_t* info, cudaStream_t st);
-isopo_status bf16_seq_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                const int32_t* order_dev, int B, const WsLayout& L, void* G, const StoreFmt& fmt,
-                                int32_t* info, cudaStream_t st);
+isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const StoredIntake& in, int B,
+                           const WsLayout& L, void* G, const StoreFmt& fmt, int32_t* info, cudaStream_t st);
 // whether a layer of this shape keeps its gradients in the split e4m3 format under the current settings
 bool use_split_store(const WsLayout& L, int B);
 StoreFmt store_fmt(const WsLayout& L, int B, void* ws);
@@ -219,12 +257,12 @@ isopo_status launch_seq_scales(const void* X, const void* dY, int d_in, int d_ou
                                float* kdiag, cudaStream_t st);
 // the same for up to three projections that read one X, in one launch (L, dY, d_out, G: one entry per projection)
 isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* const* dY, const int* d_out, int64_t T, int d_in,
-                                       const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout* L,
-                                       void* const* G, const StoreFmt* fmt, int32_t* info, cudaStream_t st);
+                                       const StoredIntake& in, int B, const WsLayout* L, void* const* G, const StoreFmt* fmt,
+                                       int32_t* info, cudaStream_t st);
 // Adds into K, which the caller has cleared on this stream.  kpart != NULL (deterministic mode): every CTA
 // stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and a second kernel sums them in order.
 constexpr int kNtkMaxPartials = 160;
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, float* kpart, const StoreFmt& fmt,
+isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead* head, float* kpart, const StoreFmt& fmt,
                       int32_t* info, cudaStream_t st);
 bool deterministic_mode();
 // K[i][j] = K[j][i] for j < i (the Gram kernels fill the upper triangle)

@@ -34,29 +34,6 @@ __device__ __forceinline__ void clear_regions(const Clear& c) {
   }
 }
 
-// Everything the bf16 stored-gradient kernels need before they start, in one launch (B <= 256):
-// CTA 0 leaves the offsets, the working order of the sequences and the workspace tag; all CTAs clear K.
-// With several projections sharing one launch (same offsets, one workspace each) every workspace gets its copy.
-struct StoredPrepArgs {
-  int64_t off[257];
-  WsTag tag[3];
-  int64_t* off_dev[3];
-  int32_t* order_dev[3];
-  WsTag* tag_dev[3];
-  float* K[3];
-  uint8_t order[256];
-};
-__global__ void __launch_bounds__(256) k_prep_stored(StoredPrepArgs a, int B, int n_proj) {
-  pdl_wait();
-  for (int h = 0; h < n_proj; ++h) {
-    if (blockIdx.x == 0) {
-      for (int i = threadIdx.x; i <= B; i += blockDim.x) a.off_dev[h][i] = a.off[i];
-      for (int i = threadIdx.x; i < B; i += blockDim.x) a.order_dev[h][i] = a.order[i];
-      if (threadIdx.x < 8) a.tag_dev[h]->v[threadIdx.x] = a.tag[h].v[threadIdx.x];
-    }
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * B; e += gridDim.x * blockDim.x) a.K[h][e] = 0.f;
-  }
-}
 // What a kernel over all tokens needs before it starts, in one launch: the offsets in the workspace, the regions it adds
 // into cleared, and per token its sequence (kOut = kTokSeq) or that sequence's coefficient (kTokScale).
 enum PrepOut { kOffsetsOnly, kTokSeq, kTokScale };
@@ -719,31 +696,19 @@ isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, co
   return prep<kOffsetsOnly>(off_host, B, 0, off_dev, nullptr, nullptr, clear, st);
 }
 
-isopo_status launch_prep_stored(const int64_t* off_host, int B, const WsTag& tag, int64_t* off_dev, int32_t* order_dev,
-                                WsTag* tag_dev, float* K, cudaStream_t st) {
-  return launch_prep_stored_multi(off_host, B, 1, &tag, &off_dev, &order_dev, &tag_dev, &K, st);
-}
-
-isopo_status launch_prep_stored_multi(const int64_t* off_host, int B, int n_proj, const WsTag* tag, int64_t* const* off_dev,
-                                      int32_t* const* order_dev, WsTag* const* tag_dev, float* const* K, cudaStream_t st) {
-  if (B > 256 || n_proj < 1 || n_proj > 3) return ISOPO_ERR_UNSUPPORTED;
-  StoredPrepArgs a;
-  for (int i = 0; i <= B; ++i) a.off[i] = off_host[i];
+void make_stored_intake(StoredIntake* a, const int64_t* off_host, int B, int n_proj, const WsTag* tag, WsHead* const* head,
+                        float* const* K) {
+  for (int i = 0; i <= B; ++i) a->off[i] = (int32_t)off_host[i];
+  a->n_proj = n_proj;
   for (int h = 0; h < 3; ++h) {
     const int hh = h < n_proj ? h : 0;
-    a.tag[h] = tag[hh]; a.off_dev[h] = off_dev[hh]; a.order_dev[h] = order_dev[hh]; a.tag_dev[h] = tag_dev[hh]; a.K[h] = K[hh];
+    a->tag[h] = tag[hh]; a->head[h] = head[hh]; a->K[h] = K[hh];
   }
-  int idx[256];
-  for (int i = 0; i < B; ++i) idx[i] = i;
-  // longest first; equal lengths keep their order
-  std::stable_sort(idx, idx + B, [&](int x, int y) { return off_host[x + 1] - off_host[x] > off_host[y + 1] - off_host[y]; });
-  for (int i = 0; i < B; ++i) a.order[i] = (uint8_t)idx[i];
-  {
-    LaunchScope scope(kIdPrep, st);
-    launch(k_prep_stored, std::max(1, (B * B + 2047) / 2048), 256, 0, st, a, B, n_proj);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
+  // longest first; equal lengths keep their order: sort (complement of the length, index)
+  uint64_t key[256];
+  for (int i = 0; i < B; ++i) key[i] = ((uint64_t)(~(uint32_t)(a->off[i + 1] - a->off[i])) << 32) | (uint32_t)i;
+  std::sort(key, key + B);
+  for (int i = 0; i < B; ++i) a->order[i] = (uint8_t)key[i];
 }
 
 template <int kTile, int kT, bool kArgOff>

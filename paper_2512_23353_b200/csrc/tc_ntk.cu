@@ -43,6 +43,10 @@ struct NtkParams {
   int32_t* info;
   int box_rows;   // rows of a piece inside a box: 32, 64, 128 or 256, >= B
   int ppb;        // pieces per box = 256 / box_rows
+  // B <= 128, float atomics: the last CTA to add its share completes the other triangle (and the diagonal of the split store)
+  uint32_t* done;
+  uint32_t n_active;  // CTAs with a share
+  const float* kdiag;
 };
 
 // kE4m3: the operand is the `hi` plane of the split store: 128 one-byte elements per 128-byte box row (two boxes
@@ -213,6 +217,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
               for (int h = 0; h < ngroups; ++h) sum += red[(((h << lr) + c) << lr) + sq];
               if (ISOPO_IN_RANGE((long long)c * p.B + sq, (long long)p.B * p.B, p.info, kIdNtk))
                 add_to_k((size_t)c * p.B + sq, unscale(sq, c, sum));
+            }
+          }
+          if (p.done) {
+            volatile int* last = abort_flag + 1;
+            __threadfence();
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (r == 0) *last = atomicAdd(p.done, 1u) == p.n_active - 1;
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (*last) {
+              __threadfence();
+              const int total = p.B * p.B;
+              for (int e0 = r; e0 < total; e0 += 128 * 8) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = e0 + u * 128 < total ? __ldcg(p.K + e0 + u * 128) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int e = e0 + u * 128, i = e / p.B, j = e - i * p.B;
+                  if (e < total && j < i) p.K[(size_t)j * p.B + i] = v[u];
+                  else if (kE4m3 && e < total && j == i) p.K[e] = p.kdiag[i];
+                }
+              }
             }
           }
         }
@@ -439,7 +465,7 @@ __global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ 
 
 }  // namespace
 
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, float* kpart, const StoreFmt& fmt,
+isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead* head, float* kpart, const StoreFmt& fmt,
                       int32_t* info, cudaStream_t st) {
   if (B > 256) return ISOPO_ERR_UNSUPPORTED;
   if (fmt.split && kpart) return ISOPO_ERR_INVALID_ARG;  // the split store's diagonal is summed with float atomics
@@ -456,26 +482,29 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, float* 
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
   NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, (pieces + ppb - 1) / ppb * (fmt.split ? 2 : 4), info, (int)rows,
-              (int)ppb};
+              (int)ppb, nullptr, 0, fmt.kdiag};
   int grid = (int)std::max<long long>(1, std::min<long long>(sms, p.nkb / 8));
   if (kpart) grid = std::min(grid, kNtkMaxPartials);
+  // CTAs whose slab of the contraction is empty take no part
+  const long long per = (p.nkb + grid - 1) / grid;
+  p.n_active = (uint32_t)((p.nkb + per - 1) / per);
+  // One CTA mirrors up to 128 sequences in about the time a launch takes (2 us); more are left to a kernel of many.
+  if (!kpart && B <= 128) p.done = &head->done;
   {
     LaunchScope scope(kIdNtk, st);
     launch(kernel, grid, kThreads, kSmemBytes, st, mapG, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
+  if (p.done) return ISOPO_OK;
   if (!kpart) {
     LaunchScope scope(kIdMirror, st);
     launch(k_mirror<true>, (B * B + 255) / 256, 256, 0, st, K, B, fmt.split ? fmt.kdiag : nullptr);
     ISOPO_CUDA_TRY(cudaGetLastError());
     return ISOPO_OK;
   }
-  // CTAs whose slab of the contraction is empty wrote nothing: sum only those that had work
-  const long long per = (p.nkb + grid - 1) / grid;
-  const int n_active = (int)((p.nkb + per - 1) / per);
   {
     LaunchScope scope(kIdMirror, st);
-    launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, n_active, B, K);
+    launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, (int)p.n_active, B, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -35,15 +35,13 @@ constexpr int kBBytes = kTileN * kKB * 2;              // 32 KB: 4 chunks
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kChunkBytes = kKB * 128;                 // one [64 tokens][64 cols] box
 constexpr int kMaxSeqs = 256;                          // sequences whose extents are staged in shared memory
-constexpr int kSeqInfoBytes = kMaxSeqs * 16;           // int64 first token, int32 length, int32 index
+constexpr int kSeqInfoBytes = kMaxSeqs * 16 + kIntakeRawBytes;  // int64 first token, int32 length, int32 index; scratch
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kSeqInfoBytes;
 constexpr int kThreads = 192;
 constexpr int kThreadsFolded = 320;                    // + 4 warps that scale the dY rows
 constexpr uint32_t kTmemCols = 512;                    // two 256-column float32 accumulators
 
 struct SeqGradParams {
-  const int64_t* off;
-  const int32_t* order;  // per-sequence mode: the k-th sequence to work on (longest first)
   __nv_bfloat16* G;
   int64_t n_pad;
   int B, tiles_m, tiles_n;
@@ -86,9 +84,16 @@ __device__ __forceinline__ void decode_unit(const SeqGradParams& p, const SeqInf
   }
 }
 
+struct NoIntake {};
+__device__ __forceinline__ void stored_extents(const NoIntake&, int, int32_t*, int64_t*, int*, int*) {}
+__device__ __forceinline__ void stored_heads(const NoIntake&, int) {}
+template <bool kFolded> struct IntakeOf { typedef StoredIntake type; };
+template <> struct IntakeOf<true> { typedef NoIntake type; };
+
 template <bool kFolded>
 __global__ void __launch_bounds__(kFolded ? kThreadsFolded : kThreads, 1)
-k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX, SeqGradParams p) {
+k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX, SeqGradParams p,
+                const __grid_constant__ typename IntakeOf<kFolded>::type in) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
@@ -120,16 +125,9 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  if (!kFolded) stored_extents(in, p.B, reinterpret_cast<int32_t*>(s_seq + kMaxSeqs), s_first, s_len, s_seq);
   pdl_begin();
-  if (!kFolded) {
-    for (int k = threadIdx.x; k < p.B; k += blockDim.x) {
-      const int i = p.order[k];
-      const int64_t t0 = p.off[i];
-      s_first[k] = t0;
-      s_len[k] = (int)(p.off[i + 1] - t0);
-      s_seq[k] = i;
-    }
-  }
+  if (!kFolded) stored_heads(in, p.B);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -344,14 +342,11 @@ static isopo_status sm_count(int* sms) {
   return ISOPO_OK;
 }
 
-isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                           const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout& L, void* G,
-                           const StoreFmt& fmt, int32_t* info, cudaStream_t st) {
-  (void)off_host;
+isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const StoredIntake& in, int B,
+                           const WsLayout& L, void* G, const StoreFmt& fmt, int32_t* info, cudaStream_t st) {
   // 2-CTA tiles (256 rows of G per pair) when they waste little: an odd number of 128-row tiles
   // leaves half of the last pair idle.
-  if (L.tiles_m % 2 == 0 || L.tiles_m >= 7)
-    return bf16_seq_grad_pair(X, dY, T, d_in, d_out, off_dev, order_dev, B, L, G, fmt, info, st);
+  if (L.tiles_m % 2 == 0 || L.tiles_m >= 7) return bf16_seq_grad_pair_shared(X, 1, &dY, &d_out, T, d_in, in, B, &L, &G, &fmt, info, st);
   if (fmt.split) return ISOPO_ERR_INVALID_ARG;  // the split store exists in the 2-CTA kernel only (use_split_store)
   CUtensorMap mapY, mapX;
   isopo_status s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out);
@@ -360,13 +355,13 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   if ((s = sm_count(&sms)) != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   SeqGradParams p{};
-  p.off = off_dev; p.order = order_dev; p.G = (__nv_bfloat16*)G; p.n_pad = L.n_pad; p.B = B; p.tiles_m = L.tiles_m; p.tiles_n = L.tiles_n;
+  p.G = (__nv_bfloat16*)G; p.n_pad = L.n_pad; p.B = B; p.tiles_m = L.tiles_m; p.tiles_n = L.tiles_n;
   p.info = info; p.d_in = d_in; p.d_out = d_out; p.grid = piece_grid(d_in, d_out);
   const long long units = (long long)B * L.tiles_m * L.tiles_n;
   const int grid = (int)std::min<long long>(units, sms);
   {
     LaunchScope scope(kIdSeqGrad, st);
-    launch(k_bf16_seq_grad<false>, grid, kThreads, kSmemBytes, st, mapY, mapX, p);
+    launch(k_bf16_seq_grad<false>, grid, kThreads, kSmemBytes, st, mapY, mapX, p, in);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -399,7 +394,7 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   const int grid = (int)std::min<long long>(tiles * nslabs, sms);
   {
     LaunchScope scope(kIdWeightGrad, st);
-    launch(k_bf16_seq_grad<true>, grid, kThreadsFolded, kSmemBytes, st, mapY, mapX, p);
+    launch(k_bf16_seq_grad<true>, grid, kThreadsFolded, kSmemBytes, st, mapY, mapX, p, NoIntake{});
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -48,7 +48,7 @@ constexpr int kChunkBytes = kKB * 128;               // one [kKB tokens][64 colu
 constexpr int kOperandBytes = 2 * kChunkBytes;       // this CTA's half of dY or of X for one stage
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kMaxSeqs = 256;                        // sequences whose extents are staged in shared memory
-constexpr int kSeqInfoBytes = kMaxSeqs * 16;         // int64 first token, int32 length, int32 index
+constexpr int kSeqInfoBytes = kMaxSeqs * 16 + kIntakeRawBytes;  // int64 first token, int32 length, int32 index; scratch
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers*/ + kSeqInfoBytes;
 constexpr int kThreads = 224;
 constexpr uint32_t kTmemCols = 512;                  // two 256-column float32 accumulators
@@ -58,8 +58,6 @@ static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 
 constexpr int kMaxProj = 3;  // projections sharing X in one launch
 struct PairParams {
-  const int64_t* off;
-  const int32_t* order;     // the k-th sequence to work on (longest first)
   __nv_bfloat16* G[kMaxProj];   // stored gradients of every projection
   PieceGrid grid[kMaxProj];     // pieces of every projection's stored gradients
   int d_in;
@@ -121,7 +119,8 @@ __device__ __forceinline__ UnitShape unit_shape(int len) {
 template <bool kSplit>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_constant__ CUtensorMap mapY1,
-                     const __grid_constant__ CUtensorMap mapY2, const __grid_constant__ CUtensorMap mapX, PairParams p) {
+                     const __grid_constant__ CUtensorMap mapY2, const __grid_constant__ CUtensorMap mapX, PairParams p,
+                     const __grid_constant__ StoredIntake in) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
@@ -156,14 +155,9 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+  stored_extents(in, p.B, reinterpret_cast<int32_t*>(s_seq + kMaxSeqs), s_first, s_len, s_seq);
   pdl_begin();
-  for (int k = threadIdx.x; k < p.B; k += kThreads) {
-    const int i = p.order[k];
-    const int64_t t0 = p.off[i];
-    s_first[k] = t0;
-    s_len[k] = (int)(p.off[i + 1] - t0);
-    s_seq[k] = i;
-  }
+  stored_heads(in, p.B);
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -442,24 +436,15 @@ isopo_status launch_seq_scales(const void* X, const void* dY, int d_in, int d_ou
   return ISOPO_OK;
 }
 
-isopo_status bf16_seq_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                const int32_t* order_dev, int B, const WsLayout& L, void* G, const StoreFmt& fmt,
-                                int32_t* info, cudaStream_t st) {
-  const void* dYs[1] = {dY};
-  const int d_outs[1] = {d_out};
-  void* Gs[1] = {G};
-  return bf16_seq_grad_pair_shared(X, 1, dYs, d_outs, T, d_in, off_dev, order_dev, B, &L, Gs, &fmt, info, st);
-}
-
 isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* const* dY, const int* d_out, int64_t T, int d_in,
-                                       const int64_t* off_dev, const int32_t* order_dev, int B, const WsLayout* L,
-                                       void* const* G, const StoreFmt* fmt, int32_t* info, cudaStream_t st) {
+                                       const StoredIntake& in, int B, const WsLayout* L, void* const* G, const StoreFmt* fmt,
+                                       int32_t* info, cudaStream_t st) {
   if (n_proj < 1 || n_proj > kMaxProj) return ISOPO_ERR_INVALID_ARG;
   for (int h = 1; h < n_proj; ++h)
     if (fmt[h].split != fmt[0].split) return ISOPO_ERR_INVALID_ARG;  // one store format per launch
   CUtensorMap mapY[kMaxProj], mapX;
   PairParams p{};
-  p.off = off_dev; p.order = order_dev; p.B = B; p.tiles_n = L[0].tiles_n; p.n_proj = n_proj; p.info = info; p.d_in = d_in;
+  p.B = B; p.tiles_n = L[0].tiles_n; p.n_proj = n_proj; p.info = info; p.d_in = d_in;
   for (int h = 0; h < kMaxProj; ++h) {
     const int hh = h < n_proj ? h : 0;  // unused slots repeat the first projection (never addressed)
     isopo_status s = make_map_2d_bf16(&mapY[h], dY[hh], (uint64_t)T, (uint64_t)d_out[hh], (uint64_t)d_out[hh], 64, kKB);
@@ -507,7 +492,7 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
   p.group_m = std::max(1, std::min(g, p.ptiles_m));
   {
     LaunchScope scope(kIdSeqGrad, st);
-    launch(kernel, 2 * npairs, kThreads, kSmemBytes, st, mapY[0], mapY[1], mapY[2], mapX, p);
+    launch(kernel, 2 * npairs, kThreads, kSmemBytes, st, mapY[0], mapY[1], mapY[2], mapX, p, in);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

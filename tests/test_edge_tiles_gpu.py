@@ -71,7 +71,7 @@ def test_stand_alone_weight_gradient(b, d_in, d_out, lens):
 
 
 # shares of the sequences in the combine: one (too few sequences / too many pieces), two, four and eight, even and uneven
-@pytest.mark.parametrize("B,d_in,d_out", [(15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
+@pytest.mark.parametrize("B,d_in,d_out", [(15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (128, 64, 48), (129, 64, 48), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
 def test_combine_shares(b, B, d_in, d_out):
     X, dY, off, c, G = _problem(d_in, d_out, [2 + i % 3 for i in range(B)], B)
     ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE)
@@ -82,3 +82,5 @@ def test_combine_shares(b, B, d_in, d_out):
     torch.cuda.synchronize()
     assert int(info.item()) == 0
     assert rel_fro(dW.cpu().numpy(), 1.0 + orc.weight_gradient(G, to_f64(c))) <= 6e-3
+    # up to 128 sequences the K pass completes the other triangle itself
+    assert torch.equal(K, K.T) and rel_fro(K.cpu().numpy(), orc.ntk(G)) <= 2e-3
