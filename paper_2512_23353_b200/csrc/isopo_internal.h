@@ -276,15 +276,22 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
                        float* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
+// 1-CTA tiles, operand rows scaled in shared memory
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              void* scaled, float* dW, int32_t* info, cudaStream_t st);
+                              float* dW, int32_t* info, cudaStream_t st);
+bool bf16_weight_grad_uses_pairs(int d_out);
 
 // dW with the per-sequence coefficient applied when a segment's accumulator is drained (no scaled operand copy)
 bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
                                    const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st);
-isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                                   void* scaled, float* dW, int32_t* info, cudaStream_t st);
+// a scaled copy of the narrower operand, then a plain GEMM in 2-CTA tiles
+isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
+                                   const float* coeffs, int B, void* scaled, float* dW, int32_t* info, cudaStream_t st);
+// plain GEMM with equal runs of stages per pair, and its modelled time in stages of 256 columns
+isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, float* dW, int32_t* info,
+                                    cudaStream_t st);
+long long bf16_weight_grad_plain_cost(int64_t T, int d_in, int d_out, int pairs);
 
 // token-sampled estimator of Algorithm 1
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,

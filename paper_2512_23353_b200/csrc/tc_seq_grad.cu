@@ -367,12 +367,14 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   return ISOPO_OK;
 }
 
+// 2-CTA tiles when they waste little (see bf16_seq_grad)
+bool bf16_weight_grad_uses_pairs(int d_out) {
+  const int tiles_m = (d_out + kTileM - 1) / kTileM;
+  return tiles_m % 2 == 0 || tiles_m >= 7;
+}
+
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              void* scaled, float* dW, int32_t* info, cudaStream_t st) {
-  {  // 2-CTA tiles when they waste little (see bf16_seq_grad)
-    const int tiles_m = (d_out + kTileM - 1) / kTileM;
-    if (tiles_m % 2 == 0 || tiles_m >= 7) return bf16_weight_grad_pair(X, dY, T, d_in, d_out, tokscale, scaled, dW, info, st);
-  }
+                              float* dW, int32_t* info, cudaStream_t st) {
   CUtensorMap mapY, mapX;
   isopo_status s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out);
   if (s != ISOPO_OK) return s;
@@ -383,10 +385,16 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   p.tiles_m = (d_out + kTileM - 1) / kTileM;
   p.tiles_n = (d_in + kTileN - 1) / kTileN;
   p.info = info; p.tokscale = tokscale; p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out;
-  // token slabs: enough (tile, slab) units to fill the machine about twice, each slab a multiple of 64 tokens
+  // token slabs: the count (up to 64) whose rounds of (tile, slab) units take least, a round costing its slab plus what a
+  // unit spends on filling its pipeline and on adding its tile into dW, about 16 stages' worth.  Every slab is a multiple of
+  // 64 tokens.
   const long long tiles = (long long)p.tiles_m * p.tiles_n;
   const long long kblocks = (T + kKB - 1) / kKB;
-  long long nslabs = std::max<long long>(1, std::min<long long>(kblocks, (2ll * sms + tiles - 1) / tiles));
+  long long nslabs = 1, best = -1;
+  for (long long n = 1; n <= std::min<long long>(64, kblocks); ++n) {
+    const long long per = (kblocks + n - 1) / n, rounds = (tiles * n + sms - 1) / sms, cost = rounds * (per + 16);
+    if (best < 0 || cost < best) { best = cost; nslabs = n; }
+  }
   const long long kb_per = (kblocks + nslabs - 1) / nslabs;
   nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;

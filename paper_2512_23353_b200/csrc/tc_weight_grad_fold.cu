@@ -19,6 +19,11 @@
 //   warps 2-9       epilogue: warp w reads TMEM lanes 32 (w mod 4) .. +31, columns 128 ((w - 2) / 4) .. +127
 //   warp 10         zeroes the dY rows past the end of a segment in its last slab
 //
+// kPlain: the same pipeline as a plain GEMM dW += dY^T X (one operand already scaled): a piece of work is one segment with
+// coefficient one.  It serves token counts for which the (256 x 512 block, slab) units of tc_weight_grad_pair.cu come out
+// in rounds that are nearly empty: here the stages of all tiles, tile after tile, are cut into one equal run per pair
+// ("stream K"), so a pair has about the same work whatever the shape, at the price of one or two drains more.
+//
 // Barriers are those of tc_seq_grad_pair.cu with "unit" read as "segment".  Every wait is bounded; a
 // CTA that gives up raises the abort flag of both CTAs, and both meet at a cluster barrier before
 // tensor memory is released.
@@ -57,6 +62,8 @@ struct FoldParams {
   int ptiles_m, tiles_n;  // 256-row and 256-column tiles of dW
   int group_m;            // tile rows per group of the tile order (see pair_tile)
   int32_t* info;
+  int kblocks;            // kPlain: stages of one tile; a pair's run is `run` stages of ptiles * kblocks
+  long long run;
 };
 
 // Tiles are visited in groups of `group_m` rows, row index fastest inside a group, so that the pairs
@@ -72,6 +79,42 @@ __device__ __forceinline__ void pair_tile(int pt, const FoldParams& p, int& ptm,
 // Columns of tile column tn that exist, in the 32-column steps of a 2-CTA MMA (see tc_seq_grad_pair.cu).
 __device__ __forceinline__ int tile_cols(const FoldParams& p, int tn) { return min(kPairN, (p.d_in - tn * kPairN + 31) & ~31); }
 
+// The pieces of work of one pair, identical in every role: (tile, tokens t0 .. t1 - 1).
+template <bool kPlain>
+struct Pieces {
+  long long at, end, step;
+  int ptiles;
+  __device__ __forceinline__ Pieces(const FoldParams& p, long long pair_id, long long npairs) : ptiles(p.ptiles_m * p.tiles_n) {
+    if (kPlain) {
+      at = pair_id * p.run;
+      end = min(at + p.run, (long long)ptiles * p.kblocks);
+      step = 0;
+    } else {
+      at = pair_id;
+      end = (long long)p.nchunks * ptiles;
+      step = npairs;
+    }
+  }
+  __device__ __forceinline__ bool next(const FoldParams& p, int& tile, int& t0, int& t1) {
+    if (at >= end) return false;
+    if (kPlain) {
+      tile = (int)(at / p.kblocks);
+      const int kb0 = (int)(at - (long long)tile * p.kblocks);
+      const int kb1 = (int)min((long long)p.kblocks, kb0 + (end - at));
+      t0 = kb0 * kKB;
+      t1 = (int)min(p.T, (int64_t)kb1 * kKB);
+      at += kb1 - kb0;
+    } else {  // chunk * ptiles + tile: the pairs running at one time read the same tokens out of L2
+      const int64_t a = (at / ptiles) * p.chunk;
+      tile = (int)(at % ptiles);
+      t0 = (int)a;
+      t1 = (int)min(p.T, a + p.chunk);
+      at += step;
+    }
+    return true;
+  }
+};
+
 // Shape of one segment's token loop, identical in every role.
 struct SegShape {
   int nkb;         // slabs
@@ -79,20 +122,24 @@ struct SegShape {
   int tail_valid;  // token rows of the last slab that belong to the segment
   bool fix;        // the last step holds rows of the next segment
 };
+template <bool kPlain>
 __device__ __forceinline__ SegShape seg_shape(int len) {
   SegShape s;
   s.nkb = (len + kKB - 1) / kKB;
   s.tail_valid = len - (s.nkb - 1) * kKB;
   s.tail_n16 = (s.tail_valid + 15) >> 4;
-  s.fix = s.tail_valid < s.tail_n16 * 16;
+  s.fix = !kPlain && s.tail_valid < s.tail_n16 * 16;  // kPlain: behind a piece that ends inside a step there are no tokens
   return s;
 }
 
-// Walks the segments of the token range [t, t_end): sequence i holds tokens off[i] .. off[i+1]-1.
+// Walks the segments of the token range [t, t_end): sequence i holds tokens off[i] .. off[i+1]-1 (kPlain: one segment).
+template <bool kPlain>
 struct SegWalk {
   const int* off;
   int t, t_end, i;
   __device__ __forceinline__ SegWalk(const int* off32, int B, int t0, int t1) : off(off32), t(t0), t_end(t1) {
+    i = 0;
+    if (kPlain) return;
     int lo = 0, hi = B;  // invariant: off[lo] <= t0 < off[hi]
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
@@ -101,7 +148,7 @@ struct SegWalk {
     i = lo;
   }
   __device__ __forceinline__ bool done() const { return t >= t_end; }
-  __device__ __forceinline__ int len() const { return min(off[i + 1], t_end) - t; }
+  __device__ __forceinline__ int len() const { return (kPlain ? t_end : min(off[i + 1], t_end)) - t; }
   __device__ __forceinline__ void next() { t += len(); ++i; }
 };
 
@@ -115,6 +162,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "memory");
 }
 
+template <bool kPlain>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX, FoldParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -151,8 +199,10 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
   pdl_begin();
-  for (int k = threadIdx.x; k <= p.B; k += kThreads) s_off[k] = (int)p.off[k];
-  for (int k = threadIdx.x; k < p.B; k += kThreads) s_coef[k] = p.coeffs[k];
+  if (!kPlain) {
+    for (int k = threadIdx.x; k <= p.B; k += kThreads) s_off[k] = (int)p.off[k];
+    for (int k = threadIdx.x; k < p.B; k += kThreads) s_coef[k] = p.coeffs[k];
+  }
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();
@@ -160,15 +210,9 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
-  const int ptiles = p.ptiles_m * p.tiles_n;
-  const long long total_units = (long long)p.nchunks * ptiles;
   const long long pair_id = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  // unit u = chunk * ptiles + tile: the pairs running at one time read the same tokens out of L2
-  auto unit_tokens = [&](long long u, int& t0, int& t1) {
-    const int64_t a = (u / ptiles) * p.chunk;
-    t0 = (int)a;
-    t1 = (int)min(p.T, a + p.chunk);
-  };
+  Pieces<kPlain> work(p, pair_id, npairs);
+  int tile, t0, t1;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
@@ -179,16 +223,15 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (long long u = pair_id; u < total_units && ok; u += npairs) {
-        int ptm, tn, t0, t1;
-        pair_tile((int)(u % ptiles), p, ptm, tn);
-        unit_tokens(u, t0, t1);
+      while (ok && work.next(p, tile, t0, t1)) {
+        int ptm, tn;
+        pair_tile(tile, p, ptm, tn);
         const int ycol = (2 * ptm + (int)rank) * kHalf, half_cols = tile_cols(p, tn) >> 1;
         const int xcol = tn * kPairN + (int)rank * half_cols;
         const bool two = half_cols > 64;  // 64-column boxes of X per CTA
         const uint32_t x_bytes = two ? kOperandBytes : kChunkBytes;
-        for (SegWalk w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
-          const SegShape ss = seg_shape(w.len());
+        for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
+          const SegShape ss = seg_shape<kPlain>(w.len());
           for (int kb = 0; kb < ss.nkb; ++kb) {
             if (!(ok = mbar_wait_pair(empty_bar(stage), phase ^ 1u, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
             const uint32_t a_dst = smem_base + stage * kStageBytes, b_dst = a_dst + kOperandBytes;
@@ -214,13 +257,12 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, fixed_phase = 0;  // fixed_phase: one bit per stage
       bool ok = true;
-      for (long long u = pair_id; u < total_units && ok; u += npairs) {
-        int ptm, tn, t0, t1;
-        pair_tile((int)(u % ptiles), p, ptm, tn);
+      while (ok && work.next(p, tile, t0, t1)) {
+        int ptm, tn;
+        pair_tile(tile, p, ptm, tn);
         const uint32_t idesc = make_idesc_bf16(256, tile_cols(p, tn), /*a_mn=*/true, /*b_mn=*/true);
-        unit_tokens(u, t0, t1);
-        for (SegWalk w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
-          const SegShape ss = seg_shape(w.len());
+        for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done() && ok; w.next()) {
+          const SegShape ss = seg_shape<kPlain>(w.len());
           if (!(ok = mbar_wait_pair(accempty_bar(acc), acc_phase ^ 1u, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
           tc_fence_after_sync();
           const uint32_t d_tmem = tmem_base + (uint32_t)acc * kPairN;
@@ -262,12 +304,11 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (long long u = pair_id; u < total_units && ok; u += npairs) {
-      int ptm, tn, t0, t1;
-      pair_tile((int)(u % ptiles), p, ptm, tn);
-      unit_tokens(u, t0, t1);
-      for (SegWalk w(s_off, p.B, t0, t1); !w.done(); w.next()) {
-        const float c = ISOPO_IN_RANGE(w.i, p.B, p.info, kIdWeightGrad) ? s_coef[w.i] : 0.f;
+    while (ok && work.next(p, tile, t0, t1)) {
+      int ptm, tn;
+      pair_tile(tile, p, ptm, tn);
+      for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done(); w.next()) {
+        const float c = kPlain ? 1.f : ISOPO_IN_RANGE(w.i, p.B, p.info, kIdWeightGrad) ? s_coef[w.i] : 0.f;
         if (!(ok = mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
         tc_fence_after_sync();
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairN + h * 128);
@@ -306,11 +347,9 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     int stage = 0;
     uint32_t tail_phase = 0;  // one bit per stage
     bool ok = true;
-    for (long long u = pair_id; u < total_units && ok; u += npairs) {
-      int t0, t1;
-      unit_tokens(u, t0, t1);
-      for (SegWalk w(s_off, p.B, t0, t1); !w.done(); w.next()) {
-        const SegShape ss = seg_shape(w.len());
+    while (ok && work.next(p, tile, t0, t1)) {
+      for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done(); w.next()) {
+        const SegShape ss = seg_shape<kPlain>(w.len());
         const int ts = (stage + ss.nkb - 1) % kStages;  // ring position of the last slab
         if (ss.fix) {
           if (!(ok = mbar_wait_pair(tail_bar(ts), (tail_phase >> ts) & 1u, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
@@ -359,20 +398,16 @@ bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B) {
          T < ((int64_t)1 << 31) - 4096;
 }
 
-isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st) {
+// Pairs of CTAs that can be resident at once.
+template <bool kPlain>
+static isopo_status resident_pairs(int* pairs) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  CUtensorMap mapY, mapX;
-  isopo_status s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
-  if (s != ISOPO_OK) return s;
-  s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
-  if (s != ISOPO_OK) return s;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  static int resident_pairs[64] = {};
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  static int resident[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
-  if (resident_pairs[dev] == 0) {
+  if (resident[dev] == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)(sms / 2));
     cfg.blockDim = dim3(kThreads);
@@ -383,10 +418,64 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    ISOPO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, k_bf16_weight_grad_fold, &cfg));
+    ISOPO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, k_bf16_weight_grad_fold<kPlain>, &cfg));
     if (n < 1) return ISOPO_ERR_UNSUPPORTED;
-    resident_pairs[dev] = std::min(n, sms / 2);
+    resident[dev] = std::min(n, sms / 2);
   }
+  *pairs = resident[dev];
+  return ISOPO_OK;
+}
+
+static isopo_status make_fold_maps(CUtensorMap* mapY, CUtensorMap* mapX, const void* X, const void* dY, int64_t T, int d_in,
+                                   int d_out) {
+  isopo_status s = make_map_2d_bf16(mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
+  return s != ISOPO_OK ? s : make_map_2d_bf16(mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
+}
+
+static void set_group(FoldParams* p, int npairs) {
+  int g = 1;
+  while ((g + 1) * (g + 1) <= npairs) ++g;  // about sqrt(npairs) rows by sqrt(npairs) columns of tiles in flight
+  p->group_m = std::max(1, std::min(g, p->ptiles_m));
+}
+
+long long bf16_weight_grad_plain_cost(int64_t T, int d_in, int d_out, int pairs) {
+  const long long ptiles = (long long)((d_out + 2 * kHalf - 1) / (2 * kHalf)) * ((d_in + kPairN - 1) / kPairN);
+  const long long kblocks = (T + kKB - 1) / kKB, run = (ptiles * kblocks + pairs - 1) / pairs;
+  return run + (run / kblocks + 2) * kUnitOverhead;  // a run touches up to run / kblocks + 2 tiles
+}
+
+isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, float* dW, int32_t* info,
+                                    cudaStream_t st) {
+  int pairs = 0;
+  isopo_status s = resident_pairs<true>(&pairs);
+  if (s != ISOPO_OK) return s;
+  CUtensorMap mapY, mapX;
+  if ((s = make_fold_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
+  FoldParams p{};
+  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info;
+  p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
+  p.tiles_n = (d_in + kPairN - 1) / kPairN;
+  p.kblocks = (int)((T + kKB - 1) / kKB);
+  const long long stages = (long long)p.ptiles_m * p.tiles_n * p.kblocks;
+  // no shorter runs than a drain takes
+  p.run = std::max<long long>((stages + pairs - 1) / pairs, std::min<long long>(kUnitOverhead, p.kblocks));
+  const int npairs = (int)((stages + p.run - 1) / p.run);
+  set_group(&p, npairs);
+  {
+    LaunchScope scope(kIdWeightGrad, st);
+    launch(k_bf16_weight_grad_fold<true>, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
+}
+
+isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
+                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st) {
+  int pairs = 0;
+  isopo_status s = resident_pairs<false>(&pairs);
+  if (s != ISOPO_OK) return s;
+  CUtensorMap mapY, mapX;
+  if ((s = make_fold_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
   FoldParams p{};
   p.off = off_dev; p.coeffs = coeffs; p.dW = dW; p.T = T; p.B = B; p.d_in = d_in; p.d_out = d_out; p.info = info;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
@@ -395,7 +484,7 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   // unit's pipeline fill and flush; ties go to fewer chunks.  Every chunk is a whole number of stages.
   // (Chunks small enough to stay in L2 while all tiles pass over them were measured slower: the float32
   // reductions into dW and the fills grow with the chunk count, and the inputs were still read 2.6 x.)
-  const long long ptiles = (long long)p.ptiles_m * p.tiles_n, pairs = resident_pairs[dev];
+  const long long ptiles = (long long)p.ptiles_m * p.tiles_n;
   const long long kblocks = (T + kKB - 1) / kKB;
   long long nchunks = 1, best = -1;
   for (long long n = 1; n <= std::min<long long>(64, kblocks); ++n) {
@@ -407,13 +496,11 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   nchunks = (kblocks + kb_per - 1) / kb_per;
   p.chunk = kb_per * kKB;
   p.nchunks = (int)nchunks;
-  const int npairs = (int)std::max<long long>(1, std::min<long long>(ptiles * nchunks, pairs));
-  int g = 1;
-  while ((g + 1) * (g + 1) <= npairs) ++g;  // about sqrt(npairs) rows by sqrt(npairs) columns of tiles in flight
-  p.group_m = std::max(1, std::min(g, p.ptiles_m));
+  const int npairs = (int)std::max<long long>(1, std::min<long long>(ptiles * nchunks, (long long)pairs));
+  set_group(&p, npairs);
   {
     LaunchScope scope(kIdWeightGrad, st);
-    launch(k_bf16_weight_grad_fold, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
+    launch(k_bf16_weight_grad_fold<false>, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -1,8 +1,8 @@
 // Stand-alone weight gradient dW = (c_seq(t) dY)^T X (Alg. 1: "grad += advantages * rescaled
 // gradient") with 2-CTA tensor-core tiles.
 //
-// The per-token scale is applied to the NARROWER operand in one streaming pass (k_scale_rows:
-// T x min(d_in, d_out) elements read and written once, round to nearest even), after which the
+// The coefficient of every token's sequence is applied to the NARROWER operand in one streaming pass (k_scale_rows:
+// T x min(d_in, d_out) elements read and written once, round to nearest even; it also clears dW), after which the
 // weight gradient is a plain GEMM over all tokens.  Scaling the landed rows in shared memory inside
 // the GEMM (what the 1-CTA kernel of tc_seq_grad.cu does for small layers) was measured 15 % slower
 // here: under the power cap the extra shared-memory traffic and the busy scaler warps cost more
@@ -222,36 +222,61 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
   if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
 }
 
-// dst[t, :] = bf16(tokscale[t] * src[t, :]) (round to nearest even), 8 elements per thread.
-__global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src, const float* __restrict__ tokscale,
-                                                    int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst) {
+// dst[t, :] = bf16(coeffs[sequence of t] * src[t, :]) (round to nearest even).  A warp takes a token: one search for its
+// sequence (offsets staged in shared memory), then 16-byte pieces of the row, four in flight per lane.  HBM stream.
+constexpr int kScaleMaxSeqs = 2048;  // offsets staged; more are searched in global memory
+__global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src, const int64_t* __restrict__ off, int B,
+                                                    const float* __restrict__ coeffs, int64_t T, int d8 /* columns / 8 */,
+                                                    uint4* __restrict__ dst) {
   pdl_wait();
-  const int64_t n = T * d8;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const float c = __ldg(tokscale + e / d8);
-    uint4 v = __ldcs(src + e);
-    uint32_t* w = reinterpret_cast<uint32_t*>(&v);
+  __shared__ int32_t s_off[kScaleMaxSeqs + 1];
+  const bool staged = B <= kScaleMaxSeqs;
+  if (staged)
+    for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = (int32_t)off[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += warps) {
+    int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if ((staged ? (int64_t)s_off[mid] : off[mid]) <= t) lo = mid; else hi = mid;
+    }
+    const float c = __ldg(coeffs + lo);
+    const uint4* from = src + t * d8;
+    uint4* to = dst + t * d8;
+    for (int e0 = lane; e0 < d8; e0 += 128) {
+      uint4 v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      w[k] = pack_bf16x2(c * __uint_as_float(w[k] << 16), c * __uint_as_float(w[k] & 0xffff0000u));
-    dst[e] = v;
+      for (int u = 0; u < 4; ++u)
+        if (e0 + 32 * u < d8) v[u] = __ldcs(from + e0 + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (e0 + 32 * u >= d8) continue;
+        uint32_t* w = reinterpret_cast<uint32_t*>(&v[u]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          w[k] = pack_bf16x2(c * __uint_as_float(w[k] << 16), c * __uint_as_float(w[k] & 0xffff0000u));
+        to[e0 + 32 * u] = v[u];
+      }
+    }
   }
 }
 
 }  // namespace
 
-isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                                   void* scaled, float* dW, int32_t* info, cudaStream_t st) {
+isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
+                                   const float* coeffs, int B, void* scaled, float* dW, int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   {  // scale the narrower operand into `scaled`
     const bool scale_y = d_out <= d_in;
     const int d8 = (scale_y ? d_out : d_in) / 8;
-    const int grid = (int)std::min<int64_t>((T * d8 + 255) / 256, (int64_t)sms * 16);
+    const int grid = (int)std::min<int64_t>((T + 7) / 8, (int64_t)sms * 16);
     {
       LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows, grid, 256, 0, st, (const uint4*)(scale_y ? dY : X), tokscale, T, d8, (uint4*)scaled);
+      launch(k_scale_rows, grid, 256, 0, st, (const uint4*)(scale_y ? dY : X), off_dev, B, coeffs, T, d8, (uint4*)scaled);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     if (scale_y) dY = scaled; else X = scaled;
@@ -295,6 +320,13 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
     const long long cost = rounds * (per + kUnitOverhead);
     if (best < 0 || cost < best) { best = cost; nslabs = n; }
   }
+  // The other kernel (256 x 256 tiles, every pair the same number of stages) where these units leave the last round too
+  // empty (a stage of 512 columns is two of 256) and the inputs stay in the L2: its pairs walk the tokens at different
+  // places.  10,496 tokens, 896 x 4864 (121 MB) 100 -> 84 us, 4864 x 896 102 -> 74 us; 40,960 tokens, 896 x 896 (147 MB)
+  // 67 -> 94 us, 35,200 tokens, 896 x 4864 (405 MB) 301 -> 445 us.
+  const bool in_l2 = 2.0 * (double)T * (d_in + d_out) <= 128e6;
+  if (in_l2 && 10 * bf16_weight_grad_plain_cost(T, d_in, d_out, (int)pairs) < 9 * 2 * best)
+    return bf16_weight_grad_plain(X, dY, T, d_in, d_out, dW, info, st);
   const long long kb_per = (kblocks + nslabs - 1) / nslabs;
   nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;

@@ -84,3 +84,20 @@ def test_combine_shares(b, B, d_in, d_out):
     assert rel_fro(dW.cpu().numpy(), 1.0 + orc.weight_gradient(G, to_f64(c))) <= 6e-3
     # up to 128 sequences the K pass completes the other triangle itself
     assert torch.equal(K, K.T) and rel_fro(K.cpu().numpy(), orc.ntk(G)) <= 2e-3
+
+
+# plain GEMM with equal runs of stages: one stage, runs inside a tile, runs across tiles and across tile rows, ragged last
+# stage, partial tiles in both directions; and more sequences than the scaling pass stages
+@pytest.mark.parametrize("lens,d_in,d_out", [([1], 256, 256), ([63, 2], 264, 200), ([3] * 21 + [1], 2120, 456), ([7] * 100, 2120, 456),
+                                             ([11] * 300, 520, 1800), ([2] * 2100, 264, 136)])
+def test_plain_gemm_runs(b, lens, d_in, d_out):
+    rng = np.random.default_rng(len(lens))
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    to = lambda a: torch.from_numpy(a.astype(np.float32)).cuda().to(torch.bfloat16)  # noqa: E731
+    X, dY = to(rng.standard_normal((off[-1], d_in))), to(0.1 * rng.standard_normal((off[-1], d_out)))
+    c = torch.from_numpy(rng.standard_normal(len(lens)).astype(np.float32)).cuda()
+    ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, len(lens), b.PATH_GRAM)
+    dW = _weight_grad(b, X, dY, off, c, ws, torch.zeros(1, dtype=torch.int32, device="cuda"), b.PATH_GRAM)
+    # dW = sum_i c_i G_i = (c_seq(t) dY)^T X, without materialising the G_i of 2100 sequences
+    want = (np.repeat(to_f64(c), lens)[:, None] * to_f64(dY)).T @ to_f64(X)
+    assert rel_fro(dW, want) <= 6e-3
