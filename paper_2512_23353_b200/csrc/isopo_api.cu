@@ -535,11 +535,8 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
     if (s != ISOPO_OK) return s;
     return bf16_weight_grad_fold(X, dY, T, d_in, d_out, off_dev, coeffs, B, dW, info, st);
   }
-  if (bf16_weight_grad_uses_pairs(d_out)) {
-    s = launch_offsets(seq_offsets_host, B, off_dev, clear, st);
-    if (s != ISOPO_OK) return s;
-    return bf16_weight_grad_pair(X, dY, T, d_in, d_out, off_dev, coeffs, B, w + L.off_scaled, dW, info, st);
-  }
+  if (bf16_weight_grad_uses_pairs(d_out))
+    return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, clear, info, st);
   // one scale per token, so that the kernel's scaler warps need a single independent load per row
   float* tokscale = (float*)tokseq;
   s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);

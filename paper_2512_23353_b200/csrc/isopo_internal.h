@@ -212,6 +212,24 @@ struct Clear {
   float* p[3];
   int64_t n[3];
 };
+// Clears the regions that the kernels behind this one add into (in place of a memset for each).
+__device__ __forceinline__ void clear_regions(const Clear& c) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (c.n[k] == 0) continue;
+    const int64_t quads = (reinterpret_cast<uintptr_t>(c.p[k]) & 15) == 0 ? c.n[k] / 4 : 0;
+    for (int64_t e = first; e < quads; e += step) reinterpret_cast<float4*>(c.p[k])[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t e = 4 * quads + first; e < c.n[k]; e += step) c.p[k][e] = 0.f;
+  }
+}
+// Token offsets as kernel arguments (no host-to-device copy); they are below 2^31 and travel as 32-bit values.
+constexpr int kArgChunk = 384;    // the usual case; 1.5 KB of arguments
+template <int kN> struct OffsetArgs { int32_t v[kN]; };
+template <int kN>
+inline void fill_offsets(OffsetArgs<kN>* a, const int64_t* off_host, int n) {
+  for (int t = 0; t < n; ++t) a->v[t] = (int32_t)off_host[t];
+}
 // offsets and the token -> sequence map to the device, `clear` cleared
 isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, const Clear& clear,
                          cudaStream_t st);
@@ -286,8 +304,10 @@ bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
                                    const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st);
 // a scaled copy of the narrower operand, then a plain GEMM in 2-CTA tiles
-isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, void* scaled, float* dW, int32_t* info, cudaStream_t st);
+// (the offsets travel with the scaling pass, through off_dev above 383 sequences; `clear` is cleared ahead of it all)
+isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, const Clear& clear,
+                                   int32_t* info, cudaStream_t st);
 // plain GEMM with equal runs of stages per pair, and its modelled time in stages of 256 columns
 isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, float* dW, int32_t* info,
                                     cudaStream_t st);

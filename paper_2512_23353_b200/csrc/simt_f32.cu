@@ -9,29 +9,14 @@ namespace isopo {
 
 namespace {
 
-// Host values travel to the device as kernel arguments (no host-to-device copy, so no hidden
-// synchronisation with the stream and nothing that reads the caller's array after the call returns).
-// Token offsets are below 2^31 and travel as 32-bit values.
-constexpr int kArgChunk = 384;    // the usual case; 1.5 KB of arguments
-constexpr int kArgLarge = 2048;   // up to here still one launch
-template <int kN> struct OffsetArgs { int32_t v[kN]; };
+// Host values travel to the device as kernel arguments: no hidden synchronisation with the stream, and nothing that reads
+// the caller's array after the call returns.
+constexpr int kArgLarge = 2048;  // offsets of one launch: 8 KB of arguments
 template <int kN>
 __global__ void __launch_bounds__(256) k_store_offsets(const __grid_constant__ OffsetArgs<kN> a, int64_t base, int n,
                                                        int64_t* __restrict__ off) {
   pdl_wait();
   for (int t = threadIdx.x; t < n; t += blockDim.x) off[base + t] = a.v[t];
-}
-
-// Clears the regions that the kernels behind this one add into (in place of a memset for each).
-__device__ __forceinline__ void clear_regions(const Clear& c) {
-  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (c.n[k] == 0) continue;
-    const int64_t quads = (reinterpret_cast<uintptr_t>(c.p[k]) & 15) == 0 ? c.n[k] / 4 : 0;
-    for (int64_t e = first; e < quads; e += step) reinterpret_cast<float4*>(c.p[k])[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t e = 4 * quads + first; e < c.n[k]; e += step) c.p[k][e] = 0.f;
-  }
 }
 
 // What a kernel over all tokens needs before it starts, in one launch: the offsets in the workspace, the regions it adds
@@ -661,17 +646,17 @@ static isopo_status prep(const int64_t* off_host, int B, int64_t T, int64_t* off
   LaunchScope scope(kIdPrep, st);
   if (B + 1 <= kArgChunk) {
     OffsetArgs<kArgChunk> a;
-    for (int t = 0; t <= B; ++t) a.v[t] = (int32_t)off_host[t];
+    fill_offsets(&a, off_host, B + 1);
     launch(k_prep<kOut, kArgChunk>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out, clear);
   } else if (B + 1 <= kArgLarge) {
     OffsetArgs<kArgLarge> a;
-    for (int t = 0; t <= B; ++t) a.v[t] = (int32_t)off_host[t];
+    fill_offsets(&a, off_host, B + 1);
     launch(k_prep<kOut, kArgLarge>, grid, 256, 0, st, a, B, T, off_dev, coeffs, out, clear);
   } else {
     for (int64_t base = 0; base <= B; base += kArgLarge) {
       OffsetArgs<kArgLarge> a;
       const int m = (int)std::min<int64_t>(kArgLarge, B + 1 - base);
-      for (int t = 0; t < m; ++t) a.v[t] = (int32_t)off_host[base + t];
+      fill_offsets(&a, off_host + base, m);
       launch(k_store_offsets<kArgLarge>, 1, 256, 0, st, a, base, m, off_dev);
     }
     ISOPO_CUDA_TRY(cudaGetLastError());

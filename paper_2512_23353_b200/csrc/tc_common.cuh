@@ -309,6 +309,25 @@ __device__ __forceinline__ uint64_t make_sdesc_sw128(uint32_t smem_addr, uint32_
          ((uint64_t)(sbo_bytes >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
+// K[j][i] = K[i][j] for the pairs of which one triangle is filled (kFromUpper: i < j), and the diagonal where `set_diag`, by
+// the 128 threads r = 0 .. 127 of one CTA once every CTA's additions are visible.  Reads run along rows; the scattered
+// writes need not be waited for.
+template <bool kFromUpper, typename Diag>
+__device__ __forceinline__ void mirror_by_cta(float* K, int B, int r, Diag diag, bool set_diag) {
+  const int total = B * B;
+  for (int e0 = r; e0 < total; e0 += 128 * 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = e0 + u * 128 < total ? __ldcg(K + e0 + u * 128) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + u * 128, i = e / B, j = e - i * B;
+      if (e < total && (kFromUpper ? j > i : j < i)) K[(size_t)j * B + i] = v[u];
+      else if (set_diag && e < total && j == i) K[e] = diag(i);
+    }
+  }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // .x = lo (low 16 bits)
   return *reinterpret_cast<uint32_t*>(&v);

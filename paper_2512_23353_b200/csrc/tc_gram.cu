@@ -63,7 +63,8 @@ __device__ __forceinline__ void decode_unit(const GramParams& p, long long u, in
 // rows a0 = X[samples] (mapRX) and g0 = dY[samples] (mapRY), the columns all tokens, and
 //   M^T[j, i] = sum_{t in sequence i} (g0_j . dY_t)(a0_j . x_t) = g0_j . G_i a0_j      (Eq. one)
 // comes out of the same product-and-segment-sum epilogue without any symmetry weights.
-template <bool kSampled>
+// kComplete (one CTA): fills K's other triangle as well.
+template <bool kSampled, bool kComplete>
 __global__ void __launch_bounds__(kThreads, 1)
 k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ CUtensorMap mapRY,
             const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY, GramParams p) {
@@ -197,6 +198,11 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       if (lane == 0) mbar_arrive(accempty_bar(acc));
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+    if (kComplete) {
+      __threadfence();
+      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+      mirror_by_cta<true>(p.K, p.B, row, [](int) { return 0.f; }, false);
+    }
   }
 
   if (*abort_flag) __nanosleep(100000);
@@ -218,17 +224,22 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   GramParams p{tokseq, K, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, 0, 0, 0};
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms);
+  // One tile of tokens: its CTA completes K, a launch less for the host, which bounds so small a layer (26 tokens, 640 x 280:
+  // 29.1 -> 26.4 us with the scaling pass's).  The last of several CTAs would be 0.7 (15 CTAs) to 1.3 us (136) slower than a
+  // kernel that is already set up when this one ends, and above 32 sequences so is one CTA.
+  const bool complete = grid == 1 && B <= 32;
+  const auto kernel = complete ? &k_bf16_gram<false, true> : &k_bf16_gram<false, false>;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   p.strip = gram_strip_width(2.0 * kTT * (d_in + d_out), grid);
   {
     LaunchScope scope(kIdGram, st);
-    launch(k_bf16_gram<false>, grid, kThreads, kSmemBytes, st, mapX, mapY, mapX, mapY, p);
+    launch(kernel, grid, kThreads, kSmemBytes, st, mapX, mapY, mapX, mapY, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
-  return mirror_upper(K, B, st);
+  return complete ? ISOPO_OK : mirror_upper(K, B, st);
 }
 
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
@@ -243,13 +254,13 @@ isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, in
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   GramParams p{tokseq, Mt, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, n_samples, (n_samples + kTT - 1) / kTT, 0};
   const long long units = (long long)p.n_row_tiles * p.nT;
   const int grid = (int)std::min<long long>(units, sms);
   {
     LaunchScope scope(kIdSampled, st);
-    launch(k_bf16_gram<true>, grid, kThreads, kSmemBytes, st, mapRX, mapRY, mapX, mapY, p);
+    launch(k_bf16_gram<true, false>, grid, kThreads, kSmemBytes, st, mapRX, mapRY, mapX, mapY, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -227,18 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (*last) {
               __threadfence();
-              const int total = p.B * p.B;
-              for (int e0 = r; e0 < total; e0 += 128 * 8) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = e0 + u * 128 < total ? __ldcg(p.K + e0 + u * 128) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                  const int e = e0 + u * 128, i = e / p.B, j = e - i * p.B;
-                  if (e < total && j < i) p.K[(size_t)j * p.B + i] = v[u];
-                  else if (kE4m3 && e < total && j == i) p.K[e] = p.kdiag[i];
-                }
-              }
+              mirror_by_cta<false>(p.K, p.B, r, [&](int i) { return p.kdiag[i]; }, kE4m3);
             }
           }
         }
@@ -488,8 +477,10 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead*
   // CTAs whose slab of the contraction is empty take no part
   const long long per = (p.nkb + grid - 1) / grid;
   p.n_active = (uint32_t)((p.nkb + per - 1) / per);
-  // One CTA mirrors up to 128 sequences in about the time a launch takes (2 us); more are left to a kernel of many.
-  if (!kpart && B <= 128) p.done = &head->done;
+  // K completed by the last CTA: a launch less (2 us for the host, which bounds a pass over little data: 128 x 128, 32
+  // sequences 18.3 -> 16.1 us), but a CTA by itself is slower than a kernel that is set up when this one ends, the more so the
+  // more sequences: 896 x 896, K and solve: 24.5 us both ways at 16, 31.5 / 30.4 at 32, 47.2 / 45.0 at 48, 127.6 / 117.1 at 128.
+  if (!kpart && (B <= 16 || (B <= 32 && per <= 16))) p.done = &head->done;
   {
     LaunchScope scope(kIdNtk, st);
     launch(kernel, grid, kThreads, kSmemBytes, st, mapG, p);

@@ -223,17 +223,28 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
 }
 
 // dst[t, :] = bf16(coeffs[sequence of t] * src[t, :]) (round to nearest even).  A warp takes a token: one search for its
-// sequence (offsets staged in shared memory), then 16-byte pieces of the row, four in flight per lane.  HBM stream.
-constexpr int kScaleMaxSeqs = 2048;  // offsets staged; more are searched in global memory
-__global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src, const int64_t* __restrict__ off, int B,
-                                                    const float* __restrict__ coeffs, int64_t T, int d8 /* columns / 8 */,
-                                                    uint4* __restrict__ dst) {
+// sequence, then 16-byte pieces of the row, four in flight per lane.  HBM stream.
+// kArgs: offsets in the arguments (read as ordinary memory, see stored_extents), so that no kernel runs ahead of this one;
+// otherwise they are staged from the workspace, above kScaleMaxSeqs searched there.
+constexpr int kScaleMaxSeqs = 2048;
+template <bool kArgs>
+__global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src,
+                                                    const __grid_constant__ OffsetArgs<kArgs ? kArgChunk : 1> args,
+                                                    const int64_t* __restrict__ off, int B, const float* __restrict__ coeffs,
+                                                    int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst,
+                                                    const __grid_constant__ Clear clear) {
+  __shared__ int32_t s_off[kArgs ? kArgChunk : kScaleMaxSeqs + 1];
+  if (kArgs) {
+    const int32_t* from = args.v;
+    asm volatile("" : "+l"(from));
+    for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = from[i];
+  }
   pdl_wait();
-  __shared__ int32_t s_off[kScaleMaxSeqs + 1];
-  const bool staged = B <= kScaleMaxSeqs;
-  if (staged)
+  const bool staged = kArgs || B <= kScaleMaxSeqs;
+  if (!kArgs && staged)
     for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = (int32_t)off[i];
   __syncthreads();
+  if (kArgs) clear_regions(clear);
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += warps) {
@@ -265,18 +276,32 @@ __global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ sr
 
 }  // namespace
 
-isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, void* scaled, float* dW, int32_t* info, cudaStream_t st) {
+isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, const Clear& clear,
+                                   int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   {  // scale the narrower operand into `scaled`
     const bool scale_y = d_out <= d_in;
     const int d8 = (scale_y ? d_out : d_in) / 8;
-    const int grid = (int)std::min<int64_t>((T + 7) / 8, (int64_t)sms * 16);
-    {
+    const uint4* src = (const uint4*)(scale_y ? dY : X);
+    int64_t ctas = (T + 7) / 8;
+    // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
+    // 4000 tokens a 4096 x 4096 dW took 10 us longer than from a kernel of its own, hence a CTA for every 16 KB as well.
+    if (B + 1 <= kArgChunk) {
+      OffsetArgs<kArgChunk> a;
+      fill_offsets(&a, off_host, B + 1);
+      ctas = std::max(ctas, clear.n[0] / 4096);
       LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows, grid, 256, 0, st, (const uint4*)(scale_y ? dY : X), off_dev, B, coeffs, T, d8, (uint4*)scaled);
+      launch(k_scale_rows<true>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, a, off_dev, B, coeffs, T, d8,
+             (uint4*)scaled, clear);
+    } else {
+      isopo_status s = launch_offsets(off_host, B, off_dev, clear, st);
+      if (s != ISOPO_OK) return s;
+      LaunchScope scope(kIdScaleRows, st);
+      launch(k_scale_rows<false>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, OffsetArgs<1>{}, off_dev, B,
+             coeffs, T, d8, (uint4*)scaled, Clear{});
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     if (scale_y) dY = scaled; else X = scaled;

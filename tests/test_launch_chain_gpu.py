@@ -92,3 +92,41 @@ def test_sample_rows(b, n):
     M = torch.stack([M[:, l.off[i]:l.off[i + 1]].sum(1) for i in range(3)], 1)
     want = (M ** 2).sum(0) / (a0.pow(2).sum(1) * g0.pow(2).sum(1)).sum()
     assert float((F2.double() - want).norm() / want.norm()) <= 4e-6
+
+
+@pytest.mark.parametrize("route", ["gram", "stored"])
+@pytest.mark.parametrize("B,d_in,d_out", [(1, 40, 24), (18, 40, 24), (15, 40, 24), (16, 40, 24), (17, 40, 24), (32, 40, 24), (33, 40, 24),
+                                          (17, 384, 512), (32, 384, 512)])
+def test_k_is_completed(b, route, B, d_in, d_out):
+    """Few sequences and little work: the only or the last CTA of the kernel completes K, otherwise a kernel of its own does.  Bounds:
+    (d_in + d_out) 2^-23, the sum of the two accumulations' worst relative errors; stored gradients are rounded to bf16, 2^-9
+    for each of the two factors."""
+    l = Layer(b, torch.bfloat16, [1 + 3 * (i % 5) for i in range(B)], d_in, d_out, B)
+    path = b.PATH_GRAM if route == "gram" else b.PATH_MATERIALISE
+    buf = {"ws": b.alloc_workspace(l.code, l.T, d_in, d_out, B, path), "K": torch.empty(B * B, device="cuda"),
+           "info": torch.zeros(1, dtype=torch.int32, device="cuda")}
+    X, dY = l.X.double(), l.dY.double()
+    G = torch.stack([dY[l.off[i]:l.off[i + 1]].T @ X[l.off[i]:l.off[i + 1]] for i in range(B)]).flatten(1)
+    want = G @ G.T
+    tol = (d_in + d_out) * 2.0 ** -23 + (2.0 ** -8 if route == "stored" else 0.0)
+    for _ in range(3):  # the counter starts anew in every pass
+        buf["K"].fill_(float("nan"))
+        b.isopo_layer_gram(l.X, l.dY, l.off, buf["K"], buf["ws"], buf["info"], path)
+        got = buf["K"].view(B, B)
+        assert torch.equal(got, got.T)
+        assert float((got.double() - want).norm() / want.norm()) <= tol
+    assert int(buf["info"].item()) == 0
+
+
+@pytest.mark.parametrize("B", [383, 384, 2047, 2048])
+def test_offsets_of_the_scaling_pass(b, B):
+    """dW of one-token sequences: (bf16(c dY))^T X.  The reference rounds c dY the same way, so only the accumulation differs:
+    T 2^-23 at worst, taken as 1e-5 of the norm."""
+    l = Layer(b, torch.bfloat16, [1] * B, 256, 256, B)
+    ws = b.alloc_workspace(b.BF16, l.T, 256, 256, B, b.PATH_GRAM)
+    c = torch.randn(B, device="cuda", generator=torch.Generator(device="cuda").manual_seed(B))
+    dW, info = torch.empty(256, 256, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    b.isopo_weight_grad(l.X, l.dY, c, l.off, dW, ws, info, b.PATH_GRAM, 0.0)
+    want = (c[:, None] * l.dY.float()).bfloat16().double().T @ l.X.double()
+    assert float((dW.double() - want).norm() / want.norm()) <= 1e-5
+    assert int(info.item()) == 0
