@@ -14,7 +14,8 @@
 //
 //   warp 0      TMA producer: [128 tokens] x [64 features] boxes of X then of dY, 6-stage ring
 //   warp 1      MMA issuer: tcgen05.mma 128 x 128 x 16, K-major operands
-//   warps 2-5   epilogue: tcgen05.ld of P and Q, product, segmented sums, float atomics into K
+//   warps 2-9   epilogue: tcgen05.ld of P and Q, product, segmented sums, float atomics into K
+//               (a warp takes 32 rows and half of the columns)
 
 #include "tc_common.cuh"
 #include "tc_gram_epilogue.cuh"
@@ -31,7 +32,10 @@ constexpr int kStages = 6;
 constexpr int kOperandBytes = kTT * 128;       // 16 KB
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
-constexpr int kThreads = 192;
+// Copy warp, MMA warp, eight epilogue warps.  With four and a walk over the units from the beginning for each, the epilogue
+// bound every layer of narrow operands or short sequences (128 x 64, 64 tokens each: 15.4 -> 11.9 us at 3840 tokens, 376 -> 207
+// at 28,800) and took 1 us longer behind the last MMA of any (896 x 896, 640 tokens: 11.1 -> 10.3).
+constexpr int kThreads = 320;
 constexpr uint32_t kTmemCols = 512;            // 2 buffers x (P 128 + Q 128) columns
 
 struct GramParams {
@@ -44,19 +48,24 @@ struct GramParams {
   int strip;                // Gram: tile columns per strip of the pair order
 };
 
-// Work unit -> (row tile I, column tile J).  Gram: pairs I <= J of token tiles in strip order.
+// The work units of a CTA: (row tile I, column tile J).  Gram: pairs I <= J of token tiles.
 // Sampled: every (sample tile, token tile).
-template <bool kSampled>
-__device__ __forceinline__ void decode_unit(const GramParams& p, long long u, int& I, int& J, bool& diag) {
-  if (kSampled) {
-    I = (int)(u % p.n_row_tiles);
-    J = (int)(u / p.n_row_tiles);
-    diag = false;
-  } else {
-    decode_pair_strips(u, p.nT, p.strip, I, J);
-    diag = I == J;
+template <bool kSampled> struct Units : PairWalk {
+  __device__ __forceinline__ Units(const GramParams& p) : PairWalk(p.nT, p.strip, blockIdx.x) {}
+  __device__ __forceinline__ void next() { PairWalk::next(gridDim.x); }
+};
+template <> struct Units<true> {
+  int rows, cols, I, J, step_i, step_j;
+  __device__ __forceinline__ Units(const GramParams& p)
+      : rows(p.n_row_tiles), cols(p.nT), I(blockIdx.x % rows), J(blockIdx.x / rows), step_i(gridDim.x % rows), step_j(gridDim.x / rows) {}
+  __device__ __forceinline__ bool more() const { return J < cols; }
+  __device__ __forceinline__ void next() {
+    I += step_i;
+    J += step_j;
+    if (I >= rows) { I -= rows; ++J; }
   }
-}
+  __device__ __forceinline__ void get(int& i, int& j) const { i = I; j = J; }
+};
 
 // kSampled = false: the Gram route, rows and columns are both token tiles (mapRX = mapX, mapRY = mapY).
 // kSampled = true: the token-sampled Fisher estimator of Algorithm 1: the rows are the sampled token
@@ -83,7 +92,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(accfull_bar(b), 1); mbar_init(accempty_bar(b), 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(accfull_bar(b), 1); mbar_init(accempty_bar(b), 8); }
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -94,7 +103,6 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
-  const long long total_units = kSampled ? (long long)p.n_row_tiles * p.nT : (long long)p.nT * (p.nT + 1) / 2;
   const int nkx = (p.d_in + kKF - 1) / kKF, nky = (p.d_out + kKF - 1) / kKF;
 
   if (warp == 0) {
@@ -108,10 +116,10 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (long long u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
+      for (Units<kSampled> u(p); u.more() && ok; u.next()) {
         int I, J;
-        bool diag;
-        decode_unit<kSampled>(p, u, I, J, diag);
+        u.get(I, J);
+        const bool diag = !kSampled && I == J;
         for (int kb = 0; kb < nkx + nky; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.info, kIdGram))) break;
           const CUtensorMap* rmap = kb < nkx ? &mapRX : &mapRY;
@@ -131,10 +139,10 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
-      for (long long u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
+      for (Units<kSampled> u(p); u.more() && ok; u.next()) {
         int I, J;
-        bool diag;
-        decode_unit<kSampled>(p, u, I, J, diag);
+        u.get(I, J);
+        const bool diag = !kSampled && I == J;
         if (!(ok = mbar_wait(accempty_bar(acc), acc_phase ^ 1u, abort_flag, p.info, kIdGram))) break;
         tc_fence_after_sync();
         for (int kb = 0; kb < nkx + nky; ++kb) {
@@ -160,13 +168,14 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       }
     }
   } else {
-    const int q = warp & 3, row = q * 32 + lane;
+    // a warp takes 32 rows (the TMEM lanes it can read) and half of the columns
+    const int q = warp & 3, row = q * 32 + lane, g0 = (warp - 2) / 4 * (kTT / 64);
     int acc = 0;
     uint32_t acc_phase = 0;
-    for (long long u = blockIdx.x; u < total_units; u += gridDim.x) {
+    for (Units<kSampled> u(p); u.more(); u.next()) {
       int I, J;
-      bool diag;
-      decode_unit<kSampled>(p, u, I, J, diag);
+      u.get(I, J);
+      const bool diag = !kSampled && I == J;
       // sequence of this thread's row token and of every column token (clamped past the end; those
       // rows and columns are zero in P and Q)
       // (sampled: the "row sequence" is the sample index, its results go to row `row_seq` of M^T;
@@ -175,7 +184,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       const int64_t trow = (int64_t)I * kTT + row;
       const int row_seq = kSampled ? (int)trow : __ldg(p.tokseq + min(trow, p.T - 1));
       auto col_seq = [&](int g) { return __ldg(p.tokseq + min((int64_t)J * kTT + g * 32 + lane, p.T - 1)); };
-      int cs = col_seq(0);  // sequence of column token 32 g + lane
+      int cs = col_seq(g0);  // sequence of column token 32 g + lane
       if (!mbar_wait(accfull_bar(acc), acc_phase, abort_flag, p.info, kIdGram)) break;
       tc_fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * 256;
@@ -183,8 +192,8 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
       int cur = __shfl_sync(0xffffffffu, cs, 0);
       float wseg = (!kSampled && row_seq == cur) ? 2.f : 1.f, run = 0.f;
 #pragma unroll 1
-      for (int g = 0; g < kTT / 32; ++g) {
-        const int cs_next = g + 1 < kTT / 32 ? col_seq(g + 1) : 0;
+      for (int g = g0; g < g0 + kTT / 64; ++g) {
+        const int cs_next = g + 1 < g0 + kTT / 64 ? col_seq(g + 1) : 0;
         uint32_t pv[32], qv[32];
         tmem_ld32(taddr + g * 32, pv);
         tmem_ld32(taddr + 128 + g * 32, qv);
@@ -200,8 +209,8 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
     }
     if (kComplete) {
       __threadfence();
-      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
-      mirror_by_cta<true>(p.K, p.B, row, [](int) { return 0.f; }, false);
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // the epilogue warps
+      if (g0 == 0) mirror_by_cta<true>(p.K, p.B, row, [](int) { return 0.f; }, false);
     }
   }
 
@@ -227,6 +236,16 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   GramParams p{tokseq, K, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, 0, 0, 0};
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms);
+  // 2-CTA tiles read 3/4 of the bytes per step (40,960 tokens, 896 x 896: 2.75 -> 2.44 ms), but take 0.7 us more to set up and
+  // give the chip coarser units.  Equal at about 160 steps of 64 features per CTA (896 x 896: 34.6 both ways at 4480 tokens,
+  // 40.4 / 39.3 us at 5120; 1536 x 1536: 32.9 / 33.4 at 3000, 44.6 / 43.3 at 3840; 512 x 88: 31 both ways at 6000, 61 / 56.5 at
+  // 9600); units of few steps are bound by their epilogue, which 1-CTA tiles spread better (128 x 64, 20,480 tokens: 119 / 134;
+  // 256 x 256, 8000: 34.5 / 39); and a last wave more costs more than a step less (896 x 896, 6080 tokens, 8 / 9 waves: 53.1 /
+  // 54.9).
+  const long long nk = (d_in + kKF - 1) / kKF + (d_out + kKF - 1) / kKF, nb = (p.nT + 1) / 2;
+  const long long waves = (units + sms - 1) / sms, pairs = sms / 2, pair_waves = (nb * (nb + 1) - p.nT % 2 * nb + pairs - 1) / pairs;
+  if (nk >= 10 && waves * nk >= 160 && 0.95 * pair_waves <= waves)
+    return bf16_gram_pair(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
   // One tile of tokens: its CTA completes K, a launch less for the host, which bounds so small a layer (26 tokens, 640 x 280:
   // 29.1 -> 26.4 us with the scaling pass's).  The last of several CTAs would be 0.7 (15 CTAs) to 1.3 us (136) slower than a
   // kernel that is already set up when this one ends, and above 32 sequences so is one CTA.

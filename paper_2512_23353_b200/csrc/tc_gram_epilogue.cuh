@@ -17,30 +17,36 @@ namespace tc {
 // Order of the tile pairs (I <= J) of the token-Gram triangle.  The tiles running at one time must
 // fit in L2 or every operand byte comes from HBM: the triangle is cut into strips of `S` tile
 // columns; inside a strip the pairs go row by row (I outer, J inner), so about n concurrent units
-// touch S column tiles and n / S row tiles.  Unit u -> (I, J).
-__device__ __forceinline__ void decode_pair_strips(long long u, int nT, int S, int& I, int& J) {
-  int J0 = 0;
-  while (true) {
-    const int w = min(S, nT - J0);
-    const long long cnt = (long long)J0 * w + (long long)w * (w + 1) / 2;
-    if (u < cnt || J0 + w >= nT) {
-      const long long rect = (long long)J0 * w;
-      if (u < rect) {
-        I = (int)(u / w);
-        J = J0 + (int)(u % w);
-      } else {
-        long long r = u - rect;
-        int k = 0;
-        while (k < w - 1 && r >= w - k) { r -= w - k; ++k; }  // row J0 + k holds w - k pairs
-        I = J0 + k;
-        J = I + (int)r;
-      }
-      return;
+// touch S column tiles and n / S row tiles.  A walk goes through the units first, first + step, ... of that order: found
+// from the one before instead of from the beginning, with 32-bit arithmetic (a strip has below 2^32 units), because every
+// warp of the epilogue decodes every unit and a narrow layer's unit is short.
+struct PairWalk {
+  int n, S, J0;  // tiles, strip width, first column of the current strip
+  unsigned r;    // unit within the strip
+  __device__ __forceinline__ PairWalk(int n_tiles, int strip, unsigned first) : n(n_tiles), S(strip), J0(0), r(first) { settle(); }
+  __device__ __forceinline__ void settle() {
+    while (J0 < n) {
+      const unsigned w = min(S, n - J0), cnt = J0 * w + w * (w + 1) / 2;
+      if (r < cnt) return;
+      r -= cnt;
+      J0 += w;
     }
-    u -= cnt;
-    J0 += w;
   }
-}
+  __device__ __forceinline__ bool more() const { return J0 < n; }
+  __device__ __forceinline__ void next(unsigned step) { r += step; settle(); }
+  __device__ __forceinline__ void get(int& I, int& J) const {
+    const unsigned w = min(S, n - J0), rect = J0 * w;
+    if (r < rect) {
+      I = r / w;
+      J = J0 + (int)(r - I * w);
+    } else {
+      unsigned left = r - rect, k = 0;
+      while (left >= w - k) { left -= w - k; ++k; }  // row J0 + k holds w - k pairs
+      I = J0 + k;
+      J = I + left;
+    }
+  }
+};
 
 // Strip width for tiles of `tile_bytes` (both operands' rows of one tile): column and row tiles of
 // ~148 concurrent units should stay within about 48 MB.
@@ -94,6 +100,11 @@ __device__ __forceinline__ void flush_rows(float* __restrict__ K, int B, const R
     atomicAdd(&K[(size_t)rows.seq * B + col_seq], v);
 }
 
+// Independent partial sums of a segment: a scheduler has two epilogue warps, which one chain of 32 dependent additions each
+// would leave idle most of the time.
+constexpr int kChains = 4;
+__device__ __forceinline__ float chain_sum(const float (&s)[kChains]) { return (s[0] + s[1]) + (s[2] + s[3]); }
+
 // One group of 32 columns.  pv/qv: this lane's 32 values of P and Q; cs: sequence of column c0 + lane;
 // cur / wseg / run: the running segment (its sequence, this lane's weight for it, this lane's sum).
 // kWeighted: the Gram route's symmetry weights (a pair inside one sequence stands for (t,s) and
@@ -102,36 +113,38 @@ __device__ __forceinline__ void flush_rows(float* __restrict__ K, int B, const R
 // (not per column), so the code stays small: this runs once per unit and a fully unrolled
 // per-column version (hundreds of KB of instructions) was bound by instruction fetch.
 template <bool kWeighted>
-__device__ __forceinline__ void gram_group(const uint32_t (&pv)[32], const uint32_t (&qv)[32], int cs, int c0, int row,
+__device__ __forceinline__ void gram_group(uint32_t (&pv)[32], uint32_t (&qv)[32], int cs, int c0, int row,
                                            bool diag, const RowSegments& rows, float* __restrict__ K, int B, int& cur,
                                            float& wseg, float& run) {
   const int lane = threadIdx.x & 31;
   const int prev = __shfl_up_sync(0xffffffffu, cs, 1);
   unsigned starts = __ballot_sync(0xffffffffu, cs != (lane == 0 ? cur : prev));  // bit e: a new sequence starts at column e
-  float h[32];
-#pragma unroll
-  for (int e = 0; e < 32; ++e) h[e] = __uint_as_float(pv[e]) * __uint_as_float(qv[e]);
   if (kWeighted && diag) {
     // column c == row is the pair (t, t): once, against the weight two of its own sequence
     const int d = row - c0;  // columns e < d are below the diagonal
 #pragma unroll
-    for (int e = 0; e < 32; ++e) h[e] = e > d ? h[e] : (e == d ? 0.5f * h[e] : 0.f);
+    for (int e = 0; e < 32; ++e) {
+      const float v = __uint_as_float(pv[e]);
+      pv[e] = __float_as_uint(e > d ? v : (e == d ? 0.5f * v : 0.f));
+      if (e < d) qv[e] = 0u;  // a non-finite entry there counts for the other half of the pair only
+    }
   }
   if (starts == 0u) {
-    float s = 0.f;
+    float s[kChains] = {};
 #pragma unroll
-    for (int e = 0; e < 32; ++e) s += h[e];
-    run = fmaf(wseg, s, run);
+    for (int e = 0; e < 32; ++e) s[e % kChains] = fmaf(__uint_as_float(pv[e]), __uint_as_float(qv[e]), s[e % kChains]);
+    run = fmaf(wseg, chain_sum(s), run);
     return;
   }
   int lo = 0;
   while (true) {
     const int hi = starts ? __ffs(starts) - 1 : 32;  // columns lo .. hi - 1 continue the running segment
     const unsigned in = (hi < 32 ? (1u << hi) - 1u : 0xffffffffu) & ~((1u << lo) - 1u);
-    float s = 0.f;
+    float s[kChains] = {};
 #pragma unroll
-    for (int e = 0; e < 32; ++e) s += ((in >> e) & 1u) ? h[e] : 0.f;
-    run = fmaf(wseg, s, run);
+    for (int e = 0; e < 32; ++e)
+      if ((in >> e) & 1u) s[e % kChains] = fmaf(__uint_as_float(pv[e]), __uint_as_float(qv[e]), s[e % kChains]);
+    run = fmaf(wseg, chain_sum(s), run);
     if (hi == 32) break;
     flush_rows(K, B, rows, cur, run);
     run = 0.f;

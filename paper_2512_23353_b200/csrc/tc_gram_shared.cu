@@ -24,7 +24,7 @@ constexpr int kStages = 6;
 constexpr int kOperandBytes = kTT * 128;       // 16 KB
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;                   // copy warp, MMA warp, eight epilogue warps
 constexpr uint32_t kTmemCols = 512;            // P0 | P1 | Q0 | Q1
 constexpr int kMaxHeads = 3;
 
@@ -58,7 +58,7 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(qfull_bar(b), 1); mbar_init(qempty_bar(b), 4); mbar_init(pempty_bar(b), 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(qfull_bar(b), 1); mbar_init(qempty_bar(b), 8); mbar_init(pempty_bar(b), 8); }
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -69,7 +69,6 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
-  const long long total_units = (long long)p.nT * (p.nT + 1) / 2;
   // stage index inside a unit -> (segment, feature block): segment 0 is X, segment 1 + h is dY^(h)
   int nk[kMaxHeads + 1];
   nk[0] = (p.d_in + kKF - 1) / kKF;
@@ -96,9 +95,9 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (long long u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
+      for (PairWalk u(p.nT, p.strip, blockIdx.x); u.more() && ok; u.next(gridDim.x)) {
         int I, J;
-        decode_pair_strips(u, p.nT, p.strip, I, J);
+        u.get(I, J);
         const bool diag = I == J;
         for (int kb = 0; kb < nk_total; ++kb) {
           int seg, kk;
@@ -120,9 +119,9 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       uint32_t phase = 0;
       unsigned ucount = 0, qcount = 0;  // units and Q accumulators started: buffer = count & 1, parity = count >> 1 & 1
       bool ok = true;
-      for (long long u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++ucount) {
+      for (PairWalk u(p.nT, p.strip, blockIdx.x); u.more() && ok; u.next(gridDim.x), ++ucount) {
         int I, J;
-        decode_pair_strips(u, p.nT, p.strip, I, J);
+        u.get(I, J);
         const bool diag = I == J;
         const unsigned pb = ucount & 1u;
         // P[pb] is free once every projection of the unit before last has been through the epilogue
@@ -160,12 +159,13 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       }
     }
   } else {
-    const int q = warp & 3, row = q * 32 + lane;
+    // a warp takes 32 rows (the TMEM lanes it can read) and half of the columns
+    const int q = warp & 3, row = q * 32 + lane, g0 = (warp - 2) / 4 * (kTT / 64);
     unsigned ucount = 0, qcount = 0;
     bool ok = true;
-    for (long long u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++ucount) {
+    for (PairWalk u(p.nT, p.strip, blockIdx.x); u.more() && ok; u.next(gridDim.x), ++ucount) {
       int I, J;
-      decode_pair_strips(u, p.nT, p.strip, I, J);
+      u.get(I, J);
       const bool diag = I == J;
       const unsigned pb = ucount & 1u;
       const int64_t trow = (int64_t)I * kTT + row;
@@ -176,15 +176,15 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
 #pragma unroll 1
       for (int h = 0; h < p.n_heads; ++h, ++qcount) {
         const unsigned qb = qcount & 1u;
-        int cs = col_seq(0);
+        int cs = col_seq(g0);
         if (!(ok = mbar_wait(qfull_bar(qb), (qcount >> 1) & 1u, abort_flag, p.info, kIdGram))) break;
         tc_fence_after_sync();
         float* Kh = p.K[h];
         int cur = __shfl_sync(0xffffffffu, cs, 0);
         float wseg = row_seq == cur ? 2.f : 1.f, run = 0.f;
 #pragma unroll 1
-        for (int g = 0; g < kTT / 32; ++g) {
-          const int cs_next = g + 1 < kTT / 32 ? col_seq(g + 1) : 0;
+        for (int g = g0; g < g0 + kTT / 64; ++g) {
+          const int cs_next = g + 1 < g0 + kTT / 64 ? col_seq(g + 1) : 0;
           uint32_t pv[32], qv[32];
           tmem_ld32(taddr + pb * 128u + g * 32, pv);
           tmem_ld32(taddr + 256u + qb * 128u + g * 32, qv);
