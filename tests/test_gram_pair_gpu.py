@@ -1,4 +1,4 @@
-"""Token-Gram kernel with 2-CTA tiles (256 rows x 128 columns of tokens): wide layers from 2049 tokens on, with an odd and an even
+"""Token-Gram kernel with 2-CTA tiles (256 x 256 tokens): wide layers from 2049 tokens on, with an odd and an even
 number of 128-token tiles, ragged last tiles, feature counts that end inside a 64-feature step, and sequences that are shorter
 than a group of 32 columns, that end on a tile's edge and that span tiles; and the widths beside the line to the 1-CTA kernel.
 
