@@ -1,4 +1,7 @@
-"""Thin ctypes binding of libisopo.so: same names as the C ABI, argument marshalling only.
+"""Thin binding of libisopo.so: same names as the C ABI, argument marshalling only.
+
+The calls of a layer's pass are marshalled natively (csrc/py_calls.c); whatever that does not take as it stands (offsets
+in a list, a wrong dtype), and the other calls, go through ctypes and the checks below.
 
 Every step of the path runs in the library's CUDA kernels.  torch is used for device memory and
 the current stream, nothing else.  Importing this module without a built library raises.
@@ -162,6 +165,25 @@ def _stream() -> int:
     return _raw_stream(_current_device())
 
 
+def _bind_calls(calls, get_device, get_stream) -> None:
+    calls.bind(tuple(ctypes.cast(f, ctypes.c_void_p).value for f in (
+        lib.isopo_layer_gram, lib.isopo_transform_advantages, lib.isopo_transform_advantages_rel, lib.isopo_reg_ema_update,
+        lib.isopo_weight_grad, lib.isopo_sampled_coefficients)), (torch.float32, torch.bfloat16, torch.int32, torch.uint8),
+        (get_device, get_stream))
+
+
+def _load_calls():
+    try:
+        from . import _calls
+    except ImportError as e:
+        raise ImportError("_calls.so is missing or does not load: build it with `python -m paper_2512_23353_b200.build`") from e
+    _bind_calls(_calls, _current_device, _raw_stream)
+    return _calls
+
+
+_calls = _load_calls()
+
+
 def _addr(a: np.ndarray) -> int:
     """Address of an array's data (`a.ctypes.data` builds two objects to get at it)."""
     return a.__array_interface__["data"][0]
@@ -195,6 +217,9 @@ def alloc_workspace(dtype: int, T: int, d_in: int, d_out: int, B: int, path: int
 
 def isopo_layer_gram(X: torch.Tensor, dY: torch.Tensor, seq_offsets, K: torch.Tensor, ws: torch.Tensor,
                      info: torch.Tensor, path: int = PATH_AUTO) -> None:
+    st = _calls.layer_gram(X, dY, seq_offsets, K, ws, info, path)
+    if st is not None:
+        return _check(st, "isopo_layer_gram")
     off = _offsets(seq_offsets)
     B = off.shape[0] - 1
     assert X.is_cuda and dY.is_cuda and X.is_contiguous() and dY.is_contiguous() and X.dtype == dY.dtype
@@ -263,6 +288,9 @@ def isopo_layer_gram_static(X: torch.Tensor, dY: torch.Tensor, seq_offsets, K: t
 
 def isopo_transform_advantages(K: torch.Tensor, A: torch.Tensor, variant: int, lam: float, coeffs: torch.Tensor,
                                info: torch.Tensor, pqr_regs=None) -> None:
+    st = _calls.transform(K, A, variant, lam, coeffs, info) if pqr_regs is None else None
+    if st is not None:
+        return _check(st, "isopo_transform_advantages")
     B = A.numel()
     assert K.dtype == torch.float32 and A.dtype == torch.float32 and coeffs.dtype == torch.float32
     assert K.is_contiguous() and K.numel() == B * B and coeffs.numel() == B
@@ -292,6 +320,9 @@ def isopo_transform_advantages_large(K: torch.Tensor, A: torch.Tensor, lam: floa
 
 def isopo_reg_ema_update(K: torch.Tensor, decay: float, state: torch.Tensor) -> None:
     """Folds this microbatch's K into the running means `state` (device float32 [4], zeroed once by the caller)."""
+    st = _calls.reg_ema(K, decay, state)
+    if st is not None:
+        return _check(st, "isopo_reg_ema_update")
     B = K.shape[0]
     assert K.dtype == torch.float32 and K.is_contiguous() and K.numel() == B * B
     assert state.dtype == torch.float32 and state.numel() == 4 and state.is_cuda
@@ -301,6 +332,9 @@ def isopo_reg_ema_update(K: torch.Tensor, decay: float, state: torch.Tensor) -> 
 def isopo_transform_advantages_rel(K: torch.Tensor, A: torch.Tensor, variant: int, factor: float, state: torch.Tensor,
                                    coeffs: torch.Tensor, info: torch.Tensor, pqr_factors=None) -> None:
     """isopo_transform_advantages with the regulariser = factor x the running mean kept in `state`."""
+    st = _calls.transform_rel(K, A, variant, factor, state, coeffs, info) if pqr_factors is None else None
+    if st is not None:
+        return _check(st, "isopo_transform_advantages_rel")
     B = A.numel()
     assert K.dtype == torch.float32 and A.dtype == torch.float32 and coeffs.dtype == torch.float32
     assert K.is_contiguous() and K.numel() == B * B and coeffs.numel() == B and state.numel() == 4
@@ -387,6 +421,9 @@ def isopo_transform_spectral_batched(Ks, A: torch.Tensor, lams, coeffs, info: to
 
 def isopo_weight_grad(X: torch.Tensor, dY: torch.Tensor, coeffs: torch.Tensor, seq_offsets, dW: torch.Tensor,
                       ws: torch.Tensor, info: torch.Tensor, path: int = PATH_AUTO, beta: float = 0.0) -> None:
+    st = _calls.weight_grad(X, dY, coeffs, seq_offsets, dW, ws, info, path, beta)
+    if st is not None:
+        return _check(st, "isopo_weight_grad")
     off = _offsets(seq_offsets)
     B = off.shape[0] - 1
     (T, d_in), d_out = X.shape, dY.shape[1]
@@ -414,6 +451,9 @@ def alloc_sampled_workspace(dtype: int, T: int, d_in: int, d_out: int, B: int, n
 def isopo_sampled_coefficients(X: torch.Tensor, dY: torch.Tensor, seq_offsets, sample_rows, A: torch.Tensor, lam: float,
                                coeffs: torch.Tensor, ws: torch.Tensor, info: torch.Tensor, F2: torch.Tensor = None) -> None:
     """Algorithm 1's coefficients from sampled token rows (the caller draws `sample_rows`)."""
+    st = _calls.sampled(X, dY, seq_offsets, sample_rows, A, lam, coeffs, ws, info, F2)
+    if st is not None:
+        return _check(st, "isopo_sampled_coefficients")
     off = _offsets(seq_offsets)
     B = off.shape[0] - 1
     rows = np.ascontiguousarray(np.asarray(sample_rows, dtype=np.int64))

@@ -1,4 +1,4 @@
-"""Builds libisopo.so (hand-written CUDA for sm_100a) in-tree with nvcc.
+"""Builds libisopo.so (hand-written CUDA for sm_100a) in-tree with nvcc, and the binding's _calls.so with gcc.
 
 Usage: python -m paper_2512_23353_b200.build [--force] [--debug] [-v]
 
@@ -13,6 +13,7 @@ import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
@@ -20,6 +21,7 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 LIB_PATH = os.path.join(PKG_DIR, "libisopo.so")
 DEBUG_LIB_PATH = os.path.join(PKG_DIR, "libisopo_debug.so")
+CALLS_PATH = os.path.join(PKG_DIR, "_calls.so")  # the binding's native marshalling (csrc/py_calls.c)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -48,8 +50,20 @@ def _compile(src, verbose, debug):
     return obj, r.stderr
 
 
+def _build_calls(force):
+    src = os.path.join(CSRC, "py_calls.c")
+    if not force and os.path.exists(CALLS_PATH) and os.path.getmtime(CALLS_PATH) >= max(
+            os.path.getmtime(p) for p in (src, os.path.join(ROOT, "include", "isopo.h"), __file__)):
+        return
+    r = subprocess.run(["gcc", "-O2", "-std=gnu11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I",
+                        os.path.join(ROOT, "include"), src, "-o", CALLS_PATH], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"gcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     """Compiles every .cu under csrc/ and links libisopo.so (libisopo_debug.so with `debug`); returns its path."""
+    _build_calls(force)
     lib_path = DEBUG_LIB_PATH if debug else LIB_PATH
     if not force and os.path.exists(lib_path) and os.path.getmtime(lib_path) >= _deps_mtime():
         return lib_path
