@@ -90,3 +90,25 @@ def test_sampled(b, n_samples, d_in, d_out, lens):
     want, _, _ = orc.isopo_layer_sampled(to_f64(X), to_f64(dY), off, to_f64(A), rows, 0.0)
     assert int(info.item()) == 0
     assert rel_fro(F2.cpu().numpy(), want) <= 2 * TOL  # a square
+
+
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 127, 128, 129, 300, 2049])
+@pytest.mark.parametrize("d_in,d_out", [(8, 8), (64, 65), (520, 260), (2048, 1280)])
+def test_weight_gradient_slabs(T, d_in, d_out):
+    """The GEMM over all tokens cuts them into as many slabs as make its waves cheapest: one, or down to 16 tokens; few tiles and
+    many.  Bound: float32 products and sums over at most T terms and the slabs' float32 additions, T 2^-24 at worst, taken as 2e-6
+    of the norm (random signs)."""
+    from paper_2512_23353_b200 import binding as b
+    B = min(T, 3)
+    off = np.linspace(0, T, B + 1).astype(np.int64)
+    g = torch.Generator(device="cuda").manual_seed(T + d_in)
+    X, dY = torch.randn(T, d_in, device="cuda", generator=g), torch.randn(T, d_out, device="cuda", generator=g)
+    c, dW = torch.randn(B, device="cuda", generator=g), torch.full((d_out, d_in), float("nan"), device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = b.alloc_workspace(b.F32, T, d_in, d_out, B, b.PATH_GRAM)
+    per_token = c.double().repeat_interleave(torch.from_numpy(np.diff(off)).cuda())[:, None]
+    want = (per_token * dY.double()).T @ X.double()
+    for beta in (0.0, 1.0):
+        b.isopo_weight_grad(X, dY, c, off, dW, ws, info, b.PATH_GRAM, beta)
+        assert float((dW.double() - (1 + beta) * want).norm() / want.norm()) <= 2e-6 * (1 + beta)
+    assert int(info.item()) == 0
