@@ -525,10 +525,11 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
   const Clear clear = beta == 0.f ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
   int64_t* off_dev = (int64_t*)(w + L.off_offsets);
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
+  float* tokscale = (float*)tokseq;  // one scale per token: a single independent load per row
   if (dtype == ISOPO_F32) {
-    s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, clear, st);
+    s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);
     if (s != ISOPO_OK) return s;
-    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, coeffs, tokseq, dW, st);
+    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, tokscale, dW, st);
   }
   if (bf16_weight_grad_fold_applies(T, d_in, d_out, B)) {
     s = launch_offsets(seq_offsets_host, B, off_dev, clear, st);
@@ -537,8 +538,6 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
   }
   if (bf16_weight_grad_uses_pairs(d_out))
     return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, clear, info, st);
-  // one scale per token, so that the kernel's scaler warps need a single independent load per row
-  float* tokscale = (float*)tokseq;
   s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);
   if (s != ISOPO_OK) return s;
   return bf16_weight_grad(X, dY, T, d_in, d_out, tokscale, dW, info, st);

@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(256) k_prep_many(const int64_t* __restrict__ o
 // Bound by the float32 pipe: 64 sequences of 72 tokens, 896 x 896: 174 us (42 TFLOP/s with the 205 MB store of G) against
 // 342 us with a 64 x 64 tile loaded synchronously.  Stages of 8 tokens waste less of a short sequence's last stage
 // (G_i: 174 against 187 us with 16); over one long token range stages of 16 synchronise half as often (dW: 197 against 212 us).
+// The copies' addresses are stepped, not computed per element, and a token's weight is copied like its row: dW of 4835 tokens
+// 190 -> 177 us, 895 x 895 (4-byte copies) 230 -> 199, G of 64 sequences of 75 tokens, 895 x 895, 285 -> 234.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool live) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
@@ -95,22 +97,33 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   return r;
 }
 
-// Stages rows [t, t + kRows) x columns [c0, c0 + kCols) of a row-major [., d] matrix into dst[kRows][kCols].
+// Stages rows [t, t + kRows) x columns [c0, c0 + kCols) of a row-major [., d] matrix into dst[kRows][kCols].  A thread keeps its
+// column (group) and steps through the rows by address.
 template <int kRows, int kCols, int kThreadsF>
 __device__ __forceinline__ void stage_rows(float* dst, const float* __restrict__ M, int64_t t, int64_t t_end, int c0, int d) {
+  const int left = (int)min((int64_t)kRows, t_end - t);  // rows that exist
   if ((d & 3) == 0) {
+    constexpr int kStep = kThreadsF / (kCols / 4);
+    const int r = threadIdx.x / (kCols / 4), c = threadIdx.x % (kCols / 4) * 4;
+    if (kStep > kRows && r >= kRows) return;
+    const bool col = c0 + c < d;
+    const float* src = M + (t + r) * d + c0 + c;
+    float* to = dst + r * kCols + c;
 #pragma unroll
-    for (int e = threadIdx.x; e < kRows * kCols / 4; e += kThreadsF) {
-      const int r = e / (kCols / 4), c = e % (kCols / 4) * 4;
-      const bool live = t + r < t_end && c0 + c < d;
-      cp_async16(dst + r * kCols + c, live ? M + (t + r) * d + c0 + c : M, live);
+    for (int i = 0; i < kRows; i += kStep, src += (int64_t)kStep * d) {
+      const bool live = col && r + i < left;
+      cp_async16(to + i * kCols, live ? src : M, live);
     }
   } else {
+    constexpr int kStep = kThreadsF / kCols;
+    const int r = threadIdx.x / kCols, c = threadIdx.x % kCols;
+    const bool col = c0 + c < d;
+    const float* src = M + (t + r) * d + c0 + c;
+    float* to = dst + r * kCols + c;
 #pragma unroll
-    for (int e = threadIdx.x; e < kRows * kCols; e += kThreadsF) {
-      const int r = e / kCols, c = e % kCols;
-      const bool live = t + r < t_end && c0 + c < d;
-      cp_async4(dst + r * kCols + c, live ? M + (t + r) * d + c0 + c : M, live);
+    for (int i = 0; i < kRows; i += kStep, src += (int64_t)kStep * d) {
+      const bool live = col && r + i < left;
+      cp_async4(to + i * kCols, live ? src : M, live);
     }
   }
 }
@@ -127,11 +140,10 @@ struct TokenGemm {
   __device__ __forceinline__ static int row(int p) { return (p / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x / kSide) * 4 + p % 4; }
   __device__ __forceinline__ static int col(int q) { return (q / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x % kSide) * 4 + q % 4; }
 
-  // kScaled: the dY row of token t counts coeffs[tokseq[t]] times (rounded once, as a scaled copy of dY would be)
+  // kScaled: the dY row of token t counts tokscale[t] times (rounded once, as a scaled copy of dY would be)
   template <bool kScaled>
   __device__ __forceinline__ void run(float* smem, const float* __restrict__ X, const float* __restrict__ dY, int d_in,
-                                      int d_out, int64_t t0, int64_t t1, int m0, int n0, const float* __restrict__ coeffs,
-                                      const int32_t* __restrict__ tokseq) {
+                                      int d_out, int64_t t0, int64_t t1, int m0, int n0, const float* __restrict__ tokscale) {
 #pragma unroll
     for (int p = 0; p < kT; ++p)
 #pragma unroll
@@ -144,8 +156,10 @@ struct TokenGemm {
         const int64_t t = t0 + (int64_t)k * kTK;
         stage_rows<kTK, kTile, kThr>(s, dY, t, t1, m0, d_out);
         stage_rows<kTK, kTile, kThr>(s + kTK * kTile, X, t, t1, n0, d_in);
-        if (kScaled && threadIdx.x < kTK)
-          sw[(k % kStages) * kTK + threadIdx.x] = t + threadIdx.x < t1 ? coeffs[tokseq[t + threadIdx.x]] : 0.f;
+        if (kScaled && threadIdx.x < kTK) {
+          const bool live = t + threadIdx.x < t1;
+          cp_async4(sw + (k % kStages) * kTK + threadIdx.x, live ? tokscale + t + threadIdx.x : tokscale, live);
+        }
       }
       cp_async_commit();
     };
@@ -222,7 +236,7 @@ k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ 
   }
   const int64_t t0 = kArgOff ? o.v[i] : a.off[i], t1 = kArgOff ? o.v[i + 1] : a.off[i + 1];
   SeqGemm<kTile, kT> g;
-  g.template run<false>(smem, a.X, a.dY, a.d_in, a.d_out, t0, t1, m0, n0, nullptr, nullptr);
+  g.template run<false>(smem, a.X, a.dY, a.d_in, a.d_out, t0, t1, m0, n0, nullptr);
   float* Gi = a.G + (size_t)i * a.gstride;
 #pragma unroll
   for (int p = 0; p < kT; ++p) {
@@ -256,13 +270,13 @@ k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ 
 template <int kTile, int kT>
 __global__ void __launch_bounds__(SlabGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
 k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int64_t T, int d_in, int d_out,
-                  const float* __restrict__ coeffs, const int32_t* __restrict__ tokseq, float* __restrict__ dW, int64_t slab) {
+                  const float* __restrict__ tokscale, float* __restrict__ dW, int64_t slab) {
   pdl_wait();
   extern __shared__ __align__(16) float smem[];
   const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t t0 = blockIdx.z * slab, t1 = min(T, t0 + slab);
   SlabGemm<kTile, kT> g;
-  g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, m0, n0, coeffs, tokseq);
+  g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, m0, n0, tokscale);
 #pragma unroll
   for (int p = 0; p < kT; ++p) {
     const int m = m0 + g.row(p);
@@ -817,7 +831,7 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
 constexpr int64_t kSlabOverhead = 64;  // tokens
 template <int kTile, int kT>
 static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out,
-                                           const float* coeffs, const int32_t* tokseq, float* dW, cudaStream_t st) {
+                                           const float* tokscale, float* dW, cudaStream_t st) {
   typedef SlabGemm<kTile, kT> Gemm;
   const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
   if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
@@ -829,7 +843,7 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
   ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
   // Token slabs, each a multiple of the staging depth: the count whose waves take least, a wave costing its slab and what a CTA
   // spends on filling its pipeline and adding its tile.  "Four CTAs per SM" instead left the last wave nearly empty: 896 x 896,
-  // 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 -> 10.1.
+  // 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 -> 10.1 (this alone).
   const int64_t tiles = (int64_t)gx * gy, slots = (int64_t)sms * std::max(per_sm, 1), most = std::max<int64_t>(1, (T + 127) / 128);
   int64_t slab = 0, best = INT64_MAX;
   for (int64_t n = 1; n <= std::min<int64_t>(most, std::max<int64_t>(8, 8 * slots / tiles)); ++n) {
@@ -841,16 +855,16 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
   if (splits > 65535) return ISOPO_ERR_UNSUPPORTED;
   {
     LaunchScope scope(kIdF32WeightGrad, st);
-    launch(kernel, dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st, X, dY, T, d_in, d_out, coeffs, tokseq, dW, slab);
+    launch(kernel, dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st, X, dY, T, d_in, d_out, tokscale, dW, slab);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 
-isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* coeffs,
-                             const int32_t* tokseq, float* dW, cudaStream_t st) {
-  return f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st)
-                                                      : launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, coeffs, tokseq, dW, st);
+isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* tokscale, float* dW,
+                             cudaStream_t st) {
+  return f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, tokscale, dW, st)
+                                                      : launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, tokscale, dW, st);
 }
 
 }  // namespace isopo
