@@ -292,9 +292,10 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
 // the sum).
 isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                        float* K, int32_t* info, cudaStream_t st);
-// 2-CTA tiles: see the rule in tc_gram.cu
-isopo_status bf16_gram_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
-                            float* K, int32_t* info, cudaStream_t st);
+// 2-CTA tiles, one projection or several that share X: where they pay
+bool bf16_gram_pair_pays(int64_t T, int d_in, const int* d_out, int n_heads, int sms);
+isopo_status bf16_gram_pair(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+                            const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 // 1-CTA tiles, operand rows scaled in shared memory

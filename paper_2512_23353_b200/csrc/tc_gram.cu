@@ -236,17 +236,7 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   GramParams p{tokseq, K, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, 0, 0, 0};
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms);
-  // 2-CTA tiles of 256 x 256 move half the bytes per flop, but take 2.5 us more to set up and drain and give the chip coarser
-  // units.  Costs in steps of 64 features of a 1-CTA tile (0.19 us); a wave is a tile per CTA or pair, which its epilogue bounds
-  // from below.  A pair's wave, twice the tokens per SM, is 1.65 of the other's, 1.45 from about 5000 tokens on.
-  // Measured (1-CTA / 2-CTA): 896 x 896: 12.4 / 18.1 us at 2048 tokens, 23.6 / 27.3 at 3328, 28.3 / 27.6 at 3840, 33.1 / 35.1 at
-  // 4352 (5 waves / 3), 39.6 / 36.8 at 5120, 137 / 121 at 10,240; 896 x 4864: 54.3 / 63.2 at 3328, 69.1 / 63.3 at 3840, 85.6 /
-  // 89.2 at 4352, 429 / 395 at 10,240; 448 x 448: 19.0 / 19.1 at 3840, 31.4 / 33.2 at 6144, 142 / 119 at 14,336; 256 x 256: 35.6 /
-  // 36.5 at 8192, 89.4 / 80.7 at 14,336; 128 x 64: 58 / 65 at 14,336; 64 x 416: 792 / 641 at 40,940.
-  const long long nk = (d_in + kKF - 1) / kKF + (d_out + kKF - 1) / kKF, nb = (p.nT + 1) / 2, pairs = sms / 2;
-  const long long waves = (units + sms - 1) / sms, pair_waves = (nb * (nb + 1) / 2 + pairs - 1) / pairs;
-  if (pair_waves * std::max((pair_waves >= 5 ? 1.45 : 1.65) * nk, 14.0) + 12 < waves * std::max((double)nk, 6.5))
-    return bf16_gram_pair(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
+  if (bf16_gram_pair_pays(T, d_in, &d_out, 1, sms)) return bf16_gram_pair(X, &dY, T, d_in, &d_out, 1, tokseq, B, &K, info, st);
   // One tile of tokens: its CTA completes K, a launch less for the host, which bounds so small a layer (26 tokens, 640 x 280:
   // 29.1 -> 26.4 us with the scaling pass's).  The last of several CTAs would be 0.7 (15 CTAs) to 1.3 us (136) slower than a
   // kernel that is already set up when this one ends, and above 32 sequences so is one CTA.

@@ -109,13 +109,14 @@ __device__ __forceinline__ float chain_sum(const float (&s)[kChains]) { return (
 // cur / wseg / run: the running segment (its sequence, this lane's weight for it, this lane's sum).
 // kWeighted: the Gram route's symmetry weights (a pair inside one sequence stands for (t,s) and
 // (s,t), weight two); on a diagonal tile only columns c >= row are used, c == row once.
+// masked: pv has been through this already, for another projection.
 // The segment boundaries of the group come from one ballot; the loop below runs once per segment
 // (not per column), so the code stays small: this runs once per unit and a fully unrolled
 // per-column version (hundreds of KB of instructions) was bound by instruction fetch.
 template <bool kWeighted>
 __device__ __forceinline__ void gram_group(uint32_t (&pv)[32], uint32_t (&qv)[32], int cs, int c0, int row,
                                            bool diag, const RowSegments& rows, float* __restrict__ K, int B, int& cur,
-                                           float& wseg, float& run) {
+                                           float& wseg, float& run, bool masked = false) {
   const int lane = threadIdx.x & 31;
   const int prev = __shfl_up_sync(0xffffffffu, cs, 1);
   unsigned starts = __ballot_sync(0xffffffffu, cs != (lane == 0 ? cur : prev));  // bit e: a new sequence starts at column e
@@ -125,7 +126,7 @@ __device__ __forceinline__ void gram_group(uint32_t (&pv)[32], uint32_t (&qv)[32
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
       const float v = __uint_as_float(pv[e]);
-      pv[e] = __float_as_uint(e > d ? v : (e == d ? 0.5f * v : 0.f));
+      if (!masked) pv[e] = __float_as_uint(e > d ? v : (e == d ? 0.5f * v : 0.f));
       if (e < d) qv[e] = 0u;  // a non-finite entry there counts for the other half of the pair only
     }
   }

@@ -6,7 +6,8 @@
 // into projection h's K, the tensor core already fills the other Q (or, after the last projection,
 // the other P for the next unit), so no epilogue is exposed.  Against one k_bf16_gram launch per
 // projection this saves the X contraction of every projection but the first, and the loads of X that
-// feed it.  Pipeline, tile order and epilogue are those of tc_gram.cu.
+// feed it.  Pipeline, tile order and epilogue are those of tc_gram.cu.  Large layers go to the 2-CTA tiles of tc_gram_pair.cu
+// (1536 -> 1536, 256, 256, 19,200 tokens 1085 -> 826 us; 896 -> 4864, 4864, 10,496 tokens 947 -> 772).
 #include <algorithm>
 
 #include "tc_common.cuh"
@@ -215,6 +216,11 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
 isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st) {
   if (n_heads < 1 || n_heads > kMaxHeads) return ISOPO_ERR_INVALID_ARG;
+  int dev = 0, sms = 0;
+  ISOPO_CUDA_TRY(cudaGetDevice(&dev));
+  ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (bf16_gram_pair_pays(T, d_in, d_out, n_heads, sms))
+    return bf16_gram_pair(X, dY, T, d_in, d_out, n_heads, tokseq, B, K, info, st);
   CUtensorMap mapX, mapY[kMaxHeads];
   isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
   if (s != ISOPO_OK) return s;
@@ -223,9 +229,6 @@ isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, i
     s = make_map_2d_bf16(&mapY[h], dY[hh], (uint64_t)T, (uint64_t)d_out[hh], (uint64_t)d_out[hh], 64, kTT);
     if (s != ISOPO_OK) return s;
   }
-  int dev = 0, sms = 0;
-  ISOPO_CUDA_TRY(cudaGetDevice(&dev));
-  ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   SharedGramParams p{};
   p.tokseq = tokseq; p.T = T; p.B = B; p.nT = (int)((T + kTT - 1) / kTT); p.d_in = d_in; p.n_heads = n_heads; p.info = info;
