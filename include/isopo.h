@@ -205,9 +205,8 @@ ISOPO_API isopo_status isopo_transform_advantages(const float* K, const float* A
 
 /*
  * isopo_transform_advantages_large: the interacting variant, (K + lambda I) c = A (Sec. 3 display; Alg. 2), for
- * up to ISOPO_MAX_LARGE_SEQS sequences.  Same blocked Cholesky and float64-residual refinement as
- * isopo_transform_advantages, with the block triangle of the factor kept in `workspace` (2.1 MB at 1024
- * sequences: it stays in the L2) instead of shared memory; one CTA, milliseconds rather than 0.1 ms.  K of more than
+ * up to ISOPO_MAX_LARGE_SEQS sequences.  Blocked Cholesky with float64-residual refinement; above 256 sequences its block
+ * rows are dealt to a cluster of sixteen CTAs and meet in `workspace`.  K of more than
  * 256 sequences comes from the GRAM path of isopo_layer_gram; the simple variants take any B in
  * isopo_transform_advantages.  A non-positive pivot k (1-based) is reported as *info = k, coeffs are then zero.
  *
@@ -281,10 +280,11 @@ ISOPO_API isopo_status isopo_transform_advantages_batched(int n_layers, const fl
  * ISOPO_VAR_INTERACTING; lambda = 0 with a cut-off gives the pseudo-inverse on the kept range, which
  * the Cholesky route cannot (it stops at a non-positive pivot).
  *
- * K is diagonalised by one-sided Jacobi rotations in float32 with float64 inner products, a cluster
- * of eight CTAs per K: milliseconds at B = 256, against ~0.1 ms for isopo_transform_advantages.  It is the
- * diagnostic variant; its float32 eigenbasis limits the coefficients to a relative error of about
- * 1e-7 * cond(K + lambda I) (kept range), the eigenvalues to ~1e-6 of the largest.
+ * Where no direction is left out and K + lambda I is well conditioned (below 1e6), the eigenvalues come from a float64
+ * tridiagonalisation and c from a Cholesky solve beside it: 0.4 ms at B = 256.  Otherwise K is diagonalised by one-sided
+ * Jacobi rotations in float32 with float64 inner products, a cluster of eight CTAs per K: milliseconds; its float32
+ * eigenbasis limits the coefficients to a relative error of about 1e-7 * cond(K + lambda I) (kept range), the
+ * eigenvalues to ~1e-6 of the largest.
  *
  *   K            dev, float32 [B, B] row-major, symmetric (as written by isopo_layer_gram); B <= 256
  *   A            dev, float32 [B]
