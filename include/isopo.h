@@ -15,7 +15,8 @@
  * Conventions shared by every entry point
  *   - "dev" pointers are CUDA device pointers of the current device, "host" pointers are ordinary
  *     host memory.  The caller owns every buffer; the library never allocates or frees device memory.
- *   - X and dY are row-major, contiguous, 16-byte aligned; row t is token t of the packed microbatch;
+ *   - X and dY are row-major, contiguous, 16-byte aligned (K, A and coeffs may start at any element, e.g.
+ *     several K carved out of one buffer); row t is token t of the packed microbatch;
  *     sequence i owns rows seq_offsets[i] .. seq_offsets[i+1]-1, with seq_offsets[0] = 0,
  *     seq_offsets[B] = T and every length >= 1.
  *   - All work is enqueued on `cuda_stream` (a cudaStream_t passed as void*; NULL = default stream)

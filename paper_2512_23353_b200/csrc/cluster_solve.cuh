@@ -344,7 +344,7 @@ __device__ __forceinline__ void cluster_solve(const TransformParams& P, float* L
       const int l = g >> 3, r0 = (g & 7) * 4, I = l == 0 ? rows[0] : rows[1];
       if (I >= nb) continue;
       double acc[4] = {};
-      if ((B & 3) == 0) {
+      if (rows_in_float4(K, B)) {
         for (int j = lane * 4; j < B; j += 128) {
           const double q0 = S.sol[j], q1 = S.sol[j + 1], q2 = S.sol[j + 2], q3 = S.sol[j + 3];
 #pragma unroll

@@ -25,6 +25,12 @@ struct TransformParams {
                            // regularisers above are then factors of these (relative regularisation)
 };
 
+// Whether the rows of a B x B matrix can be read 16 bytes at a time: callers may keep several K in one buffer, so its address
+// is a multiple of 4 bytes and no more.
+__device__ __forceinline__ bool rows_in_float4(const float* K, int B) {
+  return (B & 3) == 0 && (reinterpret_cast<uintptr_t>(K) & 15) == 0;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -224,9 +230,10 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
   const float* __restrict__ K = P.K;
   const int nb = (B + kNB - 1) / kNB, Bp = nb * kNB;
   if (tid == 0) s_fail = 0;
+  const bool vec4 = rows_in_float4(K, B);
   // load the lower block triangle.  K is symmetric, so row j of K read along i gives column j of
-  // the blocks; float4 loads, eight in flight per thread, when B is a multiple of 4.
-  if ((B & 3) == 0) {
+  // the blocks; float4 loads, eight in flight per thread, where its rows are made of them.
+  if (vec4) {
     const int nvec = B * B / 4;
     for (int base = tid; base < nvec; base += kThr * 8) {
       float4 val[8];
@@ -337,7 +344,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
     double rn2 = 0.0;
     for (int i0 = warp * 4; i0 < B; i0 += nwarps * 4) {  // four rows per warp pass: independent loads
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      if ((B & 3) == 0) {
+      if (vec4) {
         for (int j0 = lane * 4; j0 < B; j0 += 256) {  // two float4 per lane and row in flight
           float4 kv[4][2];
 #pragma unroll

@@ -47,9 +47,10 @@ __device__ __forceinline__ TransformParams layer_params(const TransformBatch& ba
 template <typename F>
 __device__ __forceinline__ void row_square_sums(const float* __restrict__ K, int B, int first, int last, F f) {
   const int lane = threadIdx.x & 31;
+  const bool vec4 = rows_in_float4(K, B);
   for (int i0 = first; i0 < last; i0 += 4) {
     double sq[4] = {};
-    if ((B & 3) == 0) {
+    if (vec4) {
 #pragma unroll 2
       for (int j = lane * 4; j < B; j += 128) {
 #pragma unroll
