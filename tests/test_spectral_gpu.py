@@ -77,6 +77,21 @@ def test_cutoff_on_a_rank_deficient_kernel(b):
     np.testing.assert_allclose(c.cpu().numpy()[:20], c.cpu().numpy()[20:], rtol=1e-3, atol=1e-6 * np.abs(c_o).max())
 
 
+@pytest.mark.parametrize("lam_rel,cutoff", [(1e-3, 0.0), (0.0, 1e-4), (1e-12, 0.0)])  # Cholesky; a cut-off; condition too large
+@pytest.mark.parametrize("B", [40, 256])
+def test_coefficients_over_the_advantages(b, B, lam_rel, cutoff):
+    """coeffs may be the array A itself: A is read to the end before anything is written over it."""
+    half = _gram(B // 2, 2, B)
+    K = np.block([[half, half], [half, half]]) if lam_rel < 1e-3 else _gram(B, 3, B)
+    Kd, A = torch.from_numpy(K).cuda(), torch.from_numpy(np.random.default_rng(B).standard_normal(B).astype(np.float32)).cuda()
+    lam = float(lam_rel * np.mean(np.diag(K)))
+    c, info = torch.empty(B, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    b.isopo_transform_spectral(Kd, A, lam, c, info, rel_cutoff=cutoff)
+    b.isopo_transform_spectral(Kd, A, lam, A, info, rel_cutoff=cutoff)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0 and bool(torch.isfinite(c).all()) and torch.equal(A, c)
+
+
 def test_time_at_full_size_and_argument_checks(b, capsys):
     K = _gram(256, 3, 1)
     Kd = torch.from_numpy(K).cuda()
