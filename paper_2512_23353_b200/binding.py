@@ -225,9 +225,8 @@ def isopo_layer_gram(X: torch.Tensor, dY: torch.Tensor, seq_offsets, K: torch.Te
     assert X.is_cuda and dY.is_cuda and X.is_contiguous() and dY.is_contiguous() and X.dtype == dY.dtype
     assert K.dtype == torch.float32 and K.is_contiguous() and K.numel() == B * B
     assert info.dtype == torch.int32 and ws.dtype == torch.uint8
-    T, d_in = X.shape
-    st = lib.isopo_layer_gram(X.data_ptr(), dY.data_ptr(), _dtype_code(X), T, d_in, dY.shape[1], _addr(off), B, path,
-                              K.data_ptr(), ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
+    st = lib.isopo_layer_gram(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1], dY.shape[1], _addr(off), B,
+                              path, K.data_ptr(), ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_layer_gram")
 
 
@@ -426,10 +425,9 @@ def isopo_weight_grad(X: torch.Tensor, dY: torch.Tensor, coeffs: torch.Tensor, s
         return _check(st, "isopo_weight_grad")
     off = _offsets(seq_offsets)
     B = off.shape[0] - 1
-    (T, d_in), d_out = X.shape, dY.shape[1]
-    assert dW.dtype == torch.float32 and dW.is_contiguous() and dW.shape == (d_out, d_in)
+    assert dW.dtype == torch.float32 and dW.is_contiguous() and dW.shape == (dY.shape[1], X.shape[1])
     assert coeffs.dtype == torch.float32 and coeffs.numel() == B
-    st = lib.isopo_weight_grad(X.data_ptr(), dY.data_ptr(), _dtype_code(X), T, d_in, d_out,
+    st = lib.isopo_weight_grad(X.data_ptr(), dY.data_ptr(), _dtype_code(X), X.shape[0], X.shape[1], dY.shape[1],
                                coeffs.data_ptr(), _addr(off), B, path, dW.data_ptr(), float(beta),
                                ws.data_ptr(), ws.numel(), info.data_ptr(), _stream())
     _check(st, "isopo_weight_grad")

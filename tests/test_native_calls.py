@@ -52,3 +52,13 @@ def test_wrong_number_of_arguments_and_other_calls():
     assert b._calls.transform_rel(K, A, b.VAR_NORMALISED, 0.0, torch.zeros(3), A, i) is None
     assert b._calls.reg_ema(K, 0.9, torch.zeros(4)) is None
     assert b._calls.sampled(torch.zeros(5, 8), torch.zeros(5, 6), OFF, [0, 1], A, 0.0, A, A, i, None) is None
+
+
+def test_trailing_dimensions_of_one_are_taken(monkeypatch):
+    """[T, d, 1] holds the same rows as [T, d]: python reads the first two sizes only, and the library sees the call."""
+    monkeypatch.setattr(b, "_stream", lambda: 0)
+    a = [torch.zeros(5, 8, 1), torch.zeros(5, 6, 1), torch.zeros(2), OFF, torch.zeros(6, 8), torch.zeros(0, dtype=torch.uint8),
+         torch.zeros(1, dtype=torch.int32), b.PATH_GRAM, 0.5]
+    assert b._calls.weight_grad(*a) is None
+    with pytest.raises(b.IsopoError, match="ISOPO_ERR_INVALID_ARG"):  # the beta, not the shapes
+        b.isopo_weight_grad(*a)
