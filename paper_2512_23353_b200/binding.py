@@ -1,7 +1,8 @@
 """Thin binding of libisopo.so: same names as the C ABI, argument marshalling only.
 
 The calls of a layer's pass are marshalled natively (csrc/py_calls.c); whatever that does not take as it stands (offsets
-in a list, a wrong dtype), and the other calls, go through ctypes and the checks below.
+in a list, a wrong dtype), the other calls, and all of them where that module is not built, go through ctypes and the checks
+below.
 
 Every step of the path runs in the library's CUDA kernels.  torch is used for device memory and
 the current stream, nothing else.  Importing this module without a built library raises.
@@ -10,6 +11,7 @@ the current stream, nothing else.  Importing this module without a built library
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 from dataclasses import dataclass
 
@@ -172,13 +174,19 @@ def _bind_calls(calls, get_device, get_stream) -> None:
         (get_device, get_stream))
 
 
+class _NoCalls:
+    """In place of the native module: leaves every call to python."""
+
+    layer_gram = transform = transform_rel = reg_ema = weight_grad = sampled = staticmethod(lambda *args: None)
+
+
 def _load_calls():
     try:
-        from . import _calls
-    except ImportError as e:
-        raise ImportError("_calls.so is missing or does not load: build it with `python -m paper_2512_23353_b200.build`") from e
-    _bind_calls(_calls, _current_device, _raw_stream)
-    return _calls
+        calls = importlib.import_module("._calls", __package__)
+    except ModuleNotFoundError:  # not built for this interpreter
+        return _NoCalls
+    _bind_calls(calls, _current_device, _raw_stream)
+    return calls
 
 
 _calls = _load_calls()

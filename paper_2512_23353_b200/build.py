@@ -1,4 +1,5 @@
-"""Builds libisopo.so (hand-written CUDA for sm_100a) in-tree with nvcc, and the binding's _calls.so with gcc.
+"""Builds libisopo.so (hand-written CUDA for sm_100a) in-tree with nvcc, and the binding's _calls module with gcc where Python's
+headers are there (without it the binding marshals through ctypes).
 
 Usage: python -m paper_2512_23353_b200.build [--force] [--debug] [-v]
 
@@ -21,7 +22,9 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 LIB_PATH = os.path.join(PKG_DIR, "libisopo.so")
 DEBUG_LIB_PATH = os.path.join(PKG_DIR, "libisopo_debug.so")
-CALLS_PATH = os.path.join(PKG_DIR, "_calls.so")  # the binding's native marshalling (csrc/py_calls.c)
+# the binding's native marshalling (csrc/py_calls.c), named for the interpreter that it is built for
+CALLS_PATH = os.path.join(PKG_DIR, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+CALLS_SRC = os.path.join(CSRC, "py_calls.c")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -34,9 +37,13 @@ def _sources():
     return sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
 
 
-def _deps_mtime():
+def _deps():
     paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "isopo.h"), __file__]
-    return max(os.path.getmtime(p) for p in paths)
+    return [p for p in paths if p != CALLS_SRC]
+
+
+def _deps_mtime():
+    return max(os.path.getmtime(p) for p in _deps())
 
 
 def _compile(src, verbose, debug):
@@ -51,14 +58,17 @@ def _compile(src, verbose, debug):
 
 
 def _build_calls(force):
-    src = os.path.join(CSRC, "py_calls.c")
-    if not force and os.path.exists(CALLS_PATH) and os.path.getmtime(CALLS_PATH) >= max(
-            os.path.getmtime(p) for p in (src, os.path.join(ROOT, "include", "isopo.h"), __file__)):
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        sys.stderr.write("Python.h not found: no _calls module, the binding marshals through ctypes\n")
         return
-    r = subprocess.run(["gcc", "-O2", "-std=gnu11", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I",
-                        os.path.join(ROOT, "include"), src, "-o", CALLS_PATH], capture_output=True, text=True)
+    if not force and os.path.exists(CALLS_PATH) and os.path.getmtime(CALLS_PATH) >= max(
+            os.path.getmtime(p) for p in (CALLS_SRC, os.path.join(ROOT, "include", "isopo.h"), __file__)):
+        return
+    r = subprocess.run(["gcc", "-O2", "-std=gnu11", "-Wall", "-shared", "-fPIC", "-I", include, "-I", os.path.join(ROOT, "include"),
+                        CALLS_SRC, "-o", CALLS_PATH], capture_output=True, text=True)
     if r.returncode != 0:
-        raise RuntimeError(f"gcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+        raise RuntimeError(f"gcc failed for {CALLS_SRC}:\n{r.stdout}\n{r.stderr}")
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:

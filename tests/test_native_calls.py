@@ -1,11 +1,17 @@
 """Native marshalling of the binding's calls: it takes an argument exactly as it stands or leaves the call to the checks in
 binding.py (None).  On the CPU the tensors stop it at `is_cuda` or the library at its argument checks."""
 
+import os
+import subprocess
+import sys
+import sysconfig
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2512_23353_b200 import binding as b
+from paper_2512_23353_b200 import build
 
 OFF = np.array([0, 2, 5], dtype=np.int64)
 
@@ -62,3 +68,36 @@ def test_trailing_dimensions_of_one_are_taken(monkeypatch):
     assert b._calls.weight_grad(*a) is None
     with pytest.raises(b.IsopoError, match="ISOPO_ERR_INVALID_ARG"):  # the beta, not the shapes
         b.isopo_weight_grad(*a)
+
+
+def test_without_the_native_module_calls_go_through_ctypes():
+    """A machine without Python's headers, or another interpreter than the one the module was built for."""
+    code = """if True:
+        import sys
+        sys.modules["paper_2512_23353_b200._calls"] = None  # as if there were no such file
+        import numpy as np, torch
+        from paper_2512_23353_b200 import binding as b
+        assert b._calls is b._NoCalls
+        b._stream = lambda: 0
+        K, A, i, off = torch.zeros(4), torch.zeros(2), torch.zeros(1, dtype=torch.int32), np.array([0, 2, 5])
+        ws = torch.zeros(0, dtype=torch.uint8)
+        for call in (lambda: b.isopo_weight_grad(torch.zeros(5, 8), torch.zeros(5, 6), A, off, torch.zeros(6, 8), ws, i, 1, 0.5),
+                     lambda: b.isopo_transform_advantages(K, A, b.VAR_NORMALISED, -1.0, A, i),
+                     lambda: b.isopo_transform_advantages_rel(K, A, b.VAR_NORMALISED, -1.0, torch.zeros(4), A, i)):
+            try:
+                call()
+            except b.IsopoError as e:
+                assert e.status == b.ERR_INVALID_ARG
+            else:
+                raise SystemExit("the library was not reached")
+        print("through ctypes")
+    """
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True)
+    assert r.returncode == 0 and "through ctypes" in r.stdout, r.stderr
+
+
+def test_module_is_named_for_its_interpreter_and_rebuilt_by_itself():
+    assert build.CALLS_PATH.endswith("_calls" + sysconfig.get_config_var("EXT_SUFFIX")) and os.path.exists(build.CALLS_PATH)
+    assert b._calls.__file__ == build.CALLS_PATH
+    assert not any(p.endswith("py_calls.c") for p in build._deps())  # an edit there leaves the CUDA objects alone
