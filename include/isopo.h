@@ -283,14 +283,14 @@ ISOPO_API isopo_status isopo_transform_advantages_batched(int n_layers, const fl
  *
  * Where no direction is left out and K + lambda I is well conditioned (below 1e6), the eigenvalues come from a float64
  * tridiagonalisation and c from a Cholesky solve beside it: 0.4 ms at B = 256.  Otherwise K is diagonalised by one-sided
- * Jacobi rotations in float32 with float64 inner products, a cluster of eight CTAs per K: milliseconds; its float32
+ * Jacobi rotations in float32 with float64 inner products, a cluster of eight CTAs per K that runs beside them: 8 ms; its float32
  * eigenbasis limits the coefficients to a relative error of about 1e-7 * cond(K + lambda I) (kept range), the
  * eigenvalues to ~1e-6 of the largest.
  *
  *   K            dev, float32 [B, B] row-major, symmetric (as written by isopo_layer_gram); B <= 256
  *   A            dev, float32 [B]
  *   lambda       >= 0;   rel_cutoff in [0, 1)
- *   coeffs       dev, float32 [B], overwritten
+ *   coeffs       dev, float32 [B], overwritten; may be the array A itself
  *   eigenvalues  dev, float32 [B], from the largest down; may be NULL
  *   ws           dev, isopo_spectral_workspace_bytes() bytes, 16-byte aligned; contents destroyed
  * If the rotations have not died out after 30 sweeps, *info = ISOPO_INFO_NO_CONVERGENCE | sweeps

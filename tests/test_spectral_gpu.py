@@ -92,6 +92,38 @@ def test_coefficients_over_the_advantages(b, B, lam_rel, cutoff):
     assert int(info.item()) == 0 and bool(torch.isfinite(c).all()) and torch.equal(A, c)
 
 
+def test_which_route_answers_does_not_depend_on_which_ends_first(b):
+    """The rotations start before the other route's verdict is there and are left when it is: small K, where either may end
+    first, K that rotations diagonalise in one sweep, and calls back to back on one workspace, which must not see each other."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    ws = torch.empty(b.lib.isopo_spectral_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for B in (1, 2, 3, 7, 32, 65, 256):
+        J = torch.randn(B, 4 * B, device="cuda", generator=g)
+        full, low = J @ J.T, J[:, :max(1, B // 2)] @ J[:, :max(1, B // 2)].T
+        diag = torch.diag(torch.arange(1.0, B + 1, device="cuda"))
+        A = torch.randn(B, device="cuda", generator=g)
+        calls = [(K, cut) for K in (full, low, diag) for cut in (0.0, 1e-3, 0.3)]
+        runs = []
+        for _ in range(3):
+            outs = [(torch.empty(B, device="cuda"), torch.empty(B, device="cuda")) for _ in calls]
+            for (K, cut), (c, e) in zip(calls, outs):
+                b.isopo_transform_spectral(K, A, 0.5, c, info, rel_cutoff=cut, eigenvalues=e, ws=ws)
+            runs.append(outs)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        for outs in runs[1:]:
+            for (c, e), (c0, e0) in zip(outs, runs[0]):
+                assert torch.equal(c, c0) and torch.equal(e, e0)
+        for (K, cut), (c, e) in zip(calls, runs[0]):
+            K64 = K.double().cpu().numpy()
+            c_o, D_o = orc.spectral_coefficients(K64, A.double().cpu().numpy(), 0.5, cut)
+            assert np.max(np.abs(e.cpu().numpy() - D_o)) <= 2e-6 * max(D_o[0], 1e-30) * max(1.0, np.sqrt(B) / 4)
+            if np.min(np.abs(D_o - cut * D_o[0])) > 1e-4 * D_o[0]:  # no direction at the cut-off itself
+                assert rel_fro(c.cpu().numpy(), c_o) <= 1e-5 + 1e-6 * D_o[0] / 0.5
+
+
 def test_time_at_full_size_and_argument_checks(b, capsys):
     K = _gram(256, 3, 1)
     Kd = torch.from_numpy(K).cuda()
