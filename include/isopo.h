@@ -415,7 +415,8 @@ ISOPO_API isopo_status isopo_layer_gram_static(const void* X, const void* dY, is
  * second kernel adds the partials in a fixed order: K, the coefficients and dW of that route are
  * then bit-identical from run to run.  The switch is process-wide and changes
  * isopo_workspace_bytes(..., MATERIALISE) (160 * B * B * 4 more bytes for bf16): set it before
- * sizing workspaces.  The GRAM route and the GEMM-route weight gradient keep their float atomics.
+ * sizing workspaces.  The GRAM route and the GEMM-route weight gradient keep their float atomics.  The
+ * ISOPO_F32 MATERIALISE route adds in a fixed order always.
  *
  * isopo_debug_build() is 1 when the library was compiled with -DISOPO_DEBUG (libisopo_debug.so): every
  * data-dependent index of the kernels is then range-checked before use, a violation skips the access

@@ -89,7 +89,8 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   L.off_tokseq = p;
   p = align_up(p + sizeof(int32_t) * (size_t)T, 1024);
   L.off_kacc = p;
-  if (dtype == ISOPO_F32) p = align_up(p + sizeof(double) * ((size_t)B * (size_t)B + 1), 1024);
+  if (dtype == ISOPO_F32)
+    p = align_up(p + (resolved == ISOPO_PATH_MATERIALISE ? sizeof(uint32_t) : sizeof(double) * (size_t)B * (size_t)B), 1024);
   L.off_scaled = p;
   if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM)
     p = align_up(p + (size_t)2 * (size_t)T * (size_t)std::min(d_in, d_out), 1024);
@@ -104,9 +105,10 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
       p = align_up(p + sizeof(float) * (size_t)kNtkMaxPartials * (size_t)B * (size_t)B, 1024);
   } else {
     L.tiles_m = L.tiles_n = 0;
-    L.off_kpart = p;
     L.n_pad = ((int64_t)d_in * d_out + 3) / 4 * 4;
     if (resolved == ISOPO_PATH_MATERIALISE) p = align_up(p + (size_t)4 * (size_t)B * (size_t)L.n_pad, 1024);
+    L.off_kpart = p;
+    if (resolved == ISOPO_PATH_MATERIALISE) p = align_up(p + f32_ntk_part_bytes(L.n_pad, B), 1024);
   }
   L.total = p;
   return L;
@@ -271,14 +273,14 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     if (s != ISOPO_OK) return s;
     return bf16_ntk(G, L, B, K, head, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
   }
-  double* kacc = (double*)(w + L.off_kacc);
   if (dtype == ISOPO_F32 && rp == ISOPO_PATH_MATERIALISE) {
     float* G = (float*)(w + L.off_G);
-    uint32_t* done = (uint32_t*)(kacc + (size_t)B * B);
-    s = f32_seq_grad((const float*)X, (const float*)dY, d_in, d_out, seq_offsets_host, off_dev, B, G, L.n_pad, kacc, done,
+    uint32_t* done = (uint32_t*)(w + L.off_kacc);
+    s = f32_seq_grad((const float*)X, (const float*)dY, d_in, d_out, seq_offsets_host, off_dev, B, G, L.n_pad, done,
                      make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host), tag_dev, st);
-    return s != ISOPO_OK ? s : f32_ntk(G, L.n_pad, B, kacc, done, K, st);
+    return s != ISOPO_OK ? s : f32_ntk(G, L.n_pad, B, (double*)(w + L.off_kpart), done, K, st);
   }
+  double* kacc = (double*)(w + L.off_kacc);
   const int64_t bb = (int64_t)B * B;
   s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, dtype == ISOPO_F32 ? Clear{{(float*)kacc}, {2 * bb}} : Clear{{K}, {bb}}, st);
   if (s != ISOPO_OK) return s;

@@ -144,10 +144,10 @@ struct WsLayout {
   size_t off_aux;      // float scales[B] | float kdiag[B]  (bf16 materialised path, split store)
   size_t off_offsets;  // int64 [B+1]
   size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here
-  size_t off_kacc;     // float64 [B*B], uint32 (float32 path: K accumulators, CTAs of the K pass that are done)
+  size_t off_kacc;     // float32 path: float64 [B*B] K accumulators (Gram), uint32 CTAs of the K pass that are done (materialised)
   size_t off_scaled;   // bf16 [T, min(d_in, d_out)]  (bf16 Gram path: the pre-scaled operand of the weight-gradient GEMM)
   size_t off_G;        // stored gradients (materialised path only)
-  size_t off_kpart;    // per-CTA partial K (bf16 materialised path in deterministic mode only)
+  size_t off_kpart;    // per-CTA partial K (materialised path; bf16: in deterministic mode only)
   size_t total;
   int tiles_m, tiles_n;  // bf16 materialised layout: tiles per gradient
   int64_t n_pad;         // elements per stored gradient (row stride of G_flat)
@@ -249,11 +249,12 @@ __device__ __forceinline__ bool ws_tag_matches(const WsTag* __restrict__ have, c
 }
 
 // float32 path.  gstride: floats between the stored gradients of two sequences (WsLayout::n_pad, a multiple of 4)
-// f32_seq_grad also leaves the tag and clears kacc [B * B] and `done`, which f32_ntk adds into
+// f32_seq_grad also leaves the tag and clears `done`, which f32_ntk counts in
 isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
-                          int B, float* G, int64_t gstride, double* kacc, uint32_t* done, const WsTag& tag, WsTag* tag_dev,
-                          cudaStream_t st);
-isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, cudaStream_t st);
+                          int B, float* G, int64_t gstride, uint32_t* done, const WsTag& tag, WsTag* tag_dev, cudaStream_t st);
+// part: f32_ntk_part_bytes of scratch
+size_t f32_ntk_part_bytes(int64_t gstride, int B);
+isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint32_t* done, float* K, cudaStream_t st);
 // M^T [n_samples, B] += of the sampled rows a0, g0
 isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
                          int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st);

@@ -203,8 +203,8 @@ struct TokenGemm {
 template <int kTile, int kT> using SeqGemm = TokenGemm<kTile, kT, 8, 4>;
 template <int kTile, int kT> using SlabGemm = TokenGemm<kTile, kT, 16, 3>;
 
-// G_i = dY_i^T X_i, one (tile, sequence) per CTA.  The launch also leaves the workspace tag and clears the accumulators
-// that the K pass behind it adds into.  Offsets come as kernel arguments when they fit (kArgOff), else from `off`.
+// G_i = dY_i^T X_i, one (tile, sequence) per CTA.  The launch also leaves the workspace tag and clears the K pass's count of
+// finished CTAs.  Offsets come as kernel arguments when they fit (kArgOff), else from `off`.
 struct F32StoredArgs {
   const float* X;
   const float* dY;
@@ -212,7 +212,6 @@ struct F32StoredArgs {
   int64_t gstride;   // floats between the gradients of two sequences (a multiple of 4)
   const int64_t* off;
   float* G;
-  double* kacc;      // [B * B]
   uint32_t* done;    // CTAs of the K pass that have finished
   WsTag tag;
   WsTag* tag_dev;
@@ -228,8 +227,6 @@ k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ 
   extern __shared__ __align__(16) float smem[];
   const int i = blockIdx.z, m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t cta = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  const int64_t threads = (int64_t)gridDim.x * gridDim.y * gridDim.z * blockDim.x;
-  for (int64_t e = cta * blockDim.x + threadIdx.x; e < (int64_t)a.B * a.B; e += threads) a.kacc[e] = 0.0;
   if (cta == 0) {
     if (threadIdx.x < 8) a.tag_dev->v[threadIdx.x] = a.tag.v[threadIdx.x];
     if (threadIdx.x == 8) *a.done = 0u;
@@ -296,8 +293,10 @@ k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int
 // accumulated in float64).  A CTA takes every gridDim.y-th 64-column chunk of a pair of row blocks of G_flat, staged by
 // cp.async as floats; its four warps share the columns of a chunk, each holding the whole block of K in registers, so a
 // fragment is read and widened once for many MMAs.  kDiag: 8 kNB rows against themselves, only the 16 x 8 blocks on and
-// above the diagonal; otherwise 16 kMA rows against 8 kNB others.  The CTAs meet in kacc by float64 atomics; with one
-// row block the last CTA to finish rounds K to float32.
+// above the diagonal; otherwise 16 kMA rows against 8 kNB others.  Every CTA stores its sums, and they are added in the order
+// of the chunks (k_f32_ntk_finish, or the last CTA to finish where there are few): K is the same to the bit from run to run,
+// which float64 atomics would not leave it where products cancel.  They were slower, too (G and K, atomics / this: 64 sequences
+// of 896 x 896 211 / 194 us, 64 of 64 x 64 31.9 / 22.3, 16 of 896 x 896 64.6 / 45.6, 256 of 512 x 512 974 / 916).
 // Bound by the float64 pipe.  One CTA per pair (i, j) with scalar float64 additions re-read G B / 2 times: 1384 us at 64
 // sequences of an 896 x 896 layer against 146 us, 3694 against 500 us at 256 sequences of 300 x 500.  One CTA of eight
 // warps per SM instead of two of four: 162 and 715 us.  Few sequences leave the pass to HBM and need more loads in flight: kPerSm.
@@ -315,12 +314,64 @@ __device__ __forceinline__ void dmma16x8x8(double (&c)[4], double a0, double a1,
       : "d"(a0), "d"(a1), "d"(a2), "d"(a3), "d"(b0), "d"(b1));
 }
 
+// 16 x 8 blocks of K in a warp's registers
+constexpr int ntk_blocks(int ma, int nb, bool diag) { return diag ? ma * (ma + 1) : ma * nb; }
+// The sums of one K pass: pairs x slabs CTAs, `doubles` of each, element (blk * 4 + q) * 32 + lane as the registers have them.
+struct NtkParts {
+  int64_t pairs, slabs;
+  int ma, nb, doubles;
+  bool diag;
+  __host__ __device__ int64_t total() const { return pairs * slabs * doubles; }
+};
+// First row of the row blocks of a pair: diagonal blocks in order; otherwise pairs I < J of 64-row blocks, I in two halves of
+// 32 rows.
+__device__ __forceinline__ void ntk_pair_rows(bool diag, int64_t pair, int& i0, int& j0) {
+  if (diag) {
+    i0 = j0 = (int)pair * kNtkRows;
+    return;
+  }
+  int J = 1, r = (int)(pair >> 1);
+  while (r >= J) { r -= J; ++J; }
+  i0 = r * kNtkRows + (int)(pair & 1) * 32;
+  j0 = J * kNtkRows;
+}
+// Adds the slabs' shares of element e of a pair's block, shares first .. last - 1 in order.
+__device__ __forceinline__ double ntk_sum(const double* part, int64_t stride, int first, int last) {
+  double s = 0.0;
+  int k = first;
+  for (; k + 8 <= last; k += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (k + u) * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  for (; k < last; ++k) s += __ldcg(part + k * stride);
+  return s;
+}
+// K[i][j] and K[j][i] of element e of a pair's block
+__device__ __forceinline__ void ntk_write(const NtkParts& P, int i0, int j0, int e, int B, float* __restrict__ K, double v) {
+  const int lane = e & 31, q = (e >> 5) & 3;
+  int p = 0, n = e >> 7;
+  if (P.diag) {
+    while (n >= P.nb - 2 * p) { n -= P.nb - 2 * p; ++p; }
+    n += 2 * p;
+  } else {
+    p = n / P.nb;
+    n -= p * P.nb;
+  }
+  const int i = i0 + p * 16 + (lane >> 2) + (q >> 1) * 8, j = j0 + n * 8 + 2 * (lane & 3) + (q & 1);
+  if (i > j || j >= B) return;
+  K[(size_t)i * B + j] = (float)v;
+  K[(size_t)j * B + i] = (float)v;
+}
+
 template <int kMA, int kNB, bool kDiag>
 struct NtkShape {
   static constexpr int kRowsStaged = kDiag ? 8 * kNB : 16 * kMA + 8 * kNB;
   static constexpr int kStageFloats = kRowsStaged * kNtkPitch;
   static constexpr int kSmemStages = kNtkStages * kStageFloats * 4;
-  static constexpr int kBlocks = kDiag ? kMA * (kMA + 1) : kMA * kNB;  // 16 x 8 blocks of K in a warp's registers
+  static constexpr int kBlocks = ntk_blocks(kMA, kNB, kDiag);
   static constexpr int kSmemRed = 2 * kBlocks * 128 * 8;               // two warps' blocks
   static constexpr int kSmem = kSmemStages > kSmemRed ? kSmemStages : kSmemRed;
   static constexpr int kPerSm = kNB == 2 ? 8 : kNB == 4 ? 4 : 2;       // resident CTAs per SM
@@ -328,21 +379,14 @@ struct NtkShape {
 
 template <int kMA, int kNB, bool kDiag>
 __global__ void __launch_bounds__(kNtkThreads, NtkShape<kMA, kNB, kDiag>::kPerSm)
-k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uint32_t* done, float* __restrict__ K) {
+k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_constant__ NtkParts parts, double* part, uint32_t* done,
+          float* __restrict__ K) {
   pdl_wait();
   typedef NtkShape<kMA, kNB, kDiag> S;
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  // the pair of row blocks: diagonal blocks in order; otherwise pairs I < J of 64-row blocks, I in two halves of 32 rows
   int i0, j0;
-  if (kDiag) {
-    i0 = j0 = blockIdx.x * kNtkRows;
-  } else {
-    int J = 1, r = blockIdx.x >> 1;
-    while (r >= J) { r -= J; ++J; }
-    i0 = r * kNtkRows + (blockIdx.x & 1) * 32;
-    j0 = J * kNtkRows;
-  }
+  ntk_pair_rows(kDiag, blockIdx.x, i0, j0);
   const int64_t nchunks = (gstride + kNtkKC - 1) / kNtkKC;
   auto fetch = [&](int64_t ch, int stage) {
     if (ch < nchunks) {
@@ -400,7 +444,7 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uin
     }
   }
   cp_async_wait<0>();
-  // the warps' shares meet in shared memory (4 -> 2 -> 1), the CTAs' in kacc
+  // the warps' shares meet in shared memory (4 -> 2 -> 1)
   double2* red = reinterpret_cast<double2*>(smem);
   for (int half = 2; half >= 1; half >>= 1) {
     __syncthreads();
@@ -427,17 +471,15 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uin
     }
   }
   if (warp == 0) {
+    double* mine = part + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * parts.doubles + lane;
 #pragma unroll
     for (int p = 0; p < kMA; ++p)
 #pragma unroll
       for (int n = kDiag ? 2 * p : 0; n < kNB; ++n)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = i0 + p * 16 + g + (q >> 1) * 8, j = j0 + n * 8 + 2 * t + (q & 1);
-          if (i <= j && j < B) atomicAdd(&kacc[(size_t)i * B + j], acc[p][n][q]);
-        }
+        for (int q = 0; q < 4; ++q, mine += 32) *mine = acc[p][n][q];
   }
-  if (kDiag && gridDim.x == 1) {
+  if (done) {  // one pair, few shares
     __shared__ bool last;
     __threadfence();
     __syncthreads();
@@ -445,11 +487,41 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, double* kacc, uin
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int e = tid; e < B * B; e += kNtkThreads) {
-      const int i = e / B, j = e % B;
-      K[e] = (float)__ldcg(&kacc[i <= j ? (size_t)i * B + j : (size_t)j * B + i]);
-    }
+    for (int e = tid; e < parts.doubles; e += kNtkThreads)
+      ntk_write(parts, i0, j0, e, B, K, ntk_sum(part + e, parts.doubles, 0, gridDim.y));
   }
+}
+
+// K from the shares of a launch on the diagonal blocks and, with more than one of them, of one on the others.  The shares of an
+// element are added in kRuns runs, a thread each: eight where they are many and a single thread's loads would be a long chain,
+// one where they are few.
+template <int kRuns>
+__global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ NtkParts diag, const __grid_constant__ NtkParts rest,
+                                                        const double* __restrict__ part, int B, float* __restrict__ K) {
+  pdl_wait();
+  constexpr int kElems = 256 / kRuns;  // of a block
+  __shared__ double sums[kRuns][kElems];
+  const int t = threadIdx.x % kElems, run = threadIdx.x / kElems;
+  const int64_t diag_blocks = diag.pairs * diag.doubles / kElems;
+  const bool on_diag = blockIdx.x < diag_blocks;
+  const NtkParts& P = on_diag ? diag : rest;
+  const int64_t x = (on_diag ? blockIdx.x : blockIdx.x - diag_blocks) * kElems;
+  const int64_t pair = x / P.doubles;
+  const int e = (int)(x - pair * P.doubles) + t;
+  const double* src = part + (on_diag ? 0 : diag.total()) + pair * P.slabs * P.doubles + e;
+  const int per = (int)((P.slabs + kRuns - 1) / kRuns), first = min((int)P.slabs, run * per);
+  double s = ntk_sum(src, P.doubles, first, min((int)P.slabs, first + per));
+  if (kRuns > 1) {
+    sums[run][t] = s;
+    __syncthreads();
+    if (run != 0) return;
+    s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kRuns; ++w) s += sums[w][t];
+  }
+  int i0, j0;
+  ntk_pair_rows(P.diag, pair, i0, j0);
+  ntk_write(P, i0, j0, e, B, K, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -731,9 +803,8 @@ static bool f32_wide_tiles(int d_in, int d_out, int64_t copies) {
 }
 
 isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
-                          int B, float* G, int64_t gstride, double* kacc, uint32_t* done, const WsTag& tag, WsTag* tag_dev,
-                          cudaStream_t st) {
-  F32StoredArgs a{X, dY, d_in, d_out, B, gstride, off_dev, G, kacc, done, tag, tag_dev};
+                          int B, float* G, int64_t gstride, uint32_t* done, const WsTag& tag, WsTag* tag_dev, cudaStream_t st) {
+  F32StoredArgs a{X, dY, d_in, d_out, B, gstride, off_dev, G, done, tag, tag_dev};
   const bool wide = f32_wide_tiles(d_in, d_out, B);
   if (B + 1 <= kArgChunk) {
     OffsetParam<true> o;
@@ -747,17 +818,36 @@ isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, 
 }
 
 template <int kMA, int kNB, bool kDiag>
-static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, int64_t pairs,
-                                   cudaStream_t st) {
-  constexpr int smem = NtkShape<kMA, kNB, kDiag>::kSmem;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_ntk<kMA, kNB, kDiag>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+static NtkParts ntk_parts(int64_t gstride, int64_t pairs) {
   // every SM full over all pairs; at least eight chunks each, or the reduction outweighs the stream
   constexpr int64_t ctas = 148 * NtkShape<kMA, kNB, kDiag>::kPerSm;
   const int64_t chunks = (gstride + kNtkKC - 1) / kNtkKC;
   const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + 7) / 8));
+  return NtkParts{pairs, slabs, kMA, kNB, NtkShape<kMA, kNB, kDiag>::kBlocks * 128, kDiag};
+}
+// The launches of the K pass of B gradients: diagonal blocks, the others (no pairs: none).
+static void ntk_plan(int64_t gstride, int B, NtkParts* diag, NtkParts* rest) {
+  const int64_t nb = (B + kNtkRows - 1) / kNtkRows;
+  *diag = B <= 16   ? ntk_parts<1, 2, true>(gstride, 1)
+          : B <= 32 ? ntk_parts<2, 4, true>(gstride, 1)
+                    : ntk_parts<4, 8, true>(gstride, nb);
+  *rest = nb == 1 ? NtkParts{} : ntk_parts<2, 8, false>(gstride, nb * (nb - 1));  // two halves of nb (nb - 1) / 2 pairs
+}
+size_t f32_ntk_part_bytes(int64_t gstride, int B) {
+  NtkParts diag, rest;
+  ntk_plan(gstride, B, &diag, &rest);
+  return sizeof(double) * (size_t)(diag.total() + rest.total());
+}
+
+template <int kMA, int kNB, bool kDiag>
+static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, const NtkParts& parts, double* part, uint32_t* done,
+                                   float* K, cudaStream_t st) {
+  constexpr int smem = NtkShape<kMA, kNB, kDiag>::kSmem;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_ntk<kMA, kNB, kDiag>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   {
     LaunchScope scope(kIdF32Ntk, st);
-    launch(k_f32_ntk<kMA, kNB, kDiag>, dim3((unsigned)pairs, (unsigned)slabs), kNtkThreads, smem, st, G, gstride, B, kacc, done, K);
+    launch(k_f32_ntk<kMA, kNB, kDiag>, dim3((unsigned)parts.pairs, (unsigned)parts.slabs), kNtkThreads, smem, st, G, gstride, B, parts,
+           part, done, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -772,14 +862,28 @@ static isopo_status launch_f32_finish(const double* kacc, int B, float* K, cudaS
   return ISOPO_OK;
 }
 
-isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* kacc, uint32_t* done, float* K, cudaStream_t st) {
-  if (B <= 16) return launch_f32_ntk<1, 2, true>(G, gstride, B, kacc, done, K, 1, st);
-  if (B <= 32) return launch_f32_ntk<2, 4, true>(G, gstride, B, kacc, done, K, 1, st);
-  const int64_t nb = (B + kNtkRows - 1) / kNtkRows;
-  isopo_status s = launch_f32_ntk<4, 8, true>(G, gstride, B, kacc, done, K, nb, st);
-  if (s != ISOPO_OK || nb == 1) return s;
-  s = launch_f32_ntk<2, 8, false>(G, gstride, B, kacc, done, K, nb * (nb - 1), st);  // two halves of nb (nb - 1) / 2 pairs
-  return s != ISOPO_OK ? s : launch_f32_finish(kacc, B, K, st);
+isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint32_t* done, float* K, cudaStream_t st) {
+  NtkParts diag, rest;
+  ntk_plan(gstride, B, &diag, &rest);
+  // the last CTA adds the shares up itself where it has 64 or fewer to load per thread: a launch less
+  const bool by_last = diag.pairs == 1 && diag.total() <= 64 * kNtkThreads;
+  if (!by_last) done = nullptr;
+  const isopo_status s = B <= 16   ? launch_f32_ntk<1, 2, true>(G, gstride, B, diag, part, done, K, st)
+                         : B <= 32 ? launch_f32_ntk<2, 4, true>(G, gstride, B, diag, part, done, K, st)
+                                   : launch_f32_ntk<4, 8, true>(G, gstride, B, diag, part, done, K, st);
+  if (s != ISOPO_OK || by_last) return s;
+  if (rest.pairs > 0) {
+    const isopo_status r = launch_f32_ntk<2, 8, false>(G, gstride, B, rest, part + diag.total(), nullptr, K, st);
+    if (r != ISOPO_OK) return r;
+  }
+  {
+    LaunchScope scope(kIdMirror, st);
+    const bool many = std::max(diag.slabs, rest.slabs) > 16;
+    const int64_t elems = diag.pairs * diag.doubles + rest.pairs * rest.doubles;  // a multiple of 256
+    launch(many ? k_f32_ntk_finish<8> : k_f32_ntk_finish<1>, (unsigned)(elems / (many ? 32 : 256)), 256, 0, st, diag, rest, part, B, K);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
 }
 
 // Tokens per tile: 64, or 32 where `tiles` of 64 would not give every SM two CTAs.

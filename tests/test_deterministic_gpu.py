@@ -47,3 +47,25 @@ def test_two_runs_are_bit_identical(b, B, d_in, d_out):
     finally:
         b.isopo_set_deterministic(False)
     assert b.isopo_workspace_bytes(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE) == plain_bytes
+
+
+@pytest.mark.parametrize("B,d", [(6, 512), (8, 64), (30, 256), (64, 512), (130, 192)])  # every K kernel; its last CTA and its finish
+def test_float32_stored_route_needs_no_mode(b, B, d):
+    """K of float32 gradients is added up in a fixed order anyway: the same to the bit where products cancel and the last bits of
+    a sum are all that is left of it."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+    h = torch.randn(B, d // 2, device="cuda", generator=g)
+    sign = 1.0 - 2.0 * (torch.arange(B, device="cuda") % 2).float()
+    X = torch.cat([h, sign[:, None] * h], 1).contiguous()  # x_i . x_j = 0 for i, j of different parity, as a sum of large terms
+    dY = torch.randn(B, d, device="cuda", generator=g).abs()
+    off, info = np.arange(B + 1), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = b.alloc_workspace(b.F32, B, d, d, B, b.PATH_MATERIALISE)
+    Ks = [torch.empty(B, B, device="cuda") for _ in range(20)]
+    for K in Ks:
+        b.isopo_layer_gram(X, dY, off, K, ws, info, b.PATH_MATERIALISE)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0 and torch.equal(Ks[0], Ks[0].T)
+    assert sum(not torch.equal(K, Ks[0]) for K in Ks) == 0
+    X64, dY64 = X.double().cpu().numpy(), dY.double().cpu().numpy()
+    assert rel_fro(Ks[0].cpu().numpy(), (X64 @ X64.T) * (dY64 @ dY64.T)) <= 1e-5
