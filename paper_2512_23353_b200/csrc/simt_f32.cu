@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "isopo_internal.h"
+#include "slab_plan.h"
 
 namespace isopo {
 
@@ -932,7 +933,8 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
   return ISOPO_OK;
 }
 
-constexpr int64_t kSlabOverhead = 64;  // tokens
+// What a CTA spends on filling its pipeline and adding its tile, in stages of 16 tokens.
+constexpr int64_t kSlabOverhead = 4;
 template <int kTile, int kT>
 static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out,
                                            const float* tokscale, float* dW, cudaStream_t st) {
@@ -941,20 +943,22 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
   if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
   const auto kernel = k_f32_weight_grad<kTile, kT>;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
-  int dev = 0, sms = 0, per_sm = 0;
+  int dev = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
-  ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
-  // Token slabs, each a multiple of the staging depth: the count whose waves take least, a wave costing its slab and what a CTA
-  // spends on filling its pipeline and adding its tile.  "Four CTAs per SM" instead left the last wave nearly empty: 896 x 896,
-  // 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 -> 10.1 (this alone).
-  const int64_t tiles = (int64_t)gx * gy, slots = (int64_t)sms * std::max(per_sm, 1), most = std::max<int64_t>(1, (T + 127) / 128);
-  int64_t slab = 0, best = INT64_MAX;
-  for (int64_t n = 1; n <= std::min<int64_t>(most, std::max<int64_t>(8, 8 * slots / tiles)); ++n) {
-    const int64_t len = ((T + n - 1) / n + 15) / 16 * 16, ctas = (T + len - 1) / len * tiles;
-    const int64_t cost = (ctas + slots - 1) / slots * (len + kSlabOverhead);
-    if (cost < best) { best = cost; slab = len; }
+  static int resident[64] = {};  // CTAs at one time
+  if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
+  if (resident[dev] == 0) {
+    int sms = 0, per_sm = 0;
+    ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
+    resident[dev] = sms * std::max(per_sm, 1);
   }
+  // Token slabs of whole stages, 128 tokens or more, up to eight waves (slab_plan.h).  "Four CTAs per SM" instead left the last
+  // wave nearly empty: 896 x 896, 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 ->
+  // 10.1 (this alone).
+  const int64_t tiles = (int64_t)gx * gy, slots = resident[dev];
+  const int64_t slab = 16 * plan_slab((T + 15) / 16, tiles, slots, kSlabOverhead,
+                                      std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles)));
   const int64_t splits = (T + slab - 1) / slab;
   if (splits > 65535) return ISOPO_ERR_UNSUPPORTED;
   {
