@@ -20,6 +20,7 @@
 //
 // The stored layout of G (pieces of 32 rows x 8 columns, sequence-minor) is described in
 // tc_common.cuh; one epilogue warp writes one 512-byte piece per store instruction.
+#include "slab_plan.h"
 #include "tc_common.cuh"
 
 namespace isopo {
@@ -385,18 +386,14 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   p.tiles_m = (d_out + kTileM - 1) / kTileM;
   p.tiles_n = (d_in + kTileN - 1) / kTileN;
   p.info = info; p.tokscale = tokscale; p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out;
-  // token slabs: the count (up to 64) whose rounds of (tile, slab) units take least, a round costing its slab plus what a
-  // unit spends on filling its pipeline and on adding its tile into dW, about 16 stages' worth.  Every slab is a multiple of
-  // 64 tokens.
+  // Token slabs of whole stages, 64 at most, or two rounds of (tile, slab) units while a slab has eight stages: a unit spends
+  // about 16 stages' worth on filling its pipeline and on adding its tile into dW, more the more units meet in a tile (16,000
+  // tokens, 256 x 128: 64 slabs 15.8 us, 125 slabs 18.6).  With 64 slabs whatever the tokens a layer of one tile had 64 CTAs:
+  // 300,000 tokens, 64 x 64 75 -> 38 us, 256 x 128 90 -> 55, 512 x 128 94 -> 85; 65,536 tokens, 64 x 64 22 -> 15.
   const long long tiles = (long long)p.tiles_m * p.tiles_n;
   const long long kblocks = (T + kKB - 1) / kKB;
-  long long nslabs = 1, best = -1;
-  for (long long n = 1; n <= std::min<long long>(64, kblocks); ++n) {
-    const long long per = (kblocks + n - 1) / n, rounds = (tiles * n + sms - 1) / sms, cost = rounds * (per + 16);
-    if (best < 0 || cost < best) { best = cost; nslabs = n; }
-  }
-  const long long kb_per = (kblocks + nslabs - 1) / nslabs;
-  nslabs = (kblocks + kb_per - 1) / kb_per;
+  const long long kb_per = plan_slab(kblocks, tiles, sms, 16, std::max<long long>(64, std::min((2ll * sms + tiles - 1) / tiles, kblocks / 8)));
+  const long long nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;
   p.nslabs = (int)nslabs;
   const int grid = (int)std::min<long long>(tiles * nslabs, sms);

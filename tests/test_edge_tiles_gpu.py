@@ -101,3 +101,18 @@ def test_plain_gemm_runs(b, lens, d_in, d_out):
     # dW = sum_i c_i G_i = (c_seq(t) dY)^T X, without materialising the G_i of 2100 sequences
     want = (np.repeat(to_f64(c), lens)[:, None] * to_f64(dY)).T @ to_f64(X)
     assert rel_fro(dW, want) <= 6e-3
+
+
+# few tiles and many tokens: as many slabs as CTAs, on both sides of eight stages per slab (64 tokens each), ragged ends
+@pytest.mark.parametrize("T,d_in,d_out", [(64 * 512 - 1, 64, 64), (64 * 512 + 1, 64, 64), (64 * 1184 + 17, 256, 128), (64 * 1300, 520, 40)])
+def test_many_slabs_of_one_tile(b, T, d_in, d_out):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    X = torch.randn(T, d_in, device="cuda", generator=g).to(torch.bfloat16)
+    dY = (0.1 * torch.randn(T, d_out, device="cuda", generator=g)).to(torch.bfloat16)
+    off = np.array([0, 1, 1000, T // 2 + 3, T - 65, T])
+    c = torch.randn(len(off) - 1, device="cuda", generator=g)
+    ws = b.alloc_workspace(b.BF16, T, d_in, d_out, len(off) - 1, b.PATH_GRAM)
+    dW = _weight_grad(b, X, dY, off, c, ws, torch.zeros(1, dtype=torch.int32, device="cuda"), b.PATH_GRAM)
+    scale = c.double().repeat_interleave(torch.from_numpy(np.diff(off)).cuda())
+    assert rel_fro(dW, ((scale[:, None] * dY.double()).T @ X.double()).cpu().numpy()) <= 6e-3
