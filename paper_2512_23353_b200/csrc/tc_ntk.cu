@@ -286,8 +286,10 @@ constexpr int kCombineInFlight = ISOPO_COMBINE_IN_FLIGHT;  // 16-byte loads a th
 // sequences) is the plain stream of a wide layer; a narrow layer has too few pieces to fill the machine that way and
 // splits the sequences instead (combine_slices below).  896 -> 128, one share against eight: 64 sequences 16.6 against
 // 11.5 us, 256 sequences 41 against 17 us.
-template <int kSlices>
-__global__ void __launch_bounds__(256, kSlices > 1 ? 4 : 1) k_bf16_combine(const uint4* __restrict__ G, long long nchunks /* n_pad / 8 */,
+// kMany: kCombineInFlight loads of a lane in flight and the remainder one by one, for long sums.  Otherwise eight, the
+// remainder together as well, and registers for twice the CTAs per SM, for short ones (kManySeqs).
+template <int kSlices, bool kMany>
+__global__ void __launch_bounds__(256, kMany ? 1 : 4) k_bf16_combine(const uint4* __restrict__ G, long long nchunks /* n_pad / 8 */,
                                                        int B, PieceGrid grid, int d_in, int d_out,
                                                        const float* __restrict__ coeffs, float* __restrict__ dW,
                                                        float beta, const WsTag* __restrict__ tag_dev, WsTag tag,
@@ -295,7 +297,8 @@ __global__ void __launch_bounds__(256, kSlices > 1 ? 4 : 1) k_bf16_combine(const
   pdl_wait();
   if (!ws_tag_matches(tag_dev, tag, info)) return;  // another layer's or microbatch's gradients: touch nothing
   constexpr int kPieces = 8 / kSlices;  // pieces a block works on at a time
-  constexpr int kF = kSlices > 1 ? 8 : kCombineInFlight;
+  constexpr int kF = kMany ? kCombineInFlight : 8;
+  static_assert(kSlices == 1 || !kMany, "a share is short");
   __shared__ float sc[256];
   __shared__ float4 part[kSlices > 1 ? 8 * 64 : 1];
   for (int i = threadIdx.x; i < B; i += blockDim.x) sc[i] = coeffs[i];
@@ -336,7 +339,15 @@ __global__ void __launch_bounds__(256, kSlices > 1 ? 4 : 1) k_bf16_combine(const
 #pragma unroll
         for (int u = 0; u < kF; ++u) add(v[u], sc[i + u]);
       }
-      for (; live && i < B; ++i) add(__ldcs(src + (size_t)i * stride), sc[i]);
+      if (kMany) {
+        for (; live && i < B; ++i) add(__ldcs(src + (size_t)i * stride), sc[i]);
+      } else if (live && i < B) {
+        uint4 v[kF];
+#pragma unroll
+        for (int u = 0; u < kF; ++u) v[u] = i + u < B ? __ldcs(src + (size_t)(i + u) * stride) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < kF; ++u) add(v[u], i + u < B ? sc[i + u] : 0.f);
+      }
     } else {
       // a share is a few loads long: all of them in flight at once, the remainder too
       for (int i = i0; i < i1; i += kF) {
@@ -382,6 +393,10 @@ inline int combine_slices(long long npieces, int B, int sms) {
   while (s < 8 && npieces * 2 * s <= 32ll * sms && B >= 16 * s) s *= 2;
   return s;
 }
+
+// Sequences from which on a whole sum is a long one.  1536 -> 4096, long / short form: 15 sequences 46.7 / 33.4 us, 60: 113 /
+// 111, 100: 177 / 181, 256: 463 / 467; 896 -> 4864: 15 sequences 36.1 / 25.2, 60: 83.2 / 77.5, 100: 125.9 / 124.5.
+constexpr int kManySeqs = 64;
 
 // Split store: dW = beta dW + sum_i (c_i / s_i) (hi_i + lo_i / 16).  One thread per PAIR of slots (two tile rows x 8
 // columns), so that every load is 16 bytes per plane: with one slot per thread the two planes cost twice the load
@@ -527,10 +542,10 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
       launch(k_e4m3_combine, grid, 256, 0, st, (const uint2*)G, chunks, B, pg, d_in, d_out, coeffs, fmt.scales, dW, beta,
                                            tag_dev, tag, info);
     else
-      launch((slices == 1   ? k_bf16_combine<1>
-       : slices == 2 ? k_bf16_combine<2>
-       : slices == 4 ? k_bf16_combine<4>
-                     : k_bf16_combine<8>), grid, 256, 0, st, (const uint4*)G, chunks, B, pg, d_in, d_out, coeffs, dW, beta,
+      launch((slices == 1   ? (B >= kManySeqs ? k_bf16_combine<1, true> : k_bf16_combine<1, false>)
+       : slices == 2 ? k_bf16_combine<2, false>
+       : slices == 4 ? k_bf16_combine<4, false>
+                     : k_bf16_combine<8, false>), grid, 256, 0, st, (const uint4*)G, chunks, B, pg, d_in, d_out, coeffs, dW, beta,
                                                                 tag_dev, tag, info);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());

@@ -70,8 +70,9 @@ def test_stand_alone_weight_gradient(b, d_in, d_out, lens):
     assert rel_fro(dW, orc.weight_gradient(G, to_f64(c))) <= 6e-3
 
 
-# shares of the sequences in the combine: one (too few sequences / too many pieces), two, four and eight, even and uneven
-@pytest.mark.parametrize("B,d_in,d_out", [(15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (128, 64, 48), (129, 64, 48), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
+# shares of the sequences in the combine: one (too few sequences / too many pieces), two, four and eight, even and uneven; one
+# share of fewer than 64 sequences and of more, whole groups of eight or sixteen and remainders
+@pytest.mark.parametrize("B,d_in,d_out", [(1, 72, 40), (8, 1024, 1000), (15, 1024, 1000), (63, 1536, 1024), (79, 1536, 1024), (15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (128, 64, 48), (129, 64, 48), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
 def test_combine_shares(b, B, d_in, d_out):
     X, dY, off, c, G = _problem(d_in, d_out, [2 + i % 3 for i in range(B)], B)
     ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE)
