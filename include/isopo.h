@@ -207,7 +207,8 @@ ISOPO_API isopo_status isopo_transform_advantages(const float* K, const float* A
 /*
  * isopo_transform_advantages_large: the interacting variant, (K + lambda I) c = A (Sec. 3 display; Alg. 2), for
  * up to ISOPO_MAX_LARGE_SEQS sequences.  Blocked Cholesky with float64-residual refinement; above 256 sequences its block
- * rows are dealt to a cluster of sixteen CTAs and meet in `workspace`.  K of more than
+ * rows are dealt to a cluster of sixteen CTAs and meet in `workspace` (0.35 ms at 1024).  A context with a part of the SMs may
+ * have no room for such a cluster: one CTA does it then (2.2 ms).  K of more than
  * 256 sequences comes from the GRAM path of isopo_layer_gram; the simple variants take any B in
  * isopo_transform_advantages.  A non-positive pivot k (1-based) is reported as *info = k, coeffs are then zero.
  *

@@ -45,10 +45,6 @@ __device__ __forceinline__ void st_async_f32x4(uint32_t addr, const float4& v, u
                : "memory");
 }
 
-template <int kC> __device__ __forceinline__ int cl_owner(int I) {
-  const int m = I % (2 * kC);
-  return m < kC ? m : 2 * kC - 1 - m;
-}
 constexpr int kMaxOwn = 2;  // block rows of a CTA: 32 / 16
 
 // Fixed part of the dynamic shared memory; the own blocks follow.

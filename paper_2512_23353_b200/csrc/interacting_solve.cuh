@@ -71,10 +71,17 @@ __device__ __forceinline__ float warp_column_sums(float (&r)[kNB]) {
   return r[0];
 }
 
+// Pointer types of the block helpers.  kShared: every block lies in this CTA's shared memory and has no other writer, so the
+// pointers may be restrict-qualified (4 % of the solve at 256 sequences).  Otherwise a block may be global memory that another
+// warp or SM wrote earlier in the same kernel: plain loads only, never the read-only path.
+template <bool kShared> struct BlkPtr { typedef float* __restrict__ rw; typedef const float* __restrict__ ro; };
+template <> struct BlkPtr<false> { typedef float* rw; typedef const float* ro; };
+
 // Factors the 32 x 32 diagonal block D (column-major, symmetric input) in place into its lower
 // Cholesky factor and writes 1 / L_kk to rd[k].  One warp.
 // Returns 0, or the 1-based local index of the first non-positive pivot.
-__device__ __noinline__ int warp_factor_diag(float* __restrict__ D, float* __restrict__ rd) {
+template <bool kShared = true>
+__device__ __noinline__ int warp_factor_diag(typename BlkPtr<kShared>::rw D, float* __restrict__ rd) {
   const int lane = threadIdx.x & 31;
   float r[kNB];
 #pragma unroll
@@ -102,7 +109,8 @@ __device__ __noinline__ int warp_factor_diag(float* __restrict__ D, float* __res
 
 // Inv = L^-1 (column-major) for the factored diagonal block D with rd[k] = 1 / L_kk.  One warp.
 // Column sweep: lane j solves L z = e_j; after step k, z[k] = Inv[k][j] is final.
-__device__ __noinline__ void warp_invert_factor(const float* __restrict__ D, const float* __restrict__ rd,
+template <bool kShared = true>
+__device__ __noinline__ void warp_invert_factor(typename BlkPtr<kShared>::ro D, const float* __restrict__ rd,
                                                 float* __restrict__ Inv) {
   const int lane = threadIdx.x & 31;
   float z[kNB];
@@ -120,7 +128,8 @@ __device__ __noinline__ void warp_invert_factor(const float* __restrict__ D, con
 
 // X L^T = A for one 32 x 32 block A (in place); lane owns a row.  L: factored diagonal block,
 // rd[k] = 1 / L_kk.  Column k of X is final after step k and is eliminated from the later columns.
-__device__ __noinline__ void warp_solve_panel(float* __restrict__ A, const float* __restrict__ L,
+template <bool kShared = true>
+__device__ __noinline__ void warp_solve_panel(typename BlkPtr<kShared>::rw A, typename BlkPtr<kShared>::ro L,
                                               const float* __restrict__ rd) {
   const int lane = threadIdx.x & 31;
   float a[kNB];
@@ -136,11 +145,7 @@ __device__ __noinline__ void warp_solve_panel(float* __restrict__ A, const float
   for (int c = 0; c < kNB; ++c) A[c * kNB + lane] = a[c];
 }
 
-// C -= A * Bm^T for 32 x 32 blocks (all column-major); lane computes a 4 x 8 sub-tile.  kShared: every block lies in this
-// CTA's shared memory and has no other writer, so the pointers may be restrict-qualified (4 % of the solve at 256
-// sequences).  Otherwise Bm may be global memory that another SM wrote earlier in the same kernel: plain loads only.
-template <bool kShared> struct BlkPtr { typedef float* __restrict__ rw; typedef const float* __restrict__ ro; };
-template <> struct BlkPtr<false> { typedef float* rw; typedef const float* ro; };
+// C -= A * Bm^T for 32 x 32 blocks (all column-major); lane computes a 4 x 8 sub-tile.
 template <bool kShared>
 __device__ __noinline__ void warp_rank32_update(typename BlkPtr<kShared>::rw C, typename BlkPtr<kShared>::ro A,
                                                 typename BlkPtr<kShared>::ro Bm) {
@@ -167,7 +172,8 @@ __device__ __noinline__ void warp_rank32_update(typename BlkPtr<kShared>::rw C, 
 }
 
 // Solves L L^T x = v in place (v in shared memory, nb*32 entries) with the blocked factor.
-__device__ __noinline__ void block_cholesky_solve(const float* __restrict__ Lb, const float* __restrict__ InvD,
+template <bool kShared = true>
+__device__ __noinline__ void block_cholesky_solve(typename BlkPtr<kShared>::ro Lb, const float* __restrict__ InvD,
                                                   float* __restrict__ v, int nb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   // forward: L y = v
@@ -220,10 +226,10 @@ __device__ __noinline__ void block_cholesky_solve(const float* __restrict__ Lb, 
 }
 
 // Interacting variant, (K + lambda I) c = A: blocked Cholesky of the lower block triangle held at Lb (nb(nb+1)/2
-// blocks of shared memory), the inverse diagonal factors at InvD, then the solve and up to
+// blocks; shared memory, or a workspace without kShared), the inverse diagonal factors at InvD, then the solve and up to
 // two refinement rounds.  Called by every thread of a CTA of kThr; `layer` tags a failed pivot in *info.
-template <int kThr = kSolveThreads>
-__device__ __forceinline__ void interacting_solve(const TransformParams& P, float* __restrict__ Lb, float* InvD,
+template <int kThr = kSolveThreads, bool kShared = true>
+__device__ __forceinline__ void interacting_solve(const TransformParams& P, typename BlkPtr<kShared>::rw Lb, float* InvD,
                                                   float* vec, double* sol, float* rdiag, double& s_trace, double& s_res,
                                                   int& s_fail, int layer) {
   const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThr / 32;
@@ -270,16 +276,16 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
   }
   __syncthreads();
   if (warp == 0) {
-    const int f = warp_factor_diag(Lb, rdiag);
+    const int f = warp_factor_diag<kShared>(Lb, rdiag);
     if (f != 0 && lane == 0) s_fail = f;
   }
   __syncthreads();
   for (int J = 0; J < nb && !s_fail; ++J) {
     const float* Ljj = Lb + blk_slot(J, J) * kBlk;
     // panel: blocks (I, J) below the diagonal on warps 0 .. nwarps-2; the last warp inverts L_JJ
-    if (warp == nwarps - 1) warp_invert_factor(Ljj, rdiag + J * kNB, InvD + J * kBlk);
+    if (warp == nwarps - 1) warp_invert_factor<kShared>(Ljj, rdiag + J * kNB, InvD + J * kBlk);
     else
-      for (int I = J + 1 + warp; I < nb; I += nwarps - 1) warp_solve_panel(Lb + blk_slot(I, J) * kBlk, Ljj, rdiag + J * kNB);
+      for (int I = J + 1 + warp; I < nb; I += nwarps - 1) warp_solve_panel<kShared>(Lb + blk_slot(I, J) * kBlk, Ljj, rdiag + J * kNB);
     __syncthreads();
     // trailing blocks (I, Kc) with I >= Kc > J; t = a(a+1)/2 + rem -> I = J+1+a, Kc = J+1+rem.
     // t = 0 is the next diagonal block: all warps update it together, then warp 0 factors it while the
@@ -303,14 +309,14 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
       for (int c = 0; c < kColsPerWarp; ++c) Dn[(warp * kColsPerWarp + c) * kNB + lane] = acc[c];
       __syncthreads();
       if (warp == 0) {
-        const int f = warp_factor_diag(Dn, rdiag + (J + 1) * kNB);
+        const int f = warp_factor_diag<kShared>(Dn, rdiag + (J + 1) * kNB);
         if (f != 0 && lane == 0) s_fail = (J + 1) * kNB + f;
       } else {
         for (int t = warp; t < ntrail; t += nwarps - 1) {
           int a = 0, rem = t;
           while (rem > a) { rem -= a + 1; ++a; }
           const int I = J + 1 + a, Kc = J + 1 + rem;
-          warp_rank32_update<true>(Lb + blk_slot(I, Kc) * kBlk, Lb + blk_slot(I, J) * kBlk, Lb + blk_slot(Kc, J) * kBlk);
+          warp_rank32_update<kShared>(Lb + blk_slot(I, Kc) * kBlk, Lb + blk_slot(I, J) * kBlk, Lb + blk_slot(Kc, J) * kBlk);
         }
       }
     }
@@ -337,7 +343,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
   __syncthreads();
   anorm2 = s_trace;
   for (int round = 0; round < 3; ++round) {
-    block_cholesky_solve(Lb, InvD, vec, nb);
+    block_cholesky_solve<kShared>(Lb, InvD, vec, nb);
     for (int i = tid; i < Bp; i += kThr) sol[i] += (double)vec[i];
     __syncthreads();
     if (round == 2) break;

@@ -330,6 +330,9 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
 size_t transform_large_workspace_bytes(int B);
 isopo_status transform_large(const float* K, const float* A, int B, float lambda, float* coeffs, float* scratch,
                              int32_t* info, cudaStream_t st);
+// the same without a cluster, any B whose diagonal blocks fit shared memory (ISOPO_MAX_LARGE_SEQS)
+isopo_status transform_one_cta(const float* K, const float* A, int B, float lambda, float* coeffs, float* scratch, int32_t* info,
+                               cudaStream_t st);
 isopo_status transform(const float* K, const float* A, int B, isopo_variant v, float lambda, const float* pqr_regs_host,
                        const float* rel_state, float* coeffs, int32_t* info, cudaStream_t st);
 isopo_status transform_batched(int n, const float* const* K, const float* A, int B, isopo_variant v, const float* lambda,

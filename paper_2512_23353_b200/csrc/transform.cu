@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_consta
 }
 
 // 257 to 1024 sequences: a cluster of sixteen, the factor's blocks also in a workspace that stays in the L2 (2.1 MB at 1024).
+// Where no such cluster can be placed (a context that has a part of the SMs): transform_one_cta.cu.
 constexpr int kMaxLargeB = ISOPO_MAX_LARGE_SEQS;
 constexpr int kLargeCluster = 16;
 __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const TransformParams P, float* scratch) {
@@ -367,6 +368,9 @@ isopo_status transform_large(const float* K, const float* A, int B, float lambda
   attr.val.clusterDim.x = kLargeCluster; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
+  int clusters = 0;  // asked at every call: a device's contexts may have different SMs
+  ISOPO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, k_transform_large, &cfg));
+  if (clusters == 0) return transform_one_cta(K, A, B, lambda, coeffs, scratch, info, st);
   {
     LaunchScope scope(kIdTransform, st);
     ISOPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_transform_large, P, scratch));

@@ -153,3 +153,28 @@ def test_block_rows_dealt_to_the_cluster(b, B):
     cond = float(np.linalg.cond(K64))
     assert rel_fro(c, np.linalg.solve(K64, A.astype(np.float64))) <= 1e-5 + 2e-7 * cond
     assert float(np.linalg.norm(K64 @ c.astype(np.float64) - A) / np.linalg.norm(A)) <= 2e-6 + 1e-7 * cond
+
+
+@pytest.mark.parametrize("B", [257, 300, 777, 1024])
+def test_a_context_without_room_for_the_cluster(b, B):
+    """Eight SMs of the device (a green context): no cluster of sixteen CTAs fits, and one CTA answers."""
+    from torch.cuda import green_contexts
+    if not green_contexts.SUPPORTED:
+        pytest.skip("no green contexts")
+    K = _spd(B, 2 * B, B)
+    A = np.random.default_rng(B).standard_normal(B).astype(np.float32)
+    lam = float(np.float32(1e-2 * np.mean(np.diag(K))))
+    bad = K.copy()
+    bad[260 % B, 260 % B] = -1e6
+    whole, _ = _solve(b, K, A, lam)
+    ctx = green_contexts.GreenContext.create(8, 0)
+    ctx.set_context()
+    try:
+        part, info = _solve(b, K, A, lam)
+        part_bad, info_bad = _solve(b, bad, A, lam)
+    finally:
+        ctx.pop_context()
+    assert info == 0 and info_bad == 260 % B + 1 and not part_bad.any()
+    want = orc.transform_advantages(K.astype(np.float64), A.astype(np.float64), orc.INTERACTING, lam)
+    cond = np.linalg.cond(K.astype(np.float64) + lam * np.eye(B))
+    assert rel_fro(part, want) <= 1e-5 + 2e-7 * cond and rel_fro(part, whole) <= 1e-5 + 2e-7 * cond
