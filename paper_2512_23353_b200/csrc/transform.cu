@@ -42,15 +42,14 @@ __device__ __forceinline__ TransformParams layer_params(const TransformBatch& ba
   return P;
 }
 
-// Sums of squares of the rows i0, i0 + step, .. of K (four at a time, so that the loads of four rows are in flight), row by
-// row to f(i, sum) in lane 0 of the calling warp.
-template <typename F>
+// Sums of squares of rows first .. last - 1 of K (four at a time, so that the loads of four rows are in flight), row by row to
+// f(i, sum) in lane 0 of the calling warp.
+template <bool kVec4, typename F>
 __device__ __forceinline__ void row_square_sums(const float* __restrict__ K, int B, int first, int last, F f) {
   const int lane = threadIdx.x & 31;
-  const bool vec4 = rows_in_float4(K, B);
   for (int i0 = first; i0 < last; i0 += 4) {
     double sq[4] = {};
-    if (vec4) {
+    if (kVec4) {
 #pragma unroll 2
       for (int j = lane * 4; j < B; j += 128) {
 #pragma unroll
@@ -104,7 +103,9 @@ __global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant_
   for (int i = tid; i < B; i += 256) tr += (double)__ldg(K + (size_t)i * B + i);
   __shared__ double s_sq[kSimpleRows];
   const int r0 = first + (tid >> 5) * 4;
-  row_square_sums(K, B, r0, min(B, r0 + 4), [&](int i, double sq) { s_sq[i - first] = sq; });
+  auto keep = [&](int i, double sq) { s_sq[i - first] = sq; };
+  if (rows_in_float4(K, B)) row_square_sums<true>(K, B, r0, min(B, r0 + 4), keep);
+  else row_square_sums<false>(K, B, r0, min(B, r0 + 4), keep);
   const double trace = block_total<8>(tr, s_part);
   const int i = first + tid;
   if (tid >= kSimpleRows || i >= B) return;
@@ -283,11 +284,14 @@ __global__ void __launch_bounds__(kEmaThreads) k_reg_ema(const float* __restrict
   const int tid = threadIdx.x, warp = tid >> 5;
   double tr = 0.0, f2 = 0.0, rel = 0.0;
   for (int i = tid; i < B; i += kEmaThreads) tr += (double)__ldg(K + (size_t)i * B + i);
-  for (int i0 = warp * 4; i0 < B; i0 += kEmaThreads / 8)
-    row_square_sums(K, B, i0, min(B, i0 + 4), [&](int i, double sq) {
-      f2 += sq;
-      rel += sq / (double)__ldg(K + (size_t)i * B + i);
-    });
+  auto add = [&](int i, double sq) {
+    f2 += sq;
+    rel += sq / (double)__ldg(K + (size_t)i * B + i);
+  };
+  if (rows_in_float4(K, B))  // outside the row loop: inside it 1024 sequences took 72 us instead of 53
+    for (int i0 = warp * 4; i0 < B; i0 += kEmaThreads / 8) row_square_sums<true>(K, B, i0, min(B, i0 + 4), add);
+  else
+    for (int i0 = warp * 4; i0 < B; i0 += kEmaThreads / 8) row_square_sums<false>(K, B, i0, min(B, i0 + 4), add);
   tr = warp_sum(tr);
   if ((tid & 31) == 0) { s_part[0][warp] = tr; s_part[1][warp] = f2; s_part[2][warp] = rel; }
   __syncthreads();
