@@ -296,11 +296,11 @@ k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int
 // fragment is read and widened once for many MMAs.  kDiag: 8 kNB rows against themselves, only the 16 x 8 blocks on and
 // above the diagonal; otherwise 16 kMA rows against 8 kNB others.  Every CTA stores its sums, and they are added in the order
 // of the chunks (k_f32_ntk_finish, or the last CTA to finish where there are few): K is the same to the bit from run to run,
-// which float64 atomics would not leave it where products cancel.  They were slower, too (G and K, atomics / this: 64 sequences
-// of 896 x 896 211 / 194 us, 64 of 64 x 64 31.9 / 22.3, 16 of 896 x 896 64.6 / 45.6, 256 of 512 x 512 974 / 916).
+// which float64 atomics would not leave it where products cancel.  G and K, atomics / this: 64 sequences of 896 x 896 210 / 193
+// us, 64 of 64 x 64 32.8 / 22.5, 16 of 896 x 896 64.8 / 40.5, 256 of 512 x 512 973 / 939, 3 of 896 x 896 24.9 / 26.6.
 // Bound by the float64 pipe.  One CTA per pair (i, j) with scalar float64 additions re-read G B / 2 times: 1384 us at 64
 // sequences of an 896 x 896 layer against 146 us, 3694 against 500 us at 256 sequences of 300 x 500.  One CTA of eight
-// warps per SM instead of two of four: 162 and 715 us.  Few sequences leave the pass to HBM and need more loads in flight: kPerSm.
+// warps per SM instead of two of four: 162 and 715 us.  Few sequences leave the pass to HBM and need more loads in flight: kGroups.
 // ---------------------------------------------------------------------------------------------
 constexpr int kNtkKC = 64;             // columns per chunk
 constexpr int kNtkPitch = kNtkKC + 4;  // floats: the 32 lanes of a fragment read hit 32 banks
@@ -320,7 +320,7 @@ constexpr int ntk_blocks(int ma, int nb, bool diag) { return diag ? ma * (ma + 1
 // The sums of one K pass: pairs x slabs CTAs, `doubles` of each, element (blk * 4 + q) * 32 + lane as the registers have them.
 struct NtkParts {
   int64_t pairs, slabs;
-  int ma, nb, doubles;
+  int ma, nb, doubles, groups;
   bool diag;
   __host__ __device__ int64_t total() const { return pairs * slabs * doubles; }
 };
@@ -336,22 +336,21 @@ __device__ __forceinline__ void ntk_pair_rows(bool diag, int64_t pair, int& i0, 
   i0 = r * kNtkRows + (int)(pair & 1) * 32;
   j0 = J * kNtkRows;
 }
-// Adds the slabs' shares of element e of a pair's block, shares first .. last - 1 in order.
+// Adds shares first .. last - 1 of an element in order, kFlight loads in flight.
+template <int kFlight>
 __device__ __forceinline__ double ntk_sum(const double* part, int64_t stride, int first, int last) {
   double s = 0.0;
-  int k = first;
-  for (; k + 8 <= last; k += 8) {
-    double v[8];
+  for (int k = first; k < last; k += kFlight) {
+    double v[kFlight];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (k + u) * stride);
+    for (int u = 0; u < kFlight; ++u) v[u] = k + u < last ? __ldcg(part + (k + u) * stride) : 0.0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) s += v[u];
+    for (int u = 0; u < kFlight; ++u) s += v[u];
   }
-  for (; k < last; ++k) s += __ldcg(part + k * stride);
   return s;
 }
-// K[i][j] and K[j][i] of element e of a pair's block
-__device__ __forceinline__ void ntk_write(const NtkParts& P, int i0, int j0, int e, int B, float* __restrict__ K, double v) {
+// Row and column of K that element e of a pair's block stands for; false where it is not of use.
+__device__ __forceinline__ bool ntk_entry(const NtkParts& P, int i0, int j0, int e, int B, int& i, int& j) {
   const int lane = e & 31, q = (e >> 5) & 3;
   int p = 0, n = e >> 7;
   if (P.diag) {
@@ -361,31 +360,53 @@ __device__ __forceinline__ void ntk_write(const NtkParts& P, int i0, int j0, int
     p = n / P.nb;
     n -= p * P.nb;
   }
-  const int i = i0 + p * 16 + (lane >> 2) + (q >> 1) * 8, j = j0 + n * 8 + 2 * (lane & 3) + (q & 1);
-  if (i > j || j >= B) return;
+  i = i0 + p * 16 + (lane >> 2) + (q >> 1) * 8;
+  j = j0 + n * 8 + 2 * (lane & 3) + (q & 1);
+  return i <= j && j < B;
+}
+// Entry e of the upper triangle of B rows (by rows), and the element of the first diagonal block that stands for it.
+__device__ __forceinline__ int ntk_triangle(const NtkParts& P, int B, int e, int& i, int& j) {
+  i = 0;
+  while (i < B && e >= B - i) { e -= B - i; ++i; }
+  j = i + e;
+  const int p = i >> 4, n = j >> 3, blk = p * (P.nb - p + 1) + n - 2 * p;
+  return (blk * 4 + ((i >> 3) & 1) * 2 + (j & 1)) * 32 + (i & 7) * 4 + ((j & 7) >> 1);
+}
+__device__ __forceinline__ void ntk_write(float* __restrict__ K, int B, int i, int j, double v) {
   K[(size_t)i * B + j] = (float)v;
   K[(size_t)j * B + i] = (float)v;
 }
 
-template <int kMA, int kNB, bool kDiag>
+template <int kMA, int kNB, bool kDiag, int kG>
 struct NtkShape {
   static constexpr int kRowsStaged = kDiag ? 8 * kNB : 16 * kMA + 8 * kNB;
   static constexpr int kStageFloats = kRowsStaged * kNtkPitch;
   static constexpr int kSmemStages = kNtkStages * kStageFloats * 4;
   static constexpr int kBlocks = ntk_blocks(kMA, kNB, kDiag);
   static constexpr int kSmemRed = 2 * kBlocks * 128 * 8;               // two warps' blocks
-  static constexpr int kSmem = kSmemStages > kSmemRed ? kSmemStages : kSmemRed;
-  static constexpr int kPerSm = kNB == 2 ? 8 : kNB == 4 ? 4 : 2;       // resident CTAs per SM
+  static constexpr int kSmemGroup = kSmemStages > kSmemRed ? kSmemStages : kSmemRed;
+  // Few sequences leave the pass to HBM: kG groups of four warps, each with a ring and chunks of its own, share a CTA, so that
+  // their sums meet in shared memory and there are few shares of K to add.  Small layers spread the groups over the SMs instead.
+  static constexpr int kGroups = kG;
+  static constexpr int kThr = kGroups * kNtkThreads;
+  static constexpr int kSmem = kGroups * kSmemGroup;
+  static constexpr int kPerSm = 2;  // resident CTAs per SM
 };
 
-template <int kMA, int kNB, bool kDiag>
-__global__ void __launch_bounds__(kNtkThreads, NtkShape<kMA, kNB, kDiag>::kPerSm)
+template <int kMA, int kNB, bool kDiag, int kG>
+__global__ void __launch_bounds__(NtkShape<kMA, kNB, kDiag, kG>::kThr, NtkShape<kMA, kNB, kDiag, kG>::kPerSm)
 k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_constant__ NtkParts parts, double* part, uint32_t* done,
           float* __restrict__ K) {
   pdl_wait();
-  typedef NtkShape<kMA, kNB, kDiag> S;
-  extern __shared__ __align__(16) float smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  typedef NtkShape<kMA, kNB, kDiag, kG> S;
+  extern __shared__ __align__(16) float smem_cta[];
+  const int group = threadIdx.x / kNtkThreads, tid = threadIdx.x % kNtkThreads, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  float* smem = smem_cta + group * (S::kSmemGroup / 4);
+  auto sync_group = [&]() {
+    if (S::kGroups == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kNtkThreads) : "memory");
+  };
+  const int64_t first_chunk = (int64_t)blockIdx.y * S::kGroups + group, chunk_step = (int64_t)gridDim.y * S::kGroups;
   int i0, j0;
   ntk_pair_rows(kDiag, blockIdx.x, i0, j0);
   const int64_t nchunks = (gstride + kNtkKC - 1) / kNtkKC;
@@ -410,12 +431,12 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[p][n][q] = 0.0;
 #pragma unroll
-  for (int k = 0; k < kNtkStages - 1; ++k) fetch(blockIdx.y + (int64_t)k * gridDim.y, k);
+  for (int k = 0; k < kNtkStages - 1; ++k) fetch(first_chunk + k * chunk_step, k);
   int stage = 0;
-  for (int64_t ch = blockIdx.y; ch < nchunks; ch += gridDim.y) {
+  for (int64_t ch = first_chunk; ch < nchunks; ch += chunk_step) {
     cp_async_wait<kNtkStages - 2>();
-    __syncthreads();
-    fetch(ch + (int64_t)(kNtkStages - 1) * gridDim.y, (stage + kNtkStages - 1) % kNtkStages);
+    sync_group();
+    fetch(ch + (kNtkStages - 1) * chunk_step, (stage + kNtkStages - 1) % kNtkStages);
     const float* s = smem + stage * S::kStageFloats;
     if (++stage == kNtkStages) stage = 0;
 #pragma unroll
@@ -448,7 +469,7 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
   // the warps' shares meet in shared memory (4 -> 2 -> 1)
   double2* red = reinterpret_cast<double2*>(smem);
   for (int half = 2; half >= 1; half >>= 1) {
-    __syncthreads();
+    sync_group();
     if (warp >= half && warp < 2 * half) {
       int blk = (warp - half) * S::kBlocks;
 #pragma unroll
@@ -459,7 +480,7 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
           red[blk * 64 + 32 + lane] = make_double2(acc[p][n][2], acc[p][n][3]);
         }
     }
-    __syncthreads();
+    sync_group();
     if (warp < half) {
       int blk = warp * S::kBlocks;
 #pragma unroll
@@ -471,7 +492,35 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
         }
     }
   }
-  if (warp == 0) {
+  if (S::kGroups > 1) {  // the groups' shares, in order
+    __syncthreads();
+    double* meet = reinterpret_cast<double*>(smem_cta) + lane;  // [group - 1][kBlocks][4][32]
+    if (group > 0 && warp == 0) {
+      double* to = meet + (group - 1) * S::kBlocks * 128;
+#pragma unroll
+      for (int p = 0; p < kMA; ++p)
+#pragma unroll
+        for (int n = kDiag ? 2 * p : 0; n < kNB; ++n)
+#pragma unroll
+          for (int q = 0; q < 4; ++q, to += 32) *to = acc[p][n][q];
+    }
+    __syncthreads();
+    if (group == 0 && warp == 0) {
+      for (int k = 0; k < S::kGroups - 1; ++k) {
+        const double* from = meet + k * S::kBlocks * 128;
+#pragma unroll
+        for (int p = 0; p < kMA; ++p)
+#pragma unroll
+          for (int n = kDiag ? 2 * p : 0; n < kNB; ++n)
+#pragma unroll
+            for (int q = 0; q < 4; ++q, from += 32) acc[p][n][q] += *from;
+      }
+    }
+  }
+  static_assert((S::kGroups - 1) * S::kBlocks * 128 * 8 <= S::kSmem, "the groups' shares");
+  // k_f32_ntk_finish is set up while the shares of a single pair are stored (of several pairs it is larger, and slower so)
+  if (kDiag && gridDim.x == 1 && !done) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (group == 0 && warp == 0) {
     double* mine = part + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * parts.doubles + lane;
 #pragma unroll
     for (int p = 0; p < kMA; ++p)
@@ -484,18 +533,47 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
     __shared__ bool last;
     __threadfence();
     __syncthreads();
-    if (tid == 0) last = atomicAdd(done, 1u) == gridDim.y - 1;
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.y - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int e = tid; e < parts.doubles; e += kNtkThreads)
-      ntk_write(parts, i0, j0, e, B, K, ntk_sum(part + e, parts.doubles, 0, gridDim.y));
+    // an entry of K to a thread, or to as many threads as there are for each, which meet in shared memory
+    const int entries = B * (B + 1) / 2, runs = S::kThr / entries, shares = (int)gridDim.y;
+    int i, j;
+    if (runs <= 1) {
+      for (int e = threadIdx.x; e < entries; e += 2 * S::kThr) {  // two at a time
+        int i1, j1;
+        const int e1 = e + S::kThr, x = ntk_triangle(parts, B, e, i, j), x1 = ntk_triangle(parts, B, min(e1, entries - 1), i1, j1);
+        double v[8], v1[8], t0 = 0.0, t1 = 0.0;
+        for (int k = 0; k < shares; k += 8) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            v[u] = k + u < shares ? __ldcg(part + (int64_t)(k + u) * parts.doubles + x) : 0.0;
+            v1[u] = k + u < shares && e1 < entries ? __ldcg(part + (int64_t)(k + u) * parts.doubles + x1) : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) { t0 += v[u]; t1 += v1[u]; }
+        }
+        ntk_write(K, B, i, j, t0);
+        if (e1 < entries) ntk_write(K, B, i1, j1, t1);
+      }
+      return;
+    }
+    const int e = threadIdx.x / runs, run = threadIdx.x % runs, per = (shares + runs - 1) / runs, first = min(shares, run * per);
+    const int x = ntk_triangle(parts, B, min(e, entries - 1), i, j);
+    double* sums = reinterpret_cast<double*>(smem_cta);
+    sums[threadIdx.x] = ntk_sum<16>(part + x, parts.doubles, first, min(shares, first + per));
+    __syncthreads();
+    if (e >= entries || run != 0) return;
+    double v = 0.0;
+    for (int k = 0; k < runs; ++k) v += sums[threadIdx.x + k];
+    ntk_write(K, B, i, j, v);
   }
 }
 
 // K from the shares of a launch on the diagonal blocks and, with more than one of them, of one on the others.  The shares of an
-// element are added in kRuns runs, a thread each: eight where they are many and a single thread's loads would be a long chain,
-// one where they are few.
+// element are added in kRuns runs, a thread each, so that a thread's loads are no long chain: one run where shares are few (up to
+// 16), 8 or, above 128 shares (there are 296 at most), 32: a thread's loads are all in flight at once.
 template <int kRuns>
 __global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ NtkParts diag, const __grid_constant__ NtkParts rest,
                                                         const double* __restrict__ part, int B, float* __restrict__ K) {
@@ -509,9 +587,12 @@ __global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ 
   const int64_t x = (on_diag ? blockIdx.x : blockIdx.x - diag_blocks) * kElems;
   const int64_t pair = x / P.doubles;
   const int e = (int)(x - pair * P.doubles) + t;
+  int i0, j0, i, j;
+  ntk_pair_rows(P.diag, pair, i0, j0);
+  const bool used = ntk_entry(P, i0, j0, e, B, i, j);
   const double* src = part + (on_diag ? 0 : diag.total()) + pair * P.slabs * P.doubles + e;
   const int per = (int)((P.slabs + kRuns - 1) / kRuns), first = min((int)P.slabs, run * per);
-  double s = ntk_sum(src, P.doubles, first, min((int)P.slabs, first + per));
+  double s = used ? ntk_sum<16>(src, P.doubles, first, min((int)P.slabs, first + per)) : 0.0;
   if (kRuns > 1) {
     sums[run][t] = s;
     __syncthreads();
@@ -520,9 +601,7 @@ __global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ 
 #pragma unroll
     for (int w = 0; w < kRuns; ++w) s += sums[w][t];
   }
-  int i0, j0;
-  ntk_pair_rows(P.diag, pair, i0, j0);
-  ntk_write(P, i0, j0, e, B, K, s);
+  if (used) ntk_write(K, B, i, j, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -818,21 +897,21 @@ isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, 
   return wide ? launch_f32_seq_grad<128, 8, false>(a, o, st) : launch_f32_seq_grad<64, 4, false>(a, o, st);
 }
 
-template <int kMA, int kNB, bool kDiag>
-static NtkParts ntk_parts(int64_t gstride, int64_t pairs) {
-  // every SM full over all pairs; at least eight chunks each, or the reduction outweighs the stream
-  constexpr int64_t ctas = 148 * NtkShape<kMA, kNB, kDiag>::kPerSm;
-  const int64_t chunks = (gstride + kNtkKC - 1) / kNtkKC;
-  const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + 7) / 8));
-  return NtkParts{pairs, slabs, kMA, kNB, NtkShape<kMA, kNB, kDiag>::kBlocks * 128, kDiag};
+// groups: of four warps in a CTA; at least eight chunks to a CTA of one group, or the reduction outweighs the stream
+static NtkParts ntk_parts(int ma, int nb, bool diag, int groups, int64_t chunks, int64_t pairs) {
+  const int64_t ctas = 148 * 2, least = groups == 1 ? 8 : 4 * groups;  // every SM full over all pairs
+  const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + least - 1) / least));
+  return NtkParts{pairs, slabs, ma, nb, ntk_blocks(ma, nb, diag) * 128, groups, diag};
 }
-// The launches of the K pass of B gradients: diagonal blocks, the others (no pairs: none).
+// The launches of the K pass of B gradients: diagonal blocks, the others (no pairs: none).  Up to 32 sequences two CTAs of one
+// group on every SM where that gives a group sixteen chunks or fewer, else two of several.
 static void ntk_plan(int64_t gstride, int B, NtkParts* diag, NtkParts* rest) {
-  const int64_t nb = (B + kNtkRows - 1) / kNtkRows;
-  *diag = B <= 16   ? ntk_parts<1, 2, true>(gstride, 1)
-          : B <= 32 ? ntk_parts<2, 4, true>(gstride, 1)
-                    : ntk_parts<4, 8, true>(gstride, nb);
-  *rest = nb == 1 ? NtkParts{} : ntk_parts<2, 8, false>(gstride, nb * (nb - 1));  // two halves of nb (nb - 1) / 2 pairs
+  const int64_t blocks = (B + kNtkRows - 1) / kNtkRows, chunks = (gstride + kNtkKC - 1) / kNtkKC;
+  const bool few_chunks = chunks <= 16 * 148 * 2;
+  *diag = B <= 16   ? ntk_parts(1, 2, true, few_chunks ? 1 : 4, chunks, 1)
+          : B <= 32 ? ntk_parts(2, 4, true, few_chunks ? 1 : 2, chunks, 1)
+                    : ntk_parts(4, 8, true, 1, chunks, blocks);
+  *rest = blocks == 1 ? NtkParts{} : ntk_parts(2, 8, false, 1, chunks, blocks * (blocks - 1));  // two halves of that many / 2 pairs
 }
 size_t f32_ntk_part_bytes(int64_t gstride, int B) {
   NtkParts diag, rest;
@@ -840,15 +919,15 @@ size_t f32_ntk_part_bytes(int64_t gstride, int B) {
   return sizeof(double) * (size_t)(diag.total() + rest.total());
 }
 
-template <int kMA, int kNB, bool kDiag>
+template <int kMA, int kNB, bool kDiag, int kG>
 static isopo_status launch_f32_ntk(const float* G, int64_t gstride, int B, const NtkParts& parts, double* part, uint32_t* done,
                                    float* K, cudaStream_t st) {
-  constexpr int smem = NtkShape<kMA, kNB, kDiag>::kSmem;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_f32_ntk<kMA, kNB, kDiag>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  typedef NtkShape<kMA, kNB, kDiag, kG> S;
+  const auto kernel = k_f32_ntk<kMA, kNB, kDiag, kG>;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem));
   {
     LaunchScope scope(kIdF32Ntk, st);
-    launch(k_f32_ntk<kMA, kNB, kDiag>, dim3((unsigned)parts.pairs, (unsigned)parts.slabs), kNtkThreads, smem, st, G, gstride, B, parts,
-           part, done, K);
+    launch(kernel, dim3((unsigned)parts.pairs, (unsigned)parts.slabs), S::kThr, S::kSmem, st, G, gstride, B, parts, part, done, K);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -866,22 +945,27 @@ static isopo_status launch_f32_finish(const double* kacc, int B, float* K, cudaS
 isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint32_t* done, float* K, cudaStream_t st) {
   NtkParts diag, rest;
   ntk_plan(gstride, B, &diag, &rest);
-  // the last CTA adds the shares up itself where it has 64 or fewer to load per thread: a launch less
-  const bool by_last = diag.pairs == 1 && diag.total() <= 64 * kNtkThreads;
+  // The last CTA adds the shares up itself, a launch less, where that takes it about as long as one round of loads: its threads
+  // are several to an entry of K, or have no more than two rounds of two entries.
+  const int threads = kNtkThreads * diag.groups, entries = B <= kNtkRows ? B * (B + 1) / 2 : INT32_MAX;
+  const bool by_last = diag.pairs == 1 && (threads >= 2 * entries ? diag.slabs <= 48 * (threads / entries)
+                                                                  : (entries + 2 * threads - 1) / (2 * threads) * ((diag.slabs + 7) / 8) <= 2);
   if (!by_last) done = nullptr;
-  const isopo_status s = B <= 16   ? launch_f32_ntk<1, 2, true>(G, gstride, B, diag, part, done, K, st)
-                         : B <= 32 ? launch_f32_ntk<2, 4, true>(G, gstride, B, diag, part, done, K, st)
-                                   : launch_f32_ntk<4, 8, true>(G, gstride, B, diag, part, done, K, st);
+  const auto launch_diag = B <= 16   ? (diag.groups == 1 ? launch_f32_ntk<1, 2, true, 1> : launch_f32_ntk<1, 2, true, 4>)
+                           : B <= 32 ? (diag.groups == 1 ? launch_f32_ntk<2, 4, true, 1> : launch_f32_ntk<2, 4, true, 2>)
+                                     : launch_f32_ntk<4, 8, true, 1>;
+  const isopo_status s = launch_diag(G, gstride, B, diag, part, done, K, st);
   if (s != ISOPO_OK || by_last) return s;
   if (rest.pairs > 0) {
-    const isopo_status r = launch_f32_ntk<2, 8, false>(G, gstride, B, rest, part + diag.total(), nullptr, K, st);
+    const isopo_status r = launch_f32_ntk<2, 8, false, 1>(G, gstride, B, rest, part + diag.total(), nullptr, K, st);
     if (r != ISOPO_OK) return r;
   }
   {
     LaunchScope scope(kIdMirror, st);
-    const bool many = std::max(diag.slabs, rest.slabs) > 16;
-    const int64_t elems = diag.pairs * diag.doubles + rest.pairs * rest.doubles;  // a multiple of 256
-    launch(many ? k_f32_ntk_finish<8> : k_f32_ntk_finish<1>, (unsigned)(elems / (many ? 32 : 256)), 256, 0, st, diag, rest, part, B, K);
+    const int64_t shares = std::max(diag.slabs, rest.slabs), elems = diag.pairs * diag.doubles + rest.pairs * rest.doubles;
+    const int runs = shares > 128 ? 32 : shares > 16 ? 8 : 1;
+    launch(runs == 32 ? k_f32_ntk_finish<32> : runs == 8 ? k_f32_ntk_finish<8> : k_f32_ntk_finish<1>,
+           (unsigned)(elems * runs / 256), 256, 0, st, diag, rest, part, B, K);  // elems: a multiple of 256
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -49,7 +49,8 @@ def test_two_runs_are_bit_identical(b, B, d_in, d_out):
     assert b.isopo_workspace_bytes(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE) == plain_bytes
 
 
-@pytest.mark.parametrize("B,d", [(6, 512), (8, 64), (30, 256), (64, 512), (130, 192)])  # every K kernel; its last CTA and its finish
+@pytest.mark.parametrize("B,d", [(3, 640), (6, 512), (8, 64), (16, 64), (16, 640), (20, 64), (30, 256), (32, 640), (40, 24),
+                                  (64, 512), (130, 192)])  # every K kernel, one group of warps and several; its last CTA, its finish
 def test_float32_stored_route_needs_no_mode(b, B, d):
     """K of float32 gradients is added up in a fixed order anyway: the same to the bit where products cancel and the last bits of
     a sum are all that is left of it."""
