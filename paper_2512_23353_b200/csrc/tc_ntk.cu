@@ -410,7 +410,10 @@ constexpr int kManySeqs = 64;
 // Split store: dW = beta dW + sum_i (c_i / s_i) (hi_i + lo_i / 16).  One thread per PAIR of slots (two tile rows x 8
 // columns), so that every load is 16 bytes per plane: with one slot per thread the two planes cost twice the load
 // instructions per byte of the bf16 store and the pass fell to 5.0 TB/s inside the step.
-__global__ void __launch_bounds__(256) k_e4m3_combine(const uint2* __restrict__ planes, long long nchunks /* n_pad / 8 */,
+// kDeep: registers for more of a thread's loads at once, on three CTAs per SM instead of four: where that takes no more waves.
+// 200 sequences, 896 x 256 66 -> 40 us (four CTAs -> three), 896 x 896 77 -> 57, 2048 x 2048 (three waves instead of two) 249 -> 259.
+template <bool kDeep>
+__global__ void __launch_bounds__(256, kDeep ? 3 : 4) k_e4m3_combine(const uint2* __restrict__ planes, long long nchunks /* n_pad / 8 */,
                                                        int B, PieceGrid grid, int d_in, int d_out,
                                                        const float* __restrict__ coeffs, const float* __restrict__ scales,
                                                        float* __restrict__ dW, float beta,
@@ -547,9 +550,10 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
   const int grid = (int)std::min<long long>((chunks * slices + 255) / 256, (long long)sms * 8);
   {
     LaunchScope scope(kIdCombine, st);
+    const int deep_waves = (grid + 3 * sms - 1) / (3 * sms), waves = (grid + 4 * sms - 1) / (4 * sms);
     if (fmt.split)
-      launch(k_e4m3_combine, grid, 256, 0, st, (const uint2*)G, chunks, B, pg, d_in, d_out, coeffs, fmt.scales, dW, beta,
-                                           tag_dev, tag, info);
+      launch(deep_waves <= waves ? k_e4m3_combine<true> : k_e4m3_combine<false>, grid, 256, 0, st, (const uint2*)G, chunks, B, pg,
+             d_in, d_out, coeffs, fmt.scales, dW, beta, tag_dev, tag, info);
     else
       launch((slices == 1   ? (B >= kManySeqs ? k_bf16_combine<1, true> : k_bf16_combine<1, false>)
        : slices == 2 ? k_bf16_combine<2, false>
