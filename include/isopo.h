@@ -191,10 +191,10 @@ ISOPO_API isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_pro
  *   c_i = A_i * reg2(F_i; g[3])^g[0] * reg2(sqrt(K_ii); g[4])^g[1] * reg2(F_i / sqrt(K_ii); g[5])^g[2],
  *   reg2(v; reg) = sqrt(v^2 + reg + 1e-8)                                         (Fig. 3),
  * with g = opt_pqr_regs = {p, q, r, reg_F, reg_G, reg_rel} (host, 6 floats; required for GENERAL,
- * ignored otherwise; `lambda` is ignored for GENERAL).  ISOPO_VAR_INTERACTING factors K + lambda*I
- * by Cholesky in shared memory (float32) and refines the solution with float64 residuals; it
+ * ignored otherwise; `lambda` is ignored for GENERAL).  ISOPO_VAR_INTERACTING eliminates K + lambda*I in float64 up to 128
+ * sequences, and above that factors it by Cholesky (float32) and refines the solution with float64 residuals; it
  * requires B <= 256 (isopo_transform_advantages_large takes up to 1024) and reports a non-positive pivot k
- * (1-based) as *info = k.
+ * (1-based) as *info = k, coeffs are then zero.
  *
  *   K       dev, float32 [B, B] row-major (as written by isopo_layer_gram)
  *   A       dev, float32 [B]

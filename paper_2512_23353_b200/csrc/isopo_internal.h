@@ -157,7 +157,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved);
 
-// Workspace of isopo_sampled_coefficients: the Gram-route prefix (offsets, order, token map), then
+// Workspace of isopo_sampled_coefficients: the Gram-route prefix (offsets, token map), then
 // the gathered rows a0 / g0, M^T and the denominator.
 struct SampledLayout {
   size_t off_a0, off_g0, off_mt, off_den, total;
@@ -175,10 +175,11 @@ void set_cuda_error(cudaError_t e, const char* where);
   } while (0)
 
 // ---- programmatic dependent launch ----
-// A layer is a chain of five to ten dependent kernels, several of them a few microseconds long.  Every kernel of the
-// library is launched so that its CTAs may be set up as soon as its predecessor in the stream lets them, and waits for
-// everything before it to be complete and visible before it touches memory (all of its CTAs do, so that the chain stays
-// ordered end to end).  Work of other origin in the stream is ordered as always.
+// A layer is a chain of five to ten dependent kernels, several of them a few microseconds long.  The kernels of the
+// library are launched so that their CTAs may be set up as soon as their predecessor in the stream lets them (not
+// k_transform_large, launched with a cluster size alone, and the self-test's k_wait_probe), and wait for everything before
+// them to be complete and visible before they touch memory: k_spectral, which runs beside its predecessor, before it ends.
+// All CTAs of a kernel wait, so that the chain stays ordered end to end.  Work of other origin in the stream is ordered as always.
 //   pdl_begin  waits, then lets the successor in while this kernel runs: kernels of one CTA per SM, which leave no room
 //              beside them, and kernels of a few CTAs
 //   pdl_wait   waits; the successor is let in when the last CTA leaves.  Kernels of several CTAs per SM: a successor let

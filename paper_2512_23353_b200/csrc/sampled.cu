@@ -135,7 +135,7 @@ isopo_status gather_samples(const T* X, const T* dY, int d_in, int d_out, const 
 SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples) {
   SampledLayout S{};
   const size_t elt = dtype == ISOPO_BF16 ? 2 : 4;
-  size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM).total;  // offsets, order, token map (+ kacc)
+  size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM).total;  // offsets, token map (+ kacc)
   S.off_a0 = p;
   p = align_up(p + elt * (size_t)n_samples * d_in, 1024);
   S.off_g0 = p;

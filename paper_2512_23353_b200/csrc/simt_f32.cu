@@ -12,6 +12,7 @@ namespace {
 
 // Host values travel to the device as kernel arguments: no hidden synchronisation with the stream, and nothing that reads
 // the caller's array after the call returns.
+constexpr int64_t kSms = 148;  // of a B200: the rules below that fill the machine
 constexpr int kArgLarge = 2048;  // offsets of one launch: 8 KB of arguments
 template <int kN>
 __global__ void __launch_bounds__(256) k_store_offsets(const __grid_constant__ OffsetArgs<kN> a, int64_t base, int n,
@@ -879,7 +880,7 @@ static isopo_status launch_f32_seq_grad(const F32StoredArgs& a, const OffsetPara
 // 128 x 128 tiles (8 x 8 per thread) where they fill the machine twice and pad little, else 64 x 64 (4 x 4).
 static bool f32_wide_tiles(int d_in, int d_out, int64_t copies) {
   const int64_t gx = (d_in + 127) / 128, gy = (d_out + 127) / 128, hx = (d_in + 63) / 64, hy = (d_out + 63) / 64;
-  return gx * gy * copies >= 296 && gx * gy * 4 * 4 <= hx * hy * 5;
+  return gx * gy * copies >= 2 * kSms && gx * gy * 4 * 4 <= hx * hy * 5;
 }
 
 isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
@@ -899,7 +900,7 @@ isopo_status f32_seq_grad(const float* X, const float* dY, int d_in, int d_out, 
 
 // groups: of four warps in a CTA; at least eight chunks to a CTA of one group, or the reduction outweighs the stream
 static NtkParts ntk_parts(int ma, int nb, bool diag, int groups, int64_t chunks, int64_t pairs) {
-  const int64_t ctas = 148 * 2, least = groups == 1 ? 8 : 4 * groups;  // every SM full over all pairs
+  const int64_t ctas = 2 * kSms, least = groups == 1 ? 8 : 4 * groups;  // every SM full over all pairs
   const int64_t slabs = std::max<int64_t>(1, std::min<int64_t>((ctas + pairs - 1) / pairs, (chunks + least - 1) / least));
   return NtkParts{pairs, slabs, ma, nb, ntk_blocks(ma, nb, diag) * 128, groups, diag};
 }
@@ -907,7 +908,7 @@ static NtkParts ntk_parts(int ma, int nb, bool diag, int groups, int64_t chunks,
 // group on every SM where that gives a group sixteen chunks or fewer, else two of several.
 static void ntk_plan(int64_t gstride, int B, NtkParts* diag, NtkParts* rest) {
   const int64_t blocks = (B + kNtkRows - 1) / kNtkRows, chunks = (gstride + kNtkKC - 1) / kNtkKC;
-  const bool few_chunks = chunks <= 16 * 148 * 2;
+  const bool few_chunks = chunks <= 16 * 2 * kSms;
   *diag = B <= 16   ? ntk_parts(1, 2, true, few_chunks ? 1 : 4, chunks, 1)
           : B <= 32 ? ntk_parts(2, 4, true, few_chunks ? 1 : 2, chunks, 1)
                     : ntk_parts(4, 8, true, 1, chunks, blocks);
@@ -972,7 +973,7 @@ isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint3
 }
 
 // Tokens per tile: 64, or 32 where `tiles` of 64 would not give every SM two CTAs.
-static bool f32_gram_small_tiles(int64_t tiles) { return tiles < 2 * 148; }
+static bool f32_gram_small_tiles(int64_t tiles) { return tiles < 2 * kSms; }
 
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                       double* kacc, float* K, cudaStream_t st) {
@@ -1008,7 +1009,7 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
   // split while whole lanes would leave the machine (about 2^17 lanes of four elements in flight) mostly empty
   const bool split = N < ((int64_t)1 << 19) && B >= 4;
   const int64_t per_block = split ? 128 : 1024;
-  const int grid = (int)std::min<int64_t>((N + per_block - 1) / per_block, 148 * 16);
+  const int grid = (int)std::min<int64_t>((N + per_block - 1) / per_block, kSms * 16);
   {
     LaunchScope scope(kIdF32Combine, st);
     launch((split ? k_f32_combine<8> : k_f32_combine<1>), grid, 256, 0, st, G, N, gstride, B, coeffs, dW, beta, tag_dev, tag, info);

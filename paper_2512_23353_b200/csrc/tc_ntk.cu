@@ -43,7 +43,8 @@ struct NtkParams {
   int32_t* info;
   int box_rows;   // rows of a piece inside a box: 32, 64, 128 or 256, >= B
   int ppb;        // pieces per box = 256 / box_rows
-  // B <= 128, float atomics: the last CTA to add its share completes the other triangle (and the diagonal of the split store)
+  // not NULL (up to 16 sequences, 32 with little data): the last CTA to add its share completes the other triangle and the
+  // diagonal of the split store
   uint32_t* done;
   uint32_t n_active;  // CTAs with a share
   const float* kdiag;

@@ -1,7 +1,8 @@
 """Deterministic mode: K of the bf16 stored-gradient route is normally reduced over the CTAs with float
 atomics, so two runs differ in their last bits; with the mode on, per-CTA partial sums are added in a
 fixed order and K, the coefficients and dW must be bit-identical from run to run - which tells a race
-(results that differ) from rounding (results that do not).  The values still match the oracle."""
+(results that differ) from rounding (results that do not).  The values still match the oracle.  The float32 stored route
+adds in a fixed order always."""
 
 import numpy as np
 import pytest

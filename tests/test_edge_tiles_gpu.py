@@ -72,7 +72,7 @@ def test_stand_alone_weight_gradient(b, d_in, d_out, lens):
 
 # shares of the sequences in the combine: one (too few sequences / too many pieces), two, four and eight, even and uneven; one
 # share of fewer than 64 sequences and of more, whole groups of eight or sixteen and remainders
-@pytest.mark.parametrize("B,d_in,d_out", [(1, 72, 40), (8, 1024, 1000), (15, 1024, 1000), (63, 1536, 1024), (79, 1536, 1024), (15, 64, 64), (16, 64, 64), (33, 128, 72), (100, 896, 128), (128, 64, 48), (129, 64, 48), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
+@pytest.mark.parametrize("B,d_in,d_out", [(1, 72, 40), (8, 1024, 1000), (15, 1024, 1000), (63, 1536, 1024), (79, 1536, 1024), (15, 64, 64), (16, 64, 64), (17, 64, 64), (32, 128, 96), (32, 1024, 1024), (33, 128, 72), (100, 896, 128), (128, 64, 48), (129, 64, 48), (65, 1536, 256), (256, 64, 40), (64, 1024, 1024)])
 def test_combine_shares(b, B, d_in, d_out):
     X, dY, off, c, G = _problem(d_in, d_out, [2 + i % 3 for i in range(B)], B)
     ws = b.alloc_workspace(b.BF16, int(off[-1]), d_in, d_out, B, b.PATH_MATERIALISE)
@@ -83,7 +83,7 @@ def test_combine_shares(b, B, d_in, d_out):
     torch.cuda.synchronize()
     assert int(info.item()) == 0
     assert rel_fro(dW.cpu().numpy(), 1.0 + orc.weight_gradient(G, to_f64(c))) <= 6e-3
-    # up to 128 sequences the K pass completes the other triangle itself
+    # the other triangle: by the K pass's last CTA up to 16 sequences, and up to 32 of little data; else by a kernel of its own
     assert torch.equal(K, K.T) and rel_fro(K.cpu().numpy(), orc.ntk(G)) <= 2e-3
 
 
