@@ -528,9 +528,15 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
 #pragma unroll
       for (int n = kDiag ? 2 * p : 0; n < kNB; ++n)
 #pragma unroll
-        for (int q = 0; q < 4; ++q, mine += 32) *mine = acc[p][n][q];
+        for (int q = 0; q < 4; ++q, mine += 32)
+          if (i0 + p * 16 + (q >> 1) * 8 < B && j0 + n * 8 < B) *mine = acc[p][n][q];  // others stand for no sequences: never read
   }
   if (done) {  // one pair, few shares
+    // an entry of K to a thread, or, of many shares, to as many threads as there are for each, which meet in shared memory
+    const int entries = B * (B + 1) / 2, shares = (int)gridDim.y, runs = shares <= 16 ? 1 : S::kThr / entries;
+    const int mine = runs > 1 ? threadIdx.x / runs : threadIdx.x;
+    int i, j;
+    int x = ntk_triangle(parts, B, min(mine, entries - 1), i, j);
     __shared__ bool last;
     __threadfence();
     __syncthreads();
@@ -538,13 +544,11 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // an entry of K to a thread, or to as many threads as there are for each, which meet in shared memory
-    const int entries = B * (B + 1) / 2, runs = S::kThr / entries, shares = (int)gridDim.y;
-    int i, j;
     if (runs <= 1) {
-      for (int e = threadIdx.x; e < entries; e += 2 * S::kThr) {  // two at a time
+      for (int e = mine; e < entries; e += 2 * S::kThr) {  // two at a time
         int i1, j1;
-        const int e1 = e + S::kThr, x = ntk_triangle(parts, B, e, i, j), x1 = ntk_triangle(parts, B, min(e1, entries - 1), i1, j1);
+        const int e1 = e + S::kThr, x1 = e1 < entries ? ntk_triangle(parts, B, e1, i1, j1) : 0;
+        if (e != mine) x = ntk_triangle(parts, B, e, i, j);
         double v[8], v1[8], t0 = 0.0, t1 = 0.0;
         for (int k = 0; k < shares; k += 8) {
 #pragma unroll
@@ -552,20 +556,19 @@ k_f32_ntk(const float* __restrict__ G, int64_t gstride, int B, const __grid_cons
             v[u] = k + u < shares ? __ldcg(part + (int64_t)(k + u) * parts.doubles + x) : 0.0;
             v1[u] = k + u < shares && e1 < entries ? __ldcg(part + (int64_t)(k + u) * parts.doubles + x1) : 0.0;
           }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) { t0 += v[u]; t1 += v1[u]; }
+          t0 += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+          t1 += ((v1[0] + v1[1]) + (v1[2] + v1[3])) + ((v1[4] + v1[5]) + (v1[6] + v1[7]));
         }
         ntk_write(K, B, i, j, t0);
         if (e1 < entries) ntk_write(K, B, i1, j1, t1);
       }
       return;
     }
-    const int e = threadIdx.x / runs, run = threadIdx.x % runs, per = (shares + runs - 1) / runs, first = min(shares, run * per);
-    const int x = ntk_triangle(parts, B, min(e, entries - 1), i, j);
+    const int run = threadIdx.x % runs, per = (shares + runs - 1) / runs, first = min(shares, run * per);
     double* sums = reinterpret_cast<double*>(smem_cta);
     sums[threadIdx.x] = ntk_sum<16>(part + x, parts.doubles, first, min(shares, first + per));
     __syncthreads();
-    if (e >= entries || run != 0) return;
+    if (mine >= entries || run != 0) return;
     double v = 0.0;
     for (int k = 0; k < runs; ++k) v += sums[threadIdx.x + k];
     ntk_write(K, B, i, j, v);
