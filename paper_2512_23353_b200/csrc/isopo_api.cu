@@ -522,27 +522,20 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
       return f32_combine((const float*)(w + L.off_G), (int64_t)d_in * d_out, L.n_pad, B, coeffs, dW, beta, tag_dev, tag, info, st);
     return bf16_combine(w + L.off_G, L, d_in, d_out, B, coeffs, dW, beta, tag_dev, tag, store_fmt(L, B, ws), info, st);
   }
-  // GEMM over all tokens: refresh the token -> sequence map so the call also works on its own.  The kernels add their
-  // token slabs into dW.
-  const Clear clear = beta == 0.f ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
+  // GEMM over all tokens; the offsets travel again so that the call also works on its own
+  const bool add = beta != 0.f;
   int64_t* off_dev = (int64_t*)(w + L.off_offsets);
-  int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
-  float* tokscale = (float*)tokseq;  // one scale per token: a single independent load per row
+  float* tokscale = (float*)(w + L.off_tokseq);  // one scale per token: a single independent load per row
   if (dtype == ISOPO_F32) {
-    s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);
+    s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, add ? Clear{} : Clear{{dW}, {(int64_t)d_in * d_out}}, st);
     if (s != ISOPO_OK) return s;
     return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, tokscale, dW, st);
   }
-  if (bf16_weight_grad_fold_applies(T, d_in, d_out, B)) {
-    s = launch_offsets(seq_offsets_host, B, off_dev, clear, st);
-    if (s != ISOPO_OK) return s;
-    return bf16_weight_grad_fold(X, dY, T, d_in, d_out, off_dev, coeffs, B, dW, info, st);
-  }
+  if (bf16_weight_grad_fold_applies(T, d_in, d_out, B))
+    return bf16_weight_grad_fold(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, dW, add, info, st);
   if (bf16_weight_grad_uses_pairs(d_out))
-    return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, clear, info, st);
-  s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, clear, st);
-  if (s != ISOPO_OK) return s;
-  return bf16_weight_grad(X, dY, T, d_in, d_out, tokscale, dW, info, st);
+    return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, add, info, st);
+  return bf16_weight_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, info, st);
 }
 
 }  // extern "C"

@@ -290,8 +290,7 @@ isopo_status mirror_upper(float* K, int B, cudaStream_t st);
 isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out, int B, const float* coeffs, float* dW,
                           float beta, const WsTag* tag_dev, const WsTag& tag, const StoreFmt& fmt, int32_t* info,
                           cudaStream_t st);
-// The Gram, sampled and weight-gradient kernels ADD into K, M^T and dW: the caller has cleared them on this stream (or wants
-// the sum).
+// The Gram and sampled kernels ADD into K and M^T: the caller has cleared them on this stream.
 isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                        float* K, int32_t* info, cudaStream_t st);
 // 2-CTA tiles, one projection or several that share X: where they pay
@@ -300,24 +299,32 @@ isopo_status bf16_gram_pair(const void* X, const void* const* dY, int64_t T, int
                             const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
-// 1-CTA tiles, operand rows scaled in shared memory
-isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              float* dW, int32_t* info, cudaStream_t st);
+// The stand-alone weight gradients prepare what they need (offsets through off_dev, a cleared dW where its shares are added up);
+// `add`: dW is added to.
+// 1-CTA tiles, operand rows scaled in shared memory by the scales per token that a launch ahead leaves in `tokscale`
+isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                              int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add, int32_t* info,
+                              cudaStream_t st);
 bool bf16_weight_grad_uses_pairs(int d_out);
 
 // dW with the per-sequence coefficient applied when a segment's accumulator is drained (no scaled operand copy)
 bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);
-isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st);
+isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                   int64_t* off_dev, const float* coeffs, int B, float* dW, bool add, int32_t* info, cudaStream_t st);
 // a scaled copy of the narrower operand, then a plain GEMM in 2-CTA tiles
-// (the offsets travel with the scaling pass, through off_dev above 383 sequences; `clear` is cleared ahead of it all)
+// (the offsets travel with the scaling pass, through off_dev above 383 sequences)
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, const Clear& clear,
-                                   int32_t* info, cudaStream_t st);
-// plain GEMM with equal runs of stages per pair, and its modelled time in stages of 256 columns
-isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, float* dW, int32_t* info,
-                                    cudaStream_t st);
-long long bf16_weight_grad_plain_cost(int64_t T, int d_in, int d_out, int pairs);
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, bool add, int32_t* info,
+                                   cudaStream_t st);
+// plain GEMM in runs of stages per pair; modelled time in stages of 256 columns
+struct PlainPlan {
+  long long run, cost;
+  bool wide;   // dW allows 32-byte accesses
+  bool clear;  // dW has to be cleared ahead of it
+};
+PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, const float* dW, bool add, int pairs);
+isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
+                                    float* dW, int32_t* info, cudaStream_t st);
 
 // token-sampled estimator of Algorithm 1
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,

@@ -52,6 +52,7 @@ struct SeqGradParams {
   float* dW;
   int64_t T, slab;  // tokens per work unit (a multiple of 64)
   int nslabs, d_in, d_out;
+  bool store;       // one slab: dW is written, nothing has cleared it
   PieceGrid grid;   // per-sequence mode
 };
 
@@ -260,7 +261,19 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
           uint32_t r[32];
           tmem_ld32(taddr + jc * 32, r);
           tmem_ld_wait();
-          if (m < p.d_out) {
+          if (p.store) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const int n = n0 + jc * 32 + v * 8;
+              if (m < p.d_out && n < p.d_in &&
+                  ISOPO_IN_RANGE((long long)m * p.d_in + n + 7, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad)) {
+                float o[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = __uint_as_float(r[v * 8 + e]);
+                st_global_8(dst + jc * 32 + v * 8, o);
+              }
+            }
+          } else if (m < p.d_out) {
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
               const int n = n0 + jc * 32 + v * 4;
@@ -374,14 +387,12 @@ bool bf16_weight_grad_uses_pairs(int d_out) {
   return tiles_m % 2 == 0 || tiles_m >= 7;
 }
 
-isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const float* tokscale,
-                              float* dW, int32_t* info, cudaStream_t st) {
-  CUtensorMap mapY, mapX;
-  isopo_status s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out);
-  if (s != ISOPO_OK) return s;
+isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                              int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add, int32_t* info,
+                              cudaStream_t st) {
   int sms = 0;
-  if ((s = sm_count(&sms)) != ISOPO_OK) return s;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  isopo_status s = sm_count(&sms);
+  if (s != ISOPO_OK) return s;
   SeqGradParams p{};
   p.tiles_m = (d_out + kTileM - 1) / kTileM;
   p.tiles_n = (d_in + kTileN - 1) / kTileN;
@@ -396,6 +407,12 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   const long long nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;
   p.nslabs = (int)nslabs;
+  p.store = !add && nslabs == 1 && ((uintptr_t)dW & 31) == 0;
+  const Clear clear = !add && !p.store ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
+  if ((s = launch_tokscale(off_host, B, T, off_dev, coeffs, tokscale, clear, st)) != ISOPO_OK) return s;
+  CUtensorMap mapY, mapX;
+  if ((s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   const int grid = (int)std::min<long long>(tiles * nslabs, sms);
   {
     LaunchScope scope(kIdWeightGrad, st);

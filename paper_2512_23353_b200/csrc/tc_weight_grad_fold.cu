@@ -64,6 +64,8 @@ struct FoldParams {
   int32_t* info;
   int kblocks;            // kPlain: stages of one tile; a pair's run is `run` stages of ptiles * kblocks
   long long run;
+  int beta;               // kPlain, 0: a tile that one pair sums alone is written, not added to
+  bool wide;              // kPlain: dW allows 32-byte accesses
 };
 
 // Tiles are visited in groups of `group_m` rows, row index fastest inside a group, so that the pairs
@@ -298,45 +300,95 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     const int q = warp & 3;            // TMEM lane quarter this warp may read
     const int h = (warp - 2) >> 2;     // column half of the tile
     const uint32_t accempty_at_leader = map_to_cta(accempty_bar(0), 0);
-    float sum[128];
-#pragma unroll
-    for (int e = 0; e < 128; ++e) sum[e] = 0.f;
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    while (ok && work.next(p, tile, t0, t1)) {
-      int ptm, tn;
-      pair_tile(tile, p, ptm, tn);
-      for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done(); w.next()) {
-        const float c = kPlain ? 1.f : ISOPO_IN_RANGE(w.i, p.B, p.info, kIdWeightGrad) ? s_coef[w.i] : 0.f;
-        if (!(ok = mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
+    if (kPlain) {
+      // A piece of work is one segment: from tensor memory straight to dW.  The loop stays rolled: its code is fetched anew in every
+      // launch and runs once or twice (unrolled, with the sums in registers as below, 896 x 896 of 1000 tokens took 18.2 us, not 14.8).
+      while (work.next(p, tile, t0, t1)) {
+        int ptm, tn;
+        pair_tile(tile, p, ptm, tn);
+        const int m = (2 * ptm + (int)rank) * kHalf + q * 32 + lane, n0 = tn * kPairN + h * 128;
+        float* const dst = p.dW + (size_t)m * p.d_in + n0;
+        const bool own = t0 == 0 && t1 == (int)p.T && p.wide;  // the whole of this tile: nobody else's
+        if (own && p.beta && m < p.d_out) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            if (n0 + v * 32 < p.d_in) asm volatile("prefetch.global.L2 [%0];" ::"l"(dst + v * 32));
+        }
+        if (!mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdWeightGrad)) break;
         tc_fence_after_sync();
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairN + h * 128);
-#pragma unroll
+#pragma unroll 1
         for (int jc = 0; jc < 8; ++jc) {
           uint32_t r[16];
           tmem_ld16(taddr + jc * 16, r);
-          tmem_ld_wait();
+          const int n = n0 + jc * 16;
+          const auto live = [&](int v, int last) {  // d_in is a multiple of 8, so a group of 4 or 8 is all in or all out
+            return m < p.d_out && n + v < p.d_in &&
+                   ISOPO_IN_RANGE((long long)m * p.d_in + n + v + last, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad);
+          };
+          if (own) {
+            float o[2][8] = {};
 #pragma unroll
-          for (int e = 0; e < 16; ++e) sum[jc * 16 + e] = fmaf(c, __uint_as_float(r[e]), sum[jc * 16 + e]);
+            for (int u = 0; u < 2; ++u)
+              if (p.beta && live(u * 8, 7)) ld_global_8(dst + jc * 16 + u * 8, o[u]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) o[u][e] = p.beta ? o[u][e] + __uint_as_float(r[u * 8 + e]) : __uint_as_float(r[u * 8 + e]);
+              if (live(u * 8, 7)) st_global_8(dst + jc * 16 + u * 8, o[u]);
+            }
+          } else {
+            tmem_ld_wait();
+#pragma unroll
+            for (int v = 0; v < 16; v += 4)
+              if (live(v, 3)) red_global_4(dst + jc * 16 + v, __uint_as_float(r[v]), __uint_as_float(r[v + 1]), __uint_as_float(r[v + 2]), __uint_as_float(r[v + 3]));
+          }
         }
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive_remote(accempty_at_leader + 8u * acc);
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
-      if (!ok) break;
-      // the unit's share of this tile: dW[m, n0 .. n0 + 127] += sum
-      const int m = (2 * ptm + (int)rank) * kHalf + q * 32 + lane, n0 = tn * kPairN + h * 128;
-      float* dst = p.dW + (size_t)m * p.d_in + n0;
+    } else {
+      float sum[128];
 #pragma unroll
-      for (int v = 0; v < 32; ++v) {
-        if (m < p.d_out && n0 + v * 4 < p.d_in &&  // d_in is a multiple of 8, so a group of 4 is all in or all out
-            ISOPO_IN_RANGE((long long)m * p.d_in + n0 + v * 4 + 3, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad))
-          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + v * 4), "f"(sum[v * 4 + 0]),
-                       "f"(sum[v * 4 + 1]), "f"(sum[v * 4 + 2]), "f"(sum[v * 4 + 3])
-                       : "memory");
-        sum[v * 4 + 0] = sum[v * 4 + 1] = sum[v * 4 + 2] = sum[v * 4 + 3] = 0.f;
+      for (int e = 0; e < 128; ++e) sum[e] = 0.f;
+      while (ok && work.next(p, tile, t0, t1)) {
+        int ptm, tn;
+        pair_tile(tile, p, ptm, tn);
+        for (SegWalk<kPlain> w(s_off, p.B, t0, t1); !w.done(); w.next()) {
+          const float c = ISOPO_IN_RANGE(w.i, p.B, p.info, kIdWeightGrad) ? s_coef[w.i] : 0.f;
+          if (!(ok = mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdWeightGrad))) break;
+          tc_fence_after_sync();
+          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairN + h * 128);
+#pragma unroll
+          for (int jc = 0; jc < 8; ++jc) {
+            uint32_t r[16];
+            tmem_ld16(taddr + jc * 16, r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sum[jc * 16 + e] = fmaf(c, __uint_as_float(r[e]), sum[jc * 16 + e]);
+          }
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote(accempty_at_leader + 8u * acc);
+          if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
+        if (!ok) break;
+        // the unit's share of this tile: dW[m, n0 .. n0 + 127] += sum
+        const int m = (2 * ptm + (int)rank) * kHalf + q * 32 + lane, n0 = tn * kPairN + h * 128;
+        float* dst = p.dW + (size_t)m * p.d_in + n0;
+#pragma unroll
+        for (int v = 0; v < 32; ++v) {
+          if (m < p.d_out && n0 + v * 4 < p.d_in &&  // d_in is a multiple of 8, so a group of 4 is all in or all out
+              ISOPO_IN_RANGE((long long)m * p.d_in + n0 + v * 4 + 3, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad))
+            red_global_4(dst + v * 4, sum[v * 4 + 0], sum[v * 4 + 1], sum[v * 4 + 2], sum[v * 4 + 3]);
+          sum[v * 4 + 0] = sum[v * 4 + 1] = sum[v * 4 + 2] = sum[v * 4 + 3] = 0.f;
+        }
       }
     }
   } else {
@@ -438,27 +490,42 @@ static void set_group(FoldParams* p, int npairs) {
   p->group_m = std::max(1, std::min(g, p->ptiles_m));
 }
 
-long long bf16_weight_grad_plain_cost(int64_t T, int d_in, int d_out, int pairs) {
+// Tiles whose sums one pair holds alone are written without a clear ahead of them and without a read of what is there: where a
+// tile has few stages, whole tiles per pair; where it has many, equal runs of stages, whose ends meet other runs in dW.
+// All in us, runs / whole tiles: 169 tokens, 3584 x 10752 140 / 44 (clear, then additions to 154 MB, against one pass of stores:
+// 3.5 TB/s), 3584 x 3584 41 / 22; 1097, 2560 x 10240 118 / 55; 2925, 2560 x 12928 204 / 169; 300, 896 x 896 12.5 / 11.5.
+// Adding (beta = 1) to what is there by loads and stores: only where dW is larger than the L2 and its tiles short, 169 tokens,
+// 3584 x 10752 140 / 95..118, but 2925, 2560 x 12928 185 / 189 and 300, 896 x 896 13.0 / 16.8.
+constexpr int kStoreStages = 8;  // stages that writing a tile takes at least, beside the MMAs of the next
+constexpr int64_t kBigWeights = (int64_t)1 << 24;
+PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, const float* dW, bool add, int pairs) {
+  PlainPlan plan{};
   const long long ptiles = (long long)((d_out + 2 * kHalf - 1) / (2 * kHalf)) * ((d_in + kPairN - 1) / kPairN);
-  const long long kblocks = (T + kKB - 1) / kKB, run = (ptiles * kblocks + pairs - 1) / pairs;
-  return run + (run / kblocks + 2) * kUnitOverhead;  // a run touches up to run / kblocks + 2 tiles
+  const long long kblocks = (T + kKB - 1) / kKB, stages = ptiles * kblocks;
+  plan.wide = ((uintptr_t)dW & 31) == 0 && (!add || (kblocks <= kStoreStages && (int64_t)d_in * d_out > kBigWeights));
+  // no shorter runs than a drain takes
+  plan.run = std::max<long long>((stages + pairs - 1) / pairs, std::min<long long>(kUnitOverhead, kblocks));
+  plan.cost = plan.run + (plan.run / kblocks + 2) * kUnitOverhead;  // a run touches up to run / kblocks + 2 tiles
+  const long long tiles = (ptiles + pairs - 1) / pairs, whole = tiles * std::max<long long>(kblocks, kStoreStages) + kUnitOverhead;
+  if (plan.wide && whole <= plan.cost) { plan.run = tiles * kblocks; plan.cost = whole; }
+  plan.clear = !add && !(plan.wide && plan.run % kblocks == 0);
+  return plan;
 }
 
-isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, float* dW, int32_t* info,
-                                    cudaStream_t st) {
+isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
+                                    float* dW, int32_t* info, cudaStream_t st) {
   int pairs = 0;
   isopo_status s = resident_pairs<true>(&pairs);
   if (s != ISOPO_OK) return s;
   CUtensorMap mapY, mapX;
   if ((s = make_fold_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
   FoldParams p{};
-  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info;
+  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add; p.wide = plan.wide;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
   p.tiles_n = (d_in + kPairN - 1) / kPairN;
   p.kblocks = (int)((T + kKB - 1) / kKB);
+  p.run = plan.run;
   const long long stages = (long long)p.ptiles_m * p.tiles_n * p.kblocks;
-  // no shorter runs than a drain takes
-  p.run = std::max<long long>((stages + pairs - 1) / pairs, std::min<long long>(kUnitOverhead, p.kblocks));
   const int npairs = (int)((stages + p.run - 1) / p.run);
   set_group(&p, npairs);
   {
@@ -469,8 +536,8 @@ isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, in
   return ISOPO_OK;
 }
 
-isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_dev,
-                                   const float* coeffs, int B, float* dW, int32_t* info, cudaStream_t st) {
+isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                   int64_t* off_dev, const float* coeffs, int B, float* dW, bool add, int32_t* info, cudaStream_t st) {
   int pairs = 0;
   isopo_status s = resident_pairs<false>(&pairs);
   if (s != ISOPO_OK) return s;
@@ -498,6 +565,7 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   p.nchunks = (int)nchunks;
   const int npairs = (int)std::max<long long>(1, std::min<long long>(ptiles * nchunks, (long long)pairs));
   set_group(&p, npairs);
+  if ((s = launch_offsets(off_host, B, off_dev, add ? Clear{} : Clear{{dW}, {(int64_t)d_in * d_out}}, st)) != ISOPO_OK) return s;
   {
     LaunchScope scope(kIdWeightGrad, st);
     launch(k_bf16_weight_grad_fold<false>, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);

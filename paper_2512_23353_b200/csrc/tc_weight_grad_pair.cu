@@ -51,6 +51,7 @@ struct FoldedPairParams {
   int nslabs, d_in, d_out;
   int ptiles_m, tiles_n;  // 256-row blocks of d_out; 512-column blocks of d_in
   int32_t* info;
+  bool store;  // a block is one unit's alone: it is written, nothing has cleared it
 };
 
 // Columns of the left / right accumulator of block column tn that exist, in the 32-column steps of a 2-CTA MMA (see
@@ -193,7 +194,19 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
         uint32_t r[32];
         tmem_ld32(taddr + jc * 32, r);
         tmem_ld_wait();
-        if (m < p.d_out) {
+        if (p.store) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int n = n0 + jc * 32 + v * 8;
+            if (m < p.d_out && n < p.d_in &&
+                ISOPO_IN_RANGE((long long)m * p.d_in + n + 7, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad)) {
+              float o[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) o[e] = __uint_as_float(r[v * 8 + e]);
+              st_global_8(dst + jc * 32 + v * 8, o);
+            }
+          }
+        } else if (m < p.d_out) {
 #pragma unroll
           for (int v = 0; v < 8; ++v) {
             const int n = n0 + jc * 32 + v * 4;
@@ -277,40 +290,11 @@ __global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ sr
 }  // namespace
 
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, const Clear& clear,
-                                   int32_t* info, cudaStream_t st) {
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, bool add, int32_t* info,
+                                   cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  {  // scale the narrower operand into `scaled`
-    const bool scale_y = d_out <= d_in;
-    const int d8 = (scale_y ? d_out : d_in) / 8;
-    const uint4* src = (const uint4*)(scale_y ? dY : X);
-    int64_t ctas = (T + 7) / 8;
-    // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
-    // 4000 tokens a 4096 x 4096 dW took 10 us longer than from a kernel of its own, hence a CTA for every 16 KB as well.
-    if (B + 1 <= kArgChunk) {
-      OffsetArgs<kArgChunk> a;
-      fill_offsets(&a, off_host, B + 1);
-      ctas = std::max(ctas, clear.n[0] / 4096);
-      LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows<true>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, a, off_dev, B, coeffs, T, d8,
-             (uint4*)scaled, clear);
-    } else {
-      isopo_status s = launch_offsets(off_host, B, off_dev, clear, st);
-      if (s != ISOPO_OK) return s;
-      LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows<false>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, OffsetArgs<1>{}, off_dev, B,
-             coeffs, T, d8, (uint4*)scaled, Clear{});
-    }
-    ISOPO_CUDA_TRY(cudaGetLastError());
-    if (scale_y) dY = scaled; else X = scaled;
-  }
-  CUtensorMap mapY, mapX;
-  isopo_status s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
-  if (s != ISOPO_OK) return s;
-  s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
-  if (s != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   static int resident_pairs[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
@@ -350,12 +334,44 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
   // places.  10,496 tokens, 896 x 4864 (121 MB) 100 -> 84 us, 4864 x 896 102 -> 74 us; 40,960 tokens, 896 x 896 (147 MB)
   // 67 -> 94 us, 35,200 tokens, 896 x 4864 (405 MB) 301 -> 445 us.
   const bool in_l2 = 2.0 * (double)T * (d_in + d_out) <= 128e6;
-  if (in_l2 && 10 * bf16_weight_grad_plain_cost(T, d_in, d_out, (int)pairs) < 9 * 2 * best)
-    return bf16_weight_grad_plain(X, dY, T, d_in, d_out, dW, info, st);
+  const PlainPlan plan = plan_weight_grad_plain(T, d_in, d_out, dW, add, (int)pairs);
+  const bool plain = in_l2 && 10 * plan.cost < 9 * 2 * best;
   const long long kb_per = (kblocks + nslabs - 1) / nslabs;
   nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;
   p.nslabs = (int)nslabs;
+  p.store = !add && nslabs == 1 && ((uintptr_t)dW & 31) == 0;
+  const Clear clear = !add && (plain ? plan.clear : !p.store) ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
+  {  // scale the narrower operand into `scaled`
+    const bool scale_y = d_out <= d_in;
+    const int d8 = (scale_y ? d_out : d_in) / 8;
+    const uint4* src = (const uint4*)(scale_y ? dY : X);
+    int64_t ctas = (T + 7) / 8;
+    // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
+    // 4000 tokens a 4096 x 4096 dW took 10 us longer than from a kernel of its own, hence a CTA for every 16 KB as well.
+    if (B + 1 <= kArgChunk) {
+      OffsetArgs<kArgChunk> a;
+      fill_offsets(&a, off_host, B + 1);
+      ctas = std::max(ctas, clear.n[0] / 4096);
+      LaunchScope scope(kIdScaleRows, st);
+      launch(k_scale_rows<true>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, a, off_dev, B, coeffs, T, d8,
+             (uint4*)scaled, clear);
+    } else {
+      isopo_status s = launch_offsets(off_host, B, off_dev, clear, st);
+      if (s != ISOPO_OK) return s;
+      LaunchScope scope(kIdScaleRows, st);
+      launch(k_scale_rows<false>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, OffsetArgs<1>{}, off_dev, B,
+             coeffs, T, d8, (uint4*)scaled, Clear{});
+    }
+    ISOPO_CUDA_TRY(cudaGetLastError());
+    if (scale_y) dY = scaled; else X = scaled;
+  }
+  if (plain) return bf16_weight_grad_plain(X, dY, T, d_in, d_out, plan, add, dW, info, st);
+  CUtensorMap mapY, mapX;
+  isopo_status s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
+  if (s != ISOPO_OK) return s;
+  s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
+  if (s != ISOPO_OK) return s;
   const int npairs = (int)std::max<long long>(1, std::min<long long>(ptiles * nslabs, pairs));
   {
     LaunchScope scope(kIdWeightGrad, st);
