@@ -219,6 +219,13 @@ isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, i
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const long long tiles = (T + kTT - 1) / kTT;
+  const int ctas = gram_split_ctas(tiles * (tiles + 1) / 2 * n_heads, d_in, *std::min_element(d_out, d_out + n_heads), sms);
+  if (ctas > 1) {
+    isopo_status r = bf16_gram_split(ctas, X, dY, T, d_in, d_out, n_heads, tokseq, B, K, false, info, st);
+    for (int h = 0; h < n_heads && r == ISOPO_OK; ++h) r = mirror_upper(K[h], B, st);
+    return r;
+  }
   if (bf16_gram_pair_pays(T, d_in, d_out, n_heads, sms))
     return bf16_gram_pair(X, dY, T, d_in, d_out, n_heads, tokseq, B, K, info, st);
   CUtensorMap mapX, mapY[kMaxHeads];
