@@ -325,10 +325,9 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
 // plain GEMM in runs of stages per pair; modelled time in stages of 256 columns
 struct PlainPlan {
   long long run, cost;
-  bool wide;   // dW allows 32-byte accesses
   bool clear;  // dW has to be cleared ahead of it
 };
-PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, const float* dW, bool add, int pairs);
+PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, bool add, int pairs);
 isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
                                     float* dW, int32_t* info, cudaStream_t st);
 

@@ -63,6 +63,10 @@ __host__ __device__ __forceinline__ size_t stored_slot(size_t piece, int i, int 
 isopo_status make_map_2d_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t row_stride_elems,
                               uint32_t box_cols, uint32_t box_rows);
 
+// Row-major float32 matrix [rows, cols], cols a multiple of 4, in boxes of 32 rows x `box_cols` (16 or 32: 64- or 128-byte swizzle):
+// what a warp adds or writes.
+isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64_t cols, uint32_t box_cols);
+
 // Stored per-sequence gradients viewed as (x = element inside a 256-element piece row, y = sequence,
 // z = piece): boxes of 64 elements x `box_rows` sequences x `box_pieces` pieces, 128-byte swizzle.  Sequences
 // past B and pieces past the last read as zero.
@@ -164,6 +168,31 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const CUtens
       ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+// A box from shared memory to where it stands in global memory, written or added; what lies outside the matrix is left out.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, uint32_t src_smem) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(src_smem)
+               : "memory");
+}
+__device__ __forceinline__ void tma_add_2d(const CUtensorMap* map, int x, int y, uint32_t src_smem) {
+  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.bulk_group [%0, {%1, %2}], [%3];"
+               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(src_smem)
+               : "memory");
+}
+// Lane's row of a 32-row box in shared memory (`box`, a multiple of 1024 bytes), its 16-byte groups where the tensor map's swizzle
+// has them; no bank conflicts.
+__device__ __forceinline__ void box_row(uint32_t box, int lane, const uint32_t (&r)[32]) {
+#pragma unroll
+  for (int v = 0; v < 8; ++v)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(box + lane * 128 + ((v ^ (lane & 7)) << 4)), "r"(r[4 * v]),
+                 "r"(r[4 * v + 1]), "r"(r[4 * v + 2]), "r"(r[4 * v + 3]) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void bulk_wait_read() {  // all but the last kPending groups of this thread have read their source
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kPending) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // generic-proxy writes to shared memory -> visible to the async proxy (TMA, tcgen05.mma)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -326,22 +355,6 @@ __device__ __forceinline__ void mirror_by_cta(float* K, int B, int r, Diag diag,
       else if (set_diag && e < total && j == i) K[e] = diag(i);
     }
   }
-}
-
-// eight floats at a 32-byte boundary: a whole sector per lane, where the lanes of a warp lie a row apart
-__device__ __forceinline__ void st_global_8(float* at, const float (&v)[8]) {
-  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(at), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
-               "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-               : "memory");
-}
-__device__ __forceinline__ void red_global_4(float* at, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
-__device__ __forceinline__ void ld_global_8(const float* at, float (&v)[8]) {
-  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-               : "l"(at)
-               : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {

@@ -37,7 +37,9 @@ constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kChunkBytes = kKB * 128;                 // one [64 tokens][64 cols] box
 constexpr int kMaxSeqs = 256;                          // sequences whose extents are staged in shared memory
 constexpr int kSeqInfoBytes = kMaxSeqs * 16 + kIntakeRawBytes;  // int64 first token, int32 length, int32 index; scratch
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kSeqInfoBytes;
+template <bool kFolded>  // behind the barriers: extents of the sequences, or folded mode two 32 x 32 boxes of each epilogue warp
+constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + (kFolded ? 1024 + 4 * 8192 : 256 + kSeqInfoBytes);
+static_assert(kSmemBytes<true> <= 227 * 1024, "shared memory");
 constexpr int kThreads = 192;
 constexpr int kThreadsFolded = 320;                    // + 4 warps that scale the dY rows
 constexpr uint32_t kTmemCols = 512;                    // two 256-column float32 accumulators
@@ -94,7 +96,8 @@ template <> struct IntakeOf<true> { typedef NoIntake type; };
 
 template <bool kFolded>
 __global__ void __launch_bounds__(kFolded ? kThreadsFolded : kThreads, 1)
-k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX, SeqGradParams p,
+k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX,
+                const __grid_constant__ CUtensorMap mapW /* dW, folded mode */, SeqGradParams p,
                 const __grid_constant__ typename IntakeOf<kFolded>::type in) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -221,7 +224,9 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
   } else if (warp < 6) {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
     const int q = warp & 3;  // TMEM lane quarter this warp may read
-    const int row = q * 32 + lane;
+    const uint32_t boxes = smem_base + kStages * kStageBytes + 1024 + (warp - 2) * 8192;  // folded mode
+    const bool issuer = elect_one();
+    uint32_t turn = 0;  // the box that is filled next
     int acc = 0;
     uint32_t acc_phase = 0;
     for (long long u = blockIdx.x; u < total_units; u += gridDim.x) {
@@ -253,38 +258,27 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
           }
         }
       } else {
-        // dW[m, n0 .. n0+255] += accumulator row; token slabs of one tile meet here, hence atomics
-        const int m = (tile / p.tiles_n) * kTileM + row, n0 = (tile % p.tiles_n) * kTileN;
-        float* dst = p.dW + (size_t)m * p.d_in + n0;
+        // dW[m .. m+31, n0 .. n0+255] += the warp's rows; token slabs of one tile meet here, hence additions.  By TMA, 32 rows of 128
+        // bytes at a time, not red.v4: 4000 tokens, 512 x 1000 16.8 -> 13.6 us, 1586, 1000 x 328 13.3 -> 12.0, 15,000, 1848 x 88 23.6 ->
+        // 22.8; 46,546, 256 x 592, 59 slabs to a tile, 39.0 -> 40.6.
+        const int m = (tile / p.tiles_n) * kTileM + q * 32, n0 = (tile % p.tiles_n) * kTileN;
 #pragma unroll 2
-        for (int jc = 0; jc < kTileN / 32; ++jc) {
+        for (int jc = 0; jc < kTileN / 32 && n0 + jc * 32 < p.d_in; ++jc) {
           uint32_t r[32];
           tmem_ld32(taddr + jc * 32, r);
+          if (issuer) bulk_wait_read<1>();  // of the two boxes that this warp fills in turn
+          __syncwarp();
           tmem_ld_wait();
-          if (p.store) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              const int n = n0 + jc * 32 + v * 8;
-              if (m < p.d_out && n < p.d_in &&
-                  ISOPO_IN_RANGE((long long)m * p.d_in + n + 7, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad)) {
-                float o[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) o[e] = __uint_as_float(r[v * 8 + e]);
-                st_global_8(dst + jc * 32 + v * 8, o);
-              }
-            }
-          } else if (m < p.d_out) {
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              const int n = n0 + jc * 32 + v * 4;
-              if (n < p.d_in &&  // d_in is a multiple of 8, so a group of 4 is all in or all out
-                  ISOPO_IN_RANGE((long long)m * p.d_in + n + 3, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad))
-                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + jc * 32 + v * 4),
-                             "f"(__uint_as_float(r[v * 4 + 0])), "f"(__uint_as_float(r[v * 4 + 1])),
-                             "f"(__uint_as_float(r[v * 4 + 2])), "f"(__uint_as_float(r[v * 4 + 3]))
-                             : "memory");
-            }
+          const uint32_t box = boxes + turn * 4096;
+          box_row(box, lane, r);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (issuer && m < p.d_out) {
+            if (p.store) tma_store_2d(&mapW, n0 + jc * 32, m, box);
+            else tma_add_2d(&mapW, n0 + jc * 32, m, box);
           }
+          if (issuer) bulk_commit();
+          turn ^= 1u;
         }
       }
       tc_fence_before_sync();
@@ -292,6 +286,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
       if (lane == 0) mbar_arrive(accempty_bar(acc));
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+    if (kFolded && issuer) bulk_wait_all();
   } else if (kFolded) {
     // ------------------------------------------------------------------ scaler (warps 6..9)
     // Thread (r, h): token row r of the stage, half h of each 128-byte row, in both dY chunks.
@@ -367,7 +362,7 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   if (s != ISOPO_OK) return s;
   int sms = 0;
   if ((s = sm_count(&sms)) != ISOPO_OK) return s;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<false>));
   SeqGradParams p{};
   p.G = (__nv_bfloat16*)G; p.n_pad = L.n_pad; p.B = B; p.tiles_m = L.tiles_m; p.tiles_n = L.tiles_n;
   p.info = info; p.d_in = d_in; p.d_out = d_out; p.grid = piece_grid(d_in, d_out);
@@ -375,7 +370,7 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   const int grid = (int)std::min<long long>(units, sms);
   {
     LaunchScope scope(kIdSeqGrad, st);
-    launch(k_bf16_seq_grad<false>, grid, kThreads, kSmemBytes, st, mapY, mapX, p, in);
+    launch(k_bf16_seq_grad<false>, grid, kThreads, kSmemBytes<false>, st, mapY, mapX, mapX, p, in);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -407,16 +402,18 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   const long long nslabs = (kblocks + kb_per - 1) / kb_per;
   p.slab = kb_per * kKB;
   p.nslabs = (int)nslabs;
-  p.store = !add && nslabs == 1 && ((uintptr_t)dW & 31) == 0;
+  p.store = !add && nslabs == 1;
   const Clear clear = !add && !p.store ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
   if ((s = launch_tokscale(off_host, B, T, off_dev, coeffs, tokscale, clear, st)) != ISOPO_OK) return s;
   CUtensorMap mapY, mapX;
   if ((s = make_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  CUtensorMap mapW;
+  if ((s = make_map_2d_f32(&mapW, dW, (uint64_t)d_out, (uint64_t)d_in, 32)) != ISOPO_OK) return s;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_seq_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<true>));
   const int grid = (int)std::min<long long>(tiles * nslabs, sms);
   {
     LaunchScope scope(kIdWeightGrad, st);
-    launch(k_bf16_seq_grad<true>, grid, kThreadsFolded, kSmemBytes, st, mapY, mapX, p, NoIntake{});
+    launch(k_bf16_seq_grad<true>, grid, kThreadsFolded, kSmemBytes<true>, st, mapY, mapX, mapW, p, NoIntake{});
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -10,7 +10,10 @@
 // accumulator, multiply by the sequence's coefficient and add into a running sum that lives in
 // REGISTERS (8 warps x 32 lanes x 128 columns = the CTA's 128 x 256 half of the tile) while the MMA
 // thread is already filling the other accumulator with the next segment.  At the end of the unit
-// the running sum is added into dW (float32 reductions: the token chunks of one tile meet there).
+// the running sum is added into dW (float32 additions: the token chunks of one tile meet there), as boxes of 32 rows that TMA adds
+// from shared memory: rows of 64 or 128 bytes at a time.  With red.v4 from the registers every instruction touched 32 rows, 16
+// bytes of each: 1000 tokens, 896 x 896 14.7 -> 12.9 us, 40,706 66.8 -> 63.5, 9000 tokens, 1536 x 1536 39.3 -> 37.3; kPlain, 10,533
+// tokens, 896 x 896 31.4 -> 29.7, 4864 x 896 82.1 -> 78.1.
 // The tile never leaves the SM between segments, so against the pre-scaled-operand GEMM this saves one
 // pass over the narrower operand (read + write) and its launch.
 //
@@ -45,13 +48,16 @@ constexpr int kOperandBytes = 2 * kChunkBytes;       // this CTA's half of dY or
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kMaxSeqs = 2048;                       // sequences whose extents and coefficients are staged in shared memory
 constexpr int kOffBytes = (kMaxSeqs + 1 + 63) / 64 * 64 * 4;
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers*/ + kOffBytes + kMaxSeqs * 4;
 constexpr int kEpiWarps = 8;
+template <bool kPlain>  // what an epilogue warp passes to dW at a time: 32 rows of 32 or 16 columns
+constexpr int kBoxBytes = kPlain ? 4096 : 2048;
+template <bool kPlain>
+constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/ + kEpiWarps * kBoxBytes<kPlain> + (kPlain ? 0 : kOffBytes + kMaxSeqs * 4);
 constexpr int kThreads = 32 * (2 + kEpiWarps + 1);
 constexpr uint32_t kTmemCols = 512;                  // two 256-column float32 accumulators
 constexpr int kPairN = 256;
 constexpr int kUnitOverhead = 6;                     // a unit's pipeline fill and flush, in stages (host cost model)
-static_assert(kSmemBytes <= 227 * 1024, "shared memory");
+static_assert(kSmemBytes<true> <= 227 * 1024 && kSmemBytes<false> <= 227 * 1024, "shared memory");
 
 struct FoldParams {
   const int64_t* off;    // [B + 1] token offsets
@@ -65,7 +71,6 @@ struct FoldParams {
   int kblocks;            // kPlain: stages of one tile; a pair's run is `run` stages of ptiles * kblocks
   long long run;
   int beta;               // kPlain, 0: a tile that one pair sums alone is written, not added to
-  bool wide;              // kPlain: dW allows 32-byte accesses
 };
 
 // Tiles are visited in groups of `group_m` rows, row index fastest inside a group, so that the pairs
@@ -166,7 +171,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 
 template <bool kPlain>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX, FoldParams p) {
+k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapX,
+                        const __grid_constant__ CUtensorMap mapW, FoldParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
@@ -182,8 +188,8 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // offsets (as 32-bit token indices) and coefficients, read once: the roles look them up at every
   // segment, and a global load there would stall the MMA thread for longer than its queue of MMAs lasts
-  int* s_off = reinterpret_cast<int*>(smem + kStages * kStageBytes + 512);
-  float* s_coef = reinterpret_cast<float*>(smem + kStages * kStageBytes + 512 + kOffBytes);
+  int* s_off = reinterpret_cast<int*>(smem + kStages * kStageBytes + 1024 + kEpiWarps * kBoxBytes<kPlain>);
+  float* s_coef = reinterpret_cast<float*>(s_off + kOffBytes / 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();  // 0 issues the MMAs
@@ -303,49 +309,33 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
+    const uint32_t box = smem_base + kStages * kStageBytes + 1024 + (warp - 2) * kBoxBytes<kPlain>;
+    const bool issuer = elect_one();
     if (kPlain) {
       // A piece of work is one segment: from tensor memory straight to dW.  The loop stays rolled: its code is fetched anew in every
-      // launch and runs once or twice (unrolled, with the sums in registers as below, 896 x 896 of 1000 tokens took 18.2 us, not 14.8).
+      // launch and runs once or twice (unrolled, with the sums in registers as below, 1000 tokens of 896 x 896 took 18 us, not 15).
       while (work.next(p, tile, t0, t1)) {
         int ptm, tn;
         pair_tile(tile, p, ptm, tn);
-        const int m = (2 * ptm + (int)rank) * kHalf + q * 32 + lane, n0 = tn * kPairN + h * 128;
-        float* const dst = p.dW + (size_t)m * p.d_in + n0;
-        const bool own = t0 == 0 && t1 == (int)p.T && p.wide;  // the whole of this tile: nobody else's
-        if (own && p.beta && m < p.d_out) {
-#pragma unroll
-          for (int v = 0; v < 4; ++v)
-            if (n0 + v * 32 < p.d_in) asm volatile("prefetch.global.L2 [%0];" ::"l"(dst + v * 32));
-        }
+        const int m = (2 * ptm + (int)rank) * kHalf + q * 32, n0 = tn * kPairN + h * 128;
+        const bool store = t0 == 0 && t1 == (int)p.T && !p.beta;  // the whole of this tile, nobody else's
         if (!mbar_wait_pair(accfull_bar(acc), acc_phase, abort_flag, peer_abort, p.info, kIdWeightGrad)) break;
         tc_fence_after_sync();
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairN + h * 128);
 #pragma unroll 1
-        for (int jc = 0; jc < 8; ++jc) {
-          uint32_t r[16];
-          tmem_ld16(taddr + jc * 16, r);
-          const int n = n0 + jc * 16;
-          const auto live = [&](int v, int last) {  // d_in is a multiple of 8, so a group of 4 or 8 is all in or all out
-            return m < p.d_out && n + v < p.d_in &&
-                   ISOPO_IN_RANGE((long long)m * p.d_in + n + v + last, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad);
-          };
-          if (own) {
-            float o[2][8] = {};
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-              if (p.beta && live(u * 8, 7)) ld_global_8(dst + jc * 16 + u * 8, o[u]);
-            tmem_ld_wait();
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) o[u][e] = p.beta ? o[u][e] + __uint_as_float(r[u * 8 + e]) : __uint_as_float(r[u * 8 + e]);
-              if (live(u * 8, 7)) st_global_8(dst + jc * 16 + u * 8, o[u]);
-            }
-          } else {
-            tmem_ld_wait();
-#pragma unroll
-            for (int v = 0; v < 16; v += 4)
-              if (live(v, 3)) red_global_4(dst + jc * 16 + v, __uint_as_float(r[v]), __uint_as_float(r[v + 1]), __uint_as_float(r[v + 2]), __uint_as_float(r[v + 3]));
+        for (int jc = 0; jc < 4; ++jc) {
+          uint32_t r[32];
+          tmem_ld32(taddr + jc * 32, r);
+          if (issuer) bulk_wait_read<0>();
+          __syncwarp();
+          tmem_ld_wait();
+          box_row(box, lane, r);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (issuer && m < p.d_out && n0 + jc * 32 < p.d_in) {
+            if (store) tma_store_2d(&mapW, n0 + jc * 32, m, box);
+            else tma_add_2d(&mapW, n0 + jc * 32, m, box);
+            bulk_commit();
           }
         }
         tc_fence_before_sync();
@@ -379,18 +369,28 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
           if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (!ok) break;
-        // the unit's share of this tile: dW[m, n0 .. n0 + 127] += sum
-        const int m = (2 * ptm + (int)rank) * kHalf + q * 32 + lane, n0 = tn * kPairN + h * 128;
-        float* dst = p.dW + (size_t)m * p.d_in + n0;
+        // the unit's share of this tile: dW[m .., n0 .. n0 + 127] += sum, 16 columns at a time
+        const int m = (2 * ptm + (int)rank) * kHalf + q * 32, n0 = tn * kPairN + h * 128;
 #pragma unroll
-        for (int v = 0; v < 32; ++v) {
-          if (m < p.d_out && n0 + v * 4 < p.d_in &&  // d_in is a multiple of 8, so a group of 4 is all in or all out
-              ISOPO_IN_RANGE((long long)m * p.d_in + n0 + v * 4 + 3, (long long)p.d_out * p.d_in, p.info, kIdWeightGrad))
-            red_global_4(dst + v * 4, sum[v * 4 + 0], sum[v * 4 + 1], sum[v * 4 + 2], sum[v * 4 + 3]);
-          sum[v * 4 + 0] = sum[v * 4 + 1] = sum[v * 4 + 2] = sum[v * 4 + 3] = 0.f;
+        for (int jc = 0; jc < 8; ++jc) {
+          if (issuer) bulk_wait_read<0>();
+          __syncwarp();
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(box + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)),
+                         "f"(sum[jc * 16 + 4 * v]), "f"(sum[jc * 16 + 4 * v + 1]), "f"(sum[jc * 16 + 4 * v + 2]), "f"(sum[jc * 16 + 4 * v + 3]) : "memory");
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (issuer && m < p.d_out && n0 + jc * 16 < p.d_in) {
+            tma_add_2d(&mapW, n0 + jc * 16, m, box);
+            bulk_commit();
+          }
         }
+#pragma unroll
+        for (int e = 0; e < 128; ++e) sum[e] = 0.f;
       }
     }
+    if (issuer) bulk_wait_all();
   } else {
     // ------------------------------------------------------------------ tail warp (warp 10, both CTAs)
     // tail[s] is used only for last slabs that need the fix, so its phase is counted per stage; it
@@ -456,14 +456,14 @@ static isopo_status resident_pairs(int* pairs) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<kPlain>));
   static int resident[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident[dev] == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)(sms / 2));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = kSmemBytes<kPlain>;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
@@ -478,9 +478,11 @@ static isopo_status resident_pairs(int* pairs) {
   return ISOPO_OK;
 }
 
-static isopo_status make_fold_maps(CUtensorMap* mapY, CUtensorMap* mapX, const void* X, const void* dY, int64_t T, int d_in,
-                                   int d_out) {
-  isopo_status s = make_map_2d_bf16(mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
+static isopo_status make_fold_maps(CUtensorMap* mapY, CUtensorMap* mapX, CUtensorMap* mapW, const void* X, const void* dY, float* dW,
+                                   int64_t T, int d_in, int d_out, uint32_t box_cols) {
+  isopo_status s = make_map_2d_f32(mapW, dW, (uint64_t)d_out, (uint64_t)d_in, box_cols);
+  if (s != ISOPO_OK) return s;
+  s = make_map_2d_bf16(mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
   return s != ISOPO_OK ? s : make_map_2d_bf16(mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
 }
 
@@ -493,22 +495,18 @@ static void set_group(FoldParams* p, int npairs) {
 // Tiles whose sums one pair holds alone are written without a clear ahead of them and without a read of what is there: where a
 // tile has few stages, whole tiles per pair; where it has many, equal runs of stages, whose ends meet other runs in dW.
 // All in us, runs / whole tiles: 169 tokens, 3584 x 10752 140 / 44 (clear, then additions to 154 MB, against one pass of stores:
-// 3.5 TB/s), 3584 x 3584 41 / 22; 1097, 2560 x 10240 118 / 55; 2925, 2560 x 12928 204 / 169; 300, 896 x 896 12.5 / 11.5.
-// Adding (beta = 1) to what is there by loads and stores: only where dW is larger than the L2 and its tiles short, 169 tokens,
-// 3584 x 10752 140 / 95..118, but 2925, 2560 x 12928 185 / 189 and 300, 896 x 896 13.0 / 16.8.
+// 3.5 TB/s), 3584 x 3584 41 / 18; 1097, 2560 x 10240 118 / 59; 2925, 2560 x 12928 204 / 162; 300, 896 x 896 12.5 / 10.2.
 constexpr int kStoreStages = 8;  // stages that writing a tile takes at least, beside the MMAs of the next
-constexpr int64_t kBigWeights = (int64_t)1 << 24;
-PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, const float* dW, bool add, int pairs) {
+PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, bool add, int pairs) {
   PlainPlan plan{};
   const long long ptiles = (long long)((d_out + 2 * kHalf - 1) / (2 * kHalf)) * ((d_in + kPairN - 1) / kPairN);
   const long long kblocks = (T + kKB - 1) / kKB, stages = ptiles * kblocks;
-  plan.wide = ((uintptr_t)dW & 31) == 0 && (!add || (kblocks <= kStoreStages && (int64_t)d_in * d_out > kBigWeights));
   // no shorter runs than a drain takes
   plan.run = std::max<long long>((stages + pairs - 1) / pairs, std::min<long long>(kUnitOverhead, kblocks));
   plan.cost = plan.run + (plan.run / kblocks + 2) * kUnitOverhead;  // a run touches up to run / kblocks + 2 tiles
   const long long tiles = (ptiles + pairs - 1) / pairs, whole = tiles * std::max<long long>(kblocks, kStoreStages) + kUnitOverhead;
-  if (plan.wide && whole <= plan.cost) { plan.run = tiles * kblocks; plan.cost = whole; }
-  plan.clear = !add && !(plan.wide && plan.run % kblocks == 0);
+  if (whole <= plan.cost) { plan.run = tiles * kblocks; plan.cost = whole; }
+  plan.clear = !add && plan.run % kblocks != 0;
   return plan;
 }
 
@@ -517,10 +515,10 @@ isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, in
   int pairs = 0;
   isopo_status s = resident_pairs<true>(&pairs);
   if (s != ISOPO_OK) return s;
-  CUtensorMap mapY, mapX;
-  if ((s = make_fold_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
+  CUtensorMap mapY, mapX, mapW;
+  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, dY, dW, T, d_in, d_out, 32)) != ISOPO_OK) return s;
   FoldParams p{};
-  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add; p.wide = plan.wide;
+  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
   p.tiles_n = (d_in + kPairN - 1) / kPairN;
   p.kblocks = (int)((T + kKB - 1) / kKB);
@@ -530,7 +528,7 @@ isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, in
   set_group(&p, npairs);
   {
     LaunchScope scope(kIdWeightGrad, st);
-    launch(k_bf16_weight_grad_fold<true>, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
+    launch(k_bf16_weight_grad_fold<true>, 2 * npairs, kThreads, kSmemBytes<true>, st, mapY, mapX, mapW, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -541,8 +539,8 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   int pairs = 0;
   isopo_status s = resident_pairs<false>(&pairs);
   if (s != ISOPO_OK) return s;
-  CUtensorMap mapY, mapX;
-  if ((s = make_fold_maps(&mapY, &mapX, X, dY, T, d_in, d_out)) != ISOPO_OK) return s;
+  CUtensorMap mapY, mapX, mapW;
+  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, dY, dW, T, d_in, d_out, 16)) != ISOPO_OK) return s;
   FoldParams p{};
   p.off = off_dev; p.coeffs = coeffs; p.dW = dW; p.T = T; p.B = B; p.d_in = d_in; p.d_out = d_out; p.info = info;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
@@ -568,7 +566,7 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   if ((s = launch_offsets(off_host, B, off_dev, add ? Clear{} : Clear{{dW}, {(int64_t)d_in * d_out}}, st)) != ISOPO_OK) return s;
   {
     LaunchScope scope(kIdWeightGrad, st);
-    launch(k_bf16_weight_grad_fold<false>, 2 * npairs, kThreads, kSmemBytes, st, mapY, mapX, p);
+    launch(k_bf16_weight_grad_fold<false>, 2 * npairs, kThreads, kSmemBytes<false>, st, mapY, mapX, mapW, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
