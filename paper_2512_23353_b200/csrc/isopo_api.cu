@@ -87,7 +87,8 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   L.off_offsets = p;
   p = align_up(p + sizeof(int64_t) * (size_t)(B + 1), 1024);
   L.off_tokseq = p;
-  p = align_up(p + sizeof(int32_t) * (size_t)T, 1024);
+  const bool stored_bf16 = dtype == ISOPO_BF16 && resolved == ISOPO_PATH_MATERIALISE;
+  p = align_up(p + sizeof(int32_t) * std::max((size_t)T, stored_bf16 ? (size_t)B * ntk_pitch(B) : 0), 1024);
   L.off_kacc = p;
   if (dtype == ISOPO_F32)
     p = align_up(p + (resolved == ISOPO_PATH_MATERIALISE ? sizeof(uint32_t) : sizeof(double) * (size_t)B * (size_t)B), 1024);
@@ -262,8 +263,11 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     WsHead* head = (WsHead*)(w + L.off_tag);
     const WsTag tag = make_ws_tag(dtype, T, d_in, d_out, B, seq_offsets_host);
     StoredIntake in;
-    make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &K);
     const StoreFmt fmt = store_fmt(L, B, ws);
+    NtkPlan plan;
+    if ((s = plan_ntk(L, B, fmt.split, deterministic_mode(), &plan)) != ISOPO_OK) return s;
+    float* acc = plan.by_last ? K : (float*)tokseq;
+    make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &acc, plan.by_last ? B * B : B * ntk_pitch(B));
     if (fmt.split) {
       s = launch_offsets(seq_offsets_host, B, off_dev, Clear{}, st);
       if (s == ISOPO_OK) s = launch_seq_scales(X, dY, d_in, d_out, off_dev, B, (float*)fmt.scales, fmt.kdiag, st);
@@ -271,7 +275,7 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     }
     s = bf16_seq_grad(X, dY, T, d_in, d_out, in, B, L, G, fmt, info, st);
     if (s != ISOPO_OK) return s;
-    return bf16_ntk(G, L, B, K, head, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
+    return bf16_ntk(plan, G, L, B, K, acc, head, deterministic_mode() ? (float*)(w + L.off_kpart) : nullptr, fmt, info, st);
   }
   if (dtype == ISOPO_F32 && rp == ISOPO_PATH_MATERIALISE) {
     float* G = (float*)(w + L.off_G);
@@ -325,6 +329,7 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
   int64_t* off_dev = nullptr;
   WsHead* head[3];
   void* G[3];
+  float* acc[3];
   StoreFmt fmt[3];
   bool pairs_fit = true;
   for (int h = 0; h < n_proj; ++h) {
@@ -341,6 +346,7 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
     head[h] = (WsHead*)(w + L[h].off_tag);
     G[h] = w + L[h].off_G;
     fmt[h] = store_fmt(L[h], B, ws[h]);
+    acc[h] = (float*)(w + L[h].off_tokseq);
     pairs_fit = pairs_fit && (L[h].tiles_m % 2 == 0 || L[h].tiles_m >= 7);
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -353,21 +359,32 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
       if (s == ISOPO_OK) s = launch_seq_scales(X, dY[h], d_in, d_out[h], off_dev, B, (float*)fmt[h].scales, fmt[h].kdiag, st);
       if (s != ISOPO_OK) return s;
     }
+  NtkPlan plan[3];
+  bool all_last = true;
+  for (int h = 0; h < n_proj; ++h) {
+    if ((s = plan_ntk(L[h], B, fmt[h].split, deterministic_mode(), &plan[h])) != ISOPO_OK) return s;
+    all_last = all_last && plan[h].by_last;
+  }
+  for (int h = 0; h < n_proj; ++h) {  // one way for all: they are cleared alike
+    plan[h].by_last = all_last;
+    if (all_last) acc[h] = K[h];
+  }
+  const int n_acc = all_last ? B * B : B * ntk_pitch(B);
   StoredIntake in;
   if (pairs_fit) {
-    make_stored_intake(&in, seq_offsets_host, B, n_proj, tag, head, K);
+    make_stored_intake(&in, seq_offsets_host, B, n_proj, tag, head, acc, n_acc);
     s = bf16_seq_grad_pair_shared(X, n_proj, dY, d_out, T, d_in, in, B, L, G, fmt, info, st);
     if (s != ISOPO_OK) return s;
   } else {  // a projection with an odd, small number of 128-row tiles would idle half of its pairs: one launch each
     for (int h = 0; h < n_proj; ++h) {
-      make_stored_intake(&in, seq_offsets_host, B, 1, tag + h, head + h, K + h);
+      make_stored_intake(&in, seq_offsets_host, B, 1, tag + h, head + h, acc + h, n_acc);
       s = bf16_seq_grad(X, dY[h], T, d_in, d_out[h], in, B, L[h], G[h], fmt[h], info, st);
       if (s != ISOPO_OK) return s;
     }
   }
   for (int h = 0; h < n_proj; ++h) {
     float* kpart = deterministic_mode() ? (float*)((char*)ws[h] + L[h].off_kpart) : nullptr;
-    s = bf16_ntk(G[h], L[h], B, K[h], head[h], kpart, fmt[h], info, st);
+    s = bf16_ntk(plan[h], G[h], L[h], B, K[h], acc[h], head[h], kpart, fmt[h], info, st);
     if (s != ISOPO_OK) return s;
   }
   return ISOPO_OK;

@@ -88,18 +88,19 @@ struct WsHead {
 };
 
 // What the bf16 gradient kernel takes as arguments besides its matrices, so that no launch of its own prepares it: the
-// token offsets, the sequences longest first, and per projection the head to leave in its workspace and the K to clear for
-// the K pass behind it.
+// token offsets, the sequences longest first, and per projection the head to leave in its workspace and what the K pass behind it
+// adds into, to be cleared.
 struct StoredIntake {
   int32_t off[257];
   uint8_t order[256];
   int n_proj;
   WsTag tag[3];
   WsHead* head[3];
-  float* K[3];
+  float* acc[3];
+  int n_acc;
 };
 void make_stored_intake(StoredIntake* a, const int64_t* off_host, int B, int n_proj, const WsTag* tag, WsHead* const* head,
-                        float* const* K);
+                        float* const* acc, int n_acc);
 // Extents of the sequences in working order to shared memory (`raw`: scratch there, kIntakeRawBytes).  Arguments are no
 // memory of any predecessor's, so this may run before the wait for them.  The arguments are read as ordinary memory, a word
 // per thread: indexing them directly goes through the constant cache, one word at a time (2.5 us at 236 sequences).
@@ -119,9 +120,9 @@ __device__ __forceinline__ void stored_extents(const StoredIntake& a, int B, int
   }
 }
 // The grid's share of the clearing; CTA 0 leaves the heads.
-__device__ __forceinline__ void stored_heads(const StoredIntake& a, int B) {
+__device__ __forceinline__ void stored_heads(const StoredIntake& a) {
   for (int h = 0; h < a.n_proj; ++h) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * B; e += gridDim.x * blockDim.x) a.K[h][e] = 0.f;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < a.n_acc; e += gridDim.x * blockDim.x) a.acc[h][e] = 0.f;
     if (blockIdx.x == 0) {
       if (threadIdx.x < 8) a.head[h]->tag.v[threadIdx.x] = a.tag[h].v[threadIdx.x];
       if (threadIdx.x == 8) a.head[h]->done = 0u;
@@ -143,7 +144,8 @@ struct WsLayout {
   size_t off_tag;      // WsHead (materialised path)
   size_t off_aux;      // float scales[B] | float kdiag[B]  (bf16 materialised path, split store)
   size_t off_offsets;  // int64 [B+1]
-  size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here
+  size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here, the bf16
+                       // stored route what its K pass adds into (float [B][ntk_pitch(B)])
   size_t off_kacc;     // float32 path: float64 [B*B] K accumulators (Gram), uint32 CTAs of the K pass that are done (materialised)
   size_t off_scaled;   // bf16 [T, min(d_in, d_out)]  (bf16 Gram path: the pre-scaled operand of the weight-gradient GEMM)
   size_t off_G;        // stored gradients (materialised path only)
@@ -279,11 +281,20 @@ isopo_status launch_seq_scales(const void* X, const void* dY, int d_in, int d_ou
 isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* const* dY, const int* d_out, int64_t T, int d_in,
                                        const StoredIntake& in, int B, const WsLayout* L, void* const* G, const StoreFmt* fmt,
                                        int32_t* info, cudaStream_t st);
-// Adds into K, which the caller has cleared on this stream.  kpart != NULL (deterministic mode): every CTA
-// stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and a second kernel sums them in order.
+// kpart != NULL (deterministic mode): every CTA of the K pass stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and
+// a second kernel sums them in order.  Otherwise they add into K (by_last) or into rows of ntk_pitch(B) floats (`acc`), from which a
+// second kernel writes K; either has been cleared on this stream.
 constexpr int kNtkMaxPartials = 160;
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead* head, float* kpart, const StoreFmt& fmt,
-                      int32_t* info, cudaStream_t st);
+inline int ntk_pitch(int B) { return (B + 3) & ~3; }
+struct NtkPlan {
+  int box_rows, ppb;  // rows of a piece inside a box, pieces per box
+  long long nkb;      // boxes
+  int grid, n_active;
+  bool by_last;       // the last CTA to add its share completes K
+};
+isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, NtkPlan* plan);
+isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int B, float* K, float* acc, WsHead* head, float* kpart,
+                      const StoreFmt& fmt, int32_t* info, cudaStream_t st);
 bool deterministic_mode();
 // K[i][j] = K[j][i] for j < i (the Gram kernels fill the upper triangle)
 isopo_status mirror_upper(float* K, int B, cudaStream_t st);

@@ -852,12 +852,13 @@ isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, co
 }
 
 void make_stored_intake(StoredIntake* a, const int64_t* off_host, int B, int n_proj, const WsTag* tag, WsHead* const* head,
-                        float* const* K) {
+                        float* const* acc, int n_acc) {
   for (int i = 0; i <= B; ++i) a->off[i] = (int32_t)off_host[i];
   a->n_proj = n_proj;
+  a->n_acc = n_acc;
   for (int h = 0; h < 3; ++h) {
     const int hh = h < n_proj ? h : 0;
-    a->tag[h] = tag[hh]; a->head[h] = head[hh]; a->K[h] = K[hh];
+    a->tag[h] = tag[hh]; a->head[h] = head[hh]; a->acc[h] = acc[hh];
   }
   // longest first; equal lengths keep their order: sort (complement of the length, index)
   uint64_t key[256];

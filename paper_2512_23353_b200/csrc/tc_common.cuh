@@ -65,7 +65,7 @@ isopo_status make_map_2d_bf16(CUtensorMap* map, const void* base, uint64_t rows,
 
 // Row-major float32 matrix [rows, cols], cols a multiple of 4, in boxes of 32 rows x `box_cols` (16 or 32: 64- or 128-byte swizzle):
 // what a warp adds or writes.
-isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64_t cols, uint32_t box_cols);
+isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, bool swizzle = true);
 
 // Stored per-sequence gradients viewed as (x = element inside a 256-element piece row, y = sequence,
 // z = piece): boxes of 64 elements x `box_rows` sequences x `box_pieces` pieces, 128-byte swizzle.  Sequences

@@ -48,7 +48,7 @@ isopo_status make_map_2d_bf16(CUtensorMap* map, const void* base, uint64_t rows,
   return ISOPO_OK;
 }
 
-isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64_t cols, uint32_t box_cols) {
+isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, bool swizzle) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) {
     set_cuda_error(cudaErrorNotSupported, "cuTensorMapEncodeTiled entry point");
@@ -60,7 +60,7 @@ isopo_status make_map_2d_f32(CUtensorMap* map, void* base, uint64_t rows, uint64
   cuuint32_t box[2] = {box_cols, 32};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  !swizzle ? CU_TENSOR_MAP_SWIZZLE_NONE : box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled (dW)");
     return ISOPO_ERR_CUDA;

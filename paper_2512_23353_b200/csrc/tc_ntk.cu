@@ -5,8 +5,10 @@
 // takes a contiguous run of the long contraction dimension, streams [B rows] x [64 elements] boxes
 // (four per piece, so a CTA walks memory front to back) through a TMA ring, and uses every box as BOTH tcgen05 operands (K-major): rows 0..127 against all rows,
 // then rows 128..255 against rows 128..255 (the lower-left block is the mirror of the upper-right).
-// The float32 accumulators stay in tensor memory for the whole slab and are added into K once, with
-// reductions across CTAs by float atomics; a last tiny kernel mirrors the triangle.
+// The float32 accumulators stay in tensor memory for the whole slab and are added up once: 32 x 32 blocks of one triangle go
+// through shared memory to TMA reductions into rows that a last tiny kernel completes K from.  (One float atomic per entry into
+// K, every CTA in the same order, was half of the pass where the layer is not large, and 8 us of any: 10,000 tokens, 480 x 448, K pass
+// of 100 sequences 24.9 -> 9.9 us, 139 23.2 -> 15.9; 896 x 128, 64 sequences 13.4 -> 7.7, 256 23.1 -> 14.7; 896 x 896, 64 25.2 -> 20.9.)
 // For B <= 128 a box holds only the rows that exist (32, 64 or 128 >= B) but spans 8, 4 or 2 pieces, so
 // that every TMA copy still moves 32 KB (small boxes cost a fixed ~100 clocks each) and the stage is
 // again 256 rows: rows 0..127 and rows 128..255 each go through ONE 128 x 128 MMA per 16 elements,
@@ -30,7 +32,7 @@ using namespace tc;
 constexpr int kKB = 64;               // contraction elements per stage (one 128-byte row)
 constexpr int kStages = 6;
 constexpr int kStageBytes = 256 * 128;  // 256 rows x 128 bytes
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
+constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256 + 1024 /* reciprocal scales of the split store */;
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
 
@@ -43,6 +45,7 @@ struct NtkParams {
   int32_t* info;
   int box_rows;   // rows of a piece inside a box: 32, 64, 128 or 256, >= B
   int ppb;        // pieces per box = 256 / box_rows
+  bool by_boxes;  // added by TMA into rows of a pitch that it can take, not into K
   // not NULL (up to 16 sequences, 32 with little data): the last CTA to add its share completes the other triangle and the
   // diagonal of the split store
   uint32_t* done;
@@ -53,7 +56,7 @@ struct NtkParams {
 // kE4m3: the operand is the `hi` plane of the split store: 128 one-byte elements per 128-byte box row (two boxes
 // per piece instead of four), kind::f8f6f4 MMAs of 32 elements each - the same number of MMAs per byte, half the bytes.
 template <bool kE4m3>
-__global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant__ CUtensorMap mapG, NtkParams p) {
+__global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ CUtensorMap mapK, NtkParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
@@ -136,25 +139,60 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
     } else {
       const int q = warp & 3;
       const int r = q * 32 + lane;
-      // every (CTA, entry of the lower triangle) is produced by exactly one thread, once.  Entry (r, c), c >= r, goes to
-      // K[c][r]: the 32 lanes of a warp own consecutive r, so one instruction adds 128 contiguous bytes.  (Adding to
-      // K[r][c] instead touched 32 rows per instruction: 89 us instead of 31 us for the whole pass at 256 sequences and
-      // a 128 x 896 layer, whose 59 MB stay in the L2.)
-      float* const mine = p.kpart ? p.kpart + (size_t)blockIdx.x * p.B * p.B : nullptr;
-      auto add_to_k = [&](size_t idx, float v) {
-        if (mine) mine[idx] = v; else atomicAdd(&p.K[idx], v);
-      };
       // `ok` is false only after a wait ran out; every thread still reaches the named barriers below
       const bool ok = mbar_wait(accfull_bar, 0, abort_flag, p.info, kIdNtk);
-      // split store: the accumulators hold s_i s_j <G_i, G_j>; 1 / s_i of every sequence goes to shared memory (the ring
-      // is idle by now), and the diagonal is left to the gradient GEMM's float32 sums
-      float* inv_s = reinterpret_cast<float*>(smem + 128 * 1024);
+      // split store: the accumulators hold s_i s_j <G_i, G_j>; 1 / s_i of every sequence goes to shared memory, and the
+      // diagonal is left to the gradient GEMM's float32 sums
+      float* inv_s = reinterpret_cast<float*>(smem + kStages * kStageBytes + 256);
       if (kE4m3) {
         for (int i = r; i < 256; i += 128) inv_s[i] = i < p.B ? 1.f / __ldg(p.scales + i) : 0.f;
         asm volatile("bar.sync 2, 128;" ::: "memory");
       }
       auto unscale = [&](int row, int col, float v) { return kE4m3 ? v * inv_s[row] * inv_s[col] : v; };
-      {
+      if (p.by_boxes) {
+        // Blocks of 32 columns c of the warp's 32 accumulator rows go through shared memory (the ring is idle by now), turned over so
+        // that box row c holds K[c][r .. r + 31], and are added by TMA into the rows of p.acc; what the diagonal blocks have
+        // above the diagonal is not read from there.  A CTA starts at a block of its own: 148 of them on one sector wait for one another.
+        tc_fence_after_sync();
+        const uint32_t tlane = (uint32_t)(q * 32) << 16, ring = smem_base + q * (kStages * kStageBytes / 4);
+        const bool issuer = elect_one();
+        // sequences of the warp's rows in the left accumulator (the right one: two pieces' groups alike, or rows 128 ..), first column
+        const int seq0 = two ? q * 32 : (q * 32) & (p.box_rows - 1), coff = two ? 0 : q * 32 - seq0;
+        const int na = ok ? max(0, ((two ? n1 : min(p.box_rows, p.B)) - seq0 + 31) >> 5) : 0;       // blocks at and right of the diagonal
+        const int nb = !ok ? 0 : two ? max(0, (n2 - seq0 + 31) >> 5) : na;
+        const int n = na + nb, first = n ? blockIdx.x % n : 0;
+#pragma unroll 1
+        for (int k = 0; k < n; ++k) {
+          const int b = first + k < n ? first + k : first + k - n;
+          const bool right = b >= na;
+          const int c = seq0 + (right ? b - na : b) * 32;                  // accumulator column (of the piece)
+          const int sr = seq0 + (two && right ? 128 : 0), sc = c + (two && right ? 128 : 0);  // sequences of row and column
+          if (sr >= p.B || sc >= p.B) continue;
+          uint32_t v[32];
+          tmem_ld32(tmem_base + tlane + (right ? 256 : 0) + coff + c, v);
+          tmem_ld_wait();
+          const uint32_t box = ring + k * 4096;
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            const float x = kE4m3 ? unscale(sr + lane, sc + e, __uint_as_float(v[e])) : __uint_as_float(v[e]);
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(box + e * 128 + lane * 4), "f"(x) : "memory");
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (issuer) {
+            tma_add_2d(&mapK, sr, sc, box);
+            bulk_commit();
+          }
+        }
+        if (issuer) bulk_wait_all();
+      } else {
+        // deterministic mode and K completed by the last CTA
+        // every (CTA, entry of the lower triangle) is produced by exactly one thread, once.  Entry (r, c), c >= r, goes to
+        // K[c][r]: the 32 lanes of a warp own consecutive r, so one instruction adds 128 contiguous bytes.
+        float* const mine = p.kpart ? p.kpart + (size_t)blockIdx.x * p.B * p.B : nullptr;
+        auto add_to_k = [&](size_t idx, float v) {
+          if (mine) mine[idx] = v; else atomicAdd(&p.K[idx], v);
+        };
         tc_fence_after_sync();
         const uint32_t tlane = (uint32_t)(q * 32) << 16;
         if (two && ok) {
@@ -266,16 +304,22 @@ __global__ void k_ntk_reduce(const float* __restrict__ kpart, int n_ctas, int B,
   K[(size_t)j * B + i] = s;
 }
 
-// Completes the triangle a K kernel left out (kFromLower: it filled i >= j, else i <= j).
-// kdiag != NULL (split store): the diagonal comes from the gradient GEMM's float32 sums of squares
-template <bool kFromLower>
-__global__ void k_mirror(float* __restrict__ K, int B, const float* __restrict__ kdiag) {
+// K[j][i] = K[i][j] for i < j: the triangle that a Gram kernel left out.
+__global__ void k_mirror(float* __restrict__ K, int B) {
   pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
   const int i = e / B, j = e % B;
-  if (kFromLower ? j > i : j < i) K[e] = K[(size_t)j * B + i];
-  else if (j == i && kdiag) K[e] = kdiag[i];
+  if (j < i) K[e] = K[(size_t)j * B + i];
+}
+// K from the triangle i >= j of the K pass's sums (rows of `ld` floats).
+// kdiag != NULL (split store): the diagonal comes from the gradient GEMM's float32 sums of squares
+__global__ void k_ntk_finish(const float* __restrict__ acc, int ld, float* __restrict__ K, int B, const float* __restrict__ kdiag) {
+  pdl_wait();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= B * B) return;
+  const int i = e / B, j = e % B;
+  K[e] = i == j && kdiag ? kdiag[i] : acc[(size_t)max(i, j) * ld + min(i, j)];
 }
 
 #ifndef ISOPO_COMBINE_IN_FLIGHT
@@ -482,48 +526,56 @@ __global__ void __launch_bounds__(256, kDeep ? 3 : 4) k_e4m3_combine(const uint2
 
 }  // namespace
 
-isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead* head, float* kpart, const StoreFmt& fmt,
-                      int32_t* info, cudaStream_t st) {
+isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, NtkPlan* plan) {
   if (B > 256) return ISOPO_ERR_UNSUPPORTED;
-  if (fmt.split && kpart) return ISOPO_ERR_INVALID_ARG;  // the split store's diagonal is summed with float atomics
-  CUtensorMap mapG;
-  const uint32_t rows = B > 128 ? 256 : B > 64 ? 128 : B > 32 ? 64 : 32, ppb = 256 / rows;
-  const long long pieces = L.n_pad / kPieceElems;
-  isopo_status s = fmt.split ? make_map_pieces_u8(&mapG, G, (uint64_t)B, (uint64_t)pieces, rows, ppb)
-                             : make_map_pieces_bf16(&mapG, G, (uint64_t)B, (uint64_t)pieces, rows, ppb);
-  if (s != ISOPO_OK) return s;
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  auto kernel = fmt.split ? k_bf16_ntk<true> : k_bf16_ntk<false>;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  plan->box_rows = B > 128 ? 256 : B > 64 ? 128 : B > 32 ? 64 : 32;
+  plan->ppb = 256 / plan->box_rows;
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
-  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, (pieces + ppb - 1) / ppb * (fmt.split ? 2 : 4), info, (int)rows,
-              (int)ppb, nullptr, 0, fmt.kdiag};
-  int grid = (int)std::max<long long>(1, std::min<long long>(sms, p.nkb / 8));
-  if (kpart) grid = std::min(grid, kNtkMaxPartials);
+  plan->nkb = (L.n_pad / kPieceElems + plan->ppb - 1) / plan->ppb * (split ? 2 : 4);
+  plan->grid = (int)std::max<long long>(1, std::min<long long>(sms, plan->nkb / 4));  // four boxes of a CTA pay for its start
+  if (deterministic) plan->grid = std::min(plan->grid, kNtkMaxPartials);
   // CTAs whose slab of the contraction is empty take no part
-  const long long per = (p.nkb + grid - 1) / grid;
-  p.n_active = (uint32_t)((p.nkb + per - 1) / per);
+  const long long per = (plan->nkb + plan->grid - 1) / plan->grid;
+  plan->n_active = (int)((plan->nkb + per - 1) / per);
   // K completed by the last CTA: a launch less (2 us for the host, which bounds a pass over little data: 128 x 128, 32
   // sequences 18.3 -> 16.1 us), but a CTA by itself is slower than a kernel that is set up when this one ends, the more so the
   // more sequences: 896 x 896, K and solve: 24.5 us both ways at 16, 31.5 / 30.4 at 32, 47.2 / 45.0 at 48, 127.6 / 117.1 at 128.
-  if (!kpart && (B <= 16 || (B <= 32 && per <= 16))) p.done = &head->done;
+  plan->by_last = !deterministic && (B <= 16 || (B <= 32 && per <= 16));
+  return ISOPO_OK;
+}
+
+isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int B, float* K, float* acc, WsHead* head, float* kpart,
+                      const StoreFmt& fmt, int32_t* info, cudaStream_t st) {
+  if (fmt.split && kpart) return ISOPO_ERR_INVALID_ARG;  // the split store's diagonal is summed with float atomics
+  CUtensorMap mapG, mapK;
+  const uint32_t rows = (uint32_t)plan.box_rows, ppb = (uint32_t)plan.ppb;
+  const uint64_t pieces = (uint64_t)(L.n_pad / kPieceElems);
+  const bool by_boxes = !kpart && !plan.by_last;
+  isopo_status s = fmt.split ? make_map_pieces_u8(&mapG, G, (uint64_t)B, pieces, rows, ppb)
+                             : make_map_pieces_bf16(&mapG, G, (uint64_t)B, pieces, rows, ppb);
+  if (s != ISOPO_OK) return s;
+  if (by_boxes) {
+    if ((s = make_map_2d_f32(&mapK, acc, (uint64_t)B, (uint64_t)ntk_pitch(B), 32, false)) != ISOPO_OK) return s;
+  } else {
+    mapK = mapG;
+  }
+  auto kernel = fmt.split ? k_bf16_ntk<true> : k_bf16_ntk<false>;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, plan.nkb, info, plan.box_rows, plan.ppb, by_boxes,
+              plan.by_last ? &head->done : nullptr, (uint32_t)plan.n_active, fmt.kdiag};
   {
     LaunchScope scope(kIdNtk, st);
-    launch(kernel, grid, kThreads, kSmemBytes, st, mapG, p);
+    launch(kernel, plan.grid, kThreads, kSmemBytes, st, mapG, mapK, p);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
-  if (p.done) return ISOPO_OK;
-  if (!kpart) {
-    LaunchScope scope(kIdMirror, st);
-    launch(k_mirror<true>, (B * B + 255) / 256, 256, 0, st, K, B, fmt.split ? fmt.kdiag : nullptr);
-    ISOPO_CUDA_TRY(cudaGetLastError());
-    return ISOPO_OK;
-  }
+  if (plan.by_last) return ISOPO_OK;
   {
     LaunchScope scope(kIdMirror, st);
-    launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, (int)p.n_active, B, K);
+    if (kpart) launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, plan.n_active, B, K);
+    else launch(k_ntk_finish, (B * B + 255) / 256, 256, 0, st, acc, ntk_pitch(B), K, B, fmt.split ? fmt.kdiag : nullptr);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
@@ -532,7 +584,7 @@ isopo_status bf16_ntk(const void* G, const WsLayout& L, int B, float* K, WsHead*
 isopo_status mirror_upper(float* K, int B, cudaStream_t st) {
   {
     LaunchScope scope(kIdMirror, st);
-    launch(k_mirror<false>, (B * B + 255) / 256, 256, 0, st, K, B, nullptr);
+    launch(k_mirror, (B * B + 255) / 256, 256, 0, st, K, B);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -90,7 +90,7 @@ __device__ __forceinline__ void decode_unit(const SeqGradParams& p, const SeqInf
 
 struct NoIntake {};
 __device__ __forceinline__ void stored_extents(const NoIntake&, int, int32_t*, int64_t*, int*, int*) {}
-__device__ __forceinline__ void stored_heads(const NoIntake&, int) {}
+__device__ __forceinline__ void stored_heads(const NoIntake&) {}
 template <bool kFolded> struct IntakeOf { typedef StoredIntake type; };
 template <> struct IntakeOf<true> { typedef NoIntake type; };
 
@@ -132,7 +132,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   if (!kFolded) stored_extents(in, p.B, reinterpret_cast<int32_t*>(s_seq + kMaxSeqs), s_first, s_len, s_seq);
   pdl_begin();
-  if (!kFolded) stored_heads(in, p.B);
+  if (!kFolded) stored_heads(in);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();

@@ -158,7 +158,7 @@ k_bf16_seq_grad_pair(const __grid_constant__ CUtensorMap mapY0, const __grid_con
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
   stored_extents(in, p.B, reinterpret_cast<int32_t*>(s_seq + kMaxSeqs), s_first, s_len, s_seq);
   pdl_begin();
-  stored_heads(in, p.B);
+  stored_heads(in);
   tc_fence_before_sync();
   __syncthreads();
   __syncwarp();

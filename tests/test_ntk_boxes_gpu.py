@@ -1,0 +1,60 @@
+"""GPU check of the K pass of the bf16 stored route around its blocks of 32 sequences: whole numbers small enough for every step to be
+exact (bf16 gradients, float32 sums), so K has to be what int64 gives, to the bit."""
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def b():
+    from paper_2512_23353_b200 import binding
+    return binding
+
+
+def _case(B, L, d_in, d_outs, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    off = np.arange(B + 1, dtype=np.int64) * L
+    draw = lambda d: torch.randint(-1, 2, (B * L, d), device="cuda", generator=gen)  # noqa: E731
+    X, dYs = draw(d_in), [draw(o) for o in d_outs]
+    Ks = []
+    for dY in dYs:
+        G = (dY.view(B, L, -1, 1) * X.view(B, L, 1, -1)).sum(1).reshape(B, -1).double()
+        assert G.abs().max() <= 256
+        Ks.append((G @ G.T).float())
+    return X.bfloat16(), [dY.bfloat16() for dY in dYs], off, Ks
+
+
+@pytest.mark.parametrize("B", [4, 16, 17, 31, 32, 33, 35, 63, 64, 65, 96, 97, 127, 128, 129, 144, 145, 160, 161, 193, 255, 256])
+@pytest.mark.parametrize("L,d_in,d_out", [(1, 72, 40), (2, 264, 296)])
+def test_exact(b, B, L, d_in, d_out):
+    X, (dY,), off, (want,) = _case(B, L, d_in, [d_out], 1000 * B + d_in)
+    raw = torch.full((B * B + 3,), float("nan"), device="cuda")
+    for shift in (0, 1, 3):  # K may start at any element
+        K = raw[shift:shift + B * B].view(B, B)
+        ws = b.alloc_workspace(b.BF16, B * L, d_in, d_out, B, b.PATH_MATERIALISE)
+        ws.fill_(0xFF)
+        info = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for _ in range(2):  # the second pass finds the first one's sums
+            b.isopo_layer_gram(X, dY, off, K, ws, info, b.PATH_MATERIALISE)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        assert torch.equal(K, want)
+
+
+@pytest.mark.parametrize("B", [30, 31, 200])
+def test_exact_shared_input(b, B):
+    """Projections of which one would complete K in its last CTA and another would not."""
+    d_outs = [8, 600, 256]
+    X, dYs, off, want = _case(B, 2, 520, d_outs, B)
+    ws = [b.alloc_workspace(b.BF16, 2 * B, 520, o, B, b.PATH_MATERIALISE) for o in d_outs]
+    Ks = [torch.full((B, B), float("nan"), device="cuda") for _ in d_outs]
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    b.isopo_layer_gram_shared_x_stored(X, dYs, off, Ks, ws, info)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    for K, w in zip(Ks, want):
+        assert torch.equal(K, w)
