@@ -620,7 +620,9 @@ __global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ 
 // boundaries are the same for all its lanes), and adds the lanes of one row sequence together before it issues one
 // float64 atomic.  Bound by the float32 pipe: 896 -> 896, 4608 tokens: 1151 us against 3246 us for 32 x 32 tiles loaded
 // synchronously with an atomic per token pair.  Too few tiles of 64 to fill the machine leave the kernel to the latency of
-// one CTA's walk over the features: tiles of 32 then (f32_gram_tile).
+// one CTA's walk over the features: tiles of 32 then, and clusters of kC CTAs that take a share of the features each and add up
+// their sums through distributed shared memory before P and Q are multiplied (f32_gram_shape).  The pairs I <= J are numbered in one
+// row: of a square grid of which half returns at once some SMs got three times the work of others (789 tokens, 251 x 1121 97 -> 74 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int kGK = 16;   // features per stage
 constexpr int kGPitch = kGK + 4;
@@ -631,7 +633,22 @@ struct GramTile {
   static constexpr int kTx = kGT / kCols, kThr = 16 * kTx;          // 64: 16 x 16 threads; 32: 16 x 8
   static constexpr int kStages = kGT == 64 ? 3 : 6;                 // 30 KB either way
 };
-template <bool kSampled, int kGT>
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float ld_cluster(const float* mine, unsigned rank) {  // what CTA `rank` has where this one has *mine
+  uint32_t at;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(mine)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+  return v;
+}
+template <bool kSampled, int kGT, int kC>
 __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
                                                   const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
                                                   int d_in, int d_out, const int32_t* __restrict__ tokseq, int B,
@@ -639,18 +656,31 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
   pdl_wait();
   constexpr int kRows = GramTile<kGT>::kRows, kTx = GramTile<kGT>::kTx, kThr = GramTile<kGT>::kThr;
   constexpr int kGramStages = GramTile<kGT>::kStages;
-  const int I = blockIdx.y, J = blockIdx.x;
-  if (!kSampled && J < I) return;
-  __shared__ __align__(16) float stage_mem[kGramStages][2][kGT * kGPitch];
+  const unsigned rank = kC > 1 ? cluster_rank() : 0, unit = blockIdx.x / kC;
+  int I, J;
+  if (kSampled) {
+    const unsigned ns = (unsigned)((n_rows + kGT - 1) / kGT);
+    J = (int)(unit / ns);
+    I = (int)(unit - (unsigned)J * ns);
+  } else {  // tile column J has tiles 0 .. J
+    J = (int)((sqrt(8.0 * unit + 1.0) - 1.0) * 0.5);
+    while ((int64_t)J * (J + 1) / 2 > unit) --J;
+    while ((int64_t)(J + 1) * (J + 2) / 2 <= unit) ++J;
+    I = (int)(unit - (int64_t)J * (J + 1) / 2);
+  }
+  constexpr int kStageFloats = kGramStages * 2 * kGT * kGPitch, kTile = kGT * (kGT + 1);
+  __shared__ __align__(16) float smem[kStageFloats > 2 * kTile ? kStageFloats : 2 * kTile];
+  auto stage_mem = [&](int k, int side) { return smem + (k % kGramStages * 2 + side) * (kGT * kGPitch); };
   __shared__ int s_col[kGT];
   const int tid = threadIdx.x, tx = tid % kTx, ty = tid / kTx;
   const int64_t r0 = (int64_t)I * kGT, c0 = (int64_t)J * kGT;
   if (tid < kGT) s_col[tid] = c0 + tid < T ? tokseq[c0 + tid] : -1;
-  const int nkx = (d_in + kGK - 1) / kGK, nky = (d_out + kGK - 1) / kGK;
+  const int nkx = (d_in + kGK - 1) / kGK, total_k = nkx + (d_out + kGK - 1) / kGK;
+  const int k0 = (int)((int64_t)total_k * rank / kC), k1 = (int)((int64_t)total_k * (rank + 1) / kC);  // this CTA's stages
   // a thread copies one column (group) of a stage, every kThr / kGK-th (4-byte copies) or 4 kThr / kGK-th row
   const int c1 = tid % kGK, r1 = tid / kGK, c4 = tid % (kGK / 4) * 4, r4 = tid / (kGK / 4);
   auto fetch = [&](int k) {
-    if (k < nkx + nky) {
+    if (k < k1) {
       const bool second = k >= nkx;
       const int d = second ? d_out : d_in, f0 = (second ? k - nkx : k) * kGK;
 #pragma unroll
@@ -658,7 +688,7 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
         const float* M = side == 0 ? (second ? RY : RX) : (second ? dY : X);
         const int64_t first = side == 0 ? r0 : c0;
         const int rows = (int)min((int64_t)kGT, (side == 0 ? n_rows : T) - first);  // rows of the tile that exist
-        float* dst = stage_mem[k % kGramStages][side];
+        float* dst = stage_mem(k - k0, side);
         if ((d & 3) == 0) {
           const float* src = M + (first + r4) * d + f0 + c4;
 #pragma unroll
@@ -678,22 +708,23 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
     }
     cp_async_commit();
   };
-  float h[kRows][4];
+  float h[kRows][4] = {};
   f32x2 acc[kRows][4] = {};
   auto total = [](f32x2 v) { float lo, hi; unpack2(v, lo, hi); return lo + hi; };
-  for (int k = 0; k < kGramStages - 1; ++k) fetch(k);
-  for (int k = 0; k < nkx + nky; ++k) {
+  auto keep_p = [&]() {  // the sums so far are of P
+#pragma unroll
+    for (int p = 0; p < kRows; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { h[p][q] = total(acc[p][q]); acc[p][q] = 0ull; }
+  };
+  for (int k = k0; k < k0 + kGramStages - 1; ++k) fetch(k);
+  for (int k = k0; k < k1; ++k) {
     cp_async_wait<kGramStages - 2>();
     __syncthreads();
     fetch(k + kGramStages - 1);
-    if (k == nkx) {
-#pragma unroll
-      for (int p = 0; p < kRows; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) { h[p][q] = total(acc[p][q]); acc[p][q] = 0ull; }
-    }
-    const float* sA = stage_mem[k % kGramStages][0];
-    const float* sB = stage_mem[k % kGramStages][1];
+    if (k == nkx) keep_p();
+    const float* sA = stage_mem(k - k0, 0);
+    const float* sB = stage_mem(k - k0, 1);
 #pragma unroll
     for (int c = 0; c < kGK; c += 4) {
       ulonglong2 a[kRows], b[4];
@@ -709,14 +740,44 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
   }
   cp_async_wait<0>();
   __syncthreads();
-  float* tile = &stage_mem[0][0][0];  // [row][kGT + 1]
-  static_assert(kGT * (kGT + 1) <= kGramStages * 2 * kGT * kGPitch, "the tile reuses the stages");
+  if (k1 <= nkx) keep_p();
+  // One CTA: the products.  Several: the sums of P and behind them those of Q, which every CTA of the cluster reads for its share
+  // of the columns and adds up in rank order.
+  float* tile = smem;  // [row][kGT + 1]
 #pragma unroll
   for (int p = 0; p < kRows; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) tile[(ty + 16 * p) * (kGT + 1) + tx + kTx * q] = h[p][q] * total(acc[p][q]);
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, row = (warp % (kGT / 32)) * 32 + lane, cb = warp / (kGT / 32) * (kGT / 4);
+    for (int q = 0; q < 4; ++q) {
+      const int e = (ty + 16 * p) * (kGT + 1) + tx + kTx * q;
+      const float y = total(acc[p][q]);
+      tile[e] = kC == 1 ? h[p][q] * y : h[p][q];
+      if (kC > 1) tile[kTile + e] = y;
+    }
+  if (kC == 1) __syncthreads();
+  else cluster_sync();
+  // a warp takes 32 rows and kWidth columns
+  constexpr int kWidth = kGT / 4 / kC;
+  const int warp = tid >> 5, lane = tid & 31, row = (warp % (kGT / 32)) * 32 + lane, cb = (int)(rank * 4 + warp / (kGT / 32)) * kWidth;
+  const float* const mine = tile + row * (kGT + 1) + cb;
+  float prod[kWidth];
+  if (kC > 1) {  // all of the loads in flight together
+    float x[kC][kWidth], y[kC][kWidth];
+#pragma unroll
+    for (int r = 0; r < kC; ++r)
+#pragma unroll
+      for (int c = 0; c < kWidth; ++c) { x[r][c] = ld_cluster(mine + c, r); y[r][c] = ld_cluster(mine + kTile + c, r); }
+#pragma unroll
+    for (int c = 0; c < kWidth; ++c) {
+      float sx = x[0][c], sy = y[0][c];
+#pragma unroll
+      for (int r = 1; r < kC; ++r) { sx += x[r][c]; sy += y[r][c]; }
+      prod[c] = sx * sy;
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // this CTA has read the others' sums
+  } else {
+#pragma unroll
+    for (int c = 0; c < kWidth; ++c) prod[c] = mine[c];
+  }
   const int64_t t = r0 + row;
   const int rseq = t < n_rows ? (kSampled ? (int)t : tokseq[t]) : -1;  // rows past the end form a run of their own, unused
   int same = 0;
@@ -728,14 +789,15 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
   const int up = __shfl_up_sync(0xffffffffu, rseq, 1);
   const bool head = (lane == 0 || up != rseq) && rseq >= 0;
   double run = 0.0;
-  for (int c = 0; c < kGT / 4; ++c) {
+#pragma unroll
+  for (int c = 0; c < kWidth; ++c) {
     const int cs = s_col[cb + c];
     if (cs < 0) break;
     const int64_t s = c0 + cb + c;
-    const double v = (double)tile[row * (kGT + 1) + cb + c];
+    const double v = (double)prod[c];
     if (kSampled) run += v;
     else if (t <= s) run += rseq == cs && t < s ? 2.0 * v : v;
-    if (c == kGT / 4 - 1 || s_col[cb + c + 1] != cs) {
+    if (c == kWidth - 1 || s_col[cb + c + 1] != cs) {
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const double o = __shfl_down_sync(0xffffffffu, run, 1 << k);
@@ -745,6 +807,7 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
       run = 0.0;
     }
   }
+  if (kC > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // nobody leaves while its sums may still be read
 }
 
 __global__ void k_f32_gram_finish(const double* __restrict__ kacc, int B, float* __restrict__ K) {
@@ -976,36 +1039,56 @@ isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint3
   return ISOPO_OK;
 }
 
-// Tokens per tile: 64, or 32 where `tiles` of 64 would not give every SM two CTAs.
-static bool f32_gram_small_tiles(int64_t tiles) { return tiles < 2 * kSms; }
+// Tokens per tile and CTAs that share a tile's features.  Tiles of 32 where those of 64 would be few; then as many CTAs to a tile as
+// make up to 240 of them: one alone is a chain of (d_in + d_out) / 16 stages.  Two CTAs to a tile of 64 where those are many features.
+// Whole call, us, 64 / 32 / 32 by two / four / eight: Gram of 115 tokens, 283 x 1288 76 / 41 / 28 / 20 / 16; 300, 896 x 896 80 / 44 / 29 /
+// 29 / 36; 789, 251 x 1121 79 / 74 / 72 / 97 / 144; 874, 296 x 577 51 / 48 / 60; 2000, 512 x 512 155 / 180.  128 samples: 128 tokens,
+// 712 x 1169 101 / 57 / 37 / 26 / 27; 938, 1539 x 185 99 / 58 / 48 / 55; 4979, 1024 x 80 90 / 80 / 87; 7032, 1481 x 1513 276, 64 by two
+// 237, 32 302.
+struct GramShape { int tile, ctas; };
+static GramShape f32_gram_shape(int64_t rows, int64_t cols, bool triangle, int d_in, int d_out) {
+  auto tiles = [&](int64_t t) {
+    const int64_t r = (rows + t - 1) / t, c = (cols + t - 1) / t;
+    return triangle ? c * (c + 1) / 2 : r * c;
+  };
+  const int stages = (d_in + kGK - 1) / kGK + (d_out + kGK - 1) / kGK;
+  const int64_t wide = tiles(64);
+  if (4 * wide >= 5 * kSms) return GramShape{64, wide < 2 * kSms && stages >= 128 ? 2 : 1};
+  GramShape g{32, 1};
+  while (g.ctas < 8 && tiles(32) * 2 * g.ctas <= 240 && stages >= 10 * g.ctas) g.ctas *= 2;
+  return g;
+}
+template <bool kSampled>
+static isopo_status launch_f32_gram(int id, const GramShape& g, int64_t units, const float* RX, const float* RY, int64_t n_rows, const float* X,
+                                    const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B, double* out, cudaStream_t st) {
+  if (units * g.ctas > INT32_MAX) return ISOPO_ERR_UNSUPPORTED;
+  {
+    LaunchScope scope(id, st);
+    const auto wide = g.ctas == 1 ? k_f32_gram<kSampled, 64, 1> : k_f32_gram<kSampled, 64, 2>;
+    const auto narrow = g.ctas == 1   ? k_f32_gram<kSampled, 32, 1>
+                        : g.ctas == 2 ? k_f32_gram<kSampled, 32, 2>
+                        : g.ctas == 4 ? k_f32_gram<kSampled, 32, 4>
+                                      : k_f32_gram<kSampled, 32, 8>;
+    launch_cluster(g.tile == 32 ? narrow : wide, (unsigned)g.ctas, dim3((unsigned)(units * g.ctas)),
+                   g.tile == 32 ? 128 : 256, 0, st, RX, RY, n_rows, X, dY, T, d_in, d_out, tokseq, B, out);
+  }
+  ISOPO_CUDA_TRY(cudaGetLastError());
+  return ISOPO_OK;
+}
 
 isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                       double* kacc, float* K, cudaStream_t st) {
-  const int64_t n64 = (T + 63) / 64;
-  const bool small = f32_gram_small_tiles(n64 * (n64 + 1) / 2);
-  const int64_t nt = small ? (T + 31) / 32 : n64;
-  if (nt > 65535) return ISOPO_ERR_UNSUPPORTED;
-  {
-    LaunchScope scope(kIdF32Gram, st);
-    launch(small ? k_f32_gram<false, 32> : k_f32_gram<false, 64>, dim3((unsigned)nt, (unsigned)nt), small ? 128 : 256, 0, st, X, dY,
-           T, X, dY, T, d_in, d_out, tokseq, B, kacc);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return launch_f32_finish(kacc, B, K, st);
+  const GramShape g = f32_gram_shape(T, T, true, d_in, d_out);
+  const int64_t nt = (T + g.tile - 1) / g.tile;
+  const isopo_status s = launch_f32_gram<false>(kIdF32Gram, g, nt * (nt + 1) / 2, X, dY, T, X, dY, T, d_in, d_out, tokseq, B, kacc, st);
+  return s != ISOPO_OK ? s : launch_f32_finish(kacc, B, K, st);
 }
 
 isopo_status f32_sampled(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* a0, const float* g0,
                          int n_samples, const int32_t* tokseq, int B, double* Mt, cudaStream_t st) {
-  const bool small = f32_gram_small_tiles((T + 63) / 64 * ((n_samples + 63) / 64));
-  const int64_t nt = small ? (T + 31) / 32 : (T + 63) / 64, ns = small ? (n_samples + 31) / 32 : (n_samples + 63) / 64;
-  if (ns > 65535) return ISOPO_ERR_UNSUPPORTED;
-  {
-    LaunchScope scope(kIdSampled, st);
-    launch(small ? k_f32_gram<true, 32> : k_f32_gram<true, 64>, dim3((unsigned)nt, (unsigned)ns), small ? 128 : 256, 0, st, a0, g0,
-           (int64_t)n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt);
-  }
-  ISOPO_CUDA_TRY(cudaGetLastError());
-  return ISOPO_OK;
+  const GramShape g = f32_gram_shape(n_samples, T, false, d_in, d_out);
+  const int64_t nt = (T + g.tile - 1) / g.tile, ns = (n_samples + g.tile - 1) / g.tile;
+  return launch_f32_gram<true>(kIdSampled, g, nt * ns, a0, g0, n_samples, X, dY, T, d_in, d_out, tokseq, B, Mt, st);
 }
 
 isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, const float* coeffs, float* dW, float beta,
