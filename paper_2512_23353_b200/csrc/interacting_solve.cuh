@@ -88,23 +88,54 @@ __device__ __noinline__ int warp_factor_diag(typename BlkPtr<kShared>::rw D, flo
   for (int c = 0; c < kNB; ++c) r[c] = D[c * kNB + lane];  // row `lane`
   int fail = 0;
   float rdiag = 0.f;  // 1 / L[lane][lane]
+  float d = __shfl_sync(0xffffffffu, r[0], 0), rs = rsqrtf(d);
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
-    const float d = __shfl_sync(0xffffffffu, r[k], k);
     if (!(d > 0.f) && fail == 0) fail = k + 1;
-    const float rs = rsqrtf(d);
     if (lane == k) rdiag = rs;
     r[k] = lane == k ? d * rs : r[k] * rs;  // L[lane][k] (rows above k hold junk, never used)
+    if (kShared) {
+      D[k * kNB + lane] = k <= lane ? r[k] : 0.f;
+      __syncwarp();
+    }
+    // the next pivot first: its chain (two shuffles, a reciprocal root) runs under the updates of the columns behind it, which read
+    // column k from shared memory four entries at a time
+    if (k + 1 < kNB) {
+      r[k + 1] = fmaf(-r[k], __shfl_sync(0xffffffffu, r[k], k + 1), r[k + 1]);
+      d = __shfl_sync(0xffffffffu, r[k + 1], k + 1);
+      rs = rsqrtf(d);
+    }
+    if (kShared) {
 #pragma unroll
-    for (int j = k + 1; j < kNB; ++j) {
-      const float ljk = __shfl_sync(0xffffffffu, r[k], j);
-      r[j] = fmaf(-r[k], ljk, r[j]);
+      for (int j = (k + 2) & ~3; j < kNB; j += 4) {
+        const float4 l = *reinterpret_cast<const float4*>(D + k * kNB + j);
+        if (j > k + 1) r[j] = fmaf(-r[k], l.x, r[j]);
+        if (j + 1 > k + 1) r[j + 1] = fmaf(-r[k], l.y, r[j + 1]);
+        if (j + 2 > k + 1) r[j + 2] = fmaf(-r[k], l.z, r[j + 2]);
+        if (j + 3 > k + 1) r[j + 3] = fmaf(-r[k], l.w, r[j + 3]);
+      }
+    } else {
+#pragma unroll
+      for (int j = k + 2; j < kNB; ++j) r[j] = fmaf(-r[k], __shfl_sync(0xffffffffu, r[k], j), r[j]);
     }
   }
+  if (!kShared)
 #pragma unroll
-  for (int c = 0; c < kNB; ++c) D[c * kNB + lane] = c <= lane ? r[c] : 0.f;
+    for (int c = 0; c < kNB; ++c) D[c * kNB + lane] = c <= lane ? r[c] : 0.f;
   rd[lane] = rdiag;
   return fail;
+}
+
+// x[j] -= L[j][k] xk for j > k; L's column k is read four entries at a time, the same for all lanes.
+__device__ __forceinline__ void below_pivot(const float* L, int k, float xk, float (&x)[kNB]) {
+#pragma unroll
+  for (int j = (k + 1) & ~3; j < kNB; j += 4) {
+    const float4 l = *reinterpret_cast<const float4*>(L + k * kNB + j);
+    if (j > k) x[j] = fmaf(-l.x, xk, x[j]);
+    if (j + 1 > k) x[j + 1] = fmaf(-l.y, xk, x[j + 1]);
+    if (j + 2 > k) x[j + 2] = fmaf(-l.z, xk, x[j + 2]);
+    if (j + 3 > k) x[j + 3] = fmaf(-l.w, xk, x[j + 3]);
+  }
 }
 
 // Inv = L^-1 (column-major) for the factored diagonal block D with rd[k] = 1 / L_kk.  One warp.
@@ -119,8 +150,7 @@ __device__ __noinline__ void warp_invert_factor(typename BlkPtr<kShared>::ro D, 
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
     z[k] *= rd[k];
-#pragma unroll
-    for (int i = k + 1; i < kNB; ++i) z[i] = fmaf(-D[k * kNB + i], z[k], z[i]);  // L[i][k], broadcast
+    below_pivot(D, k, z[k], z);
   }
 #pragma unroll
   for (int i = 0; i < kNB; ++i) Inv[lane * kNB + i] = z[i];
@@ -138,8 +168,7 @@ __device__ __noinline__ void warp_solve_panel(typename BlkPtr<kShared>::rw A, ty
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
     a[k] *= rd[k];
-#pragma unroll
-    for (int j = k + 1; j < kNB; ++j) a[j] = fmaf(-a[k], L[k * kNB + j], a[j]);  // L[j][k], broadcast
+    below_pivot(L, k, a[k], a);
   }
 #pragma unroll
   for (int c = 0; c < kNB; ++c) A[c * kNB + lane] = a[c];
@@ -235,37 +264,42 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
   const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThr / 32;
   const float* __restrict__ K = P.K;
   const int nb = (B + kNB - 1) / kNB, Bp = nb * kNB;
-  if (tid == 0) s_fail = 0;
+  __shared__ int s_taken[2];  // trailing blocks of a column that warps have taken
+  if (tid == 0) s_fail = s_taken[0] = s_taken[1] = 0;
   const bool vec4 = rows_in_float4(K, B);
-  // load the lower block triangle.  K is symmetric, so row j of K read along i gives column j of
-  // the blocks; float4 loads, eight in flight per thread, where its rows are made of them.
-  if (vec4) {
-    const int nvec = B * B / 4;
-    for (int base = tid; base < nvec; base += kThr * 8) {
-      float4 val[8];
+  // load the lower block triangle.  K is symmetric, so row j of K read along i, from the block of the diagonal on, gives column j
+  // of the blocks; a warp takes four rows at a time (float4 loads, eight in flight per lane, where rows are made of them).
+  for (int j0 = warp * 4; j0 < B; j0 += nwarps * 4) {  // four columns of one block column
+    const int J = j0 / kNB, first = J * kNB;
+    if (vec4) {
+      for (int i0 = first + lane * 4; i0 < B; i0 += 256) {
+        float4 v[4][2];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = base + u * kThr;
-        val[u] = e < nvec ? __ldg(reinterpret_cast<const float4*>(K) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = base + u * kThr;
-        if (e >= nvec) continue;
-        const int j = (e * 4) / B, i = (e * 4) % B, I = i / kNB, J = j / kNB;
-        if (I < J) continue;
-        float4 w = val[u];
-        if (i == j) w.x += P.lambda;
-        if (i + 1 == j) w.y += P.lambda;
-        if (i + 2 == j) w.z += P.lambda;
-        if (i + 3 == j) w.w += P.lambda;
-        *reinterpret_cast<float4*>(Lb + blk_slot(I, J) * kBlk + (j % kNB) * kNB + (i % kNB)) = w;
+          for (int h = 0; h < 2; ++h)
+            v[u][h] = i0 + 128 * h < B ? __ldg(reinterpret_cast<const float4*>(K + (size_t)(j0 + u) * B + i0 + 128 * h)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int i = i0 + 128 * h, j = j0 + u;
+            if (i >= B) continue;
+            float4 w = v[u][h];
+            if (i == j) w.x += P.lambda;
+            if (i + 1 == j) w.y += P.lambda;
+            if (i + 2 == j) w.z += P.lambda;
+            if (i + 3 == j) w.w += P.lambda;
+            *reinterpret_cast<float4*>(Lb + blk_slot(i / kNB, J) * kBlk + (j % kNB) * kNB + (i % kNB)) = w;
+          }
       }
-    }
-  } else {
-    for (int e = tid; e < B * B; e += kThr) {
-      const int j = e / B, i = e % B, I = i / kNB, J = j / kNB;
-      if (I >= J) Lb[blk_slot(I, J) * kBlk + (j % kNB) * kNB + (i % kNB)] = K[e] + (i == j ? P.lambda : 0.f);
+    } else {
+      for (int i = first + lane; i < B; i += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = j0 + u;
+          if (j < B) Lb[blk_slot(i / kNB, J) * kBlk + (j % kNB) * kNB + (i % kNB)] = __ldg(K + (size_t)j * B + i) + (i == j ? P.lambda : 0.f);
+        }
     }
   }
   // identity padding of the last block row / column
@@ -282,6 +316,7 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
   __syncthreads();
   for (int J = 0; J < nb && !s_fail; ++J) {
     const float* Ljj = Lb + blk_slot(J, J) * kBlk;
+    if (tid == 0) s_taken[(J + 1) & 1] = 0;
     // panel: blocks (I, J) below the diagonal on warps 0 .. nwarps-2; the last warp inverts L_JJ
     if (warp == nwarps - 1) warp_invert_factor<kShared>(Ljj, rdiag + J * kNB, InvD + J * kBlk);
     else
@@ -311,8 +346,15 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, type
       if (warp == 0) {
         const int f = warp_factor_diag<kShared>(Dn, rdiag + (J + 1) * kNB);
         if (f != 0 && lane == 0) s_fail = (J + 1) * kNB + f;
-      } else {
-        for (int t = warp; t < ntrail; t += nwarps - 1) {
+      }
+      // The other blocks, whoever is free.  Warps 4, 8, .. share warp 0's scheduler and stay away: its factorisation is the serial
+      // chain, and took 16.5 thousand clocks of the first column of 256 sequences among fifteen updating warps, 5.4 alone.
+      if (warp == 0 || (warp & 3) != 0) {
+        while (true) {
+          int t = 0;
+          if (lane == 0) t = 1 + atomicAdd(&s_taken[J & 1], 1);
+          t = __shfl_sync(0xffffffffu, t, 0);
+          if (t >= ntrail) break;
           int a = 0, rem = t;
           while (rem > a) { rem -= a + 1; ++a; }
           const int I = J + 1 + a, Kc = J + 1 + rem;

@@ -253,7 +253,7 @@ inline size_t small_smem_bytes(int B) {
 }
 
 // Interacting variant, 129 to 256 sequences: one CTA per layer, the factor in shared memory.
-__global__ void __launch_bounds__(kSolveThreads) k_transform(const __grid_constant__ TransformBatch batch) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_transform(const __grid_constant__ TransformBatch batch) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TransformParams P = layer_params(batch, blockIdx.x);
