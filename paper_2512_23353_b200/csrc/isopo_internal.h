@@ -246,8 +246,16 @@ __device__ __forceinline__ void clear_regions(const Clear& c) {
   }
 }
 // Token offsets as kernel arguments (no host-to-device copy); they are below 2^31 and travel as 32-bit values.
-constexpr int kArgChunk = 384;    // the usual case; 1.5 KB of arguments
+constexpr int kArgChunk = 384;   // the usual case; 1.5 KB of arguments
+constexpr int kArgLarge = 2048;  // 8 KB
 template <int kN> struct OffsetArgs { int32_t v[kN]; };
+// The arguments as ordinary memory, a word per thread: indexed directly they go through the constant cache, one word at a time.
+template <int kN>
+__device__ __forceinline__ const int32_t* offsets_memory(const OffsetArgs<kN>& a) {
+  const int32_t* from = a.v;
+  asm volatile("" : "+l"(from));
+  return from;
+}
 template <int kN>
 inline void fill_offsets(OffsetArgs<kN>* a, const int64_t* off_host, int n) {
   for (int t = 0; t < n; ++t) a->v[t] = (int32_t)off_host[t];

@@ -13,12 +13,12 @@ namespace {
 // Host values travel to the device as kernel arguments: no hidden synchronisation with the stream, and nothing that reads
 // the caller's array after the call returns.
 constexpr int64_t kSms = 148;  // of a B200: the rules below that fill the machine
-constexpr int kArgLarge = 2048;  // offsets of one launch: 8 KB of arguments
 template <int kN>
 __global__ void __launch_bounds__(256) k_store_offsets(const __grid_constant__ OffsetArgs<kN> a, int64_t base, int n,
                                                        int64_t* __restrict__ off) {
   pdl_wait();
-  for (int t = threadIdx.x; t < n; t += blockDim.x) off[base + t] = a.v[t];
+  const int32_t* from = offsets_memory(a);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) off[base + t] = from[t];
 }
 
 // What a kernel over all tokens needs before it starts, in one launch: the offsets in the workspace, the regions it adds
@@ -42,7 +42,8 @@ __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ OffsetArgs
                                               int64_t* __restrict__ off_dev, const float* __restrict__ coeffs,
                                               void* __restrict__ out, const __grid_constant__ Clear clear) {
   __shared__ int32_t s_off[kN];
-  for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = a.v[i];
+  const int32_t* from = offsets_memory(a);
+  for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = from[i];
   pdl_wait();
   __syncthreads();
   if (blockIdx.x == 0)

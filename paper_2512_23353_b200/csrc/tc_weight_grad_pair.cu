@@ -227,45 +227,45 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
   if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
 }
 
-// dst[t, :] = bf16(coeffs[sequence of t] * src[t, :]) (round to nearest even).  A warp takes a token: one search for its
-// sequence, then 16-byte pieces of the row, four in flight per lane.  HBM stream.
-// kArgs: offsets in the arguments (read as ordinary memory, see stored_extents), so that no kernel runs ahead of this one;
-// otherwise they are staged from the workspace, above kScaleMaxSeqs searched there.
-constexpr int kScaleMaxSeqs = 2048;
-template <bool kArgs>
-__global__ void __launch_bounds__(256) k_scale_rows(const uint4* __restrict__ src,
-                                                    const __grid_constant__ OffsetArgs<kArgs ? kArgChunk : 1> args,
+// dst[t, :] = bf16(coeffs[sequence of t] * src[t, :]) (round to nearest even).  A warp takes a token: its first 128 16-byte pieces are on
+// the way while it searches for its sequence.  HBM stream.
+// kN > 0: up to kN - 1 sequences, the offsets in the arguments, so that no kernel runs ahead of this one; otherwise they are searched in
+// the workspace.  46,546 tokens of 256 columns, 791 sequences: offsets and clear by a kernel of their own 2.6 + 16.7 us, so 15.7;
+// 40,600 of 896, 1024 sequences 9.3 + 20.6, so 23.8.  Two tokens to a warp were slower (10,533 of 896: 6.5 -> 8.3).  Registers for six
+// CTAs per SM: they wait beside the GEMM of the call before.
+template <int kN>
+__global__ void __launch_bounds__(256, 6) k_scale_rows(const uint4* __restrict__ src, const __grid_constant__ OffsetArgs<kN ? kN : 1> args,
                                                     const int64_t* __restrict__ off, int B, const float* __restrict__ coeffs,
                                                     int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst,
                                                     const __grid_constant__ Clear clear) {
-  __shared__ int32_t s_off[kArgs ? kArgChunk : kScaleMaxSeqs + 1];
-  if (kArgs) {
-    const int32_t* from = args.v;
-    asm volatile("" : "+l"(from));
+  __shared__ int32_t s_off[kN ? kN : 1];
+  if (kN) {
+    const int32_t* from = offsets_memory(args);
     for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = from[i];
   }
   pdl_wait();
-  const bool staged = kArgs || B <= kScaleMaxSeqs;
-  if (!kArgs && staged)
-    for (int i = threadIdx.x; i <= B; i += blockDim.x) s_off[i] = (int32_t)off[i];
   __syncthreads();
-  if (kArgs) clear_regions(clear);
+  if (kN) clear_regions(clear);
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += warps) {
-    int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if ((staged ? (int64_t)s_off[mid] : off[mid]) <= t) lo = mid; else hi = mid;
-    }
-    const float c = __ldg(coeffs + lo);
     const uint4* from = src + t * d8;
     uint4* to = dst + t * d8;
-    for (int e0 = lane; e0 < d8; e0 += 128) {
-      uint4 v[4];
+    uint4 v[4];
+    auto load = [&](int e0) {
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (e0 + 32 * u < d8) v[u] = __ldcs(from + e0 + 32 * u);
+    };
+    load(lane);
+    int lo = 0, hi = B;  // invariant: off[lo] <= t < off[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if ((kN ? (int64_t)s_off[mid] : off[mid]) <= t) lo = mid; else hi = mid;
+    }
+    const float c = __ldg(coeffs + lo);
+    for (int e0 = lane; e0 < d8; e0 += 128) {
+      if (e0 != lane) load(e0);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (e0 + 32 * u >= d8) continue;
@@ -341,19 +341,24 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
     int64_t ctas = (T + 7) / 8;
     // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
     // 4000 tokens a 4096 x 4096 dW took 10 us longer than from a kernel of its own, hence a CTA for every 16 KB as well.
+    ctas = std::max(ctas, clear.n[0] / 4096);
+    const int grid = (int)std::min<int64_t>(ctas, (int64_t)sms * 16);
+    auto with_args = [&](auto kernel, auto* a) {
+      fill_offsets(a, off_host, B + 1);
+      LaunchScope scope(kIdScaleRows, st);
+      launch(kernel, grid, 256, 0, st, src, *a, off_dev, B, coeffs, T, d8, (uint4*)scaled, clear);
+    };
     if (B + 1 <= kArgChunk) {
       OffsetArgs<kArgChunk> a;
-      fill_offsets(&a, off_host, B + 1);
-      ctas = std::max(ctas, clear.n[0] / 4096);
-      LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows<true>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, a, off_dev, B, coeffs, T, d8,
-             (uint4*)scaled, clear);
+      with_args(k_scale_rows<kArgChunk>, &a);
+    } else if (B + 1 <= kArgLarge) {
+      OffsetArgs<kArgLarge> a;
+      with_args(k_scale_rows<kArgLarge>, &a);
     } else {
       isopo_status s = launch_offsets(off_host, B, off_dev, clear, st);
       if (s != ISOPO_OK) return s;
       LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows<false>, (int)std::min<int64_t>(ctas, (int64_t)sms * 16), 256, 0, st, src, OffsetArgs<1>{}, off_dev, B,
-             coeffs, T, d8, (uint4*)scaled, Clear{});
+      launch(k_scale_rows<0>, grid, 256, 0, st, src, OffsetArgs<1>{}, off_dev, B, coeffs, T, d8, (uint4*)scaled, Clear{});
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
     if (scale_y) dY = scaled; else X = scaled;
