@@ -548,11 +548,11 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
     if (s != ISOPO_OK) return s;
     return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, tokscale, dW, st);
   }
+  if (!bf16_weight_grad_uses_pairs(T, d_in, d_out, B))
+    return bf16_weight_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, info, st);
   if (bf16_weight_grad_fold_applies(T, d_in, d_out, B))
     return bf16_weight_grad_fold(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, dW, add, info, st);
-  if (bf16_weight_grad_uses_pairs(d_out))
-    return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, add, info, st);
-  return bf16_weight_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, info, st);
+  return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, add, info, st);
 }
 
 }  // extern "C"

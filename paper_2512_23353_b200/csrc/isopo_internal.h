@@ -349,7 +349,7 @@ isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                               int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add, int32_t* info,
                               cudaStream_t st);
-bool bf16_weight_grad_uses_pairs(int d_out);
+bool bf16_weight_grad_uses_pairs(int64_t T, int d_in, int d_out, int B);
 
 // dW with the per-sequence coefficient applied when a segment's accumulator is drained (no scaled operand copy)
 bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);

@@ -376,10 +376,19 @@ isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, i
   return ISOPO_OK;
 }
 
-// 2-CTA tiles when they waste little (see bf16_seq_grad)
-bool bf16_weight_grad_uses_pairs(int d_out) {
+// Where the 2-CTA kernels (coefficient at the drain, or scaled operand) are the better stand-alone weight gradients: when they waste
+// little, and of an odd, small number of 128-row tiles from about a thousand stages of tiles on, because a 1-CTA tile rescales its
+// dY rows for every column of tiles and reaches two thirds of their rate.  1-CTA / 2-CTA, us, 512 x 600, 10 tiles: 3000 tokens 11.9 /
+// 13.3, 6000 15.3 / 15.7, 12,000 22.8 / 18.0; 432 x 304, 6 tiles: 12,000 16.9 / 15.2, 24,927 26.0 / 18.6; 2048 x 640, 40 tiles: 2000
+// 19.2 / 17.2, 8000 50.4 / 26.7; 4096 x 600, 80 tiles: 300 11.7 / 9.9.  Of one row of tiles half a pair is idle: one or two tiles, whose
+// tokens are all there is to split, 64 x 64: 100,000 tokens 16.5 / 14.9, 200,000 26.6 / 20.4, 512 x 128: 30,000 16.0 / 15.4, 60,000 22.8 / 19.3
+// (1000 sequences, scaled operand: 23.4 / 34.3); wide layers, 4096 x 104: 20,000 47.3 / 40.8; but 1848 x 88: 30,000 36.4 / 38.6.
+bool bf16_weight_grad_uses_pairs(int64_t T, int d_in, int d_out, int B) {
   const int tiles_m = (d_out + kTileM - 1) / kTileM;
-  return tiles_m % 2 == 0 || tiles_m >= 7;
+  if (tiles_m % 2 == 0 || tiles_m >= 7) return true;
+  const int64_t tiles = (int64_t)tiles_m * ((d_in + kTileN - 1) / kTileN), stages = tiles * ((T + kKB - 1) / kKB);
+  if (tiles_m > 1) return stages >= 1000 || tiles >= 64;
+  return tiles <= 2 ? stages >= 1500 && bf16_weight_grad_fold_applies(T, d_in, d_out, B) : d_in > 2048 && stages >= 4000;
 }
 
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,

@@ -444,9 +444,8 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
 // move a quarter fewer operand bytes from L2 per flop, which under the power cap outweighs its extra
 // pass (8960 x 1536: 7.0-8.5 against 7.9-9.1 ms; 18944 x 3584: 34-40 against 37-48 ms).
 bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B) {
-  const int tiles_m = (d_out + kHalf - 1) / kHalf;
-  // 2-CTA tiles when they waste little; segments long enough that the drain per segment stays hidden
-  return (tiles_m % 2 == 0 || tiles_m >= 7) && std::max(d_in, d_out) <= 2048 && B <= kMaxSeqs && T >= (int64_t)B * 96 &&
+  // segments long enough that the drain per segment stays hidden
+  return std::max(d_in, d_out) <= 2048 && B <= kMaxSeqs && T >= (int64_t)B * 96 &&
          T < ((int64_t)1 << 31) - 4096;
 }
 

@@ -67,3 +67,28 @@ def test_written_tiles(b, Ls, d_in, d_out, shift):
     _run(b, X, dY, c, off, dW, 1.0)
     # 2 + dW rounded to float32 once more: up to 2^-24 of the sum's size per element
     assert ((dW.double() - 2.0 - want).norm() / want.norm()).item() <= TOL + 2.0 ** -24 * dW.double().norm().item() / want.norm().item()
+
+
+@pytest.mark.parametrize("Ls,d_in,d_out", [
+    ([111] * 60, 512, 600),      # five rows of tiles: just above a thousand stages of tiles (coefficient at the drain)
+    ([50] * 140, 512, 600),      # the same through the scaled operand
+    ([64] * 99, 512, 600),       # just below
+    ([3, 5], 4104, 264),         # three rows, many columns of tiles
+    ([1001] * 50, 512, 128),     # one row, two tiles
+    ([4000] * 25, 64, 72),       # one tile
+    ([15] * 1000, 4096, 104),    # one row of a wide layer
+])
+def test_few_rows_of_tiles(b, Ls, d_in, d_out):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d_in + len(Ls))
+    off = np.concatenate([[0], np.cumsum(Ls)]).astype(np.int64)
+    X = torch.randn((int(off[-1]), d_in), device="cuda", generator=gen).bfloat16()
+    dY = torch.randn((int(off[-1]), d_out), device="cuda", generator=gen).bfloat16()
+    c = torch.randn(len(Ls), device="cuda", generator=gen)
+    rows = c[torch.from_numpy(np.repeat(np.arange(len(Ls)), Ls)).cuda()][:, None]
+    want = (rows.double() * dY.double()).T @ X.double()
+    for beta in (0.0, 1.0):
+        dW = torch.full((d_out, d_in), 0.5, device="cuda")
+        _run(b, X, dY, c, off, dW, beta)
+        # the scaled operand's rounding to bf16, 2^-9 of each product at the most
+        assert ((dW.double() - beta * 0.5 - want).norm() / want.norm()).item() <= 2.0 ** -9
