@@ -46,6 +46,7 @@ struct GramParams {
   int32_t* info;
   int n_rows, n_row_tiles;  // sampled: sample rows and their 128-row tiles
   int strip;                // Gram: tile columns per strip of the pair order
+  uint32_t row_bytes;       // sampled: of a stage's row operand (fewer than 128 samples: no more rows than there are)
 };
 
 // The work units of a CTA: (row tile I, column tile J).  Gram: pairs I <= J of token tiles.
@@ -126,7 +127,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
           const CUtensorMap* cmap = kb < nkx ? &mapX : &mapY;
           const int x = (kb < nkx ? kb : kb - nkx) * kKF;
           const uint32_t dst = smem_base + stage * kStageBytes;
-          mbar_arrive_expect_tx(full_bar(stage), diag ? kOperandBytes : kStageBytes);
+          mbar_arrive_expect_tx(full_bar(stage), kSampled ? p.row_bytes + kOperandBytes : diag ? kOperandBytes : kStageBytes);
           tma_load_2d(dst, rmap, x, I * kTT, full_bar(stage));
           if (!diag) tma_load_2d(dst + kOperandBytes, cmap, x, J * kTT, full_bar(stage));
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -267,11 +268,12 @@ isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, in
   isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
   if (s != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
-  // only the n_samples real rows are in bounds: the rest of the last 128-row tile reads as zero
-  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, kTT)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
+  const uint32_t box_rows = sample_box_rows(n_samples);
+  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, box_rows)) != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   GramParams p{tokseq, Mt, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, n_samples, (n_samples + kTT - 1) / kTT, 0};
+  p.row_bytes = box_rows * 128;
   const long long units = (long long)p.n_row_tiles * p.nT;
   const int grid = (int)std::min<long long>(units, sms);
   {

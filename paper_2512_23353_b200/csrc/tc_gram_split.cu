@@ -47,6 +47,7 @@ struct GramSplitParams {
   int d_out[kMaxProj];
   int32_t* info;
   int n_rows, n_row_tiles;  // sampled: sample rows and their 128-row tiles
+  uint32_t row_bytes;       // sampled: of a stage's row operand
   int units;                // tiles of a projection
   bool complete;            // one cluster: it fills K's other triangle as well
 };
@@ -120,7 +121,7 @@ k_bf16_gram_split(const __grid_constant__ CUtensorMap mapRX, const __grid_consta
         const CUtensorMap* rmap = kSampled ? (second ? &mapRY : &mapRX) : cmap;
         const int x = (second ? kb - nkx : kb) * kKF;
         const uint32_t dst = smem_base + stage * kStageBytes;
-        mbar_arrive_expect_tx(full_bar(stage), diag ? kOperandBytes : kStageBytes);
+        mbar_arrive_expect_tx(full_bar(stage), kSampled ? p.row_bytes + kOperandBytes : diag ? kOperandBytes : kStageBytes);
         tma_load_2d(dst, rmap, x, I * kTT, full_bar(stage));
         if (!diag) tma_load_2d(dst + kOperandBytes, cmap, x, J * kTT, full_bar(stage));
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -289,14 +290,15 @@ isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t
   isopo_status s;
   if ((s = make_map_2d_bf16(&maps[2], X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT)) != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&maps[3], dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
-  // only the n_samples real rows are in bounds: the rest of the last 128-row tile reads as zero
-  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, kTT)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
+  const uint32_t box_rows = sample_box_rows(n_samples);
+  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, box_rows)) != ISOPO_OK) return s;
   maps[4] = maps[5] = maps[3];
   GramSplitParams p{};
   for (int h = 0; h < kMaxProj; ++h) { p.K[h] = Mt; p.d_out[h] = d_out; }
   p.tokseq = tokseq; p.T = T; p.B = B; p.nT = (int)((T + kTT - 1) / kTT); p.d_in = d_in; p.info = info;
   p.n_rows = n_samples;
+  p.row_bytes = box_rows * 128;
   p.n_row_tiles = (n_samples + kTT - 1) / kTT;
   p.units = p.nT * p.n_row_tiles;
   return dispatch<true>(ctas, maps, p, 1, kIdSampled, st);

@@ -71,7 +71,8 @@ def test_gram(b, Ls, d_in, d_outs):
 
 
 @pytest.mark.parametrize("Ls,d_in,d_out,n", [([40, 48], 2160, 416, 88), ([1, 200, 7], 896, 896, 1), ([300] * 20, 512, 2360, 128),
-                                             ([90, 400], 1024, 1024, 300)])
+                                             ([90, 400], 1024, 1024, 300),
+                                             ([700] * 30, 512, 520, 9), ([700] * 30, 512, 520, 33), ([40, 48], 2160, 416, 7)])  # boxes of fewer rows
 def test_sampled(b, Ls, d_in, d_out, n):
     off, X, (dY,) = _inputs(Ls, d_in, [d_out], 5 * d_in + n)
     B, T = len(Ls), int(off[-1])
