@@ -122,7 +122,7 @@ __device__ __forceinline__ void cluster_solve(const TransformParams& P, float* L
   // Factors and inverts the diagonal block of own row l and publishes the inverse, the right-hand side and whether a pivot
   // failed.  One warp of the owner.
   auto factor = [&](int l, int J) {
-    const int f = warp_factor_diag(blk(l, J), S.rdiag);
+    const int f = warp_factor_diag<false>(blk(l, J), S.rdiag);
     __syncwarp();
     warp_invert_factor(blk(l, J), S.rdiag, S.inv_own[l]);
     __syncwarp();

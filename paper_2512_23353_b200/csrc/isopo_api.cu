@@ -77,6 +77,50 @@ LaunchScope::~LaunchScope() {
 ProfilingPause::ProfilingPause() : was_on_(g_prof_on) { g_prof_on = false; }
 ProfilingPause::~ProfilingPause() { g_prof_on = was_on_; }
 
+// Copies of the Gram route's operands at a pitch of whole lines, where theirs is none: from 1000 tokens on the token tiles' many reads of
+// them outweigh a pass over the inputs.  isopo_layer_gram as they are / copied, us: 600 tokens, 2160 x 1032 15.1 / 16.6; 1000 19.0 / 17.8;
+// 1919, 1080 x 312 17.6 / 14.8; 5000, 2136 x 968 70 / 64; 15,000, 1080 x 312 238 / 204; 40,000, 232 x 600 1184 / 885.
+static bool repitch_pays(int64_t T, int B) { return T >= 1000 && B + 1 <= kArgLarge; }
+static size_t repitch_bytes(int64_t T, int d) { return d % 64 ? align_up((size_t)2 * (size_t)T * (size_t)line_pitch(d), 1024) : 0; }
+struct GramOperands {
+  const void* X;
+  const void* dY[3];
+  int ldx, ldy[3];
+  Repitch repitch;
+};
+// What of X and the n dY has to be copied and has room there, X and the widest first.
+static GramOperands gram_operands(const void* X, int d_in, int n, const void* const* dY, const int* d_out, int64_t T, int B, char* room,
+                                  size_t bytes) {
+  GramOperands g{};
+  g.X = X;
+  g.ldx = d_in;
+  for (int h = 0; h < n; ++h) { g.dY[h] = dY[h]; g.ldy[h] = d_out[h]; }
+  if (!repitch_pays(T, B)) return g;
+  auto take = [&](const void** p, int* ld) {
+    const size_t need = repitch_bytes(T, *ld);
+    if (need == 0 || need > bytes) return;
+    const int k = g.repitch.n++;
+    g.repitch.src[k] = (const uint4*)*p;
+    g.repitch.dst[k] = (uint4*)room;
+    g.repitch.d8[k] = *ld / 8;
+    g.repitch.p8[k] = line_pitch(*ld) / 8;
+    *p = room;
+    *ld = line_pitch(*ld);
+    room += need;
+    bytes -= need;
+  };
+  take(&g.X, &g.ldx);
+  bool done[3] = {};
+  for (int k = 0; k < n; ++k) {
+    int widest = -1;
+    for (int h = 0; h < n; ++h)
+      if (!done[h] && (widest < 0 || d_out[h] > d_out[widest])) widest = h;
+    done[widest] = true;
+    take(&g.dY[widest], &g.ldy[widest]);
+  }
+  return g;
+}
+
 WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved) {
   WsLayout L{};
   size_t p = 0;
@@ -94,7 +138,8 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
     p = align_up(p + (resolved == ISOPO_PATH_MATERIALISE ? sizeof(uint32_t) : sizeof(double) * (size_t)B * (size_t)B), 1024);
   L.off_scaled = p;
   if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM)
-    p = align_up(p + (size_t)2 * (size_t)T * (size_t)std::min(d_in, d_out), 1024);
+    p = align_up(p + std::max((size_t)2 * (size_t)T * (size_t)line_pitch(std::min(d_in, d_out)),
+                              repitch_pays(T, B) ? repitch_bytes(T, d_in) + repitch_bytes(T, d_out) : 0), 1024);
   L.off_G = p;
   if (dtype == ISOPO_BF16) {
     L.tiles_m = (d_out + kTileM - 1) / kTileM;
@@ -286,10 +331,14 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
   }
   double* kacc = (double*)(w + L.off_kacc);
   const int64_t bb = (int64_t)B * B;
-  s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, dtype == ISOPO_F32 ? Clear{{(float*)kacc}, {2 * bb}} : Clear{{K}, {bb}}, st);
-  if (s != ISOPO_OK) return s;
-  if (dtype == ISOPO_F32) return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);
-  return bf16_gram(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
+  if (dtype == ISOPO_F32) {
+    s = launch_prep(seq_offsets_host, B, T, off_dev, tokseq, Clear{{(float*)kacc}, {2 * bb}}, st);
+    return s != ISOPO_OK ? s : f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);
+  }
+  const GramOperands g = gram_operands(X, d_in, 1, &dY, &d_out, T, B, w + L.off_scaled, L.off_G - L.off_scaled);
+  s = g.repitch.n ? launch_prep_repitch(seq_offsets_host, B, T, off_dev, tokseq, Clear{{K}, {bb}}, g.repitch, st)
+                  : launch_prep(seq_offsets_host, B, T, off_dev, tokseq, Clear{{K}, {bb}}, st);
+  return s != ISOPO_OK ? s : bf16_gram(g.X, g.ldx, g.dY[0], g.ldy[0], T, d_in, d_out, tokseq, B, K, info, st);
 }
 
 isopo_status isopo_layer_gram_shared_x(const void* X, int n_proj, const void* const* dY, const int* d_out, isopo_dtype dtype,
@@ -312,9 +361,11 @@ isopo_status isopo_layer_gram_shared_x(const void* X, int n_proj, const void* co
   int32_t* tokseq = (int32_t*)(w + L.off_tokseq);
   Clear clear{};
   for (int h = 0; h < n_proj; ++h) { clear.p[h] = K[h]; clear.n[h] = (int64_t)B * B; }
-  isopo_status s = launch_prep(seq_offsets_host, B, T, (int64_t*)(w + L.off_offsets), tokseq, clear, st);
-  if (s != ISOPO_OK) return s;
-  return bf16_gram_shared(X, dY, T, d_in, d_out, n_proj, tokseq, B, K, info, st);
+  const GramOperands g = gram_operands(X, d_in, n_proj, dY, d_out, T, B, w + L.off_scaled, L.off_G - L.off_scaled);
+  int64_t* off_dev = (int64_t*)(w + L.off_offsets);
+  const isopo_status s = g.repitch.n ? launch_prep_repitch(seq_offsets_host, B, T, off_dev, tokseq, clear, g.repitch, st)
+                                     : launch_prep(seq_offsets_host, B, T, off_dev, tokseq, clear, st);
+  return s != ISOPO_OK ? s : bf16_gram_shared(g.X, g.ldx, g.dY, g.ldy, T, d_in, d_out, n_proj, tokseq, B, K, info, st);
 }
 
 isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const void* const* dY, const int* d_out,

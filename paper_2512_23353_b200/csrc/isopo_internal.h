@@ -147,7 +147,8 @@ struct WsLayout {
   size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here, the bf16
                        // stored route what its K pass adds into (float [B][ntk_pitch(B)])
   size_t off_kacc;     // float32 path: float64 [B*B] K accumulators (Gram), uint32 CTAs of the K pass that are done (materialised)
-  size_t off_scaled;   // bf16 [T, min(d_in, d_out)]  (bf16 Gram path: the pre-scaled operand of the weight-gradient GEMM)
+  size_t off_scaled;   // bf16 Gram path: copies of the operands at a pitch of whole lines (repitch_bytes), later the pre-scaled operand of the
+                       // weight-gradient GEMM, bf16 [T, line_pitch(min(d_in, d_out))]
   size_t off_G;        // stored gradients (materialised path only)
   size_t off_kpart;    // per-CTA partial K (materialised path; bf16: in deterministic mode only)
   size_t total;
@@ -245,6 +246,18 @@ __device__ __forceinline__ void clear_regions(const Clear& c) {
     for (int64_t e = 4 * quads + first; e < c.n[k]; e += step) c.p[k][e] = 0.f;
   }
 }
+// Row pitch of the library's own copies of bf16 operands, in elements: whole 128-byte lines.  TMA copies 128 bytes of a row at a time;
+// where rows start anywhere, that is two lines of the L2 each: sampled estimator of 37,888 tokens, 128 samples, 2136 x 968 61 us, 2048 x
+// 1024 39 us.
+__host__ __device__ inline int line_pitch(int d) { return (d + 63) & ~63; }
+// Rows that a launch copies to a pitch of whole lines for the kernels behind it (n operands).
+constexpr int kMaxRepitch = 4;
+struct Repitch {
+  const uint4* src[kMaxRepitch];
+  uint4* dst[kMaxRepitch];
+  int d8[kMaxRepitch], p8[kMaxRepitch];  // row and pitch in 16-byte pieces
+  int n;
+};
 // Token offsets as kernel arguments (no host-to-device copy); they are below 2^31 and travel as 32-bit values.
 constexpr int kArgChunk = 384;   // the usual case; 1.5 KB of arguments
 constexpr int kArgLarge = 2048;  // 8 KB
@@ -263,6 +276,9 @@ inline void fill_offsets(OffsetArgs<kN>* a, const int64_t* off_host, int n) {
 // offsets and the token -> sequence map to the device, `clear` cleared
 isopo_status launch_prep(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, const Clear& clear,
                          cudaStream_t st);
+// the same (fewer than kArgLarge sequences), and rows copied to another pitch
+isopo_status launch_prep_repitch(const int64_t* off_host, int B, int64_t T, int64_t* off_dev, int32_t* tokseq, const Clear& clear,
+                                 const Repitch& repitch, cudaStream_t st);
 // the offsets alone
 isopo_status launch_offsets(const int64_t* off_host, int B, int64_t* off_dev, const Clear& clear, cudaStream_t st);
 // offsets and tokscale[t] = coeffs[sequence of token t] (float32 [T])
@@ -329,19 +345,20 @@ isopo_status bf16_combine(const void* G, const WsLayout& L, int d_in, int d_out,
                           float beta, const WsTag* tag_dev, const WsTag& tag, const StoreFmt& fmt, int32_t* info,
                           cudaStream_t st);
 // The Gram and sampled kernels ADD into K and M^T: the caller has cleared them on this stream.
-isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
+// (ld: elements from row to row)
+isopo_status bf16_gram(const void* X, int ldx, const void* dY, int ldy, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                        float* K, int32_t* info, cudaStream_t st);
 // 2-CTA tiles, one projection or several that share X: where they pay
 bool bf16_gram_pair_pays(int64_t T, int d_in, const int* d_out, int n_heads, int sms);
-isopo_status bf16_gram_pair(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_pair(const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                             const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
-isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_shared(const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 // The stand-alone weight gradients prepare what they need (offsets through off_dev, a cleared dW where its shares are added up);
 // `add`: dW is added to.
 // few tiles: a cluster of `ctas` CTAs shares the features of a tile (1: the kernels above are the better)
 int gram_split_ctas(long long units, int d_in, int d_out, int sms);
-isopo_status bf16_gram_split(int ctas, const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                              const int32_t* tokseq, int B, float* const* K, bool complete, int32_t* info, cudaStream_t st);
 isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                                 const void* A0, const void* G0, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
@@ -366,7 +383,7 @@ struct PlainPlan {
   bool clear;  // dW has to be cleared ahead of it
 };
 PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, bool add, int pairs);
-isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
+isopo_status bf16_weight_grad_plain(const void* X, int ldx, const void* dY, int ldy, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
                                     float* dW, int32_t* info, cudaStream_t st);
 
 // token-sampled estimator of Algorithm 1

@@ -74,8 +74,9 @@ __global__ void __launch_bounds__(256) k_gather_samples(const T* __restrict__ X,
   pdl_wait();
   const int j = blockIdx.x;
   const int64_t t = rows.v[j];
-  double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * d_in, d_in);
-  double ng = copy_row_sq(dY + t * d_out, g0 + (size_t)j * d_out, d_out);
+  constexpr bool kLines = sizeof(T) == 2;  // bf16: the tensor-core kernels' copies start at whole lines
+  double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * (kLines ? line_pitch(d_in) : d_in), d_in);
+  double ng = copy_row_sq(dY + t * d_out, g0 + (size_t)j * (kLines ? line_pitch(d_out) : d_out), d_out);
   na = block_sum_d(na);
   ng = block_sum_d(ng);
   if (threadIdx.x == 0) atomicAdd(den, na * ng);
@@ -137,9 +138,10 @@ SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, 
   const size_t elt = dtype == ISOPO_BF16 ? 2 : 4;
   size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM).total;  // offsets, token map (+ kacc)
   S.off_a0 = p;
-  p = align_up(p + elt * (size_t)n_samples * d_in, 1024);
+  const bool lines = dtype == ISOPO_BF16;  // the gathered rows lie at a pitch of whole lines
+  p = align_up(p + elt * (size_t)n_samples * (lines ? line_pitch(d_in) : d_in), 1024);
   S.off_g0 = p;
-  p = align_up(p + elt * (size_t)n_samples * d_out, 1024);
+  p = align_up(p + elt * (size_t)n_samples * (lines ? line_pitch(d_out) : d_out), 1024);
   S.off_mt = p;
   p = align_up(p + (dtype == ISOPO_BF16 ? sizeof(float) : sizeof(double)) * (size_t)n_samples * B, 1024);
   S.off_den = p;

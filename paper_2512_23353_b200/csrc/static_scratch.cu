@@ -86,5 +86,5 @@ extern "C" ISOPO_API isopo_status isopo_layer_gram_static(const void* X, const v
   if (s != ISOPO_OK) return s;
   if (dtype == ISOPO_F32)
     return f32_gram((const float*)X, (const float*)dY, T, d_in, d_out, tokseq, B, kacc, K, st);
-  return bf16_gram(X, dY, T, d_in, d_out, tokseq, B, K, info, st);
+  return bf16_gram(X, d_in, dY, d_out, T, d_in, d_out, tokseq, B, K, info, st);
 }

@@ -224,7 +224,7 @@ k_bf16_gram(const __grid_constant__ CUtensorMap mapRX, const __grid_constant__ C
 
 }  // namespace
 
-isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
+isopo_status bf16_gram(const void* X, int ldx, const void* dY, int ldy, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                        float* K, int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
@@ -233,15 +233,15 @@ isopo_status bf16_gram(const void* X, const void* dY, int64_t T, int d_in, int d
   const long long units = (long long)p.nT * (p.nT + 1) / 2;
   const int grid = (int)std::min<long long>(units, sms), ctas = gram_split_ctas(units, d_in, d_out, sms);
   if (ctas > 1) {
-    const isopo_status r = bf16_gram_split(ctas, X, &dY, T, d_in, &d_out, 1, tokseq, B, &K, units == 1 && B <= 32, info, st);
+    const isopo_status r = bf16_gram_split(ctas, X, ldx, &dY, &ldy, T, d_in, &d_out, 1, tokseq, B, &K, units == 1 && B <= 32, info, st);
     return r != ISOPO_OK || (units == 1 && B <= 32) ? r : mirror_upper(K, B, st);
   }
   CUtensorMap mapX, mapY;
-  isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
+  isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)ldx, 64, kTT);
   if (s != ISOPO_OK) return s;
-  s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT);
+  s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)ldy, 64, kTT);
   if (s != ISOPO_OK) return s;
-  if (bf16_gram_pair_pays(T, d_in, &d_out, 1, sms)) return bf16_gram_pair(X, &dY, T, d_in, &d_out, 1, tokseq, B, &K, info, st);
+  if (bf16_gram_pair_pays(T, d_in, &d_out, 1, sms)) return bf16_gram_pair(X, ldx, &dY, &ldy, T, d_in, &d_out, 1, tokseq, B, &K, info, st);
   // One tile of tokens: its CTA completes K, a launch less for the host, which bounds so small a layer (26 tokens, 640 x 280:
   // 29.1 -> 26.4 us with the scaling pass's).  The last of several CTAs would be 0.7 (15 CTAs) to 1.3 us (136) slower than a
   // kernel that is already set up when this one ends, and above 32 sequences so is one CTA.
@@ -269,8 +269,8 @@ isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, in
   if (s != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
   const uint32_t box_rows = sample_box_rows(n_samples);
-  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, box_rows)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)line_pitch(d_in), 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)line_pitch(d_out), 64, box_rows)) != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   GramParams p{tokseq, Mt, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, n_samples, (n_samples + kTT - 1) / kTT, 0};
   p.row_bytes = box_rows * 128;

@@ -242,22 +242,23 @@ bool bf16_gram_pair_pays(int64_t T, int d_in, const int* d_out, int n_heads, int
   return pair_waves * std::max((pair_waves >= 5 ? 1.45 : 1.65) * nk, 14.0 * n_heads) + 12 < waves * std::max((double)nk, 6.5 * n_heads);
 }
 
-isopo_status bf16_gram_pair(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_pair(const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                             const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st) {
   if (n_heads < 1 || n_heads > kMaxHeads) return ISOPO_ERR_INVALID_ARG;
   // P o Q = Q o P: of one projection the wider operand goes first
   const void* operand[1 + kMaxHeads] = {X, dY[0]};
-  int d[1 + kMaxHeads] = {d_in, d_out[0]}, d_sum = 0;
+  int d[1 + kMaxHeads] = {d_in, d_out[0]}, ld[1 + kMaxHeads] = {ldx, ldy[0]}, d_sum = 0;
   if (n_heads == 1 && d[1] > d[0]) {
     std::swap(operand[0], operand[1]);
     std::swap(d[0], d[1]);
+    std::swap(ld[0], ld[1]);
   }
   GramPairParams p{};
-  for (int h = 1; h < n_heads; ++h) { operand[1 + h] = dY[h]; d[1 + h] = d_out[h]; }
+  for (int h = 1; h < n_heads; ++h) { operand[1 + h] = dY[h]; d[1 + h] = d_out[h]; ld[1 + h] = ldy[h]; }
   CUtensorMap map[1 + kMaxHeads];
   for (int f = 0; f <= kMaxHeads; ++f) {
     const int ff = std::min(f, n_heads);  // unused slots repeat the last projection's map
-    isopo_status s = make_map_2d_bf16(&map[f], operand[ff], (uint64_t)T, (uint64_t)d[ff], (uint64_t)d[ff], 64, kTT);
+    isopo_status s = make_map_2d_bf16(&map[f], operand[ff], (uint64_t)T, (uint64_t)d[ff], (uint64_t)ld[ff], 64, kTT);
     if (s != ISOPO_OK) return s;
     if (f > n_heads) continue;
     p.nk[f] = (d[f] + kKF - 1) / kKF;

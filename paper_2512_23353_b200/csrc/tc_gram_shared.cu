@@ -213,7 +213,7 @@ k_bf16_gram_shared(const __grid_constant__ CUtensorMap mapX, const __grid_consta
 
 }  // namespace
 
-isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_shared(const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st) {
   if (n_heads < 1 || n_heads > kMaxHeads) return ISOPO_ERR_INVALID_ARG;
   int dev = 0, sms = 0;
@@ -222,18 +222,18 @@ isopo_status bf16_gram_shared(const void* X, const void* const* dY, int64_t T, i
   const long long tiles = (T + kTT - 1) / kTT;
   const int ctas = gram_split_ctas(tiles * (tiles + 1) / 2 * n_heads, d_in, *std::min_element(d_out, d_out + n_heads), sms);
   if (ctas > 1) {
-    isopo_status r = bf16_gram_split(ctas, X, dY, T, d_in, d_out, n_heads, tokseq, B, K, false, info, st);
+    isopo_status r = bf16_gram_split(ctas, X, ldx, dY, ldy, T, d_in, d_out, n_heads, tokseq, B, K, false, info, st);
     for (int h = 0; h < n_heads && r == ISOPO_OK; ++h) r = mirror_upper(K[h], B, st);
     return r;
   }
   if (bf16_gram_pair_pays(T, d_in, d_out, n_heads, sms))
-    return bf16_gram_pair(X, dY, T, d_in, d_out, n_heads, tokseq, B, K, info, st);
+    return bf16_gram_pair(X, ldx, dY, ldy, T, d_in, d_out, n_heads, tokseq, B, K, info, st);
   CUtensorMap mapX, mapY[kMaxHeads];
-  isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
+  isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)ldx, 64, kTT);
   if (s != ISOPO_OK) return s;
   for (int h = 0; h < kMaxHeads; ++h) {
     const int hh = std::min(h, n_heads - 1);  // unused slots repeat the last projection's map
-    s = make_map_2d_bf16(&mapY[h], dY[hh], (uint64_t)T, (uint64_t)d_out[hh], (uint64_t)d_out[hh], 64, kTT);
+    s = make_map_2d_bf16(&mapY[h], dY[hh], (uint64_t)T, (uint64_t)d_out[hh], (uint64_t)ldy[hh], 64, kTT);
     if (s != ISOPO_OK) return s;
   }
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));

@@ -264,14 +264,14 @@ int gram_split_ctas(long long units, int d_in, int d_out, int sms) {
   return c;
 }
 
-isopo_status bf16_gram_split(int ctas, const void* X, const void* const* dY, int64_t T, int d_in, const int* d_out, int n_heads,
+isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                              const int32_t* tokseq, int B, float* const* K, bool complete, int32_t* info, cudaStream_t st) {
   CUtensorMap maps[6];
-  isopo_status s = make_map_2d_bf16(&maps[2], X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
+  isopo_status s = make_map_2d_bf16(&maps[2], X, (uint64_t)T, (uint64_t)d_in, (uint64_t)ldx, 64, kTT);
   GramSplitParams p{};
   for (int h = 0; h < kMaxProj && s == ISOPO_OK; ++h) {
     const int k = h < n_heads ? h : 0;
-    s = make_map_2d_bf16(&maps[3 + h], dY[k], (uint64_t)T, (uint64_t)d_out[k], (uint64_t)d_out[k], 64, kTT);
+    s = make_map_2d_bf16(&maps[3 + h], dY[k], (uint64_t)T, (uint64_t)d_out[k], (uint64_t)ldy[k], 64, kTT);
     p.K[h] = K[k];
     p.d_out[h] = d_out[k];
   }
@@ -291,8 +291,8 @@ isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t
   if ((s = make_map_2d_bf16(&maps[2], X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT)) != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&maps[3], dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
   const uint32_t box_rows = sample_box_rows(n_samples);
-  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)d_in, 64, box_rows)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)d_out, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)line_pitch(d_in), 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)line_pitch(d_out), 64, box_rows)) != ISOPO_OK) return s;
   maps[4] = maps[5] = maps[3];
   GramSplitParams p{};
   for (int h = 0; h < kMaxProj; ++h) { p.K[h] = Mt; p.d_out[h] = d_out; }

@@ -477,12 +477,12 @@ static isopo_status resident_pairs(int* pairs) {
   return ISOPO_OK;
 }
 
-static isopo_status make_fold_maps(CUtensorMap* mapY, CUtensorMap* mapX, CUtensorMap* mapW, const void* X, const void* dY, float* dW,
+static isopo_status make_fold_maps(CUtensorMap* mapY, CUtensorMap* mapX, CUtensorMap* mapW, const void* X, int ldx, const void* dY, int ldy, float* dW,
                                    int64_t T, int d_in, int d_out, uint32_t box_cols) {
   isopo_status s = make_map_2d_f32(mapW, dW, (uint64_t)d_out, (uint64_t)d_in, box_cols);
   if (s != ISOPO_OK) return s;
-  s = make_map_2d_bf16(mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
-  return s != ISOPO_OK ? s : make_map_2d_bf16(mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
+  s = make_map_2d_bf16(mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)ldy, 64, kKB);
+  return s != ISOPO_OK ? s : make_map_2d_bf16(mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)ldx, 64, kKB);
 }
 
 static void set_group(FoldParams* p, int npairs) {
@@ -509,13 +509,13 @@ PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, bool add, int p
   return plan;
 }
 
-isopo_status bf16_weight_grad_plain(const void* X, const void* dY, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
+isopo_status bf16_weight_grad_plain(const void* X, int ldx, const void* dY, int ldy, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
                                     float* dW, int32_t* info, cudaStream_t st) {
   int pairs = 0;
   isopo_status s = resident_pairs<true>(&pairs);
   if (s != ISOPO_OK) return s;
   CUtensorMap mapY, mapX, mapW;
-  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, dY, dW, T, d_in, d_out, 32)) != ISOPO_OK) return s;
+  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, ldx, dY, ldy, dW, T, d_in, d_out, 32)) != ISOPO_OK) return s;
   FoldParams p{};
   p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
@@ -539,7 +539,7 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
   isopo_status s = resident_pairs<false>(&pairs);
   if (s != ISOPO_OK) return s;
   CUtensorMap mapY, mapX, mapW;
-  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, dY, dW, T, d_in, d_out, 16)) != ISOPO_OK) return s;
+  if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, d_in, dY, d_out, dW, T, d_in, d_out, 16)) != ISOPO_OK) return s;
   FoldParams p{};
   p.off = off_dev; p.coeffs = coeffs; p.dW = dW; p.T = T; p.B = B; p.d_in = d_in; p.d_out = d_out; p.info = info;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;

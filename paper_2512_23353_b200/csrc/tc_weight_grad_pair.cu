@@ -236,7 +236,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
 template <int kN>
 __global__ void __launch_bounds__(256, 6) k_scale_rows(const uint4* __restrict__ src, const __grid_constant__ OffsetArgs<kN ? kN : 1> args,
                                                     const int64_t* __restrict__ off, int B, const float* __restrict__ coeffs,
-                                                    int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst,
+                                                    int64_t T, int d8 /* columns / 8 */, uint4* __restrict__ dst, int p8 /* its pitch / 8 */,
                                                     const __grid_constant__ Clear clear) {
   __shared__ int32_t s_off[kN ? kN : 1];
   if (kN) {
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256, 6) k_scale_rows(const uint4* __restrict__
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += warps) {
     const uint4* from = src + t * d8;
-    uint4* to = dst + t * d8;
+    uint4* to = dst + t * p8;
     uint4 v[4];
     auto load = [&](int e0) {
 #pragma unroll
@@ -334,9 +334,10 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
   p.nslabs = (int)nslabs;
   p.store = !add && nslabs == 1;
   const Clear clear = !add && (plain ? plan.clear : !p.store) ? Clear{{dW}, {(int64_t)d_in * d_out}} : Clear{};
+  int ldx = d_in, ldy = d_out;
   {  // scale the narrower operand into `scaled`
     const bool scale_y = d_out <= d_in;
-    const int d8 = (scale_y ? d_out : d_in) / 8;
+    const int d8 = (scale_y ? d_out : d_in) / 8, p8 = line_pitch(8 * d8) / 8;
     const uint4* src = (const uint4*)(scale_y ? dY : X);
     int64_t ctas = (T + 7) / 8;
     // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
@@ -346,7 +347,7 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
     auto with_args = [&](auto kernel, auto* a) {
       fill_offsets(a, off_host, B + 1);
       LaunchScope scope(kIdScaleRows, st);
-      launch(kernel, grid, 256, 0, st, src, *a, off_dev, B, coeffs, T, d8, (uint4*)scaled, clear);
+      launch(kernel, grid, 256, 0, st, src, *a, off_dev, B, coeffs, T, d8, (uint4*)scaled, p8, clear);
     };
     if (B + 1 <= kArgChunk) {
       OffsetArgs<kArgChunk> a;
@@ -358,16 +359,16 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
       isopo_status s = launch_offsets(off_host, B, off_dev, clear, st);
       if (s != ISOPO_OK) return s;
       LaunchScope scope(kIdScaleRows, st);
-      launch(k_scale_rows<0>, grid, 256, 0, st, src, OffsetArgs<1>{}, off_dev, B, coeffs, T, d8, (uint4*)scaled, Clear{});
+      launch(k_scale_rows<0>, grid, 256, 0, st, src, OffsetArgs<1>{}, off_dev, B, coeffs, T, d8, (uint4*)scaled, p8, Clear{});
     }
     ISOPO_CUDA_TRY(cudaGetLastError());
-    if (scale_y) dY = scaled; else X = scaled;
+    if (scale_y) { dY = scaled; ldy = 8 * p8; } else { X = scaled; ldx = 8 * p8; }
   }
-  if (plain) return bf16_weight_grad_plain(X, dY, T, d_in, d_out, plan, add, dW, info, st);
+  if (plain) return bf16_weight_grad_plain(X, ldx, dY, ldy, T, d_in, d_out, plan, add, dW, info, st);
   CUtensorMap mapY, mapX;
-  isopo_status s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kKB);
+  isopo_status s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)ldy, 64, kKB);
   if (s != ISOPO_OK) return s;
-  s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kKB);
+  s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)ldx, 64, kKB);
   if (s != ISOPO_OK) return s;
   CUtensorMap mapW;
   if ((s = make_map_2d_f32(&mapW, dW, (uint64_t)d_out, (uint64_t)d_in, 32)) != ISOPO_OK) return s;

@@ -90,5 +90,6 @@ def test_few_rows_of_tiles(b, Ls, d_in, d_out):
     for beta in (0.0, 1.0):
         dW = torch.full((d_out, d_in), 0.5, device="cuda")
         _run(b, X, dY, c, off, dW, beta)
-        # the scaled operand's rounding to bf16, 2^-9 of each product at the most
-        assert ((dW.double() - beta * 0.5 - want).norm() / want.norm()).item() <= 2.0 ** -9
+        # the scaled operand is rounded to bf16, by at most 2^-8 (half of its eighth bit) of each product, however they cancel; float32 sums beside it
+        bound = (rows.double() * dY.double()).abs().T @ X.double().abs() + beta * 0.5
+        assert ((dW.double() - beta * 0.5 - want).abs() <= (2.0 ** -8 + 1e-5) * bound).all()
