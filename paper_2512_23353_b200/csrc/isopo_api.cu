@@ -311,8 +311,8 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     const StoreFmt fmt = store_fmt(L, B, ws);
     NtkPlan plan;
     if ((s = plan_ntk(L, B, fmt.split, deterministic_mode(), &plan)) != ISOPO_OK) return s;
-    float* acc = plan.by_last ? K : (float*)tokseq;
-    make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &acc, plan.by_last ? B * B : B * ntk_pitch(B));
+    float* acc = plan.by_boxes ? (float*)tokseq : K;
+    make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &acc, plan.by_boxes ? B * ntk_pitch(B) : B * B);
     if (fmt.split) {
       s = launch_offsets(seq_offsets_host, B, off_dev, Clear{}, st);
       if (s == ISOPO_OK) s = launch_seq_scales(X, dY, d_in, d_out, off_dev, B, (float*)fmt.scales, fmt.kdiag, st);
@@ -397,7 +397,6 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
     head[h] = (WsHead*)(w + L[h].off_tag);
     G[h] = w + L[h].off_G;
     fmt[h] = store_fmt(L[h], B, ws[h]);
-    acc[h] = (float*)(w + L[h].off_tokseq);
     pairs_fit = pairs_fit && (L[h].tiles_m % 2 == 0 || L[h].tiles_m >= 7);
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -410,17 +409,12 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
       if (s == ISOPO_OK) s = launch_seq_scales(X, dY[h], d_in, d_out[h], off_dev, B, (float*)fmt[h].scales, fmt[h].kdiag, st);
       if (s != ISOPO_OK) return s;
     }
-  NtkPlan plan[3];
-  bool all_last = true;
+  NtkPlan plan[3];  // by_boxes is the same for all: the number of sequences says
   for (int h = 0; h < n_proj; ++h) {
     if ((s = plan_ntk(L[h], B, fmt[h].split, deterministic_mode(), &plan[h])) != ISOPO_OK) return s;
-    all_last = all_last && plan[h].by_last;
+    acc[h] = plan[h].by_boxes ? (float*)((char*)ws[h] + L[h].off_tokseq) : K[h];
   }
-  for (int h = 0; h < n_proj; ++h) {  // one way for all: they are cleared alike
-    plan[h].by_last = all_last;
-    if (all_last) acc[h] = K[h];
-  }
-  const int n_acc = all_last ? B * B : B * ntk_pitch(B);
+  const int n_acc = plan[0].by_boxes ? B * ntk_pitch(B) : B * B;
   StoredIntake in;
   if (pairs_fit) {
     make_stored_intake(&in, seq_offsets_host, B, n_proj, tag, head, acc, n_acc);

@@ -325,15 +325,15 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
                                        const StoredIntake& in, int B, const WsLayout* L, void* const* G, const StoreFmt* fmt,
                                        int32_t* info, cudaStream_t st);
 // kpart != NULL (deterministic mode): every CTA of the K pass stores its partial triangle there ([kNtkMaxPartials][B * B] floats) and
-// a second kernel sums them in order.  Otherwise they add into K (by_last) or into rows of ntk_pitch(B) floats (`acc`), from which a
-// second kernel writes K; either has been cleared on this stream.
+// a second kernel sums them in order.  Otherwise they add one triangle into K, or by_boxes into rows of ntk_pitch(B) floats (`acc`); either
+// has been cleared on this stream, and the last CTA or a second kernel completes K.
 constexpr int kNtkMaxPartials = 160;
 inline int ntk_pitch(int B) { return (B + 3) & ~3; }
 struct NtkPlan {
   int box_rows, ppb;  // rows of a piece inside a box, pieces per box
   long long nkb;      // boxes
   int grid, n_active;
-  bool by_last;       // the last CTA to add its share completes K
+  bool by_boxes, by_last;
 };
 isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, NtkPlan* plan);
 isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int B, float* K, float* acc, WsHead* head, float* kpart,

@@ -9,10 +9,10 @@
 // through shared memory to TMA reductions into rows that a last tiny kernel completes K from.  (One float atomic per entry into
 // K, every CTA in the same order, was half of the pass where the layer is not large, and 8 us of any: 10,000 tokens, 480 x 448, K pass
 // of 100 sequences 24.9 -> 9.9 us, 139 23.2 -> 15.9; 896 x 128, 64 sequences 13.4 -> 7.7, 256 23.1 -> 14.7; 896 x 896, 64 25.2 -> 20.9.)
-// For B <= 128 a box holds only the rows that exist (32, 64 or 128 >= B) but spans 8, 4 or 2 pieces, so
+// For B <= 128 a box holds few rows that do not exist (4, 8, .. 128 >= B) but spans 64, 32, .. 2 pieces, so
 // that every TMA copy still moves 32 KB (small boxes cost a fixed ~100 clocks each) and the stage is
 // again 256 rows: rows 0..127 and rows 128..255 each go through ONE 128 x 128 MMA per 16 elements,
-// which multiplies 4, 2 or 1 pieces at once.  Only the diagonal blocks of that product (a piece
+// which multiplies up to 32 pieces at once.  Only the diagonal blocks of that product (a piece
 // against itself) are wanted; the epilogue adds them into K and skips the cross-piece blocks.  The
 // tensor pipe does up to four times the needed work this way, but in a quarter of the instructions:
 // with one 128 x 64 MMA per piece the pass was bound by the MMA issue rate (4.0 TB/s at B = 64
@@ -43,7 +43,7 @@ struct NtkParams {
   int B;
   long long nkb;  // boxes in the contraction dimension: ceil(pieces / ppb) * 4
   int32_t* info;
-  int box_rows;   // rows of a piece inside a box: 32, 64, 128 or 256, >= B
+  int box_rows;   // rows of a piece inside a box: 4, 8, .. 256, >= B
   int ppb;        // pieces per box = 256 / box_rows
   bool by_boxes;  // added by TMA into rows of a pitch that it can take, not into K
   // not NULL (up to 16 sequences, 32 with little data): the last CTA to add its share completes the other triangle and the
@@ -233,7 +233,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
           // of its two accumulator rows in shared memory (the ring is idle by now); then the 128 threads
           // walk the box_rows x box_rows block together, add the groups and update K.
           const int lr = 31 - __clz(p.box_rows), rows = 1 << lr;  // box_rows is a power of two
-          const int seq = r & (rows - 1), g = r >> lr, coff = r - seq, ngroups = 128 >> lr;
+          const int seq = r & (rows - 1), g = r >> lr, ngroups = 128 >> lr;
+          // the columns that a warp reads are the same for its lanes: of fewer than 32 sequences the whole block on its diagonal
+          const int coff = rows >= 32 ? r - seq : q * 32, mine = rows >= 32 ? 0 : lane & ~(rows - 1);
           const int ncol = min(rows, p.B);
           float* red = reinterpret_cast<float*>(smem);  // [group][column][sequence]
           if (ok) {
@@ -244,7 +246,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
               tmem_ld_wait();
               float* dst = red + ((((g << lr) + c0) << lr) + seq);
 #pragma unroll
-              for (int e = 0; e < 32; ++e) dst[e << lr] = __uint_as_float(v0[e]) + __uint_as_float(v1[e]);
+              for (int e = 0; e < 32; ++e) {
+                const int c = e - mine;
+                if (c >= 0 && c < rows) dst[c << lr] = __uint_as_float(v0[e]) + __uint_as_float(v1[e]);
+              }
             }
           }
           asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
@@ -314,7 +319,8 @@ __global__ void k_mirror(float* __restrict__ K, int B) {
 }
 // K from the triangle i >= j of the K pass's sums (rows of `ld` floats).
 // kdiag != NULL (split store): the diagonal comes from the gradient GEMM's float32 sums of squares
-__global__ void k_ntk_finish(const float* __restrict__ acc, int ld, float* __restrict__ K, int B, const float* __restrict__ kdiag) {
+// (acc may be K itself: what of it is read is written unchanged)
+__global__ void k_ntk_finish(const float* acc, int ld, float* K, int B, const float* __restrict__ kdiag) {
   pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * B) return;
@@ -531,7 +537,10 @@ isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, 
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  plan->box_rows = B > 128 ? 256 : B > 64 ? 128 : B > 32 ? 64 : 32;
+  // The least power of two that holds them, four at the least: rows of a box that do not exist are copied as slowly as any.  Boxes of 32
+  // rows / as now: 888 x 3504, 4 sequences 18.7 / 8.9 us, whole call 7 sequences 40.7 / 32.3, 4752 x 96, 14 sequences 17.7 / 16.7.
+  plan->box_rows = 256;
+  while (plan->box_rows > 4 && plan->box_rows / 2 >= B) plan->box_rows /= 2;
   plan->ppb = 256 / plan->box_rows;
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
   plan->nkb = (L.n_pad / kPieceElems + plan->ppb - 1) / plan->ppb * (split ? 2 : 4);
@@ -544,6 +553,10 @@ isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, 
   // sequences 18.3 -> 16.1 us), but a CTA by itself is slower than a kernel that is set up when this one ends, the more so the
   // more sequences: 896 x 896, K and solve: 24.5 us both ways at 16, 31.5 / 30.4 at 32, 47.2 / 45.0 at 48, 127.6 / 117.1 at 128.
   plan->by_last = !deterministic && (B <= 16 || (B <= 32 && per <= 16));
+  // Up to 32 sequences there are four groups of pieces or more in an accumulator, and two accumulators: their sums meet in shared memory
+  // first.  Eight boxes of every CTA on the same 20 x 20 entries waited for one another: 4088 x 1440, 20 sequences 154 us by
+  // atomics, 171 by boxes.
+  plan->by_boxes = !deterministic && B > 32;
   return ISOPO_OK;
 }
 
@@ -553,18 +566,17 @@ isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int
   CUtensorMap mapG, mapK;
   const uint32_t rows = (uint32_t)plan.box_rows, ppb = (uint32_t)plan.ppb;
   const uint64_t pieces = (uint64_t)(L.n_pad / kPieceElems);
-  const bool by_boxes = !kpart && !plan.by_last;
   isopo_status s = fmt.split ? make_map_pieces_u8(&mapG, G, (uint64_t)B, pieces, rows, ppb)
                              : make_map_pieces_bf16(&mapG, G, (uint64_t)B, pieces, rows, ppb);
   if (s != ISOPO_OK) return s;
-  if (by_boxes) {
+  if (plan.by_boxes) {
     if ((s = make_map_2d_f32(&mapK, acc, (uint64_t)B, (uint64_t)ntk_pitch(B), 32, false)) != ISOPO_OK) return s;
   } else {
     mapK = mapG;
   }
   auto kernel = fmt.split ? k_bf16_ntk<true> : k_bf16_ntk<false>;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, plan.nkb, info, plan.box_rows, plan.ppb, by_boxes,
+  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, plan.nkb, info, plan.box_rows, plan.ppb, plan.by_boxes,
               plan.by_last ? &head->done : nullptr, (uint32_t)plan.n_active, fmt.kdiag};
   {
     LaunchScope scope(kIdNtk, st);
@@ -575,7 +587,7 @@ isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int
   {
     LaunchScope scope(kIdMirror, st);
     if (kpart) launch(k_ntk_reduce, (B * B + 255) / 256, 256, 0, st, kpart, plan.n_active, B, K);
-    else launch(k_ntk_finish, (B * B + 255) / 256, 256, 0, st, acc, ntk_pitch(B), K, B, fmt.split ? fmt.kdiag : nullptr);
+    else launch(k_ntk_finish, (B * B + 255) / 256, 256, 0, st, acc, plan.by_boxes ? ntk_pitch(B) : B, K, B, fmt.split ? fmt.kdiag : nullptr);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

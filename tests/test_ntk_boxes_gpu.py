@@ -28,7 +28,7 @@ def _case(B, L, d_in, d_outs, seed):
     return X.bfloat16(), [dY.bfloat16() for dY in dYs], off, Ks
 
 
-@pytest.mark.parametrize("B", [4, 16, 17, 31, 32, 33, 35, 63, 64, 65, 96, 97, 127, 128, 129, 144, 145, 160, 161, 193, 255, 256])
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 5, 7, 8, 9, 13, 16, 17, 20, 31, 32, 33, 35, 63, 64, 65, 96, 97, 127, 128, 129, 144, 145, 160, 161, 193, 255, 256])
 @pytest.mark.parametrize("L,d_in,d_out", [(1, 72, 40), (2, 264, 296)])
 def test_exact(b, B, L, d_in, d_out):
     X, (dY,), off, (want,) = _case(B, L, d_in, [d_out], 1000 * B + d_in)
