@@ -189,10 +189,9 @@ __device__ __forceinline__ void box_row(uint32_t box, int lane, const uint32_t (
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int kPending>
-__device__ __forceinline__ void bulk_wait_read() {  // all but the last kPending groups of this thread have read their source
+__device__ __forceinline__ void bulk_wait_read() {  // all but the last kPending groups of this thread have read their source (what they write is complete when the kernel is)
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kPending) : "memory");
 }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // generic-proxy writes to shared memory -> visible to the async proxy (TMA, tcgen05.mma)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
             bulk_commit();
           }
         }
-        if (issuer) bulk_wait_all();
+        if (issuer) bulk_wait_read<0>();
       } else {
         // deterministic mode and K completed by the last CTA
         // every (CTA, entry of the lower triangle) is produced by exactly one thread, once.  Entry (r, c), c >= r, goes to

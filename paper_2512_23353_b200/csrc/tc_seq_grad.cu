@@ -286,7 +286,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
       if (lane == 0) mbar_arrive(accempty_bar(acc));
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
-    if (kFolded && issuer) bulk_wait_all();
+    if (kFolded && issuer) bulk_wait_read<0>();
   } else if (kFolded) {
     // ------------------------------------------------------------------ scaler (warps 6..9)
     // Thread (r, h): token row r of the stage, half h of each 128-byte row, in both dY chunks.

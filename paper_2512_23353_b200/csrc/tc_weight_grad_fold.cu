@@ -390,7 +390,7 @@ k_bf16_weight_grad_fold(const __grid_constant__ CUtensorMap mapY, const __grid_c
         for (int e = 0; e < 128; ++e) sum[e] = 0.f;
       }
     }
-    if (issuer) bulk_wait_all();
+    if (issuer) bulk_wait_read<0>();
   } else {
     // ------------------------------------------------------------------ tail warp (warp 10, both CTAs)
     // tail[s] is used only for last slabs that need the fix, so its phase is counted per stage; it

@@ -215,7 +215,7 @@ k_bf16_weight_grad_pair(const __grid_constant__ CUtensorMap mapY, const __grid_c
       if (lane == 0) mbar_arrive_remote(accempty_at_leader);
       acc_phase ^= 1u;
     }
-    if (issuer) bulk_wait_all();
+    if (issuer) bulk_wait_read<0>();
   }
 
   // ---------------------------------------------------------------------- teardown
