@@ -588,11 +588,8 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
   const bool add = beta != 0.f;
   int64_t* off_dev = (int64_t*)(w + L.off_offsets);
   float* tokscale = (float*)(w + L.off_tokseq);  // one scale per token: a single independent load per row
-  if (dtype == ISOPO_F32) {
-    s = launch_tokscale(seq_offsets_host, B, T, off_dev, coeffs, tokscale, add ? Clear{} : Clear{{dW}, {(int64_t)d_in * d_out}}, st);
-    if (s != ISOPO_OK) return s;
-    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, tokscale, dW, st);
-  }
+  if (dtype == ISOPO_F32)
+    return f32_weight_grad((const float*)X, (const float*)dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, st);
   if (!bf16_weight_grad_uses_pairs(T, d_in, d_out, B))
     return bf16_weight_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, info, st);
   if (bf16_weight_grad_fold_applies(T, d_in, d_out, B))

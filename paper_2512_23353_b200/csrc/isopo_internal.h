@@ -308,8 +308,9 @@ isopo_status f32_gram(const float* X, const float* dY, int64_t T, int d_in, int 
                       double* kacc, float* K, cudaStream_t st);
 isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, const float* coeffs, float* dW, float beta,
                          const WsTag* tag_dev, const WsTag& tag, int32_t* info, cudaStream_t st);
-isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* tokscale, float* dW,
-                             cudaStream_t st);
+// as the bf16 ones below: prepares the tokens' scales and clears dW where it has to
+isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
+                             const float* coeffs, int B, float* tokscale, float* dW, bool add, cudaStream_t st);
 
 // bf16 tcgen05 path
 isopo_status bf16_seq_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const StoredIntake& in, int B,

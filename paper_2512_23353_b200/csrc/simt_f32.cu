@@ -258,7 +258,7 @@ template <> struct OffsetParam<true> { int32_t v[kArgChunk]; };
 static_assert(sizeof(F32StoredArgs) + sizeof(OffsetParam<true>) <= 4096, "kernel arguments");
 
 template <int kTile, int kT, bool kArgOff>
-__global__ void __launch_bounds__(SeqGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
+__global__ void __launch_bounds__(SeqGemm<kTile, kT>::kThr, kT == 8 ? 2 : 3)  // 64-wide: three CTAs 297 x 651, 55 x 256 tokens 279 -> 252 us
 k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ OffsetParam<kArgOff> o) {
   pdl_wait();
   extern __shared__ __align__(16) float smem[];
@@ -300,27 +300,56 @@ k_f32_seq_grad(const __grid_constant__ F32StoredArgs a, const __grid_constant__ 
   }
 }
 
-// dW += (c_seq(t) dY)^T X over a slab of tokens (split over blockIdx.z), float atomics.
+// dW += (c_seq(t) dY)^T X over a slab of tokens (split over blockIdx.z), float atomics; one slab that nothing is added to (`store`) is
+// written.  The sums go through shared memory, so that a warp's additions are of whole lines of dW.
 template <int kTile, int kT>
 __global__ void __launch_bounds__(SlabGemm<kTile, kT>::kThr, kT == 8 ? 2 : 1)
 k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int64_t T, int d_in, int d_out,
-                  const float* __restrict__ tokscale, float* __restrict__ dW, int64_t slab) {
+                  const float* __restrict__ tokscale, float* __restrict__ dW, int64_t slab, bool store) {
   pdl_wait();
   extern __shared__ __align__(16) float smem[];
+  typedef SlabGemm<kTile, kT> Gemm;
   const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t t0 = blockIdx.z * slab, t1 = min(T, t0 + slab);
-  SlabGemm<kTile, kT> g;
+  Gemm g;
   g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, m0, n0, tokscale);
+  constexpr int kPass = kTile / (kT / 4), kPitch = kTile + 4;  // rows that four of a thread's p make up
+  static_assert(kPass * kPitch * 4 <= Gemm::kSmem, "the sums reuse the stages");
+  const bool quads = (d_in & 3) == 0 && (reinterpret_cast<uintptr_t>(dW) & 15) == 0;
 #pragma unroll
-  for (int p = 0; p < kT; ++p) {
-    const int m = m0 + g.row(p);
+  for (int p0 = 0; p0 < kT; p0 += 4) {
+    __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kT; q += 2) {
-      const int n = n0 + g.col(q);
-      float v0, v1;
-      unpack2(g.acc[p][q / 2], v0, v1);
-      if (m < d_out && n < d_in) atomicAdd(&dW[(size_t)m * d_in + n], v0);
-      if (m < d_out && n + 1 < d_in) atomicAdd(&dW[(size_t)m * d_in + n + 1], v1);
+    for (int p = p0; p < p0 + 4; ++p)
+#pragma unroll
+      for (int q = 0; q < kT; q += 4) {
+        float4 v;
+        unpack2(g.acc[p][q / 2], v.x, v.y);
+        unpack2(g.acc[p][q / 2 + 1], v.z, v.w);
+        *reinterpret_cast<float4*>(smem + (g.row(p) - p0 / 4 * kPass) * kPitch + g.col(q)) = v;
+      }
+    __syncthreads();
+    const int first = m0 + p0 / 4 * kPass, rows = min(kPass, d_out - first);
+    if (quads) {
+      constexpr int kLanes = kTile / 4;
+      const int c = threadIdx.x % kLanes * 4;
+      if (n0 + c < d_in)
+#pragma unroll 1
+        for (int r = threadIdx.x / kLanes; r < rows; r += Gemm::kThr / kLanes) {
+          const float4 v = *reinterpret_cast<const float4*>(smem + r * kPitch + c);
+          float* at = dW + (size_t)(first + r) * d_in + n0 + c;
+          if (store) *reinterpret_cast<float4*>(at) = v;
+          else asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+        }
+    } else {
+      const int c = threadIdx.x % kTile;
+      if (n0 + c < d_in)
+#pragma unroll 1
+        for (int r = threadIdx.x / kTile; r < rows; r += Gemm::kThr / kTile) {
+          float* at = dW + (size_t)(first + r) * d_in + n0 + c;
+          if (store) *at = smem[r * kPitch + c];
+          else atomicAdd(at, smem[r * kPitch + c]);
+        }
     }
   }
 }
@@ -1162,8 +1191,9 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
 // What a CTA spends on filling its pipeline and adding its tile, in stages of 16 tokens.
 constexpr int64_t kSlabOverhead = 4;
 template <int kTile, int kT>
-static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out,
-                                           const float* tokscale, float* dW, cudaStream_t st) {
+static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                           int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add,
+                                           cudaStream_t st) {
   typedef SlabGemm<kTile, kT> Gemm;
   const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
   if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
@@ -1187,18 +1217,22 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
                                       std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles)));
   const int64_t splits = (T + slab - 1) / slab;
   if (splits > 65535) return ISOPO_ERR_UNSUPPORTED;
+  const bool store = !add && splits == 1;
+  const isopo_status s = launch_tokscale(off_host, B, T, off_dev, coeffs, tokscale,
+                                         add || store ? Clear{} : Clear{{dW}, {(int64_t)d_in * d_out}}, st);
+  if (s != ISOPO_OK) return s;
   {
     LaunchScope scope(kIdF32WeightGrad, st);
-    launch(kernel, dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st, X, dY, T, d_in, d_out, tokscale, dW, slab);
+    launch(kernel, dim3(gx, gy, (unsigned)splits), Gemm::kThr, Gemm::kSmem, st, X, dY, T, d_in, d_out, tokscale, dW, slab, store);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 
-isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const float* tokscale, float* dW,
-                             cudaStream_t st) {
-  return f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, tokscale, dW, st)
-                                                      : launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, tokscale, dW, st);
+isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
+                             const float* coeffs, int B, float* tokscale, float* dW, bool add, cudaStream_t st) {
+  return (f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8> : launch_f32_weight_grad<64, 4>)(
+      X, dY, T, d_in, d_out, off_host, off_dev, coeffs, B, tokscale, dW, add, st);
 }
 
 }  // namespace isopo
