@@ -31,14 +31,6 @@ __device__ __forceinline__ bool rows_in_float4(const float* K, int B) {
   return (B & 3) == 0 && (reinterpret_cast<uintptr_t>(K) & 15) == 0;
 }
 
-// 1 / d by Newton's iteration from the hardware's approximation (about 20 bits; twice gives all 53).
-__device__ __forceinline__ double newton_rcp(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  r = fma(r, fma(-d, r, 1.0), r);
-  return fma(r, fma(-d, r, 1.0), r);
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

@@ -138,6 +138,13 @@ __global__ void __launch_bounds__(256) k_transform_simple(const __grid_constant_
 // (one reciprocal and one barrier each) took 16.4 us at 64 and 41 us at 128 sequences, this 14.7 and 36.9.  In float64 the
 // solution needs no refinement; the blocked float32 kernel below, which does, takes 21.5 and 39 us when its unrolled code
 // is in the instruction cache and about twice that when a GEMM ran before it.
+// 1 / d by Newton's iteration from the hardware's approximation (about 20 bits; twice gives all 53).
+__device__ __forceinline__ double newton_rcp(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
+}
 template <int kA>
 __global__ void __launch_bounds__(256) k_transform_small(const __grid_constant__ TransformBatch batch) {
   pdl_begin();
