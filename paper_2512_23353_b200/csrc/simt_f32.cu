@@ -680,21 +680,24 @@ __global__ void __launch_bounds__(256) k_f32_ntk_finish(const __grid_constant__ 
 //   Gram (kSampled = false): rows and columns are both tokens, tile pairs I <= J.  Only token pairs t <= s are used; a
 //     pair inside one sequence with t < s stands for (t,s) and (s,t) and counts twice.
 //   Sampled estimator (kSampled = true): the rows are the gathered sample rows, out = M^T[sample, sequence], no weights.
-// The tile's products go through shared memory; a warp owns 32 rows x kGT / 4 columns of them, walks the columns (sequence
+// The tile's products go through shared memory; a warp owns 32 rows of some columns of them, walks the columns (sequence
 // boundaries are the same for all its lanes), and adds the lanes of one row sequence together before it issues one
-// float64 atomic.  Bound by the float32 pipe: 896 -> 896, 4608 tokens: 1151 us against 3246 us for 32 x 32 tiles loaded
-// synchronously with an atomic per token pair.  Too few tiles of 64 to fill the machine leave the kernel to the latency of
-// one CTA's walk over the features: tiles of 32 then, and clusters of kC CTAs that take a share of the features each and add up
-// their sums through distributed shared memory before P and Q are multiplied (f32_gram_shape).  The pairs I <= J are numbered in one
-// row: of a square grid of which half returns at once some SMs got three times the work of others (789 tokens, 251 x 1121 97 -> 74 us).
+// float64 atomic.  Bound by the float32 pipe and, with few CTAs on an SM, by the latency of a stage.  Tiles of 64 have 8 x 4 elements a
+// thread, two thirds of the shared-memory reads of 4 x 4, and 128 threads whose registers and memory let three CTAs share an SM (two of
+// 256 threads before): 896 -> 896, 4608 tokens 1140 -> 1000 us; 128 samples of 20000 332 -> 291, 7032 tokens 1481 x 1513 236 -> 196.
+// Too few tiles of 64 to fill the machine leave the kernel to the latency of one CTA's walk over the features: tiles of 32 then, and
+// clusters of kC CTAs that take a share of the features each and add up their sums through distributed shared memory before P and Q
+// are multiplied (f32_gram_shape); those have the registers to load ahead (72 a thread -> 132: 450 tokens, 1536 x 1536 60 -> 53 us).
+// The pairs I <= J are numbered in one row: of a square grid of which half returns at once some SMs got three times the work of
+// others (789 tokens, 251 x 1121 97 -> 74 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int kGK = 16;   // features per stage
 constexpr int kGPitch = kGK + 4;
 
 template <int kGT>
 struct GramTile {
-  static constexpr int kRows = kGT / 16, kCols = 4;                 // elements of a thread
-  static constexpr int kTx = kGT / kCols, kThr = 16 * kTx;          // 64: 16 x 16 threads; 32: 16 x 8
+  static constexpr int kRows = kGT == 64 ? 8 : 2, kCols = 4;        // elements of a thread
+  static constexpr int kTx = kGT / kCols, kTy = kGT / kRows;        // 64: 8 x 16 threads; 32: 16 x 8
   static constexpr int kStages = kGT == 64 ? 3 : 6;                 // 30 KB either way
 };
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -713,12 +716,13 @@ __device__ __forceinline__ float ld_cluster(const float* mine, unsigned rank) { 
   return v;
 }
 template <bool kSampled, int kGT, int kC>
-__global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
+__global__ void __launch_bounds__(128, kGT == 64 ? 3 : kC == 1 ? 7 : 2) k_f32_gram(const float* __restrict__ RX, const float* __restrict__ RY, int64_t n_rows,
                                                   const float* __restrict__ X, const float* __restrict__ dY, int64_t T,
                                                   int d_in, int d_out, const int32_t* __restrict__ tokseq, int B,
                                                   double* __restrict__ out) {
   pdl_wait();
-  constexpr int kRows = GramTile<kGT>::kRows, kTx = GramTile<kGT>::kTx, kThr = GramTile<kGT>::kThr;
+  constexpr int kRows = GramTile<kGT>::kRows, kTx = GramTile<kGT>::kTx, kTy = GramTile<kGT>::kTy, kThr = kTx * kTy;
+  static_assert(kThr == 128, "threads");
   constexpr int kGramStages = GramTile<kGT>::kStages;
   const unsigned rank = kC > 1 ? cluster_rank() : 0, unit = blockIdx.x / kC;
   int I, J;
@@ -733,7 +737,13 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
     I = (int)(unit - (int64_t)J * (J + 1) / 2);
   }
   constexpr int kStageFloats = kGramStages * 2 * kGT * kGPitch, kTile = kGT * (kGT + 1);
-  __shared__ __align__(16) float smem[kStageFloats > 2 * kTile ? kStageFloats : 2 * kTile];
+  // The sums of Q go where the stages were, [row][kGT + 1]; those of P behind them, from tiles of 64 as soon as P's features are
+  // done (they would take 32 registers).
+  constexpr bool kParkP = kGT == 64;
+  static_assert(kParkP ? kTile <= kStageFloats : 2 * kTile <= kStageFloats, "shared memory");
+  __shared__ __align__(16) float smem[kStageFloats + (kParkP ? kTile : 0)];
+  float* const tile_q = smem;
+  float* const tile_p = smem + (kParkP ? kStageFloats : kTile);
   auto stage_mem = [&](int k, int side) { return smem + (k % kGramStages * 2 + side) * (kGT * kGPitch); };
   __shared__ int s_col[kGT];
   const int tid = threadIdx.x, tx = tid % kTx, ty = tid / kTx;
@@ -772,16 +782,23 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
     }
     cp_async_commit();
   };
-  float h[kRows][4] = {};
+  float h[kParkP ? 1 : kRows][4] = {};
   f32x2 acc[kRows][4] = {};
+  auto place = [&](int p, int q) { return (ty + kTy * p) * (kGT + 1) + tx + kTx * q; };
   auto total = [](f32x2 v) { float lo, hi; unpack2(v, lo, hi); return lo + hi; };
   auto keep_p = [&]() {  // the sums so far are of P
 #pragma unroll
     for (int p = 0; p < kRows; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { h[p][q] = total(acc[p][q]); acc[p][q] = 0ull; }
+      for (int q = 0; q < 4; ++q) {
+        const float v = total(acc[p][q]);
+        if (kParkP) tile_p[place(p, q)] = v;
+        else h[kParkP ? 0 : p][q] = v;
+        acc[p][q] = 0ull;
+      }
   };
   for (int k = k0; k < k0 + kGramStages - 1; ++k) fetch(k);
+  if (kC > 1 && kParkP && k0 > nkx) keep_p();  // no features of P here: zeros
   for (int k = k0; k < k1; ++k) {
     cp_async_wait<kGramStages - 2>();
     __syncthreads();
@@ -793,7 +810,7 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
     for (int c = 0; c < kGK; c += 4) {
       ulonglong2 a[kRows], b[4];
 #pragma unroll
-      for (int p = 0; p < kRows; ++p) a[p] = *reinterpret_cast<const ulonglong2*>(sA + (ty + 16 * p) * kGPitch + c);
+      for (int p = 0; p < kRows; ++p) a[p] = *reinterpret_cast<const ulonglong2*>(sA + (ty + kTy * p) * kGPitch + c);
 #pragma unroll
       for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(sB + (tx + kTx * q) * kGPitch + c);
 #pragma unroll
@@ -807,29 +824,28 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
   if (k1 <= nkx) keep_p();
   // One CTA: the products.  Several: the sums of P and behind them those of Q, which every CTA of the cluster reads for its share
   // of the columns and adds up in rank order.
-  float* tile = smem;  // [row][kGT + 1]
 #pragma unroll
   for (int p = 0; p < kRows; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int e = (ty + 16 * p) * (kGT + 1) + tx + kTx * q;
-      const float y = total(acc[p][q]);
-      tile[e] = kC == 1 ? h[p][q] * y : h[p][q];
-      if (kC > 1) tile[kTile + e] = y;
+      const int e = place(p, q);
+      const float y = total(acc[p][q]), x = kParkP ? (kC == 1 ? tile_p[e] : 0.0f) : h[kParkP ? 0 : p][q];
+      tile_q[e] = kC == 1 ? x * y : y;
+      if (kC > 1 && !kParkP) tile_p[e] = x;
     }
   if (kC == 1) __syncthreads();
   else cluster_sync();
   // a warp takes 32 rows and kWidth columns
-  constexpr int kWidth = kGT / 4 / kC;
-  const int warp = tid >> 5, lane = tid & 31, row = (warp % (kGT / 32)) * 32 + lane, cb = (int)(rank * 4 + warp / (kGT / 32)) * kWidth;
-  const float* const mine = tile + row * (kGT + 1) + cb;
+  constexpr int kWarpCols = 4 / (kGT / 32), kWidth = kGT / kWarpCols / kC;  // warps side by side
+  const int warp = tid >> 5, lane = tid & 31, row = (warp % (kGT / 32)) * 32 + lane, cb = (int)(rank * kWarpCols + warp / (kGT / 32)) * kWidth;
+  const int mine = row * (kGT + 1) + cb;
   float prod[kWidth];
   if (kC > 1) {  // all of the loads in flight together
     float x[kC][kWidth], y[kC][kWidth];
 #pragma unroll
     for (int r = 0; r < kC; ++r)
 #pragma unroll
-      for (int c = 0; c < kWidth; ++c) { x[r][c] = ld_cluster(mine + c, r); y[r][c] = ld_cluster(mine + kTile + c, r); }
+      for (int c = 0; c < kWidth; ++c) { x[r][c] = ld_cluster(tile_p + mine + c, r); y[r][c] = ld_cluster(tile_q + mine + c, r); }
 #pragma unroll
     for (int c = 0; c < kWidth; ++c) {
       float sx = x[0][c], sy = y[0][c];
@@ -840,7 +856,7 @@ __global__ void __launch_bounds__(GramTile<kGT>::kThr) k_f32_gram(const float* _
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // this CTA has read the others' sums
   } else {
 #pragma unroll
-    for (int c = 0; c < kWidth; ++c) prod[c] = mine[c];
+    for (int c = 0; c < kWidth; ++c) prod[c] = tile_q[mine + c];
   }
   const int64_t t = r0 + row;
   const int rseq = t < n_rows ? (kSampled ? (int)t : tokseq[t]) : -1;  // rows past the end form a run of their own, unused
@@ -1122,12 +1138,12 @@ isopo_status f32_ntk(const float* G, int64_t gstride, int B, double* part, uint3
   return ISOPO_OK;
 }
 
-// Tokens per tile and CTAs that share a tile's features.  Tiles of 32 where those of 64 would be few; then as many CTAs to a tile as
-// make up to 240 of them: one alone is a chain of (d_in + d_out) / 16 stages.  Two CTAs to a tile of 64 where those are many features.
-// Whole call, us, 64 / 32 / 32 by two / four / eight: Gram of 115 tokens, 283 x 1288 76 / 41 / 28 / 20 / 16; 300, 896 x 896 80 / 44 / 29 /
-// 29 / 36; 789, 251 x 1121 79 / 74 / 72 / 97 / 144; 874, 296 x 577 51 / 48 / 60; 2000, 512 x 512 155 / 180.  128 samples: 128 tokens,
-// 712 x 1169 101 / 57 / 37 / 26 / 27; 938, 1539 x 185 99 / 58 / 48 / 55; 4979, 1024 x 80 90 / 80 / 87; 7032, 1481 x 1513 276, 64 by two
-// 237, 32 302.
+// Tokens per tile and CTAs that share a tile's features.  Few tiles of 32: as many CTAs to each as make up to 240 of them, as one alone
+// is a chain of (d_in + d_out) / 16 stages.  Else tiles of 32, of 64, or of 64 by two CTAs, whichever costs least: us per stage with k
+// CTAs on an SM, a constant, and for two CTAs the exchange of their sums.  Kernel, us, 32 / 64 / 64 by two, features d_in + d_out: Gram of
+// 700 tokens, 512 features 22 / 29 / 25, 3072 99 / 134 / 78; 874, 3000 123 / 133 / 130; 1000, 1024 58 / 50 / 56; 1200, 1792 140 / 135 / 115;
+// 2000, 1024 180 / 142 / 186.  128 samples: 4000 tokens, 1024 61 / 52 / 59; 4979, 1104 81 / 88 / 85; 7032, 2994 300 / 241 / 197; 8000, 640
+// 66 / 55 / 77; 32 samples, which fill half of a tile of 64: 20000, 896 66 / 95 / 110.  Four CTAs to a tile of 64 were never the best.
 struct GramShape { int tile, ctas; };
 static GramShape f32_gram_shape(int64_t rows, int64_t cols, bool triangle, int d_in, int d_out) {
   auto tiles = [&](int64_t t) {
@@ -1135,11 +1151,15 @@ static GramShape f32_gram_shape(int64_t rows, int64_t cols, bool triangle, int d
     return triangle ? c * (c + 1) / 2 : r * c;
   };
   const int stages = (d_in + kGK - 1) / kGK + (d_out + kGK - 1) / kGK;
-  const int64_t wide = tiles(64);
-  if (4 * wide >= 5 * kSms) return GramShape{64, wide < 2 * kSms && stages >= 128 ? 2 : 1};
   GramShape g{32, 1};
   while (g.ctas < 8 && tiles(32) * 2 * g.ctas <= 240 && stages >= 10 * g.ctas) g.ctas *= 2;
-  return g;
+  if (g.ctas > 1) return g;
+  auto per_sm = [](int64_t ctas) { return (double)((ctas + kSms - 1) / kSms); };
+  const double k1 = per_sm(tiles(64)), k2 = per_sm(2 * tiles(64));
+  const double narrow = stages * std::max(0.48, 0.205 * per_sm(tiles(32)));
+  const double wide = stages * (0.12 + 0.52 * k1), split = 0.5 * stages * (0.12 + 0.52 * k2) + 8.0 * k2;
+  if (narrow <= wide && narrow <= split) return g;
+  return GramShape{64, wide <= split ? 1 : 2};
 }
 template <bool kSampled>
 static isopo_status launch_f32_gram(int id, const GramShape& g, int64_t units, const float* RX, const float* RY, int64_t n_rows, const float* X,
@@ -1153,7 +1173,7 @@ static isopo_status launch_f32_gram(int id, const GramShape& g, int64_t units, c
                         : g.ctas == 4 ? k_f32_gram<kSampled, 32, 4>
                                       : k_f32_gram<kSampled, 32, 8>;
     launch_cluster(g.tile == 32 ? narrow : wide, (unsigned)g.ctas, dim3((unsigned)(units * g.ctas)),
-                   g.tile == 32 ? 128 : 256, 0, st, RX, RY, n_rows, X, dY, T, d_in, d_out, tokseq, B, out);
+                   128, 0, st, RX, RY, n_rows, X, dY, T, d_in, d_out, tokseq, B, out);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;

@@ -62,3 +62,15 @@ def test_sampled(b, Ls, d_in, d_out, n):
     M = torch.zeros((n, B), dtype=torch.float64, device="cuda").index_add_(1, seq, (y[r] @ y.T) * (x[r] @ x.T))
     want = (M ** 2).sum(0) / ((y[r] ** 2).sum(1) * (x[r] ** 2).sum(1)).sum()
     assert ((F2.double() - want).norm() / want.norm()).item() <= 2 * TOL  # squares
+
+
+# tiles of 64 by two CTAs: one of them without a feature of X, without one of dY, its first stage the first of dY's
+@pytest.mark.parametrize("Ls,d_in,d_out", [([20] * 35, 48, 3000), ([350, 351], 3000, 48), ([64] * 11, 1536, 1536), ([50] * 24, 893, 899)])
+def test_gram_wide_tiles_by_two(b, Ls, d_in, d_out):
+    test_gram(b, Ls, d_in, d_out)
+
+
+# 32 samples leave half of a tile of 64 empty; 65 take tiles of 64; two CTAs to a tile
+@pytest.mark.parametrize("Ls,d_in,d_out,n", [([999] * 8, 448, 448, 32), ([999] * 8, 448, 450, 65), ([250] * 8, 896, 896, 128)])
+def test_sampled_tiles(b, Ls, d_in, d_out, n):
+    test_sampled(b, Ls, d_in, d_out, n)
