@@ -121,7 +121,7 @@ static GramOperands gram_operands(const void* X, int d_in, int n, const void* co
   return g;
 }
 
-WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved) {
+WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved, size_t have) {
   WsLayout L{};
   size_t p = 0;
   L.off_tag = p;
@@ -131,15 +131,19 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   L.off_offsets = p;
   p = align_up(p + sizeof(int64_t) * (size_t)(B + 1), 1024);
   L.off_tokseq = p;
-  const bool stored_bf16 = dtype == ISOPO_BF16 && resolved == ISOPO_PATH_MATERIALISE;
-  p = align_up(p + sizeof(int32_t) * std::max((size_t)T, stored_bf16 ? (size_t)B * ntk_pitch(B) : 0), 1024);
+  p = align_up(p + sizeof(int32_t) * (size_t)T, 1024);
   L.off_kacc = p;
   if (dtype == ISOPO_F32)
     p = align_up(p + (resolved == ISOPO_PATH_MATERIALISE ? sizeof(uint32_t) : sizeof(double) * (size_t)B * (size_t)B), 1024);
   L.off_scaled = p;
-  if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM)
-    p = align_up(p + std::max((size_t)2 * (size_t)T * (size_t)line_pitch(std::min(d_in, d_out)),
-                              repitch_pays(T, B) ? repitch_bytes(T, d_in) + repitch_bytes(T, d_out) : 0), 1024);
+  L.scaled_ld = std::min(d_in, d_out);
+  if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM) {
+    const int lines = line_pitch(L.scaled_ld);
+    const size_t copies = repitch_pays(T, B) ? repitch_bytes(T, d_in) + repitch_bytes(T, d_out) : 0;
+    const size_t full = align_up(p + std::max((size_t)2 * (size_t)T * (size_t)lines, copies), 1024);
+    if (have >= full) L.scaled_ld = lines;
+    p = have >= full ? full : align_up(p + (size_t)2 * (size_t)T * (size_t)L.scaled_ld, 1024);
+  }
   L.off_G = p;
   if (dtype == ISOPO_BF16) {
     L.tiles_m = (d_out + kTileM - 1) / kTileM;
@@ -149,6 +153,11 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
     L.off_kpart = p;
     if (resolved == ISOPO_PATH_MATERIALISE && deterministic_mode())
       p = align_up(p + sizeof(float) * (size_t)kNtkMaxPartials * (size_t)B * (size_t)B, 1024);
+    else if (resolved == ISOPO_PATH_MATERIALISE && B > kNtkSmemSums) {
+      const size_t bytes = sizeof(float) * (size_t)B * (size_t)ntk_pitch(B), full = align_up(p + bytes, 1024);
+      if (bytes <= sizeof(int32_t) * (size_t)T) L.off_ksums = L.off_tokseq;
+      else if (have >= full) { L.off_ksums = p; p = full; }
+    }
   } else {
     L.tiles_m = L.tiles_n = 0;
     L.n_pad = ((int64_t)d_in * d_out + 3) / 4 * 4;
@@ -296,7 +305,7 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
   if (s != ISOPO_OK) return s;
   const isopo_path rp = resolve_path(dtype, T, d_in, d_out, B, path);
   if (dtype == ISOPO_BF16 && rp == ISOPO_PATH_MATERIALISE && B > 256) return ISOPO_ERR_UNSUPPORTED;
-  const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, rp);
+  const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, rp, ws_bytes);
   if (ws_bytes < L.total) return ISOPO_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* w = (char*)ws;
@@ -311,7 +320,7 @@ isopo_status isopo_layer_gram(const void* X, const void* dY, isopo_dtype dtype, 
     const StoreFmt fmt = store_fmt(L, B, ws);
     NtkPlan plan;
     if ((s = plan_ntk(L, B, fmt.split, deterministic_mode(), &plan)) != ISOPO_OK) return s;
-    float* acc = plan.by_boxes ? (float*)tokseq : K;
+    float* acc = plan.by_boxes ? (float*)(w + L.off_ksums) : K;
     make_stored_intake(&in, seq_offsets_host, B, 1, &tag, &head, &acc, plan.by_boxes ? B * ntk_pitch(B) : B * B);
     if (fmt.split) {
       s = launch_offsets(seq_offsets_host, B, off_dev, Clear{}, st);
@@ -354,7 +363,7 @@ isopo_status isopo_layer_gram_shared_x(const void* X, int n_proj, const void* co
     if (s != ISOPO_OK) return s;
     d_max = std::max(d_max, d_out[h]);
   }
-  const WsLayout L = ws_layout(dtype, T, d_in, d_max, B, ISOPO_PATH_GRAM);
+  const WsLayout L = ws_layout(dtype, T, d_in, d_max, B, ISOPO_PATH_GRAM, ws_bytes);
   if (ws_bytes < L.total) return ISOPO_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* w = (char*)ws;
@@ -389,7 +398,7 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
     if (s != ISOPO_OK) return s;
     for (int g = 0; g < h; ++g)
       if (ws[g] == ws[h]) return ISOPO_ERR_INVALID_ARG;  // every projection keeps its own gradients
-    L[h] = ws_layout(dtype, T, d_in, d_out[h], B, ISOPO_PATH_MATERIALISE);
+    L[h] = ws_layout(dtype, T, d_in, d_out[h], B, ISOPO_PATH_MATERIALISE, ws_bytes[h]);
     if (ws_bytes[h] < L[h].total) return ISOPO_ERR_WORKSPACE;
     char* w = (char*)ws[h];
     tag[h] = make_ws_tag(dtype, T, d_in, d_out[h], B, seq_offsets_host);
@@ -409,10 +418,13 @@ isopo_status isopo_layer_gram_shared_x_stored(const void* X, int n_proj, const v
       if (s == ISOPO_OK) s = launch_seq_scales(X, dY[h], d_in, d_out[h], off_dev, B, (float*)fmt[h].scales, fmt[h].kdiag, st);
       if (s != ISOPO_OK) return s;
     }
-  NtkPlan plan[3];  // by_boxes is the same for all: the number of sequences says
+  NtkPlan plan[3];  // by_boxes is the same for all: the number of sequences says, and whether all have the room
+  for (int h = 0; h < n_proj; ++h)
+    if (L[h].off_ksums == 0)
+      for (int g = 0; g < n_proj; ++g) L[g].off_ksums = 0;
   for (int h = 0; h < n_proj; ++h) {
     if ((s = plan_ntk(L[h], B, fmt[h].split, deterministic_mode(), &plan[h])) != ISOPO_OK) return s;
-    acc[h] = plan[h].by_boxes ? (float*)((char*)ws[h] + L[h].off_tokseq) : K[h];
+    acc[h] = plan[h].by_boxes ? (float*)((char*)ws[h] + L[h].off_ksums) : K[h];
   }
   const int n_acc = plan[0].by_boxes ? B * ntk_pitch(B) : B * B;
   StoredIntake in;
@@ -452,7 +464,7 @@ isopo_status isopo_sampled_coefficients(const void* X, const void* dY, isopo_dty
   if (n_samples < 1 || n_samples > ISOPO_MAX_SAMPLES) return ISOPO_ERR_INVALID_ARG;
   for (int j = 0; j < n_samples; ++j)
     if (sample_rows_host[j] < 0 || sample_rows_host[j] >= T) return ISOPO_ERR_INVALID_ARG;
-  const SampledLayout S = sampled_layout(dtype, T, d_in, d_out, B, n_samples);
+  const SampledLayout S = sampled_layout(dtype, T, d_in, d_out, B, n_samples, ws_bytes);
   if (ws_bytes < S.total) return ISOPO_ERR_WORKSPACE;
   const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM);
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -572,7 +584,7 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
   if (s != ISOPO_OK) return s;
   const isopo_path rp = resolve_path(dtype, T, d_in, d_out, B, path);
   if (dtype == ISOPO_BF16 && rp == ISOPO_PATH_MATERIALISE && B > 256) return ISOPO_ERR_UNSUPPORTED;
-  const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, rp);
+  const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, rp, ws_bytes);
   if (ws_bytes < L.total) return ISOPO_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* w = (char*)ws;
@@ -594,7 +606,7 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
     return bf16_weight_grad(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, tokscale, dW, add, info, st);
   if (bf16_weight_grad_fold_applies(T, d_in, d_out, B))
     return bf16_weight_grad_fold(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, dW, add, info, st);
-  return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, dW, add, info, st);
+  return bf16_weight_grad_pair(X, dY, T, d_in, d_out, seq_offsets_host, off_dev, coeffs, B, w + L.off_scaled, L.scaled_ld, dW, add, info, st);
 }
 
 }  // extern "C"

@@ -144,28 +144,33 @@ struct WsLayout {
   size_t off_tag;      // WsHead (materialised path)
   size_t off_aux;      // float scales[B] | float kdiag[B]  (bf16 materialised path, split store)
   size_t off_offsets;  // int64 [B+1]
-  size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here, the bf16
-                       // stored route what its K pass adds into (float [B][ntk_pitch(B)])
+  size_t off_tokseq;   // int32 [T]: token -> sequence; the bf16 weight-gradient GEMM keeps float32 per-token scales here
   size_t off_kacc;     // float32 path: float64 [B*B] K accumulators (Gram), uint32 CTAs of the K pass that are done (materialised)
   size_t off_scaled;   // bf16 Gram path: copies of the operands at a pitch of whole lines (repitch_bytes), later the pre-scaled operand of the
-                       // weight-gradient GEMM, bf16 [T, line_pitch(min(d_in, d_out))]
+                       // weight-gradient GEMM, bf16 [T, scaled_ld]
   size_t off_G;        // stored gradients (materialised path only)
   size_t off_kpart;    // per-CTA partial K (materialised path; bf16: in deterministic mode only)
+  size_t off_ksums;    // bf16 materialised path above 32 sequences: what the K pass adds into, float [B][ntk_pitch(B)]; where the token map
+                       // is when it has the room; 0: none, added into K itself
   size_t total;
+  int scaled_ld;         // of the pre-scaled operand: line_pitch(min(d_in, d_out)), or the width itself in a workspace without that room
   int tiles_m, tiles_n;  // bf16 materialised layout: tiles per gradient
   int64_t n_pad;         // elements per stored gradient (row stride of G_flat)
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved);
+// In a workspace of `have` bytes: the areas that only make the kernels faster are left out where they do not fit (layout.total is then what
+// the others need), so that a workspace of 2 T min(d_in, d_out) bytes of scaled operand, or with no sums of the K pass, still serves.
+WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved, size_t have = SIZE_MAX);
 
 // Workspace of isopo_sampled_coefficients: the Gram-route prefix (offsets, token map), then
 // the gathered rows a0 / g0, M^T and the denominator.
 struct SampledLayout {
   size_t off_a0, off_g0, off_mt, off_den, total;
+  int lda, ldg;  // of the sample rows: bf16 whole lines, in a workspace of `have` bytes that has the room
 };
-SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples);
+SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples, size_t have = SIZE_MAX);
 
 void set_cuda_error(cudaError_t e, const char* where);
 #define ISOPO_CUDA_TRY(expr)                                  \
@@ -329,6 +334,7 @@ isopo_status bf16_seq_grad_pair_shared(const void* X, int n_proj, const void* co
 // a second kernel sums them in order.  Otherwise they add one triangle into K, or by_boxes into rows of ntk_pitch(B) floats (`acc`); either
 // has been cleared on this stream, and the last CTA or a second kernel completes K.
 constexpr int kNtkMaxPartials = 160;
+constexpr int kNtkSmemSums = 32;  // sequences up to which a CTA adds its groups of pieces in shared memory and then into K
 inline int ntk_pitch(int B) { return (B + 3) & ~3; }
 struct NtkPlan {
   int box_rows, ppb;  // rows of a piece inside a box, pieces per box
@@ -362,7 +368,7 @@ int gram_split_ctas(long long units, int d_in, int d_out, int sms);
 isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                              const int32_t* tokseq, int B, float* const* K, bool complete, int32_t* info, cudaStream_t st);
 isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
-                                const void* A0, const void* G0, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
+                                const void* A0, int lda, const void* G0, int ldg, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
 // 1-CTA tiles, operand rows scaled in shared memory by the scales per token that a launch ahead leaves in `tokscale`
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                               int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add, int32_t* info,
@@ -376,8 +382,8 @@ isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int
 // a scaled copy of the narrower operand, then a plain GEMM in 2-CTA tiles
 // (the offsets travel with the scaling pass, through off_dev above 383 sequences)
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, bool add, int32_t* info,
-                                   cudaStream_t st);
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, int scaled_ld, float* dW, bool add,
+                                   int32_t* info, cudaStream_t st);
 // plain GEMM in runs of stages per pair; modelled time in stages of 256 columns
 struct PlainPlan {
   long long run, cost;
@@ -389,7 +395,7 @@ isopo_status bf16_weight_grad_plain(const void* X, int ldx, const void* dY, int 
 
 // token-sampled estimator of Algorithm 1
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
-                          const void* A0, const void* G0, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
+                          const void* A0, int lda, const void* G0, int ldg, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
 isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dtype, int64_t T, int d_in, int d_out,
                                   const int32_t* tokseq, int B, const int64_t* rows_host, int n_samples, char* ws,
                                   const SampledLayout& S, const float* A, float lambda, float* coeffs, float* F2,

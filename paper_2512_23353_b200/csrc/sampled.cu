@@ -69,14 +69,13 @@ template <int kN> struct RowArgs { int32_t v[kN]; };
 template <typename T, int kN>
 __global__ void __launch_bounds__(256) k_gather_samples(const T* __restrict__ X, const T* __restrict__ dY, int d_in,
                                                         int d_out, const __grid_constant__ RowArgs<kN> rows,
-                                                        T* __restrict__ a0, T* __restrict__ g0,
+                                                        T* __restrict__ a0, int lda, T* __restrict__ g0, int ldg,
                                                         double* __restrict__ den) {
   pdl_wait();
   const int j = blockIdx.x;
   const int64_t t = rows.v[j];
-  constexpr bool kLines = sizeof(T) == 2;  // bf16: the tensor-core kernels' copies start at whole lines
-  double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * (kLines ? line_pitch(d_in) : d_in), d_in);
-  double ng = copy_row_sq(dY + t * d_out, g0 + (size_t)j * (kLines ? line_pitch(d_out) : d_out), d_out);
+  double na = copy_row_sq(X + t * d_in, a0 + (size_t)j * lda, d_in);
+  double ng = copy_row_sq(dY + t * d_out, g0 + (size_t)j * ldg, d_out);
   na = block_sum_d(na);
   ng = block_sum_d(ng);
   if (threadIdx.x == 0) atomicAdd(den, na * ng);
@@ -113,41 +112,47 @@ __global__ void __launch_bounds__(32 * kFinishSlices) k_sampled_finish(const TM*
 }
 
 template <int kN, typename T>
-isopo_status gather_with(const T* X, const T* dY, int d_in, int d_out, const int64_t* rows_host, int n_samples, T* a0, T* g0,
+isopo_status gather_with(const T* X, const T* dY, int d_in, int d_out, const int64_t* rows_host, int n_samples, T* a0, T* g0, const SampledLayout& S,
                          double* den, cudaStream_t st) {
   RowArgs<kN> rows;
   for (int j = 0; j < n_samples; ++j) rows.v[j] = (int32_t)rows_host[j];
   {
     LaunchScope scope(kIdSampledAux, st);
-    launch(k_gather_samples<T, kN>, n_samples, 256, 0, st, X, dY, d_in, d_out, rows, a0, g0, den);
+    launch(k_gather_samples<T, kN>, n_samples, 256, 0, st, X, dY, d_in, d_out, rows, a0, S.lda, g0, S.ldg, den);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
 }
 template <typename T>
 isopo_status gather_samples(const T* X, const T* dY, int d_in, int d_out, const int64_t* rows_host, int n_samples, T* a0, T* g0,
-                            double* den, cudaStream_t st) {
-  return n_samples <= 256 ? gather_with<256>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st)
-                          : gather_with<ISOPO_MAX_SAMPLES>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st);
+                            const SampledLayout& S, double* den, cudaStream_t st) {
+  return n_samples <= 256 ? gather_with<256>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, S, den, st)
+                          : gather_with<ISOPO_MAX_SAMPLES>(X, dY, d_in, d_out, rows_host, n_samples, a0, g0, S, den, st);
 }
 
 }  // namespace
 
-SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples) {
-  SampledLayout S{};
+SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples, size_t have) {
   const size_t elt = dtype == ISOPO_BF16 ? 2 : 4;
-  size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM).total;  // offsets, token map (+ kacc)
-  S.off_a0 = p;
-  const bool lines = dtype == ISOPO_BF16;  // the gathered rows lie at a pitch of whole lines
-  p = align_up(p + elt * (size_t)n_samples * (lines ? line_pitch(d_in) : d_in), 1024);
-  S.off_g0 = p;
-  p = align_up(p + elt * (size_t)n_samples * (lines ? line_pitch(d_out) : d_out), 1024);
-  S.off_mt = p;
-  p = align_up(p + (dtype == ISOPO_BF16 ? sizeof(float) : sizeof(double)) * (size_t)n_samples * B, 1024);
-  S.off_den = p;
-  p = align_up(p + sizeof(double), 1024);
-  S.total = p;
-  return S;
+  auto lay = [&](bool lines) {
+    SampledLayout S{};
+    S.lda = lines ? line_pitch(d_in) : d_in;
+    S.ldg = lines ? line_pitch(d_out) : d_out;
+    size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM, lines ? SIZE_MAX : 0).total;  // offsets, token map (+ kacc)
+    S.off_a0 = p;
+    p = align_up(p + elt * (size_t)n_samples * S.lda, 1024);
+    S.off_g0 = p;
+    p = align_up(p + elt * (size_t)n_samples * S.ldg, 1024);
+    S.off_mt = p;
+    p = align_up(p + (dtype == ISOPO_BF16 ? sizeof(float) : sizeof(double)) * (size_t)n_samples * B, 1024);
+    S.off_den = p;
+    p = align_up(p + sizeof(double), 1024);
+    S.total = p;
+    return S;
+  };
+  // bf16: the tensor-core kernels' copies of the sample rows start at whole lines
+  const SampledLayout S = lay(dtype == ISOPO_BF16);
+  return have >= S.total ? S : lay(false);
 }
 
 isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dtype, int64_t T, int d_in, int d_out,
@@ -160,7 +165,7 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
     float* a0 = (float*)(ws + S.off_a0);
     float* g0 = (float*)(ws + S.off_g0);
     double* Mt = (double*)(ws + S.off_mt);
-    if ((s = gather_samples((const float*)X, (const float*)dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st)) != ISOPO_OK) return s;
+    if ((s = gather_samples((const float*)X, (const float*)dY, d_in, d_out, rows_host, n_samples, a0, g0, S, den, st)) != ISOPO_OK) return s;
     s = f32_sampled((const float*)X, (const float*)dY, T, d_in, d_out, a0, g0, n_samples, tokseq, B, Mt, st);
     if (s != ISOPO_OK) return s;
     {
@@ -173,9 +178,9 @@ isopo_status sampled_coefficients(const void* X, const void* dY, isopo_dtype dty
   __nv_bfloat16* a0 = (__nv_bfloat16*)(ws + S.off_a0);
   __nv_bfloat16* g0 = (__nv_bfloat16*)(ws + S.off_g0);
   float* Mt = (float*)(ws + S.off_mt);
-  s = gather_samples((const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out, rows_host, n_samples, a0, g0, den, st);
+  s = gather_samples((const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, d_in, d_out, rows_host, n_samples, a0, g0, S, den, st);
   if (s != ISOPO_OK) return s;
-  s = bf16_sampled(X, dY, T, d_in, d_out, tokseq, B, a0, g0, n_samples, Mt, info, st);
+  s = bf16_sampled(X, dY, T, d_in, d_out, tokseq, B, a0, S.lda, g0, S.ldg, n_samples, Mt, info, st);
   if (s != ISOPO_OK) return s;
   {
     LaunchScope scope(kIdSampledAux, st);

@@ -258,19 +258,19 @@ isopo_status bf16_gram(const void* X, int ldx, const void* dY, int ldy, int64_t 
 }
 
 isopo_status bf16_sampled(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
-                          const void* A0, const void* G0, int n_samples, float* Mt, int32_t* info, cudaStream_t st) {
+                          const void* A0, int lda, const void* G0, int ldg, int n_samples, float* Mt, int32_t* info, cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int ctas = gram_split_ctas((T + kTT - 1) / kTT * ((n_samples + kTT - 1) / kTT), d_in, d_out, sms);
-  if (ctas > 1) return bf16_sampled_split(ctas, X, dY, T, d_in, d_out, tokseq, B, A0, G0, n_samples, Mt, info, st);
+  if (ctas > 1) return bf16_sampled_split(ctas, X, dY, T, d_in, d_out, tokseq, B, A0, lda, G0, ldg, n_samples, Mt, info, st);
   CUtensorMap mapX, mapY, mapRX, mapRY;
   isopo_status s = make_map_2d_bf16(&mapX, X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT);
   if (s != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&mapY, dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
   const uint32_t box_rows = sample_box_rows(n_samples);
-  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)line_pitch(d_in), 64, box_rows)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)line_pitch(d_out), 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&mapRX, A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)lda, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&mapRY, G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)ldg, 64, box_rows)) != ISOPO_OK) return s;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_gram<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   GramParams p{tokseq, Mt, T, B, (int)((T + kTT - 1) / kTT), d_in, d_out, info, n_samples, (n_samples + kTT - 1) / kTT, 0};
   p.row_bytes = box_rows * 128;

@@ -285,14 +285,14 @@ isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const
 }
 
 isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
-                                const void* A0, const void* G0, int n_samples, float* Mt, int32_t* info, cudaStream_t st) {
+                                const void* A0, int lda, const void* G0, int ldg, int n_samples, float* Mt, int32_t* info, cudaStream_t st) {
   CUtensorMap maps[6];
   isopo_status s;
   if ((s = make_map_2d_bf16(&maps[2], X, (uint64_t)T, (uint64_t)d_in, (uint64_t)d_in, 64, kTT)) != ISOPO_OK) return s;
   if ((s = make_map_2d_bf16(&maps[3], dY, (uint64_t)T, (uint64_t)d_out, (uint64_t)d_out, 64, kTT)) != ISOPO_OK) return s;
   const uint32_t box_rows = sample_box_rows(n_samples);
-  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)line_pitch(d_in), 64, box_rows)) != ISOPO_OK) return s;
-  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)line_pitch(d_out), 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&maps[0], A0, (uint64_t)n_samples, (uint64_t)d_in, (uint64_t)lda, 64, box_rows)) != ISOPO_OK) return s;
+  if ((s = make_map_2d_bf16(&maps[1], G0, (uint64_t)n_samples, (uint64_t)d_out, (uint64_t)ldg, 64, box_rows)) != ISOPO_OK) return s;
   maps[4] = maps[5] = maps[3];
   GramSplitParams p{};
   for (int h = 0; h < kMaxProj; ++h) { p.K[h] = Mt; p.d_out[h] = d_out; }

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
         }
         if (issuer) bulk_wait_read<0>();
       } else {
-        // deterministic mode and K completed by the last CTA
+        // deterministic mode, few sequences, no room for padded rows
         // every (CTA, entry of the lower triangle) is produced by exactly one thread, once.  Entry (r, c), c >= r, goes to
         // K[c][r]: the 32 lanes of a warp own consecutive r, so one instruction adds 128 contiguous bytes.
         float* const mine = p.kpart ? p.kpart + (size_t)blockIdx.x * p.B * p.B : nullptr;
@@ -556,7 +556,7 @@ isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, 
   // Up to 32 sequences there are four groups of pieces or more in an accumulator, and two accumulators: their sums meet in shared memory
   // first.  Eight boxes of every CTA on the same 20 x 20 entries waited for one another: 4088 x 1440, 20 sequences 154 us by
   // atomics, 171 by boxes.
-  plan->by_boxes = !deterministic && B > 32;
+  plan->by_boxes = !deterministic && B > kNtkSmemSums && L.off_ksums != 0;
   return ISOPO_OK;
 }
 

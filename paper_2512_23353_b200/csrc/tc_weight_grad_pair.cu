@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256, 6) k_scale_rows(const uint4* __restrict__
 }  // namespace
 
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, float* dW, bool add, int32_t* info,
+                                   int64_t* off_dev, const float* coeffs, int B, void* scaled, int scaled_ld, float* dW, bool add, int32_t* info,
                                    cudaStream_t st) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
@@ -337,7 +337,7 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
   int ldx = d_in, ldy = d_out;
   {  // scale the narrower operand into `scaled`
     const bool scale_y = d_out <= d_in;
-    const int d8 = (scale_y ? d_out : d_in) / 8, p8 = line_pitch(8 * d8) / 8;
+    const int d8 = (scale_y ? d_out : d_in) / 8, p8 = scaled_ld / 8;
     const uint4* src = (const uint4*)(scale_y ? dY : X);
     int64_t ctas = (T + 7) / 8;
     // One launch less (1 to 3 us of a small layer's pass).  The clear needs its share of the chip: with one CTA for every 8 of
