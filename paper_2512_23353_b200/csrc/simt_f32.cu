@@ -1210,31 +1210,49 @@ isopo_status f32_combine(const float* G, int64_t N, int64_t gstride, int B, cons
 
 // What a CTA spends on filling its pipeline and adding its tile, in stages of 16 tokens.
 constexpr int64_t kSlabOverhead = 4;
+struct F32Slabs { int64_t stages; double us; };  // of a token slab; what its CTAs take
+// Token slabs of whole stages, 128 tokens or more, up to eight waves (slab_plan.h).  "Four CTAs per SM" instead left the last
+// wave nearly empty: 896 x 896, 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 ->
+// 10.1 (this alone).  Two CTAs of 128 x 128 on an SM take twice the time of one (a stage of the SM 1.83 us each, 0.57 for 64 x 64), so where
+// few units leave most SMs with one, slabs for one to an SM are better: 500 tokens, 896 x 896 31.8 -> 23.8 us, 20,000 tokens, 128 x 128 31.6 -> 21.7.
 template <int kTile, int kT>
-static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
-                                           int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add,
-                                           cudaStream_t st) {
+static isopo_status plan_f32_weight_grad(int64_t T, int d_in, int d_out, F32Slabs* plan) {
   typedef SlabGemm<kTile, kT> Gemm;
-  const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
-  if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
   const auto kernel = k_f32_weight_grad<kTile, kT>;
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   int dev = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
-  static int resident[64] = {};  // CTAs at one time
+  static int resident[64] = {}, sms[64] = {};  // CTAs at one time
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident[dev] == 0) {
-    int sms = 0, per_sm = 0;
-    ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int per_sm = 0;
+    ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
     ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
-    resident[dev] = sms * std::max(per_sm, 1);
+    resident[dev] = sms[dev] * std::max(per_sm, 1);
   }
-  // Token slabs of whole stages, 128 tokens or more, up to eight waves (slab_plan.h).  "Four CTAs per SM" instead left the last
-  // wave nearly empty: 896 x 896, 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 ->
-  // 10.1 (this alone).
-  const int64_t tiles = (int64_t)gx * gy, slots = resident[dev];
-  const int64_t slab = 16 * plan_slab((T + 15) / 16, tiles, slots, kSlabOverhead,
-                                      std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles)));
+  const int64_t tiles = (int64_t)((d_in + kTile - 1) / kTile) * ((d_out + kTile - 1) / kTile), slots = resident[dev], n = sms[dev];
+  const int64_t blocks = (T + 15) / 16, most = std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles));
+  auto us = [&](int64_t stages) {
+    const int64_t units = (blocks + stages - 1) / stages * tiles, on_sm = (units + n - 1) / n, waves = (units + slots - 1) / slots;
+    return (double)(on_sm * stages + 2 * waves) * (kTile == 128 ? 1.83 : 0.57);
+  };
+  plan->stages = plan_slab(blocks, tiles, slots, kSlabOverhead, most);
+  if (kTile == 128) {
+    const int64_t alone = plan_slab(blocks, tiles, n, 2, most);
+    if (us(alone) < 0.93 * us(plan->stages)) plan->stages = alone;
+  }
+  plan->us = us(plan->stages);
+  return ISOPO_OK;
+}
+template <int kTile, int kT>
+static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
+                                           int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add,
+                                           const F32Slabs& plan, cudaStream_t st) {
+  typedef SlabGemm<kTile, kT> Gemm;
+  const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
+  if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
+  const auto kernel = k_f32_weight_grad<kTile, kT>;
+  const int64_t slab = 16 * plan.stages;
   const int64_t splits = (T + slab - 1) / slab;
   if (splits > 65535) return ISOPO_ERR_UNSUPPORTED;
   const bool store = !add && splits == 1;
@@ -1251,8 +1269,15 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
 
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
                              const float* coeffs, int B, float* tokscale, float* dW, bool add, cudaStream_t st) {
-  return (f32_wide_tiles(d_in, d_out, (T + 255) / 256) ? launch_f32_weight_grad<128, 8> : launch_f32_weight_grad<64, 4>)(
-      X, dY, T, d_in, d_out, off_host, off_dev, coeffs, B, tokscale, dW, add, st);
+  // Tiles by the time that their CTAs take.  128 x 128 only where they filled the machine twice (64 x 64 / 128 x 128 us): 500 tokens,
+  // 1536 x 1536 76.7 / 58.7; 1000, 896 x 896 52.3 / 41.6; 100, 1536 x 1536 20.1 / 16.3; 2500, 384 x 640 49.4 / 34.8; 12,000, 128 x 128 16.2 / 19.0.
+  F32Slabs narrow, wide;
+  isopo_status s = plan_f32_weight_grad<64, 4>(T, d_in, d_out, &narrow);
+  if (s == ISOPO_OK) s = plan_f32_weight_grad<128, 8>(T, d_in, d_out, &wide);
+  if (s != ISOPO_OK) return s;
+  return narrow.us <= wide.us
+             ? launch_f32_weight_grad<64, 4>(X, dY, T, d_in, d_out, off_host, off_dev, coeffs, B, tokscale, dW, add, narrow, st)
+             : launch_f32_weight_grad<128, 8>(X, dY, T, d_in, d_out, off_host, off_dev, coeffs, B, tokscale, dW, add, wide, st);
 }
 
 }  // namespace isopo
