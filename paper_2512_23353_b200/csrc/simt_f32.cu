@@ -1219,13 +1219,13 @@ template <int kTile, int kT>
 static isopo_status plan_f32_weight_grad(int64_t T, int d_in, int d_out, F32Slabs* plan) {
   typedef SlabGemm<kTile, kT> Gemm;
   const auto kernel = k_f32_weight_grad<kTile, kT>;
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   int dev = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   static int resident[64] = {}, sms[64] = {};  // CTAs at one time
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident[dev] == 0) {
     int per_sm = 0;
+    ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
     ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
     ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
     resident[dev] = sms[dev] * std::max(per_sm, 1);
@@ -1252,6 +1252,7 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
   const int gx = (d_in + kTile - 1) / kTile, gy = (d_out + kTile - 1) / kTile;
   if (gy > 65535) return ISOPO_ERR_UNSUPPORTED;
   const auto kernel = k_f32_weight_grad<kTile, kT>;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
   const int64_t slab = 16 * plan.stages;
   const int64_t splits = (T + slab - 1) / slab;
   if (splits > 65535) return ISOPO_ERR_UNSUPPORTED;
