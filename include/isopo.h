@@ -336,7 +336,8 @@ ISOPO_API isopo_status isopo_transform_spectral_batched(int n_layers, const floa
  * GEMM, or, for layers with few rows, to the rows as they land in shared memory.
  *
  *   coeffs  dev, float32 [B]
- *   dW      dev, float32 [d_out, d_in] row-major (the layout of `grad_out.T @ act_in`)
+ *   dW      dev, float32 [d_out, d_in] row-major (the layout of `grad_out.T @ act_in`); 16-byte
+ *           aligned for ISOPO_BF16 (otherwise ISOPO_ERR_INVALID_ARG, dW untouched), any float for ISOPO_F32
  *   beta    0 (overwrite) or 1 (accumulate into the existing gradient)
  * Other arguments as for isopo_layer_gram; seq_offsets_host must hold the same offsets.
  */

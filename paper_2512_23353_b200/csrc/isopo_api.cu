@@ -580,6 +580,8 @@ isopo_status isopo_weight_grad(const void* X, const void* dY, isopo_dtype dtype,
   ApiRange nvtx_range("isopo_weight_grad");
   if (!coeffs || !dW || !info) return ISOPO_ERR_INVALID_ARG;
   if (beta != 0.0f && beta != 1.0f) return ISOPO_ERR_INVALID_ARG;
+  // the bf16 kernels write dW in pieces of 16 bytes and by TMA; refused here, before anything of dW is cleared
+  if (dtype == ISOPO_BF16 && ((uintptr_t)dW & 15)) return ISOPO_ERR_INVALID_ARG;
   isopo_status s = check_layer_args(X, dY, dtype, T, d_in, d_out, seq_offsets_host, B, path, ws);
   if (s != ISOPO_OK) return s;
   const isopo_path rp = resolve_path(dtype, T, d_in, d_out, B, path);

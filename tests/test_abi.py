@@ -102,6 +102,21 @@ def test_argument_validation_happens_on_the_host(binding):
     assert wg == b.ERR_INVALID_ARG                                     # beta must be 0 or 1
 
 
+def test_weight_gradient_alignment_is_checked_on_the_host(binding):
+    """bf16 dW off a 16-byte boundary is refused on both routes before any CUDA call (so with nothing enqueued); float32 dW is not."""
+    b = binding
+    off = np.array([0, 3, 5], dtype=np.int64)
+    fake = 1 << 20
+    grad = lambda dtype, path, dW, beta, ws_bytes=1 << 30: b.lib.isopo_weight_grad(  # noqa: E731
+        fake, fake, dtype, 5, 8, 8, fake, off.ctypes.data, 2, path, dW, beta, fake, ws_bytes, fake, None)
+    for path in (b.PATH_GRAM, b.PATH_MATERIALISE, b.PATH_AUTO):
+        for beta in (0.0, 1.0):
+            for shift in (4, 8, 12):
+                assert grad(b.BF16, path, fake + shift, beta) == b.ERR_INVALID_ARG
+                assert grad(b.F32, path, fake + shift, beta, 16) == b.ERR_WORKSPACE  # past the check, stopped by the next
+            assert grad(b.BF16, path, fake + 16, beta, 16) == b.ERR_WORKSPACE
+
+
 def test_new_entry_points_validate_on_the_host(binding):
     """The entry points added around the three calls reject bad arguments before any CUDA call, and the
     process-wide switches change what they say they change (workspace size, nothing else)."""
