@@ -2,6 +2,7 @@
 // dtypes use.  Token contractions are float32 FMA; everything that sums over many products of
 // products (K) is accumulated in float64.
 #include <algorithm>
+#include <atomic>
 
 #include "isopo_internal.h"
 #include "slab_plan.h"
@@ -1219,18 +1220,20 @@ template <int kTile, int kT>
 static isopo_status plan_f32_weight_grad(int64_t T, int d_in, int d_out, F32Slabs* plan) {
   typedef SlabGemm<kTile, kT> Gemm;
   const auto kernel = k_f32_weight_grad<kTile, kT>;
-  int dev = 0;
+  int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
-  static int resident[64] = {}, sms[64] = {};  // CTAs at one time
+  ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // CTAs at one time on an SM.  One word, all that a thread takes from another: beside the SMs in a second one, a thread could have seen the
+  // first set and the second not yet, and divided by zero.
+  static std::atomic<int> resident[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
-  if (resident[dev] == 0) {
-    int per_sm = 0;
+  int per_sm = resident[dev].load(std::memory_order_relaxed);
+  if (per_sm == 0) {
     ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gemm::kSmem));
-    ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
     ISOPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, Gemm::kThr, Gemm::kSmem));
-    resident[dev] = sms[dev] * std::max(per_sm, 1);
+    resident[dev].store(per_sm = std::max(per_sm, 1), std::memory_order_relaxed);
   }
-  const int64_t tiles = (int64_t)((d_in + kTile - 1) / kTile) * ((d_out + kTile - 1) / kTile), slots = resident[dev], n = sms[dev];
+  const int64_t tiles = (int64_t)((d_in + kTile - 1) / kTile) * ((d_out + kTile - 1) / kTile), slots = (int64_t)sms * per_sm, n = sms;
   const int64_t blocks = (T + 15) / 16, most = std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles));
   auto us = [&](int64_t stages) {
     const int64_t units = (blocks + stages - 1) / stages * tiles, on_sm = (units + n - 1) / n, waves = (units + slots - 1) / slots;
