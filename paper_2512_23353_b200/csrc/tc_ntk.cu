@@ -153,25 +153,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
         // Blocks of 32 columns c of the warp's 32 accumulator rows go through shared memory (the ring is idle by now), turned over so
         // that box row c holds K[c][r .. r + 31], and are added by TMA into the rows of p.acc; what the diagonal blocks have
         // above the diagonal is not read from there.  A CTA starts at a block of its own: 148 of them on one sector wait for one another.
+        // Up to 128 sequences both accumulators hold sums of the same blocks, up to 64 so do warps q and q + 2: they are added up here, so
+        // that an entry of K is a sum of one float32 addition per CTA (four of them had twice the error: 64 sequences 3.5e-7 against 1.8e-7).
         tc_fence_after_sync();
-        const uint32_t tlane = (uint32_t)(q * 32) << 16, ring = smem_base + q * (kStages * kStageBytes / 4);
-        const bool issuer = elect_one();
-        // sequences of the warp's rows in the left accumulator (the right one: two pieces' groups alike, or rows 128 ..), first column
+        constexpr int kRingBytes = kStages * kStageBytes / 4;
+        const uint32_t tlane = (uint32_t)(q * 32) << 16, ring = smem_base + q * kRingBytes, partner = smem_base + (q ^ 2) * kRingBytes;
+        const bool issuer = elect_one(), halves = p.box_rows == 64;
+        // sequences of the warp's rows in the left accumulator (the right one: the same, or rows 128 ..), first column of their piece
         const int seq0 = two ? q * 32 : (q * 32) & (p.box_rows - 1), coff = two ? 0 : q * 32 - seq0;
         const int na = ok ? max(0, ((two ? n1 : min(p.box_rows, p.B)) - seq0 + 31) >> 5) : 0;       // blocks at and right of the diagonal
-        const int nb = !ok ? 0 : two ? max(0, (n2 - seq0 + 31) >> 5) : na;
-        const int n = na + nb, first = n ? blockIdx.x % n : 0;
-#pragma unroll 1
-        for (int k = 0; k < n; ++k) {
-          const int b = first + k < n ? first + k : first + k - n;
-          const bool right = b >= na;
-          const int c = seq0 + (right ? b - na : b) * 32;                  // accumulator column (of the piece)
-          const int sr = seq0 + (two && right ? 128 : 0), sc = c + (two && right ? 128 : 0);  // sequences of row and column
-          if (sr >= p.B || sc >= p.B) continue;
-          uint32_t v[32];
-          tmem_ld32(tmem_base + tlane + (right ? 256 : 0) + coff + c, v);
-          tmem_ld_wait();
-          const uint32_t box = ring + k * 4096;
+        auto send = [&](int sr, int sc, uint32_t box, const uint32_t (&v)[32]) {  // sequences of the block's first row and column
 #pragma unroll
           for (int e = 0; e < 32; ++e) {
             const float x = kE4m3 ? unscale(sr + lane, sc + e, __uint_as_float(v[e])) : __uint_as_float(v[e]);
@@ -182,6 +173,59 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
           if (issuer) {
             tma_add_2d(&mapK, sr, sc, box);
             bulk_commit();
+          }
+        };
+        if (two) {
+          const int nb = ok ? max(0, (n2 - seq0 + 31) >> 5) : 0, n = na + nb, first = n ? blockIdx.x % n : 0;
+#pragma unroll 1
+          for (int k = 0; k < n; ++k) {
+            const int b = first + k < n ? first + k : first + k - n;
+            const bool right = b >= na;
+            const int c = seq0 + (right ? b - na : b) * 32;                  // accumulator column
+            const int sr = seq0 + (right ? 128 : 0), sc = c + (right ? 128 : 0);
+            if (sr >= p.B || sc >= p.B) continue;
+            uint32_t v[32];
+            tmem_ld32(tmem_base + tlane + (right ? 256 : 0) + c, v);
+            tmem_ld_wait();
+            send(sr, sc, ring + k * 4096, v);
+          }
+        } else {
+          auto load = [&](int c, uint32_t (&v)[32]) {  // accumulator column c of the piece
+            uint32_t w[32];
+            tmem_ld32(tmem_base + tlane + coff + c, v);
+            tmem_ld32(tmem_base + tlane + 256 + coff + c, w);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
+          };
+          auto others = [&](int b) { return halves && ((b ^ (q >> 1)) & 1); };  // block b is warp q ^ 2's to send
+          if (halves) {
+#pragma unroll 1
+            for (int b = 0; b < na; ++b) {
+              if (!others(b)) continue;
+              uint32_t v[32];
+              load(seq0 + b * 32, v);
+#pragma unroll
+              for (int e = 0; e < 32; ++e) asm volatile("st.shared.b32 [%0], %1;" ::"r"(ring + b * 4096 + e * 128 + lane * 4), "r"(v[e]) : "memory");
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+          }
+          const int first = na ? blockIdx.x % na : 0;
+#pragma unroll 1
+          for (int k = 0; k < na; ++k) {
+            const int b = first + k < na ? first + k : first + k - na, c = seq0 + b * 32;
+            if (seq0 >= p.B || c >= p.B || others(b)) continue;
+            uint32_t v[32];
+            load(c, v);
+            if (halves) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) {
+                float x;
+                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(partner + b * 4096 + e * 128 + lane * 4) : "memory");
+                v[e] = __float_as_uint(__uint_as_float(v[e]) + x);
+              }
+            }
+            send(seq0, c, ring + b * 4096, v);
           }
         }
         if (issuer) bulk_wait_read<0>();
@@ -544,7 +588,9 @@ isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, 
   plan->ppb = 256 / plan->box_rows;
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
   plan->nkb = (L.n_pad / kPieceElems + plan->ppb - 1) / plan->ppb * (split ? 2 : 4);
-  plan->grid = (int)std::max<long long>(1, std::min<long long>(sms, plan->nkb / 4));  // four boxes of a CTA pay for its start
+  // Four boxes of a CTA pay for its start, eight above 32 sequences: half of the CTAs are half of the additions to an entry of K (896 x 128,
+  // 64 sequences: error 1.0e-7 with 56 of them, 1.4e-7 with 112; isopo_layer_gram 15.4 / 14.3 us).
+  plan->grid = (int)std::max<long long>(1, std::min<long long>(sms, plan->nkb / (B > kNtkSmemSums ? 8 : 4)));
   if (deterministic) plan->grid = std::min(plan->grid, kNtkMaxPartials);
   // CTAs whose slab of the contraction is empty take no part
   const long long per = (plan->nkb + plan->grid - 1) / plan->grid;
