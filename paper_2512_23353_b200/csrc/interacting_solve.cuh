@@ -71,17 +71,19 @@ __device__ __forceinline__ float warp_column_sums(float (&r)[kNB]) {
   return r[0];
 }
 
-// Pointer types of the block helpers.  kShared: every block lies in this CTA's shared memory and has no other writer, so the
-// pointers may be restrict-qualified (4 % of the solve at 256 sequences).  Otherwise a block may be global memory that another
-// warp or SM wrote earlier in the same kernel: plain loads only, never the read-only path.
+// Pointer types of the block helpers.  kShared: every block lies in this CTA's shared memory, is written by one warp at a time, and a
+// lane of a helper reads of it what others left before the call or what it wrote itself, so the pointers may be restrict-qualified
+// (4 % of the solve at 256 sequences).  Otherwise a block may be global memory that another warp or SM wrote earlier in the same
+// kernel: plain loads only, never the read-only path.
 template <bool kShared> struct BlkPtr { typedef float* __restrict__ rw; typedef const float* __restrict__ ro; };
 template <> struct BlkPtr<false> { typedef float* rw; typedef const float* ro; };
 
 // Factors the 32 x 32 diagonal block D (column-major, symmetric input) in place into its lower
-// Cholesky factor and writes 1 / L_kk to rd[k].  One warp.
+// Cholesky factor and writes 1 / L_kk to rd[k].  One warp.  D is not restrict-qualified: in shared memory its lanes read columns that the
+// others have just written, and a load through such a pointer could be moved ahead of the __syncwarp between.
 // Returns 0, or the 1-based local index of the first non-positive pivot.
 template <bool kShared = true>
-__device__ __noinline__ int warp_factor_diag(typename BlkPtr<kShared>::rw D, float* __restrict__ rd) {
+__device__ __noinline__ int warp_factor_diag(float* D, float* __restrict__ rd) {
   const int lane = threadIdx.x & 31;
   float r[kNB];
 #pragma unroll
@@ -200,10 +202,10 @@ __device__ __noinline__ void warp_rank32_update(typename BlkPtr<kShared>::rw C, 
   for (int c = 0; c < 8; ++c) *reinterpret_cast<float4*>(C + (c0 + c) * kNB + r0) = acc[c];
 }
 
-// Solves L L^T x = v in place (v in shared memory, nb*32 entries) with the blocked factor.
+// Solves L L^T x = v in place (v in shared memory, nb*32 entries, written by all warps in turn) with the blocked factor.
 template <bool kShared = true>
 __device__ __noinline__ void block_cholesky_solve(typename BlkPtr<kShared>::ro Lb, const float* __restrict__ InvD,
-                                                  float* __restrict__ v, int nb) {
+                                                  float* v, int nb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   // forward: L y = v
   for (int J = 0; J < nb; ++J) {
@@ -258,7 +260,7 @@ __device__ __noinline__ void block_cholesky_solve(typename BlkPtr<kShared>::ro L
 // blocks; shared memory, or a workspace without kShared), the inverse diagonal factors at InvD, then the solve and up to
 // two refinement rounds.  Called by every thread of a CTA of kThr; `layer` tags a failed pivot in *info.
 template <int kThr = kSolveThreads, bool kShared = true>
-__device__ __forceinline__ void interacting_solve(const TransformParams& P, typename BlkPtr<kShared>::rw Lb, float* InvD,
+__device__ __forceinline__ void interacting_solve(const TransformParams& P, float* Lb, float* InvD,
                                                   float* vec, double* sol, float* rdiag, double& s_trace, double& s_res,
                                                   int& s_fail, int layer) {
   const int B = P.B, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThr / 32;
