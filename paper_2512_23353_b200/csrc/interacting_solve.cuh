@@ -350,8 +350,9 @@ __device__ __forceinline__ void interacting_solve(const TransformParams& P, floa
         if (f != 0 && lane == 0) s_fail = (J + 1) * kNB + f;
       }
       // The other blocks, whoever is free.  Warps 4, 8, .. share warp 0's scheduler and stay away: its factorisation is the serial
-      // chain, and took 16.5 thousand clocks of the first column of 256 sequences among fifteen updating warps, 5.4 alone.
-      if (warp == 0 || (warp & 3) != 0) {
+      // chain, and took 16.5 thousand clocks of the first column of 256 sequences among fifteen updating warps, 5.4 alone.  Not where the
+      // updates are the longer (more than 64 blocks, which only the solve by one CTA above 256 sequences has: 1024 of them 2302 / 2182 us).
+      if ((!kShared && ntrail > 64) || warp == 0 || (warp & 3) != 0) {
         while (true) {
           int t = 0;
           if (lane == 0) t = 1 + atomicAdd(&s_taken[J & 1], 1);

@@ -1,6 +1,6 @@
 // Interacting solve for 257 to 1024 sequences by one CTA, the factor in a workspace that stays in the L2: what
 // isopo_transform_advantages_large does where a cluster of sixteen CTAs (transform.cu) cannot be placed, i.e. in a context that
-// has a part of the SMs.  512 sequences 398 us (the cluster 145), 1024 2207 us (340).  A file of its own: in transform.cu the
+// has a part of the SMs.  512 sequences 398 us (the cluster 148), 1024 2182 us (338).  A file of its own: in transform.cu the
 // cluster's kernel, whose helpers it shares, took 4 us longer at 1024 sequences.
 #include "interacting_solve.cuh"
 
