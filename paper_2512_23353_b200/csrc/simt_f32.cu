@@ -175,8 +175,10 @@ struct TokenGemm {
   static_assert(kSmem <= 99 * 1024, "two CTAs per SM");
   f32x2 acc[kT][kT / 2];
   // tile row of acc[p][.], tile column of the first element of a pair acc[.][q / 2]
-  __device__ __forceinline__ static int row(int p) { return (p / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x / kSide) * 4 + p % 4; }
-  __device__ __forceinline__ static int col(int q) { return (q / 4) * (kTile / (kT / 4)) + (int)(threadIdx.x % kSide) * 4 + q % 4; }
+  __device__ __forceinline__ static int row(int p, unsigned tid) { return (p / 4) * (kTile / (kT / 4)) + (int)(tid / kSide) * 4 + p % 4; }
+  __device__ __forceinline__ static int row(int p) { return row(p, threadIdx.x); }
+  __device__ __forceinline__ static int col(int q, unsigned tid) { return (q / 4) * (kTile / (kT / 4)) + (int)(tid % kSide) * 4 + q % 4; }
+  __device__ __forceinline__ static int col(int q) { return col(q, threadIdx.x); }
 
   // kScaled: the dY row of token t counts tokscale[t] times (rounded once, as a scaled copy of dY would be)
   template <bool kScaled>
@@ -310,12 +312,16 @@ k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int
   pdl_wait();
   extern __shared__ __align__(16) float smem[];
   typedef SlabGemm<kTile, kT> Gemm;
-  const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   const int64_t t0 = blockIdx.z * slab, t1 = min(T, t0 + slab);
   Gemm g;
-  g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, m0, n0, tokscale);
+  g.template run<true>(smem, X, dY, d_in, d_out, t0, t1, blockIdx.y * kTile, blockIdx.x * kTile, tokscale);
   constexpr int kPass = kTile / (kT / 4), kPitch = kTile + 4;  // rows that four of a thread's p make up
   static_assert(kPass * kPitch * 4 <= Gemm::kSmem, "the sums reuse the stages");
+  // 128 x 128: read anew, as keeping them through the GEMM takes registers that are not there (40 bytes of spills for 12: 7032 tokens, 1481 x
+  // 1513 830 -> 768 us)
+  unsigned tid = threadIdx.x, bx = blockIdx.x, by = blockIdx.y;
+  if (kTile == 128) asm volatile("mov.u32 %0, %%tid.x;\nmov.u32 %1, %%ctaid.x;\nmov.u32 %2, %%ctaid.y;" : "=r"(tid), "=r"(bx), "=r"(by));
+  const int m0 = by * kTile, n0 = bx * kTile;
   const bool quads = (d_in & 3) == 0 && (reinterpret_cast<uintptr_t>(dW) & 15) == 0;
 #pragma unroll
   for (int p0 = 0; p0 < kT; p0 += 4) {
@@ -327,26 +333,26 @@ k_f32_weight_grad(const float* __restrict__ X, const float* __restrict__ dY, int
         float4 v;
         unpack2(g.acc[p][q / 2], v.x, v.y);
         unpack2(g.acc[p][q / 2 + 1], v.z, v.w);
-        *reinterpret_cast<float4*>(smem + (g.row(p) - p0 / 4 * kPass) * kPitch + g.col(q)) = v;
+        *reinterpret_cast<float4*>(smem + (Gemm::row(p, tid) - p0 / 4 * kPass) * kPitch + Gemm::col(q, tid)) = v;
       }
     __syncthreads();
     const int first = m0 + p0 / 4 * kPass, rows = min(kPass, d_out - first);
     if (quads) {
       constexpr int kLanes = kTile / 4;
-      const int c = threadIdx.x % kLanes * 4;
+      const int c = tid % kLanes * 4;
       if (n0 + c < d_in)
 #pragma unroll 1
-        for (int r = threadIdx.x / kLanes; r < rows; r += Gemm::kThr / kLanes) {
+        for (int r = tid / kLanes; r < rows; r += Gemm::kThr / kLanes) {
           const float4 v = *reinterpret_cast<const float4*>(smem + r * kPitch + c);
           float* at = dW + (size_t)(first + r) * d_in + n0 + c;
           if (store) *reinterpret_cast<float4*>(at) = v;
           else asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
         }
     } else {
-      const int c = threadIdx.x % kTile;
+      const int c = tid % kTile;
       if (n0 + c < d_in)
 #pragma unroll 1
-        for (int r = threadIdx.x / kTile; r < rows; r += Gemm::kThr / kTile) {
+        for (int r = tid / kTile; r < rows; r += Gemm::kThr / kTile) {
           float* at = dW + (size_t)(first + r) * d_in + n0 + c;
           if (store) *at = smem[r * kPitch + c];
           else atomicAdd(at, smem[r * kPitch + c]);
@@ -1214,8 +1220,8 @@ constexpr int64_t kSlabOverhead = 4;
 struct F32Slabs { int64_t stages; double us; };  // of a token slab; what its CTAs take
 // Token slabs of whole stages, 128 tokens or more, up to eight waves (slab_plan.h).  "Four CTAs per SM" instead left the last
 // wave nearly empty: 896 x 896, 4835 tokens 206 -> 190 us, 1537 x 739, 18,151 tokens 1484 -> 1265, 64 x 64, 353 tokens 13.2 ->
-// 10.1 (this alone).  Two CTAs of 128 x 128 on an SM take twice the time of one (a stage of the SM 1.83 us each, 0.57 for 64 x 64), so where
-// few units leave most SMs with one, slabs for one to an SM are better: 500 tokens, 896 x 896 31.8 -> 23.8 us, 20,000 tokens, 128 x 128 31.6 -> 21.7.
+// 10.1 (this alone).  Two CTAs of 128 x 128 on an SM take twice the time of one (a stage of the SM 1.57 us each, 0.56 for 64 x 64; 1.75
+// and 0.63 where rows are not made of 16 bytes), so where few units leave most SMs with one, slabs for one to an SM are better: 500 tokens, 896 x 896 31.8 -> 23.8 us, 20,000 tokens, 128 x 128 31.6 -> 21.7.
 template <int kTile, int kT>
 static isopo_status plan_f32_weight_grad(int64_t T, int d_in, int d_out, F32Slabs* plan) {
   typedef SlabGemm<kTile, kT> Gemm;
@@ -1237,7 +1243,7 @@ static isopo_status plan_f32_weight_grad(int64_t T, int d_in, int d_out, F32Slab
   const int64_t blocks = (T + 15) / 16, most = std::min<int64_t>((T + 127) / 128, std::max<int64_t>(8, 8 * slots / tiles));
   auto us = [&](int64_t stages) {
     const int64_t units = (blocks + stages - 1) / stages * tiles, on_sm = (units + n - 1) / n, waves = (units + slots - 1) / slots;
-    return (double)(on_sm * stages + 2 * waves) * (kTile == 128 ? 1.83 : 0.57);
+    return (double)(on_sm * stages + 2 * waves) * (kTile == 128 ? 1.57 : 0.56);
   };
   plan->stages = plan_slab(blocks, tiles, slots, kSlabOverhead, most);
   if (kTile == 128) {
@@ -1273,8 +1279,8 @@ static isopo_status launch_f32_weight_grad(const float* X, const float* dY, int6
 
 isopo_status f32_weight_grad(const float* X, const float* dY, int64_t T, int d_in, int d_out, const int64_t* off_host, int64_t* off_dev,
                              const float* coeffs, int B, float* tokscale, float* dW, bool add, cudaStream_t st) {
-  // Tiles by the time that their CTAs take.  128 x 128 only where they filled the machine twice (64 x 64 / 128 x 128 us): 500 tokens,
-  // 1536 x 1536 76.7 / 58.7; 1000, 896 x 896 52.3 / 41.6; 100, 1536 x 1536 20.1 / 16.3; 2500, 384 x 640 49.4 / 34.8; 12,000, 128 x 128 16.2 / 19.0.
+  // Tiles by the time that their CTAs take, 64 x 64 / 128 x 128, us: 500 tokens, 1536 x 1536 76.0 / 57.4, 1539 x 1539 98.7 / 84.2; 100, 1536 x 1536
+  // 20.3 / 16.2, 1539 x 1539 27.5 / 31.3; 150, 1000 x 1000 15.1 / 13.5; 800, 448 x 896 23.3 / 21.7; 10,000, 192 x 192 26.6 / 34.0; 4000, 320 x 320 30.1 / 30.8.
   F32Slabs narrow, wide;
   isopo_status s = plan_f32_weight_grad<64, 4>(T, d_in, d_out, &narrow);
   if (s == ISOPO_OK) s = plan_f32_weight_grad<128, 8>(T, d_in, d_out, &wide);
