@@ -233,6 +233,11 @@ inline void launch_cluster(void (*kernel)(Params...), unsigned cluster, dim3 gri
   cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
+// The largest cluster of up to `wanted` (8, 4, 2 or 1) CTAs, each with an SM to itself, that the current context can place: where it has a
+// part of a device, SMs of one group may be too few for it.  Asked at every call, as contexts of a device differ (0.2 us, where a kernel
+// in clusters of more than one is to be launched).
+int placed_cluster(int wanted);
+
 // ---- launchers (each enqueues on `st` and returns a status; none synchronises) ----
 
 // Up to three float32 regions that a launch clears for the kernels behind it (n = 0: none).
@@ -364,7 +369,7 @@ isopo_status bf16_gram_shared(const void* X, int ldx, const void* const* dY, con
 // The stand-alone weight gradients prepare what they need (offsets through off_dev, a cleared dW where its shares are added up);
 // `add`: dW is added to.
 // few tiles: a cluster of `ctas` CTAs shares the features of a tile (1: the kernels above are the better)
-int gram_split_ctas(long long units, int d_in, int d_out, int sms);
+int gram_split_ctas(long long units, int d_in, int d_out, int sms);  // asks placed_cluster
 isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                              const int32_t* tokseq, int B, float* const* K, bool complete, int32_t* info, cudaStream_t st);
 isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,

@@ -1160,13 +1160,13 @@ static GramShape f32_gram_shape(int64_t rows, int64_t cols, bool triangle, int d
   const int stages = (d_in + kGK - 1) / kGK + (d_out + kGK - 1) / kGK;
   GramShape g{32, 1};
   while (g.ctas < 8 && tiles(32) * 2 * g.ctas <= 240 && stages >= 10 * g.ctas) g.ctas *= 2;
-  if (g.ctas > 1) return g;
+  if (g.ctas > 1 && (g.ctas = placed_cluster(g.ctas)) > 1) return g;
   auto per_sm = [](int64_t ctas) { return (double)((ctas + kSms - 1) / kSms); };
   const double k1 = per_sm(tiles(64)), k2 = per_sm(2 * tiles(64));
   const double narrow = stages * std::max(0.48, 0.205 * per_sm(tiles(32)));
   const double wide = stages * (0.12 + 0.52 * k1), split = 0.5 * stages * (0.12 + 0.52 * k2) + 8.0 * k2;
   if (narrow <= wide && narrow <= split) return g;
-  return GramShape{64, wide <= split ? 1 : 2};
+  return GramShape{64, wide <= split ? 1 : placed_cluster(2)};
 }
 template <bool kSampled>
 static isopo_status launch_f32_gram(int id, const GramShape& g, int64_t units, const float* RX, const float* RY, int64_t n_rows, const float* X,

@@ -250,7 +250,34 @@ isopo_status dispatch(int ctas, const CUtensorMap (&maps)[6], const GramSplitPar
   }
 }
 
+template <int kC>
+bool placed() {
+  const auto kernel = &k_bf16_gram_split<false, kC>;  // its CTAs leave no room for another on their SMs
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kC);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = split_smem(kC);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kC;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, split_smem(kC)) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess)
+    return n >= 1;
+  (void)cudaGetLastError();  // an answer, no failure of the call that asks
+  return false;
+}
+
 }  // namespace
+
+int placed_cluster(int wanted) {
+  if (wanted >= 8 && placed<8>()) return 8;
+  if (wanted >= 4 && placed<4>()) return 4;
+  return wanted >= 2 && placed<2>() ? 2 : 1;
+}
 
 // CTAs per tile: 1 where the kernels of tc_gram.cu and tc_gram_shared.cu are the better.  As many as leave a CTA six stages and
 // all clusters resident at one time: clusters of four or eight find fewer than 148 SMs (1000 tokens, 3584 x 8192, 36 tiles: 38.2 us
@@ -261,7 +288,7 @@ int gram_split_ctas(long long units, int d_in, int d_out, int sms) {
   const int stages = (d_in + kKF - 1) / kKF + (d_out + kKF - 1) / kKF;
   int c = 1;
   while (c < 8 && units * 2 * c <= (c == 1 ? sms : sms * 7 / 8) && stages >= 12 * c) c *= 2;
-  return c;
+  return c > 1 ? placed_cluster(c) : 1;
 }
 
 isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,

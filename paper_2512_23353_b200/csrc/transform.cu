@@ -276,27 +276,27 @@ __global__ void __launch_bounds__(kClThreads, 1) k_transform_large(const Transfo
 // Running means for the relative regulariser.  state = {E[F^2], E[||G||^2], E[F^2 / ||G||^2], number of updates};
 // the first update stores this microbatch's means, later ones blend: s <- decay * s + (1 - decay) * mean.
 // One pass: F_i^2 = sum_j K_ij^2 / tr K, so all three means follow from sums of row sums.
-// A cluster shares the rows (four to a warp at a time) and its first CTA adds up.  Bound by latency: 156 sequences 7.4 -> 4.9 us against
+// The grid is one cluster, which shares the rows (four to a warp at a time), and its first CTA adds up.  Bound by latency: 156 sequences 7.4 -> 4.9 us against
 // one CTA of 1024 threads, 255 9.1 -> 6.4, 1024 49.8 -> 20.2; up to 100 sequences 4.9 either way (the call's host time).
 constexpr int kEmaThreads = 256;
 constexpr int kEmaCluster = 8;
-__global__ void __cluster_dims__(kEmaCluster, 1, 1) __launch_bounds__(kEmaThreads)
+__global__ void __launch_bounds__(kEmaThreads)
 k_reg_ema(const float* __restrict__ K, int B, float decay, float* __restrict__ state) {
   pdl_begin();
   constexpr int kWarps = kEmaThreads / 32;
   __shared__ double s_part[kEmaCluster * kWarps][3];  // first CTA: of every warp of the cluster
   const int tid = threadIdx.x, lane = tid & 31, rank = (int)tc::cluster_ctarank(), warp = rank * kWarps + (tid >> 5);
-  constexpr int kStep = kEmaCluster * kWarps * 4;
+  const int ctas = gridDim.x, step = ctas * kWarps * 4;
   double tr = 0.0, f2 = 0.0, rel = 0.0;
-  for (int i = rank * kEmaThreads + tid; i < B; i += kEmaCluster * kEmaThreads) tr += (double)__ldg(K + (size_t)i * B + i);
+  for (int i = rank * kEmaThreads + tid; i < B; i += ctas * kEmaThreads) tr += (double)__ldg(K + (size_t)i * B + i);
   auto add = [&](int i, double sq) {
     f2 += sq;
     rel += sq / (double)__ldg(K + (size_t)i * B + i);
   };
   if (rows_in_float4(K, B))  // outside the row loop: inside it 1024 sequences took 72 us instead of 53 in one CTA
-    for (int i0 = warp * 4; i0 < B; i0 += kStep) row_square_sums<true>(K, B, i0, min(B, i0 + 4), add);
+    for (int i0 = warp * 4; i0 < B; i0 += step) row_square_sums<true>(K, B, i0, min(B, i0 + 4), add);
   else
-    for (int i0 = warp * 4; i0 < B; i0 += kStep) row_square_sums<false>(K, B, i0, min(B, i0 + 4), add);
+    for (int i0 = warp * 4; i0 < B; i0 += step) row_square_sums<false>(K, B, i0, min(B, i0 + 4), add);
   tr = warp_sum(tr);
   cl_arrive();
   cl_wait();  // the first CTA runs
@@ -310,7 +310,7 @@ k_reg_ema(const float* __restrict__ K, int B, float decay, float* __restrict__ s
   if (rank != 0 || tid >= 32) return;
   double sum[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) sum[k] = warp_sum(s_part[lane][k] + s_part[lane + 32][k]);
+  for (int k = 0; k < 3; ++k) sum[k] = warp_sum((lane < ctas * kWarps ? s_part[lane][k] : 0.0) + (lane + 32 < ctas * kWarps ? s_part[lane + 32][k] : 0.0));
   static_assert(kEmaCluster * kWarps == 64, "two partial sums to a lane");
   const double trace = sum[0];
   if (lane == 0) {
@@ -325,9 +325,10 @@ k_reg_ema(const float* __restrict__ K, int B, float decay, float* __restrict__ s
 }  // namespace
 
 isopo_status reg_ema_update(const float* K, int B, float decay, float* state, cudaStream_t st) {
+  const unsigned ctas = B <= 4 * kEmaThreads / 32 ? 1 : (unsigned)placed_cluster(kEmaCluster);  // one has a row for every warp
   {
     LaunchScope scope(kIdTransform, st);
-    launch(k_reg_ema, kEmaCluster, kEmaThreads, 0, st, K, B, decay, state);
+    launch_cluster(k_reg_ema, ctas, ctas, kEmaThreads, 0, st, K, B, decay, state);
   }
   ISOPO_CUDA_TRY(cudaGetLastError());
   return ISOPO_OK;
