@@ -115,8 +115,8 @@ ISOPO_API isopo_path isopo_choose_path(isopo_dtype dtype, int64_t T, int d_in, i
  * in a piece-blocked order private to the library; on the bf16 Gram path, the per-token-scaled
  * copy of the narrower of X and dY that isopo_weight_grad feeds to its GEMM
  * (2 * T * min(d_in, d_out) bytes).  With widths that are no multiple of 64, or fewer tokens than B * B, bf16 asks for more,
- * which only makes the kernels faster (copies of X and dY, and that copy, at rows of whole 128-byte lines; rows for the sums
- * of K): a workspace without it is accepted.  It must be 1024-byte aligned (cudaMalloc promises 256 bytes only: allocate
+ * which only makes the kernels faster (copies of X and dY, up to 2 GiB of them, and that copy, at rows of whole 128-byte lines;
+ * rows for the sums of K): a workspace without it, or with a part of it, is accepted.  It must be 1024-byte aligned (cudaMalloc promises 256 bytes only: allocate
  * 1024 bytes more and round the pointer up).  Returns 0 for invalid sizes.
  */
 ISOPO_API size_t isopo_workspace_bytes(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path path);

@@ -82,6 +82,15 @@ ProfilingPause::~ProfilingPause() { g_prof_on = was_on_; }
 // 1919, 1080 x 312 17.6 / 14.8; 5000, 2136 x 968 70 / 64; 15,000, 1080 x 312 238 / 204; 40,000, 232 x 600 1184 / 885.
 static bool repitch_pays(int64_t T, int B) { return T >= 1000 && B + 1 <= kArgLarge; }
 static size_t repitch_bytes(int64_t T, int d) { return d % 64 ? align_up((size_t)2 * (size_t)T * (size_t)line_pitch(d), 1024) : 0; }
+// What is asked for to hold them: X's and dY's, each unless it takes the two past 2 GiB.  (300,000 tokens of 8200 x 72, which need 0.04 GB
+// without copies, asked for 5.0; now 0.08.)  They pay for lopsided layers too: in place / copied, 30,000 tokens, 8200 x 72 (0.5 GB) 8.4 /
+// 6.5 ms, 1000 x 8200 9.6 / 7.1; 3000, 8200 x 72 148 / 94 us.
+constexpr size_t kRepitchMost = (size_t)2 << 30;
+static size_t repitch_room(int64_t T, int d_in, int d_out, int B) {
+  if (!repitch_pays(T, B)) return 0;
+  const size_t x = repitch_bytes(T, d_in), y = repitch_bytes(T, d_out), first = x <= kRepitchMost ? x : 0;
+  return first + y <= kRepitchMost ? first + y : first;
+}
 struct GramOperands {
   const void* X;
   const void* dY[3];
@@ -138,11 +147,12 @@ WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, iso
   L.off_scaled = p;
   L.scaled_ld = std::min(d_in, d_out);
   if (dtype == ISOPO_BF16 && resolved == ISOPO_PATH_GRAM) {
-    const int lines = line_pitch(L.scaled_ld);
-    const size_t copies = repitch_pays(T, B) ? repitch_bytes(T, d_in) + repitch_bytes(T, d_out) : 0;
-    const size_t full = align_up(p + std::max((size_t)2 * (size_t)T * (size_t)lines, copies), 1024);
-    if (have >= full) L.scaled_ld = lines;
-    p = have >= full ? full : align_up(p + (size_t)2 * (size_t)T * (size_t)L.scaled_ld, 1024);
+    auto scaled = [&](int ld) { return align_up((size_t)2 * (size_t)T * (size_t)ld, 1024); };
+    const size_t bare = scaled(L.scaled_ld), lines = scaled(line_pitch(L.scaled_ld));
+    const size_t left = have < p + bare ? bare : (have - p) / 1024 * 1024;
+    const size_t room = std::min(left, std::max(lines, repitch_room(T, d_in, d_out, B)));  // as much of it as there is
+    if (room >= lines) L.scaled_ld = line_pitch(L.scaled_ld);
+    p += room;
   }
   L.off_G = p;
   if (dtype == ISOPO_BF16) {

@@ -160,8 +160,9 @@ struct WsLayout {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// In a workspace of `have` bytes: the areas that only make the kernels faster are left out where they do not fit (layout.total is then what
-// the others need), so that a workspace of 2 T min(d_in, d_out) bytes of scaled operand, or with no sums of the K pass, still serves.
+// In a workspace of `have` bytes: the areas that only make the kernels faster are left out, or hold fewer copies, where they do not fit
+// (layout.total is then at most `have`, or what the others need), so that a workspace of 2 T min(d_in, d_out) bytes of scaled operand, or
+// with no sums of the K pass, still serves.
 WsLayout ws_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, isopo_path resolved, size_t have = SIZE_MAX);
 
 // Workspace of isopo_sampled_coefficients: the Gram-route prefix (offsets, token map), then

@@ -134,11 +134,13 @@ isopo_status gather_samples(const T* X, const T* dY, int d_in, int d_out, const 
 
 SampledLayout sampled_layout(isopo_dtype dtype, int64_t T, int d_in, int d_out, int B, int n_samples, size_t have) {
   const size_t elt = dtype == ISOPO_BF16 ? 2 : 4;
+  const WsLayout L = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM, 0);  // offsets, token map (+ kacc), scaled operand
   auto lay = [&](bool lines) {
     SampledLayout S{};
     S.lda = lines ? line_pitch(d_in) : d_in;
     S.ldg = lines ? line_pitch(d_out) : d_out;
-    size_t p = ws_layout(dtype, T, d_in, d_out, B, ISOPO_PATH_GRAM, lines ? SIZE_MAX : 0).total;  // offsets, token map (+ kacc)
+    // the scaled operand of the weight gradient behind it at lines as well; no copies of X and dY, which are read in place
+    size_t p = lines ? L.off_scaled + align_up((size_t)2 * (size_t)T * (size_t)line_pitch(std::min(d_in, d_out)), 1024) : L.total;
     S.off_a0 = p;
     p = align_up(p + elt * (size_t)n_samples * S.lda, 1024);
     S.off_g0 = p;

@@ -72,6 +72,25 @@ def test_workspace_bytes(binding):
     assert f32 >= 4 * 8 * 64 * 64
 
 
+def test_workspace_bytes_of_lopsided_layers(binding):
+    """Copies of the Gram route's operands at whole lines are asked for up to 2 GiB, and not at all by the sampled estimator, which reads
+    its operands in place."""
+    b = binding
+    T, B = 300000, 300
+    other = 1024 + 8 * (B + 1) + 1024 + 4 * T + 1024  # offsets and token map
+    up = lambda n: -(-n // 1024) * 1024  # noqa: E731
+    for d_in, d_out, copies in [(8200, 72, 2 * T * 128), (72, 8200, 2 * T * 128),      # the wide operand's would be 4.9 GB
+                                (1000, 8200, 2 * T * 1024), (8200, 8192, 0), (2000, 1000, 2 * T * (2048 + 1024))]:
+        gram = b.isopo_workspace_bytes(b.BF16, T, d_in, d_out, B, b.PATH_GRAM)
+        scaled = 2 * T * (-(-min(d_in, d_out) // 64) * 64)
+        assert abs(gram - other - max(copies, scaled)) < 8192
+        assert copies <= 2 << 30
+        n = 128
+        sampled = b.isopo_sampled_workspace_bytes(b.BF16, T, d_in, d_out, B, n)
+        rows = up(2 * n * (-(-d_in // 64) * 64)) + up(2 * n * (-(-d_out // 64) * 64)) + up(4 * n * B)
+        assert abs(sampled - other - scaled - rows) < 8192
+
+
 def test_argument_validation_happens_on_the_host(binding):
     """Bad arguments are rejected before any CUDA call, so this runs without a GPU."""
     b = binding

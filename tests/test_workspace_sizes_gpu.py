@@ -43,15 +43,20 @@ def test_least_workspace(b, Ls, d_in, d_out, stored):
     full = b.isopo_workspace_bytes(b.BF16, T, d_in, d_out, B, path)
     assert full > least or T >= B * B
     got = []
-    for n in (full, least):
+    between = [least + 1024 + 1000, (least + full) // 2 + 1, full - 1] if full > least + 4096 else []  # fewer copies, or none
+    for n in (full, least, *between):
         K, dW, info = torch.empty((B, B), device="cuda"), torch.empty((d_out, d_in), device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
-        ws = _ws(n)
+        raw = _ws(n + 4096)
+        raw[n:] = 77
+        ws = raw[:n]
         b.isopo_layer_gram(X, dY, off, K, ws, info, path)
         b.isopo_weight_grad(X, dY, c, off, dW, ws, info, path)
         torch.cuda.synchronize()
         assert int(info.item()) == 0
+        assert (raw[n:] == 77).all()  # nothing behind it is written
         got.append((K, dW))
-    assert _rel(got[1][0], got[0][0]) <= 2e-6 and _rel(got[1][1], got[0][1]) <= 2.0 ** -8
+    for K, dW in got[1:]:
+        assert _rel(K, got[0][0]) <= 2e-6 and _rel(dW, got[0][1]) <= 2.0 ** -8
     with pytest.raises(Exception):
         b.isopo_layer_gram(X, dY, off, K, _ws(least - 1024), info, path)
     with pytest.raises(Exception):
