@@ -57,12 +57,11 @@ def test_gram(b, T, B, d_in, d_outs):
         assert ((K.double() - want).norm() / want.norm()).item() <= TOL
         assert torch.equal(K, K.T)
     assert all(torch.equal(a, t) for a, t in zip(before, [X, *dYs]))
-    # the scaled operand of the weight gradient lies at such a pitch too
-    c = torch.randn(B, device="cuda")
-    dW = torch.full((d_outs[0], d_in), float("nan"), device="cuda")
-    b.isopo_weight_grad(X, dYs[0], c, off, dW, ws[0], info, b.PATH_GRAM, 0.0)
+    # the scaled operand of the weight gradient lies at such a pitch too: whole numbers small enough for every step to be exact
+    X, dY, c = (torch.randint(-n, n + 1, shape, device="cuda") for n, shape in [(1, X.shape), (1, dYs[0].shape), (8, (B,))])
     rows = c[torch.from_numpy(np.repeat(np.arange(B), np.diff(off))).cuda()][:, None]
-    want = (rows.double() * dYs[0].double()).T @ X.double()
-    # the scaled operand is rounded to bf16, by at most 2^-8 (half of its eighth bit) of each product, however they cancel; float32 sums beside it
-    bound = (rows.double() * dYs[0].double()).abs().T @ X.double().abs()
-    assert ((dW.double() - want).abs() <= (2.0 ** -8 + 1e-5) * bound).all()
+    want = (rows.double() * dY.double()).T @ X.double()
+    for beta in (0.0, 1.0):
+        dW = torch.full((d_outs[0], d_in), 500.0 if beta else float("nan"), device="cuda")
+        b.isopo_weight_grad(X.bfloat16(), dY.bfloat16(), c.float(), off, dW, ws[0], info, b.PATH_GRAM, beta)
+        assert torch.equal(dW.double(), want + 500.0 * beta)

@@ -48,8 +48,8 @@ def _run(b, X, dY, c, off, dW, beta):
     ([1], 2304, 2560),                 # one token, more tiles than pairs
     ([3, 60, 1], 2056, 4104),          # one stage exactly; widths 8 past the tile grid
     ([20, 45], 4104, 2056),            # a second stage of one token
-    ([5] * 100, 3072, 6144),           # eight stages; more than 2^24 elements: beta = 1 by loads and stores
-    ([7] * 80, 3072, 6144),            # nine stages: beta = 1 by additions
+    ([5] * 100, 3072, 6144),           # eight stages, as many as writing a tile takes; more than 2^24 elements
+    ([7] * 80, 3072, 6144),            # nine stages
     ([30, 30], 896, 256),              # two tiles of one stage
     ([33, 7, 1], 1000, 328),           # one row of CTAs, no pairs
     ([9] * 30, 200, 72),               # one CTA
@@ -79,17 +79,19 @@ def test_written_tiles(b, Ls, d_in, d_out, shift):
     ([15] * 1000, 4096, 104),    # one row of a wide layer
 ])
 def test_few_rows_of_tiles(b, Ls, d_in, d_out):
+    """Whole numbers small enough for every step of every kernel to be exact (a scaled operand of at most 8, float32 sums below 2^24): dW
+    has to be what float64 gives, to the bit, whether the coefficient is applied to an operand or at the drain."""
     gen = torch.Generator(device="cuda")
     gen.manual_seed(d_in + len(Ls))
     off = np.concatenate([[0], np.cumsum(Ls)]).astype(np.int64)
-    X = torch.randn((int(off[-1]), d_in), device="cuda", generator=gen).bfloat16()
-    dY = torch.randn((int(off[-1]), d_out), device="cuda", generator=gen).bfloat16()
-    c = torch.randn(len(Ls), device="cuda", generator=gen)
+    draw = lambda n, *shape: torch.randint(-n, n + 1, shape, device="cuda", generator=gen)  # noqa: E731
+    X, dY, c = draw(1, int(off[-1]), d_in).bfloat16(), draw(1, int(off[-1]), d_out).bfloat16(), draw(8, len(Ls)).float()
     rows = c[torch.from_numpy(np.repeat(np.arange(len(Ls)), Ls)).cuda()][:, None]
     want = (rows.double() * dY.double()).T @ X.double()
-    for beta in (0.0, 1.0):
-        dW = torch.full((d_out, d_in), 0.5, device="cuda")
-        _run(b, X, dY, c, off, dW, beta)
-        # the scaled operand is rounded to bf16, by at most 2^-8 (half of its eighth bit) of each product, however they cancel; float32 sums beside it
-        bound = (rows.double() * dY.double()).abs().T @ X.double().abs() + beta * 0.5
-        assert ((dW.double() - beta * 0.5 - want).abs() <= (2.0 ** -8 + 1e-5) * bound).all()
+    dW = torch.full((d_out, d_in), float("nan"), device="cuda")
+    _run(b, X, dY, c, off, dW, 0.0)
+    assert torch.equal(dW.double(), want)
+    before = draw(1 << 12, d_out, d_in).float()
+    dW.copy_(before)
+    _run(b, X, dY, c, off, dW, 1.0)
+    assert torch.equal(dW.double(), before.double() + want)
