@@ -331,9 +331,10 @@ ISOPO_API isopo_status isopo_transform_spectral_batched(int n_layers, const floa
  * GRAM: one GEMM over all tokens, dW = (coeffs[seq(t)] * dY)^T X.  bf16, layers whose wider side is
  * at most 2048 (and sequences of about 100 tokens or more): every run of tokens of one sequence is
  * accumulated on its own in tensor memory and multiplied by its coefficient when the accumulator
- * is drained, so no operand is rounded a second time.  Wider bf16 layers: the per-token scale is
+ * is drained, so no operand is rounded a second time.  Other bf16 layers: the per-token scale is
  * applied to the narrower operand (rounded to nearest even in bf16) in one pass before a plain
- * GEMM, or, for layers with few rows, to the rows as they land in shared memory.
+ * GEMM.  bf16 layers of an odd number of 128-row tiles below seven (d_out up to 128, 257 to 384, 513
+ * to 640) with few tokens, or of one such tile and not very wide: to the rows as they land in shared memory.
  *
  *   coeffs  dev, float32 [B]
  *   dW      dev, float32 [d_out, d_in] row-major (the layout of `grad_out.T @ act_in`); 16-byte

@@ -367,14 +367,14 @@ isopo_status bf16_gram_pair(const void* X, int ldx, const void* const* dY, const
                             const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
 isopo_status bf16_gram_shared(const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                               const int32_t* tokseq, int B, float* const* K, int32_t* info, cudaStream_t st);
-// The stand-alone weight gradients prepare what they need (offsets through off_dev, a cleared dW where its shares are added up);
-// `add`: dW is added to.
 // few tiles: a cluster of `ctas` CTAs shares the features of a tile (1: the kernels above are the better)
 int gram_split_ctas(long long units, int d_in, int d_out, int sms);  // asks placed_cluster
 isopo_status bf16_gram_split(int ctas, const void* X, int ldx, const void* const* dY, const int* ldy, int64_t T, int d_in, const int* d_out, int n_heads,
                              const int32_t* tokseq, int B, float* const* K, bool complete, int32_t* info, cudaStream_t st);
 isopo_status bf16_sampled_split(int ctas, const void* X, const void* dY, int64_t T, int d_in, int d_out, const int32_t* tokseq, int B,
                                 const void* A0, int lda, const void* G0, int ldg, int n_samples, float* Mt, int32_t* info, cudaStream_t st);
+// The stand-alone weight gradients prepare what they need (offsets through off_dev, a cleared dW where its shares are added up);
+// `add`: dW is added to.
 // 1-CTA tiles, operand rows scaled in shared memory by the scales per token that a launch ahead leaves in `tokscale`
 isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                               int64_t* off_dev, const float* coeffs, int B, float* tokscale, float* dW, bool add, int32_t* info,
@@ -386,7 +386,7 @@ bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B);
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                                    int64_t* off_dev, const float* coeffs, int B, float* dW, bool add, int32_t* info, cudaStream_t st);
 // a scaled copy of the narrower operand, then a plain GEMM in 2-CTA tiles
-// (the offsets travel with the scaling pass, through off_dev above 383 sequences)
+// (the offsets travel with the scaling pass, through off_dev above 2047 sequences)
 isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                                    int64_t* off_dev, const float* coeffs, int B, void* scaled, int scaled_ld, float* dW, bool add,
                                    int32_t* info, cudaStream_t st);

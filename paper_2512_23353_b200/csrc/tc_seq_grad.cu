@@ -51,7 +51,6 @@ struct SeqGradParams {
   int32_t* info;
   // folded weight-gradient GEMM only
   const float* tokscale;  // coefficient of every token's sequence
-  float* dW;
   int64_t T, slab;  // tokens per work unit (a multiple of 64)
   int nslabs, d_in, d_out;
   bool store;       // one slab: dW is written, nothing has cleared it
@@ -259,8 +258,7 @@ k_bf16_seq_grad(const __grid_constant__ CUtensorMap mapY, const __grid_constant_
         }
       } else {
         // dW[m .. m+31, n0 .. n0+255] += the warp's rows; token slabs of one tile meet here, hence additions.  By TMA, 32 rows of 128
-        // bytes at a time, not red.v4: 4000 tokens, 512 x 1000 16.8 -> 13.6 us, 1586, 1000 x 328 13.3 -> 12.0, 15,000, 1848 x 88 23.6 ->
-        // 22.8; 46,546, 256 x 592, 59 slabs to a tile, 39.0 -> 40.6.
+        // bytes at a time, not red.v4: 1586 tokens, 1000 x 328 13.3 -> 12.0 us, 15,000, 1848 x 88 23.6 -> 22.8.
         const int m = (tile / p.tiles_n) * kTileM + q * 32, n0 = (tile % p.tiles_n) * kTileN;
 #pragma unroll 2
         for (int jc = 0; jc < kTileN / 32 && n0 + jc * 32 < p.d_in; ++jc) {
@@ -400,7 +398,7 @@ isopo_status bf16_weight_grad(const void* X, const void* dY, int64_t T, int d_in
   SeqGradParams p{};
   p.tiles_m = (d_out + kTileM - 1) / kTileM;
   p.tiles_n = (d_in + kTileN - 1) / kTileN;
-  p.info = info; p.tokscale = tokscale; p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out;
+  p.info = info; p.tokscale = tokscale; p.T = T; p.d_in = d_in; p.d_out = d_out;
   // Token slabs of whole stages, 64 at most, or two rounds of (tile, slab) units while a slab has eight stages: a unit spends
   // about 16 stages' worth on filling its pipeline and on adding its tile into dW, more the more units meet in a tile (16,000
   // tokens, 256 x 128: 64 slabs 15.8 us, 125 slabs 18.6).  With 64 slabs whatever the tokens a layer of one tile had 64 CTAs:

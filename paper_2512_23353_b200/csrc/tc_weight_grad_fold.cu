@@ -62,7 +62,6 @@ static_assert(kSmemBytes<true> <= 227 * 1024 && kSmemBytes<false> <= 227 * 1024,
 struct FoldParams {
   const int64_t* off;    // [B + 1] token offsets
   const float* coeffs;   // [B]
-  float* dW;
   int64_t T, chunk;      // tokens per work unit (a multiple of kKB)
   int nchunks, B, d_in, d_out;
   int ptiles_m, tiles_n;  // 256-row and 256-column tiles of dW
@@ -449,27 +448,26 @@ bool bf16_weight_grad_fold_applies(int64_t T, int d_in, int d_out, int B) {
          T < ((int64_t)1 << 31) - 4096;
 }
 
-// Pairs of CTAs that can be resident at once.
-template <bool kPlain>
+// Pairs of CTAs of the kernel with segments that can be resident at once.
 static isopo_status resident_pairs(int* pairs) {
   int dev = 0, sms = 0;
   ISOPO_CUDA_TRY(cudaGetDevice(&dev));
   ISOPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<kPlain>));
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<false>));
   static int resident[64] = {};
   if (dev < 0 || dev >= 64) return ISOPO_ERR_UNSUPPORTED;
   if (resident[dev] == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)(sms / 2));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes<kPlain>;
+    cfg.dynamicSmemBytes = kSmemBytes<false>;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    ISOPO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, k_bf16_weight_grad_fold<kPlain>, &cfg));
+    ISOPO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, k_bf16_weight_grad_fold<false>, &cfg));
     if (n < 1) return ISOPO_ERR_UNSUPPORTED;
     resident[dev] = std::min(n, sms / 2);
   }
@@ -511,13 +509,12 @@ PlainPlan plan_weight_grad_plain(int64_t T, int d_in, int d_out, bool add, int p
 
 isopo_status bf16_weight_grad_plain(const void* X, int ldx, const void* dY, int ldy, int64_t T, int d_in, int d_out, const PlainPlan& plan, bool add,
                                     float* dW, int32_t* info, cudaStream_t st) {
-  int pairs = 0;
-  isopo_status s = resident_pairs<true>(&pairs);
-  if (s != ISOPO_OK) return s;
+  ISOPO_CUDA_TRY(cudaFuncSetAttribute(k_bf16_weight_grad_fold<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<true>));
+  isopo_status s;
   CUtensorMap mapY, mapX, mapW;
   if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, ldx, dY, ldy, dW, T, d_in, d_out, 32)) != ISOPO_OK) return s;
   FoldParams p{};
-  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add;
+  p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info; p.beta = add;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
   p.tiles_n = (d_in + kPairN - 1) / kPairN;
   p.kblocks = (int)((T + kKB - 1) / kKB);
@@ -536,12 +533,12 @@ isopo_status bf16_weight_grad_plain(const void* X, int ldx, const void* dY, int 
 isopo_status bf16_weight_grad_fold(const void* X, const void* dY, int64_t T, int d_in, int d_out, const int64_t* off_host,
                                    int64_t* off_dev, const float* coeffs, int B, float* dW, bool add, int32_t* info, cudaStream_t st) {
   int pairs = 0;
-  isopo_status s = resident_pairs<false>(&pairs);
+  isopo_status s = resident_pairs(&pairs);
   if (s != ISOPO_OK) return s;
   CUtensorMap mapY, mapX, mapW;
   if ((s = make_fold_maps(&mapY, &mapX, &mapW, X, d_in, dY, d_out, dW, T, d_in, d_out, 16)) != ISOPO_OK) return s;
   FoldParams p{};
-  p.off = off_dev; p.coeffs = coeffs; p.dW = dW; p.T = T; p.B = B; p.d_in = d_in; p.d_out = d_out; p.info = info;
+  p.off = off_dev; p.coeffs = coeffs; p.T = T; p.B = B; p.d_in = d_in; p.d_out = d_out; p.info = info;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
   p.tiles_n = (d_in + kPairN - 1) / kPairN;
   // token chunks: the count (up to 64) whose rounds of units take least, a round costing its chunk plus the

@@ -49,7 +49,6 @@ constexpr int kUnitOverhead = 16;  // a unit's epilogue and pipeline fill, in 64
 static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 
 struct FoldedPairParams {
-  float* dW;
   int64_t T, slab;  // tokens per work unit (a multiple of kKB)
   int nslabs, d_in, d_out;
   int ptiles_m, tiles_n;  // 256-row blocks of d_out; 512-column blocks of d_in
@@ -306,7 +305,7 @@ isopo_status bf16_weight_grad_pair(const void* X, const void* dY, int64_t T, int
     resident_pairs[dev] = std::min(n, sms / 2);
   }
   FoldedPairParams p{};
-  p.dW = dW; p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info;
+  p.T = T; p.d_in = d_in; p.d_out = d_out; p.info = info;
   p.ptiles_m = ((d_out + kHalf - 1) / kHalf + 1) / 2;
   p.tiles_n = (d_in + 2 * kPairN - 1) / (2 * kPairN);
   // token slabs: the count (up to 64) whose rounds of units take least, a round costing its slab plus the
