@@ -894,7 +894,10 @@ __global__ void __launch_bounds__(128, kGT == 64 ? 3 : kC == 1 ? 7 : 2) k_f32_gr
       run = 0.0;
     }
   }
-  if (kC > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // nobody leaves while its sums may still be read
+  if (kC > 1) {
+    __syncwarp();  // the barrier wants the warp together
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // nobody leaves while its sums may still be read
+  }
 }
 
 __global__ void k_f32_gram_finish(const double* __restrict__ kacc, int B, float* __restrict__ K) {

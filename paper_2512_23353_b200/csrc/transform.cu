@@ -305,6 +305,7 @@ k_reg_ema(const float* __restrict__ K, int B, float decay, float* __restrict__ s
 #pragma unroll
     for (int k = 0; k < 3; ++k) st_cluster_f64(tc::map_to_cta(tc::smem_u32(&s_part[warp][k]), 0), part[k]);
   }
+  __syncwarp();  // the barrier wants the warp together
   cl_arrive();
   cl_wait();
   if (rank != 0 || tid >= 32) return;
