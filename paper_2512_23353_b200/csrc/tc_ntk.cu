@@ -45,7 +45,6 @@ struct NtkParams {
   int32_t* info;
   int box_rows;   // rows of a piece inside a box: 4, 8, .. 256, >= B
   int ppb;        // pieces per box = 256 / box_rows
-  bool by_boxes;  // added by TMA into rows of a pitch that it can take, not into K
   // not NULL (up to 16 sequences, 32 with little data): the last CTA to add its share completes the other triangle and the
   // diagonal of the split store
   uint32_t* done;
@@ -55,7 +54,10 @@ struct NtkParams {
 
 // kE4m3: the operand is the `hi` plane of the split store: 128 one-byte elements per 128-byte box row (two boxes
 // per piece instead of four), kind::f8f6f4 MMAs of 32 elements each - the same number of MMAs per byte, half the bytes.
-template <bool kE4m3>
+// The end of it, by kSums: kFew (boxes of fewer than 32 rows) and kRows add into K or store partial sums, kBoxes adds boxes by TMA.  Each a
+// kernel of its own, as their code is fetched anew in every launch and runs once.
+enum NtkSums { kFew, kRows, kBoxes };
+template <bool kE4m3, NtkSums kSums>
 __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ CUtensorMap mapK, NtkParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
         asm volatile("bar.sync 2, 128;" ::: "memory");
       }
       auto unscale = [&](int row, int col, float v) { return kE4m3 ? v * inv_s[row] * inv_s[col] : v; };
-      if (p.by_boxes) {
+      if (kSums == kBoxes) {
         // Blocks of 32 columns c of the warp's 32 accumulator rows go through shared memory (the ring is idle by now), turned over so
         // that box row c holds K[c][r .. r + 31], and are added by TMA into the rows of p.acc; what the diagonal blocks have
         // above the diagonal is not read from there.  A CTA starts at a block of its own: 148 of them on one sector wait for one another.
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
         };
         tc_fence_after_sync();
         const uint32_t tlane = (uint32_t)(q * 32) << 16;
-        if (two && ok) {
+        if (kSums == kRows && two && ok) {
           // block A: rows 0..127 x columns 0..255 of K; keep the upper triangle c >= r
           for (int c0 = 0; c0 < n1; c0 += 32) {
             uint32_t v[32];
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
           const int lr = 31 - __clz(p.box_rows), rows = 1 << lr;  // box_rows is a power of two
           const int seq = r & (rows - 1), g = r >> lr, ngroups = 128 >> lr;
           // the columns that a warp reads are the same for its lanes: of fewer than 32 sequences the whole block on its diagonal
-          const int coff = rows >= 32 ? r - seq : q * 32, mine = rows >= 32 ? 0 : lane & ~(rows - 1);
+          const int coff = (q * 32) & ~(rows - 1), mine = lane & ~(rows - 1);
           const int ncol = min(rows, p.B);
           float* red = reinterpret_cast<float*>(smem);  // [group][column][sequence]
           if (ok) {
@@ -289,10 +291,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_bf16_ntk(const __grid_constant_
               tmem_ld32(tmem_base + tlane + 256 + coff + c0, v1);
               tmem_ld_wait();
               float* dst = red + ((((g << lr) + c0) << lr) + seq);
+              if (kSums == kRows) {
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                const int c = e - mine;
-                if (c >= 0 && c < rows) dst[c << lr] = __uint_as_float(v0[e]) + __uint_as_float(v1[e]);
+                for (int e = 0; e < 32; ++e) dst[e << lr] = __uint_as_float(v0[e]) + __uint_as_float(v1[e]);
+              } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                  const int c = e - mine;
+                  if (c >= 0 && c < rows) dst[c << lr] = __uint_as_float(v0[e]) + __uint_as_float(v1[e]);
+                }
               }
             }
           }
@@ -588,9 +595,9 @@ isopo_status plan_ntk(const WsLayout& L, int B, bool split, bool deterministic, 
   plan->ppb = 256 / plan->box_rows;
   // boxes along the contraction: four per piece group of bf16 (64 elements a row), two of e4m3 (128 elements a row)
   plan->nkb = (L.n_pad / kPieceElems + plan->ppb - 1) / plan->ppb * (split ? 2 : 4);
-  // Four boxes of a CTA pay for its start, eight above 32 sequences: half of the CTAs are half of the additions to an entry of K (896 x 128,
-  // 64 sequences: error 1.0e-7 with 56 of them, 1.4e-7 with 112; isopo_layer_gram 15.4 / 14.3 us).
-  plan->grid = (int)std::max<long long>(1, std::min<long long>(sms, plan->nkb / (B > kNtkSmemSums ? 8 : 4)));
+  // Four boxes of a CTA pay for its start, eight above 16 sequences: half of the CTAs are half of the additions to an entry of K (896 x 128,
+  // 64 sequences: error 1.0e-7 with 56 of them, 1.4e-7 with 112, isopo_layer_gram 15.3 / 14.3 us; 512 x 512, 32: 1.2e-7 / 1.6e-7, 17.5 / 17.3).
+  plan->grid = (int)std::max<long long>(1, std::min<long long>(sms, plan->nkb / (B > 16 ? 8 : 4)));
   if (deterministic) plan->grid = std::min(plan->grid, kNtkMaxPartials);
   // CTAs whose slab of the contraction is empty take no part
   const long long per = (plan->nkb + plan->grid - 1) / plan->grid;
@@ -620,9 +627,11 @@ isopo_status bf16_ntk(const NtkPlan& plan, const void* G, const WsLayout& L, int
   } else {
     mapK = mapG;
   }
-  auto kernel = fmt.split ? k_bf16_ntk<true> : k_bf16_ntk<false>;
+  auto kernel = plan.by_boxes ? (fmt.split ? k_bf16_ntk<true, kBoxes> : k_bf16_ntk<false, kBoxes>)
+                : rows < 32   ? (fmt.split ? k_bf16_ntk<true, kFew> : k_bf16_ntk<false, kFew>)
+                              : (fmt.split ? k_bf16_ntk<true, kRows> : k_bf16_ntk<false, kRows>);
   ISOPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, plan.nkb, info, plan.box_rows, plan.ppb, plan.by_boxes,
+  NtkParams p{kpart, fmt.split ? fmt.scales : nullptr, K, B, plan.nkb, info, plan.box_rows, plan.ppb,
               plan.by_last ? &head->done : nullptr, (uint32_t)plan.n_active, fmt.kdiag};
   {
     LaunchScope scope(kIdNtk, st);

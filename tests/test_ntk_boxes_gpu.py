@@ -61,7 +61,8 @@ def test_exact_shared_input(b, B):
 
 
 @pytest.mark.parametrize("B,d_in,d_out,n", [(40, 512, 640, 148), (64, 512, 640, 148), (100, 512, 320, 148), (128, 512, 320, 148),
-                                            (160, 512, 160, 148), (256, 512, 160, 148), (64, 896, 128, 56), (100, 896, 128, 112)])
+                                            (160, 512, 160, 148), (256, 512, 160, 148), (64, 896, 128, 56), (100, 896, 128, 112),
+                                            (20, 512, 512, 64), (32, 512, 512, 64)])
 def test_one_addition_per_cta(b, B, d_in, d_out, n):
     """K of gradients of one sign, exact in bf16, is a sum of up to n positive float32 additions, one per CTA of eight boxes or more.
     Rounding an addition to S errs by ulp(S) / sqrt(12), ulp(S)^2 is 0.54 * 2^-46 S^2 in the mean, and S grows evenly: n additions leave
